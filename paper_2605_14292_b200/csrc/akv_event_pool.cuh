@@ -59,8 +59,9 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
     int* pool_holder = reinterpret_cast<int*>(smem + sp.misc + 20);
     int* pick_holder = reinterpret_cast<int*>(smem + sp.misc + 24);
     int* redi = reinterpret_cast<int*>(smem + sp.misc + 32);
-    uint32_t* bound_holder = reinterpret_cast<uint32_t*>(smem + sp.misc + 28);  // large size: key no left-out candidate exceeds
-    float* thr_holder = reinterpret_cast<float*>(smem + sp.misc + 56);          // large size: the pool's score threshold
+    uint32_t* bound_holder = reinterpret_cast<uint32_t*>(smem + sp.misc + 28);  // key that no candidate outside the active set exceeds
+    float* thr_holder = reinterpret_cast<float*>(smem + sp.misc + 56);          // the pool's score threshold
+    int* tie_holder = reinterpret_cast<int*>(smem + sp.misc + 60);              // see picks_cosine: tie_slot
     const uint32_t tile_u32 = smem_u32(tile);
     const uint32_t half_bytes = kPoolTileBytes / 2u;  // the operand's two 128-byte column halves
 
@@ -277,31 +278,37 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
             }
         }
         const float sb = from_orderable(kb);
-        // -inf keeps everyone
-        const float thr = a.no_prune ? -INFINITY : fmaf(-1.001f, a.lam, sb) - 1e-6f * fabsf(sb);
-        // Active set: the pool's best-scored rows, at most kPoolActive of them; bound is the best key left out (0: none is).
-        // A candidate's Eq. 2 value never exceeds its score: the loop over the active set is exact as long as its winning
-        // value stays above the bound (it nearly always does: with lambda = 0.5 the picks reach a few ranks beyond the
-        // budget).
-        uint32_t bound = 0u;
+        // -inf keeps everyone (also where kb, whose low bits are open, is below every finite value's key)
+        const float thr = a.no_prune || kb < 0x00800000u ? -INFINITY : fmaf(-1.001f, a.lam, sb) - 1e-6f * fabsf(sb);
+        // Active set: the pool's best-scored rows, at most kPoolActive of them; no key left out is above bound.key (0: none
+        // is left out). A candidate's Eq. 2 value never exceeds its score: the loop over the active set is exact as long as
+        // its winning value stays above the bound (it nearly always does: with lambda = 0.5 the picks reach a few ranks
+        // beyond the budget).
+        ActiveBound bound{0u, 0};
         if (similarity) {
             int pool_size = 0;
 #pragma unroll
             for (int k = 0; k < 8; ++k) pool_size += kk[k] != 0u && !(from_orderable(kk[k]) < thr);
             pool_size = __reduce_add_sync(0xFFFFFFFFu, pool_size);
-            if (pool_size > kPoolActive) bound = active_bound(kk, orderable(thr), kb, kPoolActive);
+            if (pool_size > kPoolActive) bound = warp_active_bound(kk, orderable(thr), kb, kPoolActive);
         }
         int base = 0;
+        if (lane == 0) *tie_holder = 0;
+        __syncwarp();
+        if (bound.ties) {
+            base = list_with_ties(key, np4, bound.key, bound.ties, bypool, tie_holder);
+        } else {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const bool in = kk[k] != 0u && (similarity ? !(from_orderable(kk[k]) < thr) && kk[k] > bound : kk[k] >= kb);
-            const uint32_t mask = __ballot_sync(0xFFFFFFFFu, in);
-            if (in) bypool[base + __popc(mask & ((1u << lane) - 1u))] = (unsigned short)(lane + 32 * k);
-            base += __popc(mask);
+            for (int k = 0; k < 8; ++k) {
+                const bool in = kk[k] != 0u && (similarity ? !(from_orderable(kk[k]) < thr) && kk[k] > bound.key : kk[k] >= kb);
+                const uint32_t mask = __ballot_sync(0xFFFFFFFFu, in);
+                if (in) bypool[base + __popc(mask & ((1u << lane) - 1u))] = (unsigned short)(lane + 32 * k);
+                base += __popc(mask);
+            }
         }
         if (lane == 0) {
             *pool_holder = base;
-            *bound_holder = bound;
+            *bound_holder = bound.key;
             *thr_holder = thr;
         }
     }
@@ -365,7 +372,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
     // by symmetry
     const bool product = similarity && !G;  // the cosine matrix comes off the tensor core
     const int nb = (product && P > 128) ? P - 128 : 0;
-    const int ncols = (P + 15) & ~15, base2 = ncols - 128;
+    const int ncols = max((P + 15) & ~15, 16), base2 = ncols - 128;   // (a shape with no columns is not allowed)
     if (product) {
         if (tid == 0) {
             tc_fence_after();
@@ -469,7 +476,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
     } else {
         if (warp == 0) {
             const bool ok = picks_cosine<kPoolCpl, true>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order, *bound_holder,
-                                                         reinterpret_cast<float*>(tile + kContMact), redi);
+                                                         reinterpret_cast<float*>(tile + kContMact), redi, nullptr, tie_holder);
             if (lane == 0) *pick_holder = ok ? picks : *redi;
         }
         __syncthreads();

@@ -22,6 +22,7 @@
 //   5. Kept rows are written back in place: K and V rows are re-read (L2) into the tile, which is
 //      free by then, and stored after a barrier; positions come from their shared-memory copy.
 #pragma once
+#include "akv_active_set.cuh"
 #include "akv_event_tc.cuh"
 
 namespace akv {
@@ -173,17 +174,11 @@ __device__ __forceinline__ void picks_by_rank(int tid, int P, int picks, const u
     }
 }
 
-// The best key v with at most max_pool keys above it, from below: for a warp's keys (8 per lane) of which more than
-// max_pool reach the threshold's key `low`, and fewer than max_pool the key kb (14 low bits open). The common leading bits
-// of the two are v's own, and fourteen more place it well enough.
-__device__ __forceinline__ uint32_t active_bound(const uint32_t (&kk)[8], uint32_t low, uint32_t kb, int max_pool) {
-    const uint32_t diff = (kb | 0x3FFFu) ^ low;
-    const int top = max((31 - __clz(diff)) | 1, 1);   // an odd bit number: two bits a round
-    const int last = max(top - 13, 0);
-    uint32_t v = top == 31 ? 0u : low & ~((2u << top) - 1u);
-    for (int lo = top - 1; lo >= last; lo -= 2) {
-        const uint32_t v1 = v | (1u << lo), v2 = v | (2u << lo), v3 = v | (3u << lo);
-        int c1 = 0, c2 = 0, c3 = 0;
+// active_bound for a warp's keys (8 per lane, 0: no row). (A row fewer than the set could hold costs nothing; from an eighth
+// fewer on the search goes on to the last bit.)
+__device__ __forceinline__ ActiveBound warp_active_bound(const uint32_t (&kk)[8], uint32_t low, uint32_t kb, int cap) {
+    return active_bound(low, kb, cap, cap + 1, cap - cap / 8, [&](uint32_t v1, uint32_t v2, uint32_t v3, int& c1, int& c2, int& c3) {
+        c1 = c2 = c3 = 0;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             c1 += kk[k] >= v1;
@@ -193,9 +188,30 @@ __device__ __forceinline__ uint32_t active_bound(const uint32_t (&kk)[8], uint32
         c1 = __reduce_add_sync(0xFFFFFFFFu, c1);
         c2 = __reduce_add_sync(0xFFFFFFFFu, c2);
         c3 = __reduce_add_sync(0xFFFFFFFFu, c3);
-        v = c3 > max_pool ? v3 : (c2 > max_pool ? v2 : (c1 > max_pool ? v1 : v));
+    });
+}
+
+// The active set in slot order where keys equal to its bound belong to it, by one warp: the keys above the bound and the
+// `ties` lowest slots of those equal to it. Returns its size; *tie_slot: the lowest slot that equals the bound and is left
+// out. Out of line: few events come here.
+__device__ __noinline__ int list_with_ties(const uint32_t* key, int np4, uint32_t bound, int ties, unsigned short* bypool, int* tie_slot) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t below = (1u << lane) - 1u;
+    int base = 0, seen = 0;
+    for (int j0 = 0; j0 < np4; j0 += 32) {
+        const int j = j0 + lane;
+        const uint32_t kj = j < np4 ? key[j] : 0u;
+        const bool tie = kj == bound;
+        const uint32_t tmask = __ballot_sync(0xFFFFFFFFu, tie);
+        const int rank = seen + __popc(tmask & below);
+        const bool in = kj > bound || (tie && rank < ties);
+        const uint32_t mask = __ballot_sync(0xFFFFFFFFu, in);
+        if (in) bypool[base + __popc(mask & below)] = (unsigned short)j;
+        if (tie && rank == ties) *tie_slot = j;
+        base += __popc(mask);
+        seen += __popc(tmask);
     }
-    return v | ((1u << last) - 1u);   // more than max_pool keys are >= v; at most that many are above this
+    return base;
 }
 
 // Warp-wide maximum of a float (sm_100a has the reduction for f32).
@@ -232,13 +248,15 @@ __device__ __forceinline__ int lowest_free_row(const int* picked, int t) {
 //
 // BOUNDED: the P rows are only the best-scored part of the pool, and every candidate left out scores at most
 // `bound_key` (as an order-preserving key), so its Eq. 2 value can never exceed that. The loop is exact as long as the
-// winning value stays above the bound; at the first pick that does not, it stops and returns false. The picks made so
+// winning value stays above the bound, or equals it at a slot below *tie_slot (null: none), the lowest one of the candidates
+// left out that may equal it; at the first pick that does not, it stops and returns false. The picks made so
 // far stand; with m_out / t_out given the running maxima (by pool row; +inf for the rows already picked) and the number
 // of picks are left for the caller to continue from. m_in: maxima to start from (null: 0). `tri` (its diagonal) and `r` are modified. At most 256 rows.
 template <int CPL, bool BOUNDED>
 __device__ __forceinline__ bool picks_cosine(int lane, int P, int picks, const float* s, const unsigned short* bypool, float* r, float lam,
                                              float* tri, uint32_t* park_key, int* park_row, uint32_t bound_key = 0u,
-                                             float* m_out = nullptr, int* t_out = nullptr, const float* m_in = nullptr) {
+                                             float* m_out = nullptr, int* t_out = nullptr, const float* m_in = nullptr,
+                                             const int* tie_slot = nullptr) {
     constexpr int kGroup = 4;   // picks per look at the bound (divides 32)
     const uint32_t tb = smem_u32(tri), rb = smem_u32(r);
     const float ninf = __int_as_float(0xff800000), pinf = __int_as_float(0x7f800000);
@@ -318,7 +336,7 @@ __device__ __forceinline__ bool picks_cosine(int lane, int P, int picks, const f
                 for (int u = 0; u < kGroup && t < t1; ++u, ++t) {
                     uint32_t w;
                     winner(whi, w);
-                    at_bound = !(whi > bound);
+                    at_bound = !(whi > bound || (BOUNDED && tie_slot && whi == bound && whi > ninf && (int)bypool[w & 255u] < *tie_slot));
                     if (at_bound) break;
                     const bool mine = lane == t - t0;
                     my_val = mine ? whi : my_val;
@@ -537,6 +555,7 @@ __global__ void __launch_bounds__(kTcThreads) event_tri_kernel(const __grid_cons
     int* pick_holder = reinterpret_cast<int*>(smem + sp.misc + 24);
     uint32_t* bound_holder = reinterpret_cast<uint32_t*>(smem + sp.misc + 28);  // key that no candidate outside the active set exceeds
     float* thr_holder = reinterpret_cast<float*>(smem + sp.misc + 56);          // the pool's score threshold
+    int* tie_holder = reinterpret_cast<int*>(smem + sp.misc + 60);              // see picks_cosine: tie_slot
     int* redi = reinterpret_cast<int*>(smem + sp.misc + 32);
     const uint32_t tile_u32 = smem_u32(tile);
     const uint32_t half_bytes = (uint32_t)kTriTileRows * 128u;
@@ -727,28 +746,34 @@ __global__ void __launch_bounds__(kTcThreads) event_tri_kernel(const __grid_cons
             }
         }
         const float sb = from_orderable(kb);
-        // -inf keeps everyone
-        const float thr = a.no_prune ? -INFINITY : fmaf(-1.001f, a.lam, sb) - 1e-6f * fabsf(sb);
-        // active set: bound is the best key left out (0: none is)
-        uint32_t bound = 0u;
+        // -inf keeps everyone (also where kb, whose low bits are open, is below every finite value's key)
+        const float thr = a.no_prune || kb < 0x00800000u ? -INFINITY : fmaf(-1.001f, a.lam, sb) - 1e-6f * fabsf(sb);
+        // active set: no key left out is above bound.key (0: none is left out)
+        ActiveBound bound{0u, 0};
         if (similarity) {
             int pool_size = 0;
 #pragma unroll
             for (int k = 0; k < 8; ++k) pool_size += kk[k] != 0u && !(from_orderable(kk[k]) < thr);
             pool_size = __reduce_add_sync(0xFFFFFFFFu, pool_size);
-            if (pool_size > kTriMaxPool) bound = active_bound(kk, orderable(thr), kb, kTriMaxPool);
+            if (pool_size > kTriMaxPool) bound = warp_active_bound(kk, orderable(thr), kb, kTriMaxPool);
         }
         int base = 0;
+        if (lane == 0) *tie_holder = 0;
+        __syncwarp();
+        if (bound.ties) {
+            base = list_with_ties(key, np4, bound.key, bound.ties, bypool, tie_holder);
+        } else {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const bool in = kk[k] != 0u && (similarity ? !(from_orderable(kk[k]) < thr) && kk[k] > bound : kk[k] >= kb);
-            const uint32_t mask = __ballot_sync(0xFFFFFFFFu, in);
-            if (in) bypool[base + __popc(mask & ((1u << lane) - 1u))] = (unsigned short)(lane + 32 * k);
-            base += __popc(mask);
+            for (int k = 0; k < 8; ++k) {
+                const bool in = kk[k] != 0u && (similarity ? !(from_orderable(kk[k]) < thr) && kk[k] > bound.key : kk[k] >= kb);
+                const uint32_t mask = __ballot_sync(0xFFFFFFFFu, in);
+                if (in) bypool[base + __popc(mask & ((1u << lane) - 1u))] = (unsigned short)(lane + 32 * k);
+                base += __popc(mask);
+            }
         }
         if (lane == 0) {
             *pool_holder = base;
-            *bound_holder = bound;
+            *bound_holder = bound.key;
             *thr_holder = thr;
         }
     }
@@ -778,7 +803,7 @@ __global__ void __launch_bounds__(kTcThreads) event_tri_kernel(const __grid_cons
     if (similarity) {
         if (tid == 0) {
             tc_fence_after();
-            const uint32_t idesc = umma_idesc_bf16(128, (P + 15) & ~15);
+            const uint32_t idesc = umma_idesc_bf16(128, max((P + 15) & ~15, 16));   // (a shape with no columns is not allowed)
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) {
                 const uint32_t koff = (uint32_t)(kk >> 2) * half_bytes + (uint32_t)(kk & 3) * 32u;
@@ -840,7 +865,7 @@ __global__ void __launch_bounds__(kTcThreads) event_tri_kernel(const __grid_cons
     } else {
         if (warp == 0) {
             const bool ok = picks_cosine<4, true>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order, *bound_holder,
-                                                  reinterpret_cast<float*>(tile + kContMact), redi);
+                                                  reinterpret_cast<float*>(tile + kContMact), redi, nullptr, tie_holder);
             if (lane == 0) *pick_holder = ok ? picks : *redi;
         }
         __syncthreads();

@@ -630,6 +630,45 @@ def test_small_event_kernel_with_more_than_127_pool_rows(N, budget, lam):
     check_all(plain, run_fused(plain, lam=lam), lam)
 
 
+def _close_scores(N, budget, lam, width, seed, B=2, L=1, H=2):
+    """Scores of 0.3 + width * N(0, 1): the statistic looks at two coordinates, one constant in all keys, and every key
+    sits at the reference position. width = 0: all scores equal."""
+    ev = synth.make_plain(B, L, H, N, 128, budget, lam, dtype=synth.BF16, seed=seed)
+    rng = np.random.default_rng(seed)
+    ev.qstat[...] = 0
+    ev.qstat[..., 0], ev.qstat[..., 1] = np.sqrt(128.0), np.sqrt(128.0) / 256
+    ev.K[..., 0] = synth.f32_to_bf16_bits(np.float32(0.3))
+    ev.K[..., 1] = synth.f32_to_bf16_bits((256 * width * rng.standard_normal(ev.K.shape[:-1])).astype(np.float32))
+    ev.pos[...] = 7
+    ev.p_ref[...] = 7
+    return ev
+
+
+@pytest.mark.parametrize("lam", [0.5, 1.0])
+@pytest.mark.parametrize("width", [0.0, 1e-3, 3e-3])
+@pytest.mark.parametrize("N,budget", [(192, 64), (128, 128), (256, 128)])
+def test_scores_close_together(N, budget, width, lam):
+    """The best-scored rows that an active set holds are then told apart by the last bits of their scores, or by their slots."""
+    ev = _close_scores(N, budget, lam, width, seed=N)
+    check_all(ev, run_fused(ev), lam)
+
+
+@pytest.mark.parametrize("N,budget", [(192, 64), (256, 128)])
+def test_zero_cache_and_non_finite_scores(N, budget):
+    """A zero-filled cache keeps its lowest slots; so does one whose scores are all NaN, with status 1."""
+    ev = synth.make_plain(1, 2, 2, N, 128, budget, 0.5, dtype=synth.BF16, seed=N)
+    nan = synth.make_plain(1, 2, 2, N, 128, budget, 0.5, dtype=synth.BF16, seed=N)
+    ev.K[...], ev.V[...] = 0, 0
+    nan.K[..., 3] = synth.f32_to_bf16_bits(np.float32(np.nan))
+    for e, status in ((ev, 0), (nan, 1)):
+        g = run_fused(e)
+        assert np.all(g["status"] == status)
+        assert np.array_equal(g["order"], np.broadcast_to(np.arange(budget), g["order"].shape))
+        assert np.array_equal(g["idx"], g["order"])
+        for k in ("K", "V", "pos"):
+            assert np.array_equal(g[k], getattr(e, k))
+
+
 @pytest.mark.parametrize("N,budget", [(192, 64), (256, 128)])
 def test_topk_order_with_equal_scores(N, budget):
     """lambda = 0 with every key row four times at one position: equal scores go to the lower slot, in the picks made and
