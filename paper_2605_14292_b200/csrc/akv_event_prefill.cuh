@@ -12,8 +12,9 @@
 //      winning values stay above that. Where one does not (4096 random rows to 128 at lambda = 0.5: about one event in a
 //      hundred), the picks made stand and the next active set is formed: Eq. 2's values only fall, so a row's value
 //      when it was last known, or its score, is an upper bound, and the rows with the best of those make up the set; their
-//      running maxima come from one more product, against the rows picked. Should such a round make no pick (more equal
-//      values than a set holds), the event is done over the whole pool with plain dot products.
+//      running maxima come from one more product, against the rows picked. A round may make no pick (all of its rows have
+//      fallen below one left out), but it leaves their values known: 4096 scores close together take about 40 rounds for 128
+//      picks. Where infinite value rows make picks impossible, the event is done over the whole pool with plain dot products.
 //   4. Kept K and V rows are staged on chip and written to slots 0..b-1 of the same buffers.
 //
 // FUSED: score + select + compact; otherwise selection only (scores are read from a.scores and nothing is rewritten).
@@ -26,6 +27,7 @@ constexpr int kPfStages = 4;
 constexpr unsigned kPfRing = kPfStages * kStStageBytes;
 constexpr int kPfActive = 192;              // rows of the active set: 2 x 192 - 128 columns of tensor memory for its products
 constexpr int kPfEnough = 184;              // rows that an active set is content with
+constexpr int kPfLeast = 160;               // the same once the search has gone on for fourteen bits
 constexpr uint32_t kPfCols = 256;
 constexpr int kPfKeys = 21;                 // most keys per thread (an odd run per thread: no bank conflicts)
 constexpr int kPfMaxN = 5120;
@@ -90,7 +92,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
     float2* sect = reinterpret_cast<float2*>(smem + sp.sect);
     const uint32_t bar_full = smem_u32(smem + sp.misc), bar_empty = bar_full + 8 * kPfStages, barM = bar_full + 64;
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + sp.misc + 72);
-    int* cnt = reinterpret_cast<int*>(smem + sp.misc + 80);  // [0] a wait ran out, [1] newest position, [2] irregular positions, [3] a round's picks, [4] the same at a bound
+    int* cnt = reinterpret_cast<int*>(smem + sp.misc + 80);  // [0] a wait ran out, [1] newest position, [2] irregular positions, [3] a round's picks, [4] the same at a bound, [5] see picks_cosine: tie_slot
     const uint32_t region_u32 = smem_u32(region);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -419,8 +421,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
         const int quarter = warp & 3, rho = 32 * quarter + lane;            // row of a product this thread reads
         const uint32_t lanes = tbase + ((uint32_t)(32 * quarter) << 16);
         uint32_t phase = 0u;
-        int made = 0;
-        bool stuck = false;
+        int made = 0, idle = 0;   // idle: rounds without a pick since the last one
         // a product of the tile rows from row_a on with those from row_b on, into the columns from col on
         auto product = [&](int row_a, int row_b, int cols, uint32_t col) {
             const uint32_t idesc = umma_idesc_bf16(128, cols);
@@ -436,27 +437,30 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
             phase ^= 1u;
             tc_fence_after();
         };
-        while (made < picks && !stuck) {
-            // ---- the active set: at most 192 rows; bound: the best key with at most that many above it, from below (see
-            // active_bound; 0: the pool is no larger)
+        // A round without a pick makes the values of its rows known, and the next set holds the rows between the best of
+        // those and the bound, all of them unknown, until they fit a set: n / 192 + 1 such rounds at most. (The limit is a
+        // safeguard.)
+        while (made < picks && idle <= n / kPfActive + 2) {
+            // ---- the active set: at most 192 rows (bound 0: the pool is no larger)
             int pool_size, unused1, unused2;
             count3(low, 0xFFFFFFFFu, 0xFFFFFFFFu, pool_size, unused1, unused2);
-            uint32_t bound = 0u;
-            if (pool_size > kPfActive) {
-                // (the counts fall towards the set's size; a key that 184 to 192 rows reach will do)
-                const uint32_t diff = (kb | 0x3FFFu) ^ low;
-                const int top = max((31 - __clz(diff)) | 1, 1), last = max(top - 13, 0);
-                uint32_t v = top == 31 ? 0u : low & ~((2u << top) - 1u);
-                for (int lo = top - 1; lo >= last && bound == 0u; lo -= 2) {
-                    const uint32_t v1 = v | (1u << lo), v2 = v | (2u << lo), v3 = v | (3u << lo);
-                    int t1, t2, t3;
-                    count3(v1, v2, v3, t1, t2, t3);
-                    if (t1 <= kPfActive) bound = t1 >= kPfEnough ? v1 - 1u : 0u;
-                    else if (t2 <= kPfActive) { bound = t2 >= kPfEnough ? v2 - 1u : 0u; v = v1; }
-                    else if (t3 <= kPfActive) { bound = t3 >= kPfEnough ? v3 - 1u : 0u; v = v2; }
-                    else v = v3;
-                }
-                if (bound == 0u) bound = v | ((1u << last) - 1u);   // more than 192 keys are >= v; at most that many are above this
+            ActiveBound found{0u, 0};
+            if (pool_size > kPfActive) found = active_bound(low, kb, kPfActive, kPfEnough, kPfLeast, count3);
+            const uint32_t bound = found.key;
+            if (tid == 0) cnt[5] = 0;
+            if (found.ties) {
+                // the lowest slots of those that equal the bound move above it (a key may lie above its row's value)
+                uint32_t c = 0u, total;
+#pragma unroll
+                for (int i = 0; i < kPfKeys; ++i) c += key[i] == bound;
+                int eq = (int)scan2(c, total);
+#pragma unroll
+                for (int i = 0; i < kPfKeys; ++i)
+                    if (key[i] == bound) {
+                        if (eq < found.ties) ++key[i];
+                        else if (eq == found.ties) cnt[5] = j0 + i;
+                        ++eq;
+                    }
             }
             const int R = list(bound, act);
             if (bound == 0u && R < picks - made) break;   // (values lost to overflowed cosines)
@@ -574,7 +578,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
             if (warp == 0) {
                 const bool ok = picks_cosine<kPfActive / 32, true>(lane, R, picks - made, s, act, ar, a.lam, tri,
                                                                    reinterpret_cast<uint32_t*>(gain) + made, order + made, bound, am,
-                                                                   cnt + 4, made > 0 ? am : nullptr);
+                                                                   cnt + 4, made > 0 ? am : nullptr, cnt + 5);
                 if (lane == 0) cnt[3] = ok ? picks - made : cnt[4];
             }
             work_barrier();
@@ -606,7 +610,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
                 work_barrier();
             }
             made += got;
-            stuck = got == 0;
+            idle = got ? 0 : idle + 1;
         }
         tc_fence_before();
         work_barrier();

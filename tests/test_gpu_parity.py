@@ -646,14 +646,14 @@ def _close_scores(N, budget, lam, width, seed, B=2, L=1, H=2):
 
 @pytest.mark.parametrize("lam", [0.5, 1.0])
 @pytest.mark.parametrize("width", [0.0, 1e-3, 3e-3])
-@pytest.mark.parametrize("N,budget", [(192, 64), (128, 128), (256, 128)])
+@pytest.mark.parametrize("N,budget", [(192, 64), (128, 128), (256, 128), (300, 128), (1000, 64), (5120, 128)])
 def test_scores_close_together(N, budget, width, lam):
     """The best-scored rows that an active set holds are then told apart by the last bits of their scores, or by their slots."""
     ev = _close_scores(N, budget, lam, width, seed=N)
     check_all(ev, run_fused(ev), lam)
 
 
-@pytest.mark.parametrize("N,budget", [(192, 64), (256, 128)])
+@pytest.mark.parametrize("N,budget", [(192, 64), (256, 128), (1000, 128)])
 def test_zero_cache_and_non_finite_scores(N, budget):
     """A zero-filled cache keeps its lowest slots; so does one whose scores are all NaN, with status 1."""
     ev = synth.make_plain(1, 2, 2, N, 128, budget, 0.5, dtype=synth.BF16, seed=N)
