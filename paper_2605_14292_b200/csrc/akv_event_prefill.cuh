@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
                 if (tid < R) {
                     const float m = am[tid];
                     upper[act[tid]] = m == __int_as_float(0x7f800000) ? 0u
-                                                                      : orderable(fmaf(-fmaxf(a.lam * ar[tid], 1e-30f), m, fmaxf(s[act[tid]], kLowestScore)));
+                                                                      : orderable(fmaf(-fmaxf(penalty_rate(a.lam, ar[tid]), 1e-30f), m, fmaxf(s[act[tid]], kLowestScore)));
                 }
             }
             for (int t = made + tid; t < made + got; t += kStWork) {
@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
                         mm = fmaxf(mm, fminf(r[last] * vdot(pool[q], pool[last]), 1e30f));
                         m[q] = mm;
                     }
-                    const uint32_t k = orderable(fmaf(-a.lam * r[q], mm, ps[q]));
+                    const uint32_t k = orderable(fmaf(-penalty_rate(a.lam, r[q]), mm, ps[q]));
                     if (k > hi) { hi = k; lo = 0xFFFFFFFFu - (uint32_t)pool[q]; row = (uint32_t)q; }
                 }
                 // block-wide arg-max, ties to the lower slot; the row travels with it

@@ -634,7 +634,7 @@ __global__ void __launch_bounds__(kStThreads, 1) event_stream_kernel(const Event
                         dot8_bf16(v, v, acc);
                     }
                     rr[k] = 1.f / (sqrtf(acc.x + acc.y) + a.eps);
-                    lr[k] = a.lam * rr[k];
+                    lr[k] = penalty_rate(a.lam, rr[k]);
                 }
             }
             // a row beyond the tile stays in its thread's registers for the whole loop (256 bytes)
@@ -650,7 +650,7 @@ __global__ void __launch_bounds__(kStThreads, 1) event_stream_kernel(const Event
                     dot8_bf16(own[c], own[c], acc);
                 }
                 xr[tid] = 1.f / (sqrtf(acc.x + acc.y) + a.eps);
-                xlr[tid] = a.lam * xr[tid];
+                xlr[tid] = penalty_rate(a.lam, xr[tid]);
             }
             const int nblk = (resident + 127) >> 7;
             // window: 128 tile rows when the pool has at most four blocks (4 x 128 columns of tensor memory), else 64;

@@ -459,7 +459,7 @@ __global__ void __launch_bounds__(kTcThreads, 4) event_tc_kernel(const EventArgs
                 }
                 const float rr = 1.f / (sqrtf(ss) + a.eps);
                 r[rho[u]] = rr;
-                lr[u] = a.lam * rr;
+                lr[u] = penalty_rate(a.lam, rr);
             }
         }
     }

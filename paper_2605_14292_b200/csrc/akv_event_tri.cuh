@@ -114,7 +114,7 @@ struct GreedyLane {
             sv[k] = 0.f; lr[k] = 0.f; M[k] = 0.f; am[k] = 0u;
             if (rho < P) {
                 sv[k] = s[bypool[rho]];
-                lr[k] = use_r ? lam * r[rho] : 0.f;
+                lr[k] = use_r ? penalty_rate(lam, r[rho]) : 0.f;
                 am[k] = 0xFFFFFFFFu;
             }
         }
@@ -272,7 +272,7 @@ __device__ __forceinline__ bool picks_cosine(int lane, int P, int picks, const f
         sv[k] = in ? fmaxf(s[bypool[rc]], kLowestScore) : ninf;
         M[k] = m_in && in ? m_in[rc] : 0.f;
         const float rk = fmaxf(r[rc], 1e-30f);   // positive, so that a maximum of +inf and a value of -inf come about
-        lr[k] = in ? fmaxf(lam * rk, 1e-30f) : 1.f;
+        lr[k] = in ? fmaxf(penalty_rate(lam, rk), 1e-30f) : 1.f;   // (finite: no value below is ever NaN, so a winner's row is always found)
         rc4[k] = 4 * rc;
         trow[k] = (int)(tb + 4u * (uint32_t)tri_row(rc));
         tag[k] = ((4u * (uint32_t)tri_row(rc)) << 8) | (uint32_t)rc;

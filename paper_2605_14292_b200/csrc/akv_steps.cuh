@@ -90,6 +90,10 @@ __device__ __forceinline__ float sumsq_row(const T* vrow, bool valid, int d, int
     return group_sum(acc, G);
 }
 
+// lambda times a row's reciprocal norm r, kept finite: with eps = 0 a zero row has r = inf, and inf times a maximum of 0
+// would be a NaN that competes as a candidate's value
+__device__ __forceinline__ float penalty_rate(float lam, float r) { return fminf(lam * r, 3.0e38f); }
+
 // ---- greedy selection (Algorithm 1) ---------------------------------------------------------------
 // s, m, taken, order, gain and red live in shared memory. s holds sanitised scores (non-finite ->
 // -inf), m starts at 0, taken at 0. r holds 1/(||V_j||+eps) per candidate, or nullptr when the

@@ -669,6 +669,21 @@ def test_zero_cache_and_non_finite_scores(N, budget):
             assert np.array_equal(g[k], getattr(e, k))
 
 
+@pytest.mark.parametrize("dtype,N,budget", [(synth.BF16, 192, 64), (synth.BF16, 256, 128), (synth.BF16, 256, 140), (synth.BF16, 1000, 128),
+                                            (synth.BF16, 1000, 140), (synth.F32, 128, 64), (synth.F32, 128, 128)])
+def test_zero_value_rows_with_eps_zero(dtype, N, budget):
+    """eps = 0 and zero value rows: their reciprocal norm is infinite, their cosine counts as 0 (the oracle's with a tiny eps).
+    In one event every value row is zero: no penalty, and the kept rows are the top-k."""
+    ev = synth.make_plain(2, 1, 2, N, 128, budget, 0.5, dtype=dtype, seed=N + budget)
+    ev.V[:, :, :, 3::7] = 0
+    ev.V[0, 0, 0] = 0
+    ev.eps = 0.0
+    g = run_fused(ev)
+    ev.eps = 1e-30
+    check_all(ev, g, ev.lam)
+    assert g["order"][0, 0, 0].tolist() == O.topk_indices(g["scores"][0, 0, 0].astype(np.float64), budget).tolist()
+
+
 @pytest.mark.parametrize("N,budget", [(192, 64), (256, 128)])
 def test_topk_order_with_equal_scores(N, budget):
     """lambda = 0 with every key row four times at one position: equal scores go to the lower slot, in the picks made and
