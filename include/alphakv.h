@@ -112,8 +112,9 @@ typedef struct {
     /* Grouped-query attention: qstat holds gqa_group statistics per KV head, [L, H * gqa_group, d] (0 and 1 both
      * mean one). The score of a key is the mean over the group's query heads of their scores (gqa_reduce = 0;
      * the same as scoring with the averaged statistic, the score being linear in it) or the largest of them
-     * (gqa_reduce = 1: a key that any query head of the group wants is kept). At most 8 per group. Groups
-     * larger than one run on the general kernels (the resident one or three launches). */
+     * (gqa_reduce = 1: a key that any query head of the group wants is kept). At most 8 per group. The mean runs on
+     * the kernels of ungrouped calls, with every row's rotation taken afresh (as with AKV_FLAG_NO_CHAIN); the maximum
+     * runs on the general kernels (the resident one or three launches). */
     int32_t gqa_group;
     int32_t gqa_reduce;
 } akv_options_t;

@@ -738,6 +738,19 @@ def test_mean_of_grouped_statistics_on_the_tensor_memory_kernels(N, budget, G):
                                 sel.idx_sorted[b, l, h].cpu().numpy(), Kn[b, l, h], Vn[b, l, h], pn[b, l, h])
 
 
+@pytest.mark.parametrize("N,budget", [(192, 64), (256, 128), (256, 140), (700, 60), (5200, 60)])
+def test_grouped_statistics_are_scored_with_fresh_rotations(N, budget):
+    """The scores of grouped calls keep the general kernels' precision: no rotation is carried from row to row."""
+    ev = synth.make_plain(1, 2, 2, N, 128, budget, 0.5, dtype=synth.BF16, seed=N)
+    Q = np.random.default_rng(N).standard_normal((2, 2 * 4, 128)).astype(np.float32)
+    s = []
+    for flags in (0, akv.FLAG_NO_CHAIN):
+        sel = akv.alpha_compress_event(dev(ev.K), dev(ev.V), dev(ev.pos), dev(Q), budget, akv.Options(lam=0.5, gqa_group=4, flags=flags),
+                                       p_ref=dev(ev.p_ref), want_scores=True)
+        s.append(sel.scores.cpu().numpy())
+    assert np.array_equal(s[0], s[1])
+
+
 @pytest.mark.parametrize("reduce", ["mean", "max"])
 @pytest.mark.parametrize("dtype,N,d", [(synth.BF16, 150, 128), (synth.F32, 600, 64)])
 def test_grouped_query_statistics(reduce, dtype, N, d):
