@@ -135,6 +135,25 @@ def test_nonfinite_scores_are_flagged_and_never_preferred():
     assert len(set(g["idx"][0, 0, 0].tolist())) == 20
 
 
+@pytest.mark.parametrize("d", [128, 256])
+def test_resident_kernel_norms_are_summed_in_a_tree(d):
+    """The second pick's value is -lambda x_0 r, with r the reciprocal norm of its row x: the first row is a unit vector, so the
+    dot product is exact. Errors of r: half of the squared norm's, and one rounding each for root, division and product. In
+    fp32 emulation the whole is 4.8e-8 (d = 128) and 5.0e-8 (d = 256) root mean square for sums of eight squares in a tree,
+    9.3e-8 and 1.2e-7 for one chain of d squares."""
+    ev = synth.make_plain(8, 32, 8, 2, d, 2, 1.0, dtype=synth.F32, seed=d)
+    ev.K[...] = 0
+    ev.V[..., 0, :] = 0
+    ev.V[..., 0, 0] = 1
+    ev.V[..., 1, 0] = np.abs(ev.V[..., 1, 0]) + 0.5
+    x = ev.V[..., 1, :].astype(np.float64)
+    want = -x[..., 0] / np.sqrt((x * x).sum(-1))
+    g = run_fused(ev)
+    assert np.all(g["order"] == [0, 1])
+    err = g["gain"][..., 1] / want - 1
+    assert np.sqrt(np.mean(err ** 2)) < 7e-8
+
+
 # ------------------------------------------------------------------ stand-alone entry points
 @pytest.mark.parametrize("dtype", [synth.BF16, synth.F32])
 def test_score_select_compact_chain_equals_fused(dtype):
