@@ -5,8 +5,10 @@
 // Selection, when lambda > 0: the exact pool (s_i >= s_(b) - lambda (1 + slack), see akv_select_pool.cuh) is
 // formed, and when the lower triangle of its cosine matrix fits, into the shared memory left beside the tiles or else over
 // the K tile, which scoring is done with (the kept K rows are then read again for the compaction), the triangle is filled
-// by plain fp32 dot products and Algorithm 1 runs as the one-warp loop of the tensor-memory kernels. Otherwise, and for
-// lambda = 0, the CTA-wide loop with rows of the cosine matrix on demand (greedy_cta).
+// by plain fp32 dot products and Algorithm 1 runs as the one-warp loop of the tensor-memory kernels. A pool that does not
+// fit is taken in rounds of active sets (picks_in_rounds). Otherwise, and for lambda = 0, the CTA-wide loop with rows of the
+// cosine matrix on demand (greedy_cta). (896 events of 256 bf16 rows of 64, 128 kept, lambda = 0.5: 345 us in rounds, 1471 in
+// the CTA-wide loop, 556 with the whole triangle and one CTA per SM.)
 //
 // The dot products are bound by shared-memory reads, so a thread takes 8 x 4 pairs of rows at a time (12 reads for
 // 128 multiply-adds a step instead of 2 for 4), walking the head dimension from its own starting column so that a warp's loads
@@ -35,14 +37,223 @@ __device__ __forceinline__ void cp_async_wait_pending() {
     asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
 }
 
-constexpr int kResidentCtas = 2;   // most CTAs per SM that the kernel's registers allow
+constexpr int kResidentCtas = 2;       // most CTAs per SM that the registers of the kernel with the penalty allow
+constexpr int kResidentCtasTopk = 3;   // ... and of the one without: no triangle (896 events of 128 bf16 rows of 64: 107 us, with the
+                                       // other's 128 registers 156)
+constexpr int kResidentLeastSet = 64;  // rows from which an active set is worth its triangle
+
+// Raw dot products of every pair of the R rows listed in `rows` (i >= j) -> the triangle `tri`, 8 x 4 at a time: thread x
+// takes blocks x, x + 256, ...; row band b of eight rows has 2 b + 2 blocks, so it starts at block b (b + 1). row_of: slot ->
+// values.
+template <typename RowOf>
+__device__ __forceinline__ void fill_triangle(RowOf row_of, const unsigned short* rows, int R, int d, float* tri) {
+    const int tid = threadIdx.x, G4 = d >> 2;   // G4: groups of four elements per row
+    const int bands = (R + 7) >> 3, blocks = bands * (bands + 1);
+    for (int x = tid; x < blocks; x += kThreads) {
+        int bi = (int)sqrtf((float)x);
+        while (bi * (bi + 1) > x) --bi;
+        while ((bi + 1) * (bi + 2) <= x) ++bi;
+        const int bj = x - bi * (bi + 1);
+        float acc[8][4] = {};
+        decltype(row_of(0)) vi[8], vj[4];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) vi[q] = row_of(rows[min(8 * bi + q, R - 1)]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) vj[q] = row_of(rows[min(4 * bj + q, R - 1)]);
+        int gq = tid % G4;
+        for (int c = 0; c < G4; ++c) {
+            float xj[4][4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) load4(vj[q] + 4 * gq, xj[q]);
+#pragma unroll
+            for (int p = 0; p < 8; ++p) {
+                float xi[4];
+                load4(vi[p] + 4 * gq, xi);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) acc[p][q] = fmaf(xi[e], xj[q][e], acc[p][q]);
+            }
+            gq = gq + 1 == G4 ? 0 : gq + 1;
+        }
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (8 * bi + p < R && 4 * bj + q <= 8 * bi + p) tri[tri_row(8 * bi + p) + 4 * bj + q] = acc[p][q];
+    }
+}
+
+// State of the rounds over active sets, in the shared memory beside the tiles or else at the head of the K tile.
+struct ResidentState {
+    unsigned key, seen, row, in, r, m, total;
+};
+__host__ __device__ inline ResidentState plan_resident_state(int N) {
+    ResidentState p;
+    unsigned o = 0;
+    p.key = o;  o += align16((unsigned)N * 4);   // by slot: the most that the row's value can be, 0 once it is picked
+    p.seen = o; o += align16((unsigned)N * 2);   // by slot: how many picks its running maximum covers
+    p.row = o;  o += align16((unsigned)N * 2);   // the active set's slots
+    p.in = o;   o += align16((unsigned)N);       // by slot: 1 in the active set
+    p.r = o;    o += 1024;                       // the set's norms
+    p.m = o;    o += 1024;                       // and running maxima
+    p.total = o;
+    return p;
+}
+
+// Algorithm 1 in rounds over the best rows of a pool whose triangle does not fit (`low`: the pool's threshold, as a key).
+// At the bound of an active set the picks made stand, and the next set is formed from what is known of every row's value,
+// as in akv_event_prefill.cuh. All threads call, after a barrier; s and r by slot, taken 0. Leaves order[], gain[] and
+// taken[] and returns kRoundsDone; leaves taken 0 and returns without that bit where a set would be too small or values are
+// lost to infinite cosines. kRoundsOverK: the K tile was written over. Out of line: registers and code of the kernel stay
+// those of the pool that fits.
+constexpr int kRoundsDone = 1, kRoundsOverK = 2;
+template <typename T>
+__device__ __noinline__ int picks_in_rounds(const EventArgs& a, unsigned char* smem, int n, int picks, uint32_t low, int extra_bytes) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int d = a.lay.d, N = a.lay.N, G4 = d >> 2;
+    const EventId id = decode_event(a.lay, blockIdx.x);
+    const SmemPlan sp = plan_smem(N, d, sizeof(T), a.budget, true, true);
+    const T* Vt = reinterpret_cast<const T*>(smem + sp.tileV);
+    const float* s = reinterpret_cast<const float*>(smem + sp.s);
+    const float* r = reinterpret_cast<const float*>(smem + sp.r);
+    float* m = reinterpret_cast<float*>(smem + sp.m);
+    int* order = reinterpret_cast<int*>(smem + sp.order);
+    float* gain = reinterpret_cast<float*>(smem + sp.gain);
+    uint32_t* park_key = reinterpret_cast<uint32_t*>(gain);
+    unsigned char* taken = smem + sp.taken;
+    const float* sig = a.flat_sig ? event_sig(a, id) : nullptr;
+    // state and triangle: beside the tiles what fits there, the rest over the K tile
+    const ResidentState rs = plan_resident_state(N);
+    const bool state_beside = (int)rs.total <= extra_bytes;
+    unsigned char* state = state_beside ? smem + sp.total : smem + sp.tileK;
+    const int room_beside = extra_bytes - (state_beside ? (int)rs.total : 0);
+    const int room_over = N * d * (int)sizeof(T) - (state_beside ? 0 : (int)rs.total);
+    const int room = max(room_beside, room_over);
+    int cap = min((int)sqrtf((float)room * 0.5f), 256);   // rows whose triangle fits
+    while (2 * cap * (cap + 1) > room) --cap;
+    if (cap < kResidentLeastSet) return 0;
+    int over_k = state_beside ? 0 : kRoundsOverK;
+    uint32_t* key = reinterpret_cast<uint32_t*>(state + rs.key);
+    unsigned short* seen = reinterpret_cast<unsigned short*>(state + rs.seen);
+    unsigned short* act = reinterpret_cast<unsigned short*>(state + rs.row);
+    unsigned char* in_set = state + rs.in;
+    float* ar = reinterpret_cast<float*>(state + rs.r);
+    float* am = reinterpret_cast<float*>(state + rs.m);
+    uint32_t* bound_holder = reinterpret_cast<uint32_t*>(smem + sp.red);
+    int* tie_holder = reinterpret_cast<int*>(smem + sp.red) + 1;    // see picks_cosine: tie_slot
+    int* made_holder = reinterpret_cast<int*>(smem + sp.red) + 2;
+    for (int j = tid; j < n; j += kThreads) {
+        key[j] = orderable(s[j]);
+        seen[j] = 0;
+        m[j] = 0.f;
+    }
+    __syncthreads();
+    int made = 0, idle = 0;   // idle: rounds without a pick since the last one (the limit is a safeguard)
+    while (made < picks && idle <= n / cap + 2) {
+        // ---- the active set: the pool's rows with the largest keys, equal ones by slot
+        int P = 0;
+        for (int j0 = 0; j0 < n; j0 += kThreads) P += __syncthreads_count(j0 + tid < n && key[j0 + tid] >= low);
+        for (int j = tid; j < n; j += kThreads) {
+            const uint32_t kj = key[j];
+            bool in = kj >= low;
+            if (in && P > cap) {
+                int rank = 0;
+                for (int i = 0; i < n; ++i) {
+                    const uint32_t ki = key[i];
+                    rank += ki > kj || (ki == kj && i < j);
+                }
+                in = rank < cap;
+                if (rank == cap) {   // the best row left out
+                    *bound_holder = kj;
+                    *tie_holder = j;
+                }
+            }
+            in_set[j] = in;
+        }
+        __syncthreads();
+        const int R = min(P, cap);
+        const uint32_t bound = P > cap ? *bound_holder : 0u;
+        if (bound == 0u && R < picks - made) break;   // (values lost to overflowed cosines)
+        if (warp == 0) {
+            int base = 0;
+            for (int j0 = 0; j0 < n; j0 += 32) {
+                const int j = j0 + lane;
+                const bool in = j < n && in_set[j];
+                const uint32_t mask = __ballot_sync(0xFFFFFFFFu, in);
+                if (in) act[base + __popc(mask & ((1u << lane) - 1u))] = (unsigned short)j;
+                base += __popc(mask);
+            }
+        }
+        __syncthreads();
+        if (tid < R) {
+            ar[tid] = sig ? 1.f : r[act[tid]];
+            am[tid] = m[act[tid]];
+        }
+        __syncthreads();
+        // running maxima over the picks that a row has not seen yet: a dot product per (row, pick), the maximum by an integer
+        // atomic (the values are non-negative floats)
+        for (int x = tid; x < R * made; x += kThreads) {
+            const int row = x / made, t = x - row * made, j = act[row], i = order[t];
+            if (t < seen[j]) continue;
+            float acc = 0.f;
+            int gq = tid % G4;
+            for (int c = 0; c < G4; ++c) {
+                float xi[4], xj[4];
+                if (sig) {
+                    load4(sig + (long long)i * d + 4 * gq, xi);
+                    load4(sig + (long long)j * d + 4 * gq, xj);
+                } else {
+                    load4(Vt + (size_t)i * d + 4 * gq, xi);
+                    load4(Vt + (size_t)j * d + 4 * gq, xj);
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc = fmaf(xi[e], xj[e], acc);
+                gq = gq + 1 == G4 ? 0 : gq + 1;
+            }
+            atomicMax(reinterpret_cast<int*>(am) + row, __float_as_int(fmaxf((sig ? 1.f : r[i]) * acc, 0.f)));
+        }
+        const bool beside = 2 * R * (R + 1) <= room_beside;
+        if (!beside) over_k = kRoundsOverK;
+        float* tri = reinterpret_cast<float*>(beside ? smem + sp.total + (state_beside ? rs.total : 0u) : smem + sp.tileK + (state_beside ? 0u : rs.total));
+        if (sig) fill_triangle([&](int j) { return sig + (long long)j * d; }, act, R, d, tri);
+        else fill_triangle([&](int j) { return Vt + (size_t)j * d; }, act, R, d, tri);
+        __syncthreads();
+        if (warp == 0) {
+            const bool ok = picks_cosine<8, true>(lane, R, picks - made, s, act, ar, a.lam, tri, park_key + made, order + made, bound, am, made_holder, am,
+                                                  tie_holder);
+            if (ok && lane == 0) *made_holder = picks - made;
+        }
+        __syncthreads();
+        const int got = *made_holder;
+        for (int t = made + tid; t < made + got; t += kThreads) {
+            const int j = act[order[t]];
+            gain[t] = from_orderable(park_key[t]);
+            order[t] = j;
+            taken[j] = 1;
+        }
+        __syncthreads();
+        made += got;
+        if (made < picks && tid < R) {
+            const int j = act[tid];
+            m[j] = am[tid];
+            seen[j] = (unsigned short)made;
+            key[j] = taken[j] ? 0u : orderable(fmaf(-fmaxf(penalty_rate(a.lam, ar[tid]), 1e-30f), am[tid], fmaxf(s[j], kLowestScore)));
+        }
+        idle = got ? 0 : idle + 1;
+        __syncthreads();
+    }
+    if (made == picks) return kRoundsDone | over_k;
+    for (int j = tid; j < n; j += kThreads) taken[j] = 0;
+    return over_k;
+}
 
 // ---------------------------------------------------------------------------------------------
 // Fused event, tiles resident in shared memory: K and V are read from HBM once and the kept rows
 // are written once. One CTA per (sequence, layer, KV head).
 // ---------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(kThreads, kResidentCtas) event_resident_kernel(const EventArgs a, const __grid_constant__ ScoreTab tab, int extra_bytes) {
+template <typename T, bool PENALTY>
+__global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentCtasTopk) event_resident_kernel(const __grid_constant__ EventArgs a, const __grid_constant__ ScoreTab tab, int extra_bytes) {
     extern __shared__ __align__(16) unsigned char smem[];
     const DevLayout& lay = a.lay;
     const EventId id = decode_event(lay, blockIdx.x);
@@ -130,7 +341,7 @@ __global__ void __launch_bounds__(kThreads, kResidentCtas) event_resident_kernel
     // reciprocal norms: a thread per row, each lane from its own block of eight elements on (different banks). A block's
     // squares in two chains of four, the blocks in eight sums: an error of 4.2e-8 at d = 128, as from sixteen lanes' partial
     // sums; one chain of all squares has 1.6e-7.
-    if (!a.flat_sig) {
+    if (PENALTY && !a.flat_sig) {
         const int nb = d >> 3, half = lane & 4;
         for (int j = tid; j < n; j += kThreads) {
             float u[8] = {};
@@ -161,7 +372,7 @@ __global__ void __launch_bounds__(kThreads, kResidentCtas) event_resident_kernel
     const int picks = min(bud, n);
     // ---- pool + triangle + one-warp loop, when it fits --------------------------------------------------------
     bool done = false, k_tile = true;   // k_tile: the K rows are still in theirs
-    if (a.greedy != 0 && picks > 1) {
+    if (PENALTY && picks > 1) {
         unsigned short* bypool = reinterpret_cast<unsigned short*>(m);
         float* sb_holder = reinterpret_cast<float*>(red);
         int* pool_holder = redi;
@@ -208,47 +419,8 @@ __global__ void __launch_bounds__(kThreads, kResidentCtas) event_resident_kernel
             const float own_r = tid < P && !sig ? r[bypool[tid]] : 1.f;
             __syncthreads();
             if (tid < P) r[tid] = own_r;
-            // raw dot products of every pair of pool rows (i >= j), 8 x 4 at a time: thread x takes blocks x, x + 256, ...;
-            // row band b of eight rows has 2 b + 2 blocks, so it starts at block b (b + 1)
-            const int G4 = d >> 2;  // groups of four elements per row
-            const int bands = (P + 7) >> 3, blocks = bands * (bands + 1);
-            auto block_dots = [&](auto row_of, int bi, int bj, float (&acc)[8][4]) {
-                decltype(row_of(0)) vi[8], vj[4];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) vi[q] = row_of(bypool[min(8 * bi + q, P - 1)]);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) vj[q] = row_of(bypool[min(4 * bj + q, P - 1)]);
-                int gq = tid % G4;
-                for (int c = 0; c < G4; ++c) {
-                    float xj[4][4];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) load4(vj[q] + 4 * gq, xj[q]);
-#pragma unroll
-                    for (int p = 0; p < 8; ++p) {
-                        float xi[4];
-                        load4(vi[p] + 4 * gq, xi);
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) acc[p][q] = fmaf(xi[e], xj[q][e], acc[p][q]);
-                    }
-                    gq = gq + 1 == G4 ? 0 : gq + 1;
-                }
-            };
-            for (int x = tid; x < blocks; x += kThreads) {
-                int bi = (int)sqrtf((float)x);
-                while (bi * (bi + 1) > x) --bi;
-                while ((bi + 1) * (bi + 2) <= x) ++bi;
-                const int bj = x - bi * (bi + 1);
-                float acc[8][4] = {};
-                if (sig) block_dots([&](int j) { return sig + (long long)j * d; }, bi, bj, acc);
-                else block_dots([&](int j) { return (const T*)Vt + (size_t)j * d; }, bi, bj, acc);
-#pragma unroll
-                for (int p = 0; p < 8; ++p)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        if (8 * bi + p < P && 4 * bj + q <= 8 * bi + p) tri[tri_row(8 * bi + p) + 4 * bj + q] = acc[p][q];
-            }
+            if (sig) fill_triangle([&](int j) { return sig + (long long)j * d; }, bypool, P, d, tri);
+            else fill_triangle([&](int j) { return (const T*)Vt + (size_t)j * d; }, bypool, P, d, tri);
             __syncthreads();
             uint32_t* park_key = reinterpret_cast<uint32_t*>(gain);
             if (warp == 0) {
@@ -264,17 +436,23 @@ __global__ void __launch_bounds__(kThreads, kResidentCtas) event_resident_kernel
             }
             __syncthreads();
         } else {
-            for (int j = tid; j < n; j += kThreads) m[j] = 0.f;   // (the list stood there)
+            const int rounds = picks_in_rounds<T>(a, smem, n, picks, orderable(thr), extra_bytes);
+            done = rounds & kRoundsDone;
+            k_tile = !(rounds & kRoundsOverK);
             __syncthreads();
+            if (!done) {
+                for (int j = tid; j < n; j += kThreads) m[j] = 0.f;
+                __syncthreads();
+            }
         }
     }
     if (!done) {
         if (a.flat_sig) {
             StridedRows<float> rows{event_sig(a, id), d};
-            greedy_cta<float>(n, picks, a.lam, a.greedy != 0, d, s, nullptr, m, taken, order, gain, rows, red);
+            greedy_cta<float>(n, picks, a.lam, PENALTY, d, s, nullptr, m, taken, order, gain, rows, red);
         } else {
             StridedRows<T> rows{Vt, d};
-            greedy_cta<T>(n, picks, a.lam, a.greedy != 0, d, s, r, m, taken, order, gain, rows, red);
+            greedy_cta<T>(n, picks, a.lam, PENALTY, d, s, r, m, taken, order, gain, rows, red);
         }
     }
     ordered_indices(n, a.budget, taken, idx);

@@ -644,22 +644,20 @@ static akv_status_t alpha_compress_event_impl(akv_handle_t* h, const akv_layout_
         const int es = lay->dtype == AKV_BF16 ? 2 : 4;
         const SmemPlan res = plan_smem(lay->N, lay->d, es, budget, true, true);
         const int E = a.lay.B * a.lay.L * a.lay.H;
-        // Beside the tiles: as much of a cosine triangle (at most the whole event's) as leaves room for as many CTAs per
-        // SM as without it; a triangle that does not fit there takes the K tile's place.
+        // Beside the tiles, with a penalty: as much of a cosine triangle (at most the whole event's) as leaves room for as
+        // many CTAs per SM as without; a triangle that does not fit there takes the K tile's place.
         const long long whole = (long long)lay->N * (lay->N + 1) / 2 * 4;
         const long long sm_bytes = (long long)h->smem_optin + 1024;   // an SM's shared memory; each CTA takes 1 KB more than it asks for
         long long per_sm = sm_bytes / ((long long)res.total + 1024);
         if (per_sm > kResidentCtas) per_sm = kResidentCtas;
+        if (E <= h->sm_count) per_sm = 1;   // (a second one would not come)
         const long long room = sm_bytes / per_sm - 1024 - (long long)res.total;
-        const int extra = (int)((room < whole ? room : whole) & ~15ll);
+        const int extra = a.greedy ? (int)((room < whole ? room : whole) & ~15ll) : 0;
         const unsigned total = res.total + (unsigned)(extra > 0 ? extra : 0);
-        if (lay->dtype == AKV_BF16) {
-            if ((s = set_smem(event_resident_kernel<__nv_bfloat16>, total)) != AKV_OK) return s;
-            event_resident_kernel<__nv_bfloat16><<<E, kThreads, total, st>>>(a, h->tab, extra > 0 ? extra : 0);
-        } else {
-            if ((s = set_smem(event_resident_kernel<float>, total)) != AKV_OK) return s;
-            event_resident_kernel<float><<<E, kThreads, total, st>>>(a, h->tab, extra > 0 ? extra : 0);
-        }
+        auto kernel = lay->dtype == AKV_BF16 ? (a.greedy ? event_resident_kernel<__nv_bfloat16, true> : event_resident_kernel<__nv_bfloat16, false>)
+                                             : (a.greedy ? event_resident_kernel<float, true> : event_resident_kernel<float, false>);
+        if ((s = set_smem(kernel, total)) != AKV_OK) return s;
+        kernel<<<E, kThreads, total, st>>>(a, h->tab, extra > 0 ? extra : 0);
         return launched("event");
     }
     // The event does not fit on chip: score -> select -> compact as three launches, scores held in

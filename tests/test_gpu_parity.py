@@ -154,6 +154,42 @@ def test_resident_kernel_norms_are_summed_in_a_tree(d):
     assert np.sqrt(np.mean(err ** 2)) < 7e-8
 
 
+@pytest.mark.parametrize("dtype,d,N,budget,lam", [(synth.BF16, 64, 256, 128, 0.5), (synth.BF16, 64, 256, 128, 2.0), (synth.BF16, 96, 192, 64, 2.0),
+                                                  (synth.F32, 64, 256, 128, 2.0), (synth.F32, 40, 192, 64, 2.0), (synth.F32, 64, 430, 64, 4.0),
+                                                  (synth.BF16, 64, 700, 300, 1.0), (synth.BF16, 16, 400, 70, 1.0)])
+@pytest.mark.parametrize("close", [False, True])
+def test_resident_kernel_with_a_pool_larger_than_its_triangle(dtype, d, N, budget, lam, close):
+    """Rounds of active sets, their state beside the tiles or (N = 430) at the head of the K tile; a set too small for them
+    (d = 16, N = 400) leaves the event to the CTA-wide loop. close: scores that differ in their last bits, one event's not at all."""
+    for shape in ((2, 1, 2), (10, 4, 4)):        # one CTA per SM, and two
+        ev = synth.make_plain(*shape, N, d, budget, lam, dtype=dtype, seed=N + d)
+        if close:
+            ev.qstat *= np.float32(1e-6)
+            ev.K[0, 0, 0] = 0
+            ev.V[..., N - N // 4:, :] = ev.V[..., :N // 4, :]
+        g = run_fused(ev, n_cand=[N, N - 5] + [N] * (shape[0] - 2))
+        check_all(ev, g, lam, n_cand=[N, N - 5] + [N] * (shape[0] - 2), events=range(4))
+
+
+@pytest.mark.parametrize("mode", ["flat", "layer"])
+def test_resident_kernel_rounds_on_shared_signatures(mode):
+    ev = synth.make_plain(2, 2, 2, 256, 64, 128, 1.5, dtype=synth.BF16, seed=17)
+    V = dev(ev.V)
+    sig = akv.alpha_signature_flat(V) if mode == "flat" else akv.alpha_signature_layer(V)
+    K, pos = dev(ev.K), dev(ev.pos)
+    opts = akv.Options(lam=1.5, sig_mode=akv.SIG_FLAT if mode == "flat" else akv.SIG_PER_LAYER)
+    sel = akv.alpha_compress_event(K, V, pos, dev(ev.qstat), 128, opts, p_ref=dev(ev.p_ref), flat_sig=sig, want_scores=True)
+    torch.cuda.synchronize()
+    Kn, Vn, pn = akv.to_host_bits(K), akv.to_host_bits(V), pos.cpu().numpy()
+    for b in range(2):
+        for l in range(2):
+            ref = O.signatures_flat(ev.V[b]) if mode == "flat" else O.signatures_per_layer(ev.V[b, l])
+            for h in range(2):
+                chk.check_event(ev.K[b, l, h], ev.V[b, l, h], ev.pos[b, l, h], ev.qstat[l, h], int(ev.p_ref[b]), 128, 1.5,
+                                sel.scores[b, l, h].cpu().numpy(), sel.pick_order[b, l, h].cpu().numpy(),
+                                sel.idx_sorted[b, l, h].cpu().numpy(), Kn[b, l, h], Vn[b, l, h], pn[b, l, h], sig=ref)
+
+
 # ------------------------------------------------------------------ stand-alone entry points
 @pytest.mark.parametrize("dtype", [synth.BF16, synth.F32])
 def test_score_select_compact_chain_equals_fused(dtype):
