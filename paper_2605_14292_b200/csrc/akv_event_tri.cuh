@@ -401,7 +401,9 @@ __device__ __noinline__ void picks_over_whole_pool(const EventArgs& a, unsigned 
     int* holders = reinterpret_cast<int*>(smem + sp.misc + 32);
     const float thr = *reinterpret_cast<const float*>(smem + sp.misc + 56);
     const __nv_bfloat16* Vg = reinterpret_cast<const __nv_bfloat16*>(a.V);
-    auto vrow_of = [&](int j) { return Vg + row_offset(lay, id.b, id.l, id.h, j); };
+    const bool dense = lay.page_size == 0;
+    const __nv_bfloat16* Ve = Vg + (dense ? id.b * lay.sb + id.l * lay.sl + id.h * lay.sh : 0);
+    auto vrow_of = [&](int j) { return dense ? Ve + (long long)j * lay.sn : Vg + row_offset(lay, id.b, id.l, id.h, j); };
     float* rowbuf = reinterpret_cast<float*>(tile);
     const float* m_act = reinterpret_cast<const float*>(tile + kContMact);   // by old pool row (from the loop)
     float* m_slot = reinterpret_cast<float*>(tile + kContScratch);           // by slot
@@ -459,9 +461,8 @@ __device__ __noinline__ void picks_over_whole_pool(const EventArgs& a, unsigned 
     __syncthreads();
     for (int t = tid; t < made; t += kTcThreads) order[t] = inv[chosen[t]];
     __syncthreads();
-    auto dot = [&](int i, int c) -> float {   // of two pool rows
+    auto dot = [&](int i, const __nv_bfloat16* vi, int c) -> float {   // of two pool rows (vi: row i's values)
         if (G) return G[(long long)bypool[i] * lay.N + bypool[c]];
-        const __nv_bfloat16* vi = vrow_of(bypool[i]);
         const __nv_bfloat16* vc = vrow_of(bypool[c]);
         float acc = 0.f;
 #pragma unroll 4
@@ -479,7 +480,7 @@ __device__ __noinline__ void picks_over_whole_pool(const EventArgs& a, unsigned 
     const int pairs = *n_left * made;
     for (int x = tid; x < pairs; x += kTcThreads) {
         const int c = left[x / made], i = order[x % made];
-        const float v = fmaxf(r[i] * dot(i, c), 0.f);
+        const float v = fmaxf(r[i] * dot(i, vrow_of(bypool[i]), c), 0.f);
         atomicMax(reinterpret_cast<int*>(m_init) + c, __float_as_int(v));
     }
     __syncthreads();
@@ -509,7 +510,8 @@ __device__ __noinline__ void picks_over_whole_pool(const EventArgs& a, unsigned 
         __syncthreads();
         const int irho = holders[1];
         // row irho of the cosine matrix
-        for (int rho = tid; rho < P; rho += kTcThreads) rowbuf[rho] = dot(irho, rho);
+        const __nv_bfloat16* vpick = vrow_of(bypool[irho]);
+        for (int rho = tid; rho < P; rho += kTcThreads) rowbuf[rho] = dot(irho, vpick, rho);
         __syncthreads();
         if (warp == 0) {
             const float ri = r[irho];
