@@ -259,10 +259,13 @@ __global__ void __launch_bounds__(kThreads) compact_kernel(const CompactArgs a) 
 // Eq. 1: shared signatures. u = mean over (l, h) of the V rows of one (sequence, slot), v = u / (||u|| + eps),
 // written as fp32 [B, N, d]; per_layer: one signature per (sequence, layer, slot), the mean runs over the heads
 // of that layer only, written as fp32 [B, L, N, d]. One CTA per (group, 32 / G slots), G = lanes per row: its
-// eight warps split the (layer, head) pairs among themselves (every thread has a dozen independent 16-byte
-// loads in flight), partial sums meet in shared memory in a fixed order.
+// eight warps split the (layer, head) pairs among themselves, partial sums meet in shared memory in a fixed order.
+// AHEAD: rows that a warp requests before it adds the first, and those that are left one by one. Four where every warp
+// has four (32 pairs or more): 16 sequences of 112 pairs, 256 slots 37.2 -> 31.9 us (eight: 33 to 39, and half of the
+// resident warps); with fewer pairs one, which needs the fewest registers (4 pairs per layer: 196 us, with eight 292).
 // ---------------------------------------------------------------------------------------------
-template <typename T>
+constexpr int kSigAhead = 4;
+template <typename T, int AHEAD>
 __global__ void __launch_bounds__(kThreads) flat_signature_kernel(const DevLayout lay, const void* V, const int* n_cand,
                                                                  float eps, float* out, int per_layer) {
     __shared__ float part[kWarps][32][8];
@@ -284,20 +287,24 @@ __global__ void __launch_bounds__(kThreads) flat_signature_kernel(const DevLayou
     const int pairs = (l1 - l0) * lay.H;
     float u[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     if (act) {
-        // eight rows requested before the first is added (in the order of the pairs)
-        for (int p0 = warp; p0 < pairs; p0 += 8 * kWarps) {
-            float x[8][8];
+        auto row = [&](int p) { return Vg + row_offset(lay, b, l0 + p / lay.H, p % lay.H, j) + lig * 8; };
+        int p = warp;
+        if constexpr (AHEAD > 1) {
+            for (; p + (AHEAD - 1) * kWarps < pairs; p += AHEAD * kWarps) {
+                float x[AHEAD][8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int p = min(p0 + i * kWarps, pairs - 1);
-                load8(Vg + row_offset(lay, b, l0 + p / lay.H, p % lay.H, j) + lig * 8, x[i]);
-            }
+                for (int i = 0; i < AHEAD; ++i) load8(row(p + i * kWarps), x[i]);
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if (p0 + i * kWarps < pairs) {
+                for (int i = 0; i < AHEAD; ++i)
 #pragma unroll
                     for (int q = 0; q < 8; ++q) u[q] += x[i][q];
-                }
+            }
+        }
+        for (; p < pairs; p += kWarps) {
+            float x[8];
+            load8(row(p), x);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) u[q] += x[q];
         }
     }
 #pragma unroll

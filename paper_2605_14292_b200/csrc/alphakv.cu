@@ -511,8 +511,10 @@ static akv_status_t alpha_signature_flat_impl(akv_handle_t* h, const akv_layout_
     if (blocks > INT_MAX) return fail(AKV_ERR_UNSUPPORTED, "alpha_signature: %lld blocks exceed the grid limit", blocks);
     const unsigned grid = (unsigned)blocks;
     cudaStream_t st = (cudaStream_t)stream;
-    if (y.dtype == AKV_BF16) flat_signature_kernel<__nv_bfloat16><<<grid, kThreads, 0, st>>>(y, V, n_cand, opt->eps, flat_sig, per_layer);
-    else flat_signature_kernel<float><<<grid, kThreads, 0, st>>>(y, V, n_cand, opt->eps, flat_sig, per_layer);
+    const bool many = (per_layer ? 1 : y.L) * y.H >= kSigAhead * kWarps;
+    auto kernel = y.dtype == AKV_BF16 ? (many ? flat_signature_kernel<__nv_bfloat16, kSigAhead> : flat_signature_kernel<__nv_bfloat16, 1>)
+                                      : (many ? flat_signature_kernel<float, kSigAhead> : flat_signature_kernel<float, 1>);
+    kernel<<<grid, kThreads, 0, st>>>(y, V, n_cand, opt->eps, flat_sig, per_layer);
     return launched(per_layer ? "layer_signature" : "flat_signature");
 }
 

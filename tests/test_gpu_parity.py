@@ -590,6 +590,20 @@ def test_chained_and_fresh_scores_agree_on_the_tensor_memory_kernels():
 
 
 # ------------------------------------------------------------------ shared signatures with one cosine matrix per sequence
+@pytest.mark.parametrize("L,H", [(1, 1), (1, 31), (4, 8), (3, 11), (9, 7), (1, 64), (5, 13)])
+@pytest.mark.parametrize("dtype", [synth.BF16, synth.F32])
+def test_signatures_over_any_number_of_pairs(dtype, L, H):
+    """Rows requested four at a time from 32 (layer, head) pairs on, and a remainder one by one. fp32 sums of unit-scale rows:
+    a unit row is within 1e-6 of the float64 one."""
+    ev = synth.make_plain(2, L, H, 37, 64, 5, 0.5, dtype=dtype, seed=L * H)
+    V = dev(ev.V)
+    flat, layer = akv.alpha_signature_flat(V).cpu().numpy(), akv.alpha_signature_layer(V).cpu().numpy()
+    for b in range(2):
+        assert np.max(np.abs(flat[b] - O.signatures_flat(ev.V[b]))) < 1e-6
+        for l in range(L):
+            assert np.max(np.abs(layer[b, l] - O.signatures_per_layer(ev.V[b, l]))) < 1e-6
+
+
 @pytest.mark.parametrize("mode", ["flat", "layer"])
 @pytest.mark.parametrize("N", [96, 256, 300])
 def test_shared_cosine_matrix(mode, N):
