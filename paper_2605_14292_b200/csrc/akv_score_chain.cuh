@@ -180,13 +180,19 @@ __global__ void __launch_bounds__(kThreads, 3) score_rows_kernel(const EventArgs
     __syncthreads();
     const int f0 = (lane & 7) * 8;
     ChainScore ca, cb;   // (their rotations only, no chain)
+    if (!rotate) {       // keys that are rotated already: the statistic itself, for every row
+        ca.anchor(0, gtab + f0, phitab + f0, sect);
+        cb = ca;
+    }
     int bad = 0;
     for (int st = 0; 64 * st < rows; ++st) {
         uint4 next[4];
         if (64 * (st + 1) < rows) request(st + 1, next);
         const int ja = 64 * st + ja0, jb = ja + 32;
-        ca.anchor(pref - (long long)spos[min(ja, rows - 1)], gtab + f0, phitab + f0, sect);
-        cb.anchor(pref - (long long)spos[min(jb, rows - 1)], gtab + f0, phitab + f0, sect);
+        if (rotate) {
+            ca.anchor(pref - (long long)spos[min(ja, rows - 1)], gtab + f0, phitab + f0, sect);
+            cb.anchor(pref - (long long)spos[min(jb, rows - 1)], gtab + f0, phitab + f0, sect);
+        }
         const float acca = ca.dot4(cur[0], cur[1]), accb = cb.dot4(cur[2], cur[3]);
         // both rows' sums in three exchanges: lanes 0..3 of a group go on with the first, lanes 4..7 with the second
         const bool second = lane & 4;
