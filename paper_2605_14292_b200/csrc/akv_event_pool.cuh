@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
     const int nb = (product && P > 128) ? P - 128 : 0;
     const int ncols = max((P + 15) & ~15, 16), base2 = ncols - 128;   // (a shape with no columns is not allowed)
     if (product) {
-        if (tid == 0) {
+        if (tid == 0 && (FUSED || !a.starve)) {
             tc_fence_after();
             const uint32_t idesc = umma_idesc_bf16(128, ncols);
 #pragma unroll
@@ -399,6 +399,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
     timeout = __syncthreads_or(timeout);  // also: the product has read the whole tile before the triangle lands on it
     if (timeout) {
         if (tid == 0 && a.status) a.status[id.e] = 3;
+        if (!FUSED) select_gave_up(a, id.e, kTcThreads);
         if (have_tmem && warp == 0) tmem_dealloc(tbase, kPoolCols);
         return;
     }

@@ -507,7 +507,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
                 work_barrier();   // the columns have been read
                 tc_fence_after();
             }
-            if (tid == 0) {
+            if (tid == 0 && (FUSED || !a.starve)) {
                 product(0, 0, ncols, 0u);
                 // the second block against rows 128.. gives their cosines against one another; those against rows < 128
                 // are those rows' columns from 128 on
@@ -519,6 +519,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
             if (cnt[0]) {
                 if (warp == 0) tmem_dealloc(tbase, kPfCols);
                 if (tid == 0 && a.status) a.status[id.e] = 3;
+                if (!FUSED) select_gave_up(a, id.e, kStWork);
                 return;
             }
             // lower triangle -> shared memory: warps 0..3 the first product's columns up to the row itself, warps 4..7 its

@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(kTcThreads, 4) event_tc_kernel(const EventArgs
 
     phase_stamp(id.e, 3);
     const bool do_mma = use_tc && picks > 1;
-    if (do_mma && tid == 0) {
+    if (do_mma && tid == 0 && (FUSED || !a.starve)) {
         tc_fence_after();
         const uint32_t idesc = umma_idesc_bf16(128, ncols);
 #pragma unroll 1
@@ -468,6 +468,7 @@ __global__ void __launch_bounds__(kTcThreads, 4) event_tc_kernel(const EventArgs
     timeout = __syncthreads_or(timeout);
     if (timeout) {
         if (tid == 0 && a.status) a.status[id.e] = 3;
+        if (!FUSED) select_gave_up(a, id.e, kTcThreads);
         if (use_tc && warp == 0) tmem_dealloc(tbase, tcols);
         return;
     }

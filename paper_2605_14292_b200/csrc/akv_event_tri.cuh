@@ -803,7 +803,7 @@ __global__ void __launch_bounds__(kTcThreads) event_tri_kernel(const __grid_cons
     }
     phase_stamp(id.e, 4);
     if (similarity) {
-        if (tid == 0) {
+        if (tid == 0 && (FUSED || !a.starve)) {
             tc_fence_after();
             const uint32_t idesc = umma_idesc_bf16(128, max((P + 15) & ~15, 16));   // (a shape with no columns is not allowed)
 #pragma unroll
@@ -819,6 +819,7 @@ __global__ void __launch_bounds__(kTcThreads) event_tri_kernel(const __grid_cons
     timeout = __syncthreads_or(timeout);  // also: the product has read the whole tile before the triangle lands on it
     if (timeout) {
         if (tid == 0 && a.status) a.status[id.e] = 3;
+        if (!FUSED) select_gave_up(a, id.e, kTcThreads);
         if (use_tc && warp == 0) tmem_dealloc(tbase, kTcCols);
         return;
     }

@@ -25,7 +25,7 @@ struct EventArgs {
     int no_chain;           // testing aid: score every row from scratch even when positions are regular
     int gqa_group;          // query statistics per KV head (>= 1)
     int gqa_max;            // 1: a key's score is the largest over the group, 0: their mean
-    int starve;             // testing aid: request no K row, so that the bounded waits run out
+    int starve;             // testing aid: request no K row and, where there is no K to read, issue no product, so that the bounded waits run out
     int wait_polls;         // polls after which a bounded wait gives up
     int* idx_sorted;
     int* pick_order;
@@ -45,6 +45,12 @@ __device__ __forceinline__ int event_budget(const EventArgs& a, const EventId& i
     if (!a.head_budgets) return a.budget;
     const int b = a.head_budgets[id.l * a.lay.H + id.h];
     return b < 1 ? 1 : (b > a.budget ? a.budget : b);
+}
+// What a selection by itself leaves when one of its bounded waits gave up: status 3 and no row, so that a compaction that
+// follows moves none (the fused kernels leave the cache alone themselves).
+__device__ __forceinline__ void select_gave_up(const EventArgs& a, int e, int threads) {
+    for (int t = threadIdx.x; t < a.budget; t += threads) a.idx_sorted[(long long)e * a.budget + t] = -1;
+    if (threadIdx.x == 0 && a.n_kept) a.n_kept[e] = 0;
 }
 // shared signature rows of this event's (sequence, layer)
 __device__ __forceinline__ const float* event_sig(const EventArgs& a, const EventId& id) {

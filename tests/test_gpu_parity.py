@@ -386,6 +386,22 @@ def test_reference_position_behind_some_keys():
     check_all(ev, g, ev.lam)
 
 
+@pytest.mark.parametrize("N,budget", [(192, 64), (256, 128), (256, 140), (1000, 100)])
+def test_a_selection_that_gives_up_lists_no_row(N, budget):
+    """With the starve flag alpha_select issues no product: its waits run out, it reports status 3 and lists no row, and the
+    compaction behind it (the three launches of the static variant) leaves the cache alone."""
+    ev = synth.make_plain(1, 2, 2, N, 128, budget, 0.5, dtype=synth.BF16, seed=N)
+    K, V, pos, q, pref = dev(ev.K), dev(ev.V), dev(ev.pos), dev(ev.qstat), dev(ev.p_ref)
+    opts = akv.Options(lam=0.5, flags=akv.FLAG_TEST_STARVE_WAIT)
+    s = akv.alpha_score(K, q, pos=pos, p_ref=pref, opts=opts)
+    sel = akv.alpha_select(s, V, budget, opts, layout=akv.Layout.dense(V))
+    assert bool((sel.status == 3).all()) and bool((sel.idx_sorted == -1).all()) and bool((sel.n_kept == 0).all())
+    sel = akv.alpha_compress_event_static(K, V, pos, q, budget, opts, p_ref=pref)
+    assert bool((sel.status == 3).all())
+    for x, name in ((akv.to_host_bits(K), "K"), (akv.to_host_bits(V), "V"), (pos.cpu().numpy(), "pos")):
+        assert np.array_equal(x, getattr(ev, name))
+
+
 # ------------------------------------------------------------------ per-layer signatures, per-head budgets (Section 6)
 @pytest.mark.parametrize("dtype,N,d", [(synth.BF16, 80, 128), (synth.F32, 600, 64)])
 def test_per_layer_signature_mode(dtype, N, d):
