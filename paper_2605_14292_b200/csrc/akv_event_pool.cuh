@@ -1,12 +1,12 @@
 // Event kernel for bf16, d = 128, per-head signatures, N <= 256 and budgets up to 128 (the shapes of the
 // Qwen-7B-shaped batch and of the decode cadence: 256 candidates -> 128). Same structure as event_tri_kernel
-// (K rows scored from a 128-row tile, pool by bisection, cosine matrix on tcgen05, its lower triangle in shared
+// (K rows scored from shared memory, here all of them at once, pool by bisection, cosine matrix on tcgen05, its lower triangle in shared
 // memory, Algorithm 1 as a one-warp loop), for an ACTIVE SET instead of the whole pool:
 //
 //   The picks hardly ever reach beyond the best-scored few dozen rows past the budget. The cosine matrix is
-//   therefore formed only for the pool's best-scored rows, at most 180 of them (64 KB of triangle: three CTAs
-//   per SM), and only their V rows are read. Every candidate left out scores at most `bound`, the 181st largest
-//   key, and its Eq. 2 value never exceeds its score: the loop over the active set is exact as long as its
+//   therefore formed only for the pool's best-scored rows, 158 to 180 of them (64 KB of triangle: three CTAs
+//   per SM), and only their V rows are read. Every candidate left out scores at most `bound` (see active_bound),
+//   and its Eq. 2 value never exceeds its score: the loop over the active set is exact as long as its
 //   winning value stays above that bound. In the rare event where it does not, the picks made so far stand and
 //   the remaining ones (a few, as a rule) are taken over the whole pool with rows of the cosine matrix as plain
 //   dot products, starting from the running maxima the loop had reached.
@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
         tc_fence_after();
     }
     phase_stamp(id.e, 4);
-    // large size, rows from 128 on (nb of them): a second product, the last 128 rows of the operand against those
+    // rows from 128 on (nb of them): a second product, the last 128 rows of the operand against those
     // rows, gives their cosines against one another; what lies left of column 128 comes from the first product
     // by symmetry
     const bool product = similarity && !G;  // the cosine matrix comes off the tensor core
@@ -535,7 +535,8 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
             *reinterpret_cast<uint4*>(Kg + off) = *reinterpret_cast<const uint4*>(src);
             *reinterpret_cast<uint4*>(Vg + off) = *reinterpret_cast<const uint4*>(src + 16384);
         }
-    } else if ((unsigned)picks * 512u <= kPoolTileBytes) {
+    } else {
+        static_assert(128u * 512u <= kPoolTileBytes, "the kept rows of the largest budget fit the tile");
         // The tile holds the kept rows of K and of V side by side: one round of 16-byte gathers, one barrier.
         // Stores: slots 0..picks-1 are contiguous in a dense cache (and page by page in a paged one), so one
         // thread writes them back with a few bulk copies. (Gathering by one bulk copy per row measured slower.)
@@ -566,18 +567,6 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
                 copy16(reinterpret_cast<char*>(Kg + off), tile + x * 16);
                 copy16(reinterpret_cast<char*>(Vg + off), tile + vhalf + x * 16);
             }
-        }
-    } else {
-#pragma unroll 1
-        for (int pass = 0; pass < 2; ++pass) {
-            __nv_bfloat16* X = pass ? Vg : Kg;
-            __syncthreads();  // the tile is free (greedy loop, or the previous pass, is done with it)
-            for (int x = tid; x < picks * 16; x += kTcThreads)
-                cp_async16(tile_u32 + (uint32_t)x * 16u, X + rowoff(idx[x >> 4]) + (x & 15) * 8);
-            cp_async_wait_all();
-            __syncthreads();
-            for (int x = tid; x < picks * 16; x += kTcThreads)
-                copy16(reinterpret_cast<char*>(X + rowoff(x >> 4)) + (x & 15) * 16, tile + x * 16);
         }
     }
     if (wpos)

@@ -1,14 +1,13 @@
-// One-launch event kernel for large candidate pools (bf16, d = 128, per-head signatures, N beyond the
-// 256 rows that the other tensor-memory kernels hold): prefill compression, N = 4096 -> budget 128.
-// One CTA of nine warps per event.
+// One-launch event kernel for large candidate pools (bf16, d = 128, per-head signatures, N > 256) that
+// event_prefill_kernel does not take: N > 5120, or budgets above 128. One CTA of nine warps per event.
 //
-//   1. K streams through a ring of eight 64-row stages (cp.async.bulk + full/empty mbarriers, one
-//      producer warp, eight scoring warps); every row is scored as it lands and only its score stays
-//      on chip. K is read from HBM exactly once.
+//   1. K streams through a ring of eight 64-row stages (four from about N = 5040 on, where the scores take
+//      their place; cp.async.bulk + full/empty mbarriers, one producer warp, eight scoring warps); every row is scored
+//      as it lands and only its score stays on chip. K is read from HBM exactly once.
 //   2. s_(b) by a radix-4 bisection over the score keys (all eight warps), then either the top-k
 //      flags (lambda = 0) or the pool of candidates that can ever be an arg-max of Eq. 2
 //      (s_i >= s_(b) - lambda (1 + slack), see akv_select_pool.cuh), in slot order.
-//   3. Only the pool's V rows are read (about 350 of 4096 at lambda = 0.5), into a K-major,
+//   3. Only the pool's V rows are read (about 350 of 4096 random rows at lambda = 0.5), into a K-major,
 //      128-byte-swizzled operand tile in shared memory.
 //   4. Algorithm 1 over the pool, every thread owning up to four candidates (score, norm and running
 //      maximum in registers). After a pick, the cosines of the picked row against the whole pool are

@@ -9,9 +9,9 @@
 //      (the running maximum m never exceeds 1, so every still unchosen member of the top-b scores
 //      beats the others). s_(b) comes from a bisection over the score keys; that pool of P rows,
 //      in slot order, is the only part of V that is read for the selection.
-//      A pool of more than 127 rows (a strong penalty) is cut to its best-scored ones, the active set; no candidate
-//      left out scores above `bound`, so the loop is exact while its winning values stay above that, and the rare event
-//      where one does not is finished by picks_over_whole_pool.
+//      A pool of more than 127 rows (a strong penalty) is cut to its best-scored ones, the active set (112 to 127 rows);
+//      no candidate left out scores above `bound`, so the loop is exact while its winning values stay above that, and
+//      the rare event where one does not is finished by picks_over_whole_pool.
 //   3. The pool's V rows form a K-major, 128-byte-swizzled operand tile, one
 //      tcgen05.mma sequence writes the pool's cosine matrix (raw dot products, fp32) into tensor
 //      memory, and the four warps move its lower triangle to shared memory (tcgen05.ld), taking
@@ -35,11 +35,11 @@ struct TriSmem {
     unsigned tile, s, key, spos, bypool, taken, order, gain, idx, sect, misc, total;
 };
 // Layout after the 1024-byte aligned base. `key` (score keys) and `r` (reciprocal norms) share storage.
-__host__ __device__ inline TriSmem plan_tri_smem(int N, int budget) {
+__host__ __device__ inline TriSmem plan_event_smem(int N, int budget, unsigned tile_bytes) {
     TriSmem p;
     const unsigned np = (unsigned)((N + 3) & ~3);
     unsigned o = 0;
-    p.tile = o;   o += kTriTileBytes;
+    p.tile = o;   o += tile_bytes;
     p.s = o;      o += align16(np * 4);
     p.key = o;    o += align16(np * 4);
     p.spos = o;   o += align16(np * 4);
@@ -50,10 +50,11 @@ __host__ __device__ inline TriSmem plan_tri_smem(int N, int budget) {
     p.idx = o;    o += align16((unsigned)budget * 4);
     if (o - p.bypool < 1024u) o = p.bypool + 1024u;  // bypool..idx also hold the folded statistic and the phase steps (1 KB) while scoring
     p.sect = o;   o += 256;       // cosine and sine of the 32 sector angles
-    p.misc = o;   o += 64;        // mbarriers (K, product, late K rows), tmem base, pool size, block-max scratch
+    p.misc = o;   o += 64;        // mbarriers (K, product, late K rows), tmem base, pool size, bound, threshold, block-max scratch
     p.total = o + 1024;           // room to align the base to 1024 bytes
     return p;
 }
+__host__ __device__ inline TriSmem plan_tri_smem(int N, int budget) { return plan_event_smem(N, budget, kTriTileBytes); }
 
 // event_pool_kernel's (akv_event_pool.cuh): a tile of 64 KB, for a whole event's K rows, then the triangle of an active set of up to 180 rows (see the kernel);
 // three CTAs per SM.
@@ -62,26 +63,7 @@ constexpr int kPoolActive = 180;            // most rows whose cosine matrix goe
 constexpr uint32_t kPoolCols = 256u;        // tensor-memory columns (a power of two >= the matrix's columns)
 constexpr int kPoolCpl = 6;                 // candidates per lane of the one-warp loop
 
-// Layout after the 1024-byte aligned base. `key` (score keys) and `r` (reciprocal norms) share storage.
-__host__ __device__ inline TriSmem plan_pool_event_smem(int N, int budget) {
-    TriSmem p;
-    const unsigned np = (unsigned)((N + 3) & ~3);
-    unsigned o = 0;
-    p.tile = o;   o += kPoolTileBytes;
-    p.s = o;      o += align16(np * 4);
-    p.key = o;    o += align16(np * 4);
-    p.spos = o;   o += align16(np * 4);
-    p.bypool = o; o += align16(np * 2);
-    p.taken = o;  o += align16(np);
-    p.order = o;  o += align16((unsigned)budget * 4);
-    p.gain = o;   o += align16((unsigned)budget * 4);
-    p.idx = o;    o += align16((unsigned)budget * 4);
-    if (o - p.bypool < 1024u) o = p.bypool + 1024u;  // bypool..idx also hold the folded statistic and the phase steps (1 KB) while scoring
-    p.sect = o;   o += 256;       // cosine and sine of the 32 sector angles
-    p.misc = o;   o += 64;        // mbarriers (K, product, late K rows), tmem base, pool size, block-max scratch
-    p.total = o + 1024;           // room to align the base to 1024 bytes
-    return p;
-}
+__host__ __device__ inline TriSmem plan_pool_event_smem(int N, int budget) { return plan_event_smem(N, budget, kPoolTileBytes); }
 
 // 32 consecutive columns of this thread's TMEM lane.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {

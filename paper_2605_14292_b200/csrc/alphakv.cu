@@ -338,7 +338,7 @@ static akv_status_t launch_tc(akv_handle* h, const EventArgs& a0, cudaStream_t s
 // maximum takes the general kernels.
 static bool tri_path_ok(const EventArgs& a) { return tc_path_ok(a) && (a.lay.N <= 128 || a.budget <= 64); }
 static bool tri_big_ok(const EventArgs& a) { return tc_path_ok(a) && !tri_path_ok(a) && a.budget <= 128; }
-// shared signatures with their cosine matrix at hand: the large size, which gathers its triangle from that matrix
+// shared signatures with their cosine matrix at hand: event_pool_kernel, which gathers its triangle from that matrix
 static bool pool_shared_ok(const EventArgs& a) {
     return a.gram != nullptr && a.lay.dtype == AKV_BF16 && a.lay.d == kTcD && a.lay.N <= kTcMaxN && a.budget <= 128 && !a.gqa_max;
 }
@@ -539,9 +539,9 @@ static akv_status_t kv_compact_impl(akv_handle_t* h, const akv_layout_t* lay, vo
     return launch_compact(h, a, (cudaStream_t)stream);
 }
 
-// Which kernels the fused call runs for a shape: the two tensor-memory kernels (bf16, d = 128, N <= 256,
-// per-head signatures), the resident kernel when an event's K and V tiles fit in shared memory, else
-// three launches with the scores in global memory.
+// Which kernels the fused call runs for a shape: one of the tensor-memory kernels (bf16, d = 128, per-head signatures or a
+// shared cosine matrix), the resident kernel when an event's K and V tiles fit in shared memory, else three launches with the
+// scores in global memory.
 enum EventRoute { ROUTE_TRI, ROUTE_TRI_BIG, ROUTE_TC, ROUTE_PREFILL, ROUTE_STREAM, ROUTE_RESIDENT, ROUTE_THREE };
 // shared memory the streaming kernel may plan with: what the device allows minus its static arrays
 static int stream_smem_limit(int smem_optin) { return smem_optin - 1024; }
@@ -573,7 +573,6 @@ extern "C" akv_status_t akv_workspace_bytes(const akv_layout_t* lay, int32_t bud
     if ((s = check_budget(budget, lay->N)) != AKV_OK) return s;
     a.budget = budget;
     a.greedy = (opt->lambda > 0.f || (opt->flags & AKV_FLAG_FORCE_GREEDY)) ? 1 : 0;
-    a.lam = opt->lambda;
     // only whether shared signatures are in use matters for the route, not where they live
     a.flat_sig = opt->sig_mode != AKV_SIG_PER_HEAD ? reinterpret_cast<const float*>(bytes) : nullptr;
     a.gram = opt->sig_mode != AKV_SIG_PER_HEAD ? opt->shared_gram : nullptr;

@@ -100,12 +100,12 @@ def make_plain(B, L, H, N, d, budget, lam, dtype=BF16, seed=0, name="plain") -> 
 
 
 def make_c1(seed=0) -> EventBatch:
-    """configs[0]: a single (layer, KV head), fp32, N=192 -> b=64, lambda=0.5."""
+    """C1: a single (layer, KV head), fp32, N=192 -> b=64, lambda=0.5."""
     return make_plain(1, 1, 1, 192, 128, 64, 0.5, dtype=F32, seed=seed, name="C1-single-fp32")
 
 
 def make_c2(seed=0, B=1, L=28, H=4) -> EventBatch:
-    """configs[1]: Qwen-7B-shaped, bf16, per-channel scale U(0.5,2) drawn per
+    """C2: Qwen-7B-shaped, bf16, per-channel scale U(0.5,2) drawn per
     (layer, head) separately for K and V, N=256 -> b=128."""
     N, d = 256, 128
     rng = np.random.default_rng(seed)
@@ -120,7 +120,7 @@ def make_c2(seed=0, B=1, L=28, H=4) -> EventBatch:
 
 
 def make_c3(seed=0, B=16, L=32, H=8, N=192, budget=64, dup_frac=0.05, noise=0.01) -> EventBatch:
-    """configs[2]: Llama-8B-shaped, bf16, batch 16, N=192 -> b=64. In every event
+    """C3: Llama-8B-shaped, bf16, batch 16, N=192 -> b=64. In every event
     round(dup_frac*N) V rows are overwritten by another row's V plus N(0, noise^2)
     before bf16 rounding (K untouched), which makes the redundancy penalty bite."""
     d = 128
@@ -140,14 +140,14 @@ def make_c3(seed=0, B=16, L=32, H=8, N=192, budget=64, dup_frac=0.05, noise=0.01
 
 
 def make_c4(seed=0, B=8, L=28, H=4, N=4096, lam=0.5) -> EventBatch:
-    """configs[3]: large candidate pool (prefill compression), Qwen-7B shape,
+    """C4: large candidate pool (prefill compression), Qwen-7B shape,
     N=4096 -> b=128, lambda in {0, 0.5, 1.0} chosen by the caller."""
     return make_plain(B, L, H, N, 128, 128, lam, dtype=BF16, seed=seed, name="C4-large-pool")
 
 
 @dataclass
 class PagedCadence:
-    """configs[4]: decode-cadence stress in a fixed-size paged KV buffer.
+    """C5: decode-cadence stress in a fixed-size paged KV buffer.
 
     pool_K / pool_V: uint16 (bf16 bits) [L, n_pages, H, page, d].
     block_table: int32 [B, pages_per_seq]; slot n of sequence b lives in page

@@ -1,4 +1,4 @@
-"""(1) The stored oracle outputs for configs[0] still come out of the oracle.
+"""(1) The stored oracle outputs for the single event (C1) still come out of the oracle.
 (2) The pins have teeth: plausible mistakes planted in a copy of the selection
 loop (on the CPU, in this file) are each caught by one of the closed-form pins."""
 import json
