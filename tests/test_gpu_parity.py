@@ -1,4 +1,7 @@
 """GPU-vs-oracle parity, through the C ABI (via the thin binding), element by element."""
+import os
+import re
+
 import numpy as np
 import pytest
 import torch
@@ -501,8 +504,9 @@ def test_score_with_more_events_than_a_grid_dimension_holds():
 @pytest.mark.parametrize("N,budget,lam", [(257, 40, 0.5), (300, 128, 0.0), (1000, 64, 0.5), (1000, 100, 1.5), (2050, 128, 1.0), (5041, 128, 1.0),
                                           (5042, 128, 1.0), (9000, 128, 1.0)])
 def test_large_pool_stream_kernel(N, budget, lam):
-    """bf16, d = 128, N > 256: K streams through a ring, scores stay on chip, pool rows of V only. Ragged
-    candidate counts put the end of an event inside a ring stage, at its edge, and below the budget."""
+    """bf16, d = 128, N > 256: K streams through a ring, scores stay on chip, pool rows of V only (up to N = 5120 in the
+    prefill kernel, beyond in the stream kernel). Ragged candidate counts put the end of an event inside a ring stage, at
+    its edge, and below the budget."""
     ev = synth.make_c3(seed=N, B=4, L=1, H=2, N=N, budget=budget)
     before = akv.launch_count()
     g = run_fused(ev, lam=lam)
@@ -514,7 +518,7 @@ def test_large_pool_stream_kernel(N, budget, lam):
 
 
 def test_large_pool_stream_kernel_variants():
-    """Same kernel: no pruning (the pool outgrows the on-chip tile, the rest of V is read in place), the greedy
+    """The prefill kernel: no pruning (the pool outgrows the active set), the greedy
     loop forced at lambda = 0, per-head budgets, irregular positions with the default reference position, every
     row scored from scratch, and the bounded waits running out."""
     ev = synth.make_c3(seed=71, B=2, L=2, H=2, N=900, budget=48)
@@ -541,8 +545,8 @@ def test_large_pool_stream_kernel_variants():
 
 @pytest.mark.parametrize("N,budget", [(700, 128), (1500, 128)])
 def test_large_pool_active_set_bound_reached(N, budget):
-    """Every V row exists twice and the penalty is strong: the loop over the best-scored rows reaches its bound and the
-    event is redone over the whole pool, which at N = 1500 outgrows the operand tile."""
+    """Every V row exists twice and the penalty is strong: the prefill kernel's loop over the best-scored rows reaches its
+    bound and goes on with further active sets."""
     ev = synth.make_plain(2, 1, 2, N, 128, budget, 2.0, dtype=synth.BF16, seed=N)
     ev.V[..., N // 2:, :] = ev.V[..., :N // 2, :]
     check_all(ev, run_fused(ev), ev.lam)
@@ -552,8 +556,8 @@ def test_large_pool_active_set_bound_reached(N, budget):
                                                   (5120, 128, 0.3, True), (5121, 128, 1.0, False), (1000, 1, 1.0, False), (300, 128, 1e-9, True)])
 def test_prefill_sized_pool_beyond_the_active_set(N, budget, scale, twice):
     """Two events per SM, an active set of 192 rows. Statistics scaled down (scores then differ less than the penalty) and
-    every V row twice send the picks beyond it, to one or many more rounds with further active sets; where more than 192
-    scores are equal no round makes a pick, and the plain route over the whole pool takes over."""
+    every V row twice send the picks beyond it, to one or many more rounds with further active sets, also where more than
+    192 scores are equal."""
     ev = synth.make_plain(2, 1, 2, N, 128, budget, 0.5, dtype=synth.BF16, seed=N + budget)
     ev.qstat[...] *= scale
     if twice:
@@ -574,6 +578,88 @@ def test_prefill_sized_pool_beyond_the_active_set(N, budget, scale, twice):
             rep = O.replay_pick_order(sn[b, 0, h].astype(np.float64), O.signatures_per_head(ev.V[b, 0, h], ev.eps), 0.5,
                                       order[b, 0, h].astype(np.int64), chk.MARGIN_TOL)
             assert rep.ok, rep.log[:3]
+
+
+def _takes_stream_kernel(N, budget):
+    """bf16, d = 128, per-head signatures: what the prefill kernel's limits leave"""
+    text = open(os.path.join(os.path.dirname(akv.__file__), "csrc", "akv_event_prefill.cuh")).read()
+    limit = {k: int(re.search(r"constexpr int %s = (\d+);" % k, text).group(1)) for k in ("kPfMaxN", "kPfMaxBudget")}
+    return N > 256 and (N > limit["kPfMaxN"] or budget > limit["kPfMaxBudget"])
+
+
+@pytest.mark.parametrize("N,budget,lam", [(300, 129, 0.5), (900, 200, 1.0), (1500, 150, 0.0), (5041, 129, 1.0), (5042, 140, 1.0), (5121, 64, 0.5)])
+@pytest.mark.parametrize("twice", [False, True])
+def test_stream_kernel(N, budget, lam, twice):
+    """Budgets above 128 and N above 5120, rings of eight and of four stages. twice: every V row twice, so that the loop over the
+    active set reaches its bound and the route over the whole pool follows (the one within the operand tile, or plain dot
+    products where the pool outgrows it)."""
+    assert _takes_stream_kernel(N, budget)
+    ev = synth.make_plain(4, 1, 2, N, 128, budget, 2 * lam if twice else lam, dtype=synth.BF16, seed=N + budget)
+    if twice:
+        ev.V[..., N - N // 2:, :] = ev.V[..., :N // 2, :]
+    before = akv.launch_count()
+    g = run_fused(ev)
+    assert akv.launch_count() == before + 1
+    check_all(ev, g, ev.lam)
+    n_cand = [N, N - 63, 64 * (N // 64), budget - 3]
+    check_all(ev, run_fused(ev, n_cand=n_cand), ev.lam, n_cand=n_cand)
+
+
+def test_stream_kernel_variants():
+    """No pruning, the loop forced at lambda = 0, per-head budgets, scores taken afresh, irregular positions with the default
+    reference position, close and equal scores, starved waits."""
+    N, budget = 900, 140
+    assert _takes_stream_kernel(N, budget)
+    ev = synth.make_c3(seed=75, B=2, L=2, H=2, N=N, budget=budget)
+    base = run_fused(ev)
+    check_all(ev, base, ev.lam)
+    full = run_fused(ev, flags=akv.FLAG_NO_PRUNE)
+    for k in ("order", "idx", "K", "V", "pos"):
+        assert np.array_equal(base[k], full[k]), k
+    fast, loop = run_fused(ev, lam=0.0), run_fused(ev, lam=0.0, flags=akv.FLAG_FORCE_GREEDY)
+    assert np.array_equal(fast["order"], loop["order"]) and np.array_equal(fast["K"], loop["K"])
+    budgets = np.array([[140, 1], [17, 130]], dtype=np.int32)
+    check_all(ev, run_fused(ev, budgets=budgets), ev.lam, budgets=budgets)
+    fresh = run_fused(ev, flags=akv.FLAG_NO_CHAIN)
+    assert np.max(np.abs(fresh["scores"] - base["scores"])) < 2e-6
+    for width in (0.0, 1e-3):
+        close = _close_scores(N, budget, 0.5, width, seed=76)
+        check_all(close, run_fused(close), 0.5)
+    ev.pos[:] = np.sort(np.random.default_rng(77).choice(200_000, size=N, replace=False)).astype(np.int32)
+    check_all(ev, run_fused(ev, p_ref=False), ev.lam, p_ref=False)
+    starved = run_fused(ev, flags=akv.FLAG_TEST_STARVE_WAIT)
+    assert np.all(starved["status"] == 3)
+    assert np.array_equal(starved["K"], ev.K) and np.array_equal(starved["V"], ev.V) and np.array_equal(starved["pos"], ev.pos)
+
+
+@pytest.mark.parametrize("budget,lam,twice", [(150, 0.5, False), (150, 1.5, True), (100, 1.5, True)])
+def test_paged_large_pools(budget, lam, twice):
+    """A paged cache of N = 576 in the stream kernel (150 kept) and in the prefill kernel beyond its first active set (100
+    kept, every V row twice), under budgets per head."""
+    c5 = synth.make_c5(seed=78, B=2, L=2, H=2, page=64, pages_per_seq=9, budget=budget, rounds=1)
+    L, H, N, d = c5.L, c5.H, c5.N, c5.d
+    assert _takes_stream_kernel(N, budget) == (budget > 128)
+    if twice:
+        for bb in range(c5.B):
+            pages = c5.block_table[bb]
+            c5.pool_V[:, pages[5:]] = c5.pool_V[:, pages[:4]]
+    hostK = synth.paged_gather_dense(c5.pool_K, c5.block_table)
+    hostV = synth.paged_gather_dense(c5.pool_V, c5.block_table)
+    pool_K, pool_V = dev(c5.pool_K), dev(c5.pool_V)
+    pos = dev(c5.pos)
+    budgets = np.array([[budget, 60], [budget - 1, 90]], dtype=np.int32)
+    sel = akv.alpha_compress_event(pool_K, pool_V, pos, dev(c5.qstat), budget, akv.Options(lam=lam, head_budgets=dev(budgets)),
+                                   layout=akv.Layout.paged(pool_K, dev(c5.block_table)), want_scores=True)
+    torch.cuda.synchronize()
+    idx, order, sc, posn = (x.cpu().numpy() for x in (sel.idx_sorted, sel.pick_order, sel.scores, pos))
+    for bb in range(c5.B):
+        pages = c5.block_table[bb].tolist()
+        for l in range(L):
+            for h in range(H):
+                Kn = akv.to_host_bits(pool_K[l, pages, h]).reshape(N, d)
+                Vn = akv.to_host_bits(pool_V[l, pages, h]).reshape(N, d)
+                chk.check_event(hostK[bb, l, h], hostV[bb, l, h], c5.pos[bb, l, h], c5.qstat[l, h], None, int(budgets[l, h]), lam,
+                                sc[bb, l, h], order[bb, l, h], idx[bb, l, h], Kn, Vn, posn[bb, l, h], log=[])
 
 
 def test_large_pool_stream_kernel_paged():
@@ -753,6 +839,25 @@ def test_zero_cache_and_non_finite_scores(N, budget):
         assert np.array_equal(g["idx"], g["order"])
         for k in ("K", "V", "pos"):
             assert np.array_equal(g[k], getattr(e, k))
+
+
+@pytest.mark.parametrize("lam", [0.0, 0.5])
+@pytest.mark.parametrize("N,budget", [(192, 64), (256, 128), (256, 140), (1000, 100), (1000, 140), (5200, 100)])
+def test_a_few_non_finite_scores_on_the_tensor_memory_kernels(N, budget, lam):
+    """Flagged and never preferred: with the rows of infinite and NaN scores out of the candidates the result is the same."""
+    ev = synth.make_plain(1, 1, 2, N, 128, budget, lam, dtype=synth.BF16, seed=N + budget)
+    bad = [0, 5, 9, N // 2, N - 1]
+    ev.K[0, 0, 0, bad[:3], 3] = synth.f32_to_bf16_bits(np.float32(np.inf))
+    ev.K[0, 0, 0, bad[3:], 100] = synth.f32_to_bf16_bits(np.float32(np.nan))
+    g = run_fused(ev)
+    assert g["status"][0, 0].tolist() == [1, 0]
+    order = g["order"][0, 0, 0].astype(np.int64)
+    assert not set(bad) & set(order.tolist()) and len(set(order.tolist())) == budget
+    good = np.setdiff1d(np.arange(N), bad)
+    with np.errstate(invalid="ignore"):
+        s = O.triattention_score(ev.K[0, 0, 0], ev.pos[0, 0, 0], ev.qstat[0, 0], int(ev.p_ref[0]))
+    rep = O.replay_pick_order(s[good], O.signatures_per_head(ev.V[0, 0, 0][good], ev.eps), lam, np.searchsorted(good, order), chk.MARGIN_TOL)
+    assert rep.ok, rep.log[:3]
 
 
 @pytest.mark.parametrize("dtype,N,budget", [(synth.BF16, 192, 64), (synth.BF16, 256, 128), (synth.BF16, 256, 140), (synth.BF16, 1000, 128),
