@@ -1,6 +1,6 @@
 // Fast event kernel for bf16, d = 128, per-head signatures, N <= 256, used when the pool that
 // survives pruning is expected to stay within 127 rows (N <= 128 or budget <= 64). One CTA of four
-// warps per event, six CTAs resident per SM (37 KB of shared memory and 72 registers each).
+// warps per event, six CTAs resident per SM (37 KB of shared memory and 80 registers each).
 //
 //   1. K rows arrive in shared memory by bulk copies (cp.async.bulk + mbarrier) and are scored there
 //      (fused RoPE rotate-and-dot against the folded query statistic). The tile holds 128 rows: rows
