@@ -46,7 +46,7 @@ WORKLOADS = {
 }
 # kernel(s) one call of the fused entry point launches for each workload
 KERNELS = {"C1": "event_resident_kernel<float>", "C2": "event_pool_kernel<fused>", "C3": "event_tri_kernel<fused>",
-           "C4": "event_stream_kernel", "C5": "event_pool_kernel<fused>",
+           "C4": "event_prefill_kernel<fused>", "C5": "event_pool_kernel<fused>",
            "C6": "flat_signature_kernel + gram_shared_kernel + event_pool_kernel<fused>"}
 
 # dram__bytes_read.sum + dram__bytes_write.sum per step from the ncu captures summarised under profiles/,
@@ -54,15 +54,17 @@ KERNELS = {"C1": "event_resident_kernel<float>", "C2": "event_pool_kernel<fused>
 # capture of another revision is reported as null.
 NCU_TRAFFIC = {
     # one launch of 4096 events captured whole (profiles/event_tri_kernel_bf16_C3.md)
-    "C3": {"bytes": 323675904 + 98740992, "revision": "2ef03d00f108"},
+    "C3": {"bytes": 320790272 + 97728000, "revision": "7942d50ef41b"},
     # one launch of 4096 events (16 sequences) captured; a step is 4 x 32 launches of that size
     # (profiles/event_pool_kernel_bf16_C5.md)
-    "C5": {"bytes": (489861376 + 230915584) * 128, "revision": "2ef03d00f108"},
+    "C5": {"bytes": (488350976 + 229420288) * 128, "revision": "7942d50ef41b"},
     # the same kernel and capture, scaled to 112 events
-    "C2": {"bytes": (489861376 + 230915584) * 112 // 4096, "revision": "2ef03d00f108"},
+    "C2": {"bytes": (488350976 + 229420288) * 112 // 4096, "revision": "7942d50ef41b"},
     # the three launches (lambda 0, 0.5, 1) of a 2-sequence batch captured; the bench batch has 8 sequences
-    # (profiles/event_stream_kernel_bf16_C4.md)
-    "C4": {"bytes": ((249109504 + 12716032) + (256418560 + 10868480) + (256417536 + 11575296)) * 4, "revision": "2ef03d00f108"},
+    # (profiles/event_prefill_kernel_bf16_C4.md)
+    "C4": {"bytes": ((251866112 + 3623168) + (255989760 + 3400704) + (262314752 + 3449856)) * 4, "revision": "7942d50ef41b"},
+    # the step's three launches captured whole (profiles/gram_shared_kernel_f32_C6.md)
+    "C6": {"bytes": (117467904 + 3454976) + 2136320 + (180876544 + 70199040), "revision": "7942d50ef41b"},
 }
 
 
