@@ -18,6 +18,8 @@
 //   4. Kept K and V rows are staged on chip and written to slots 0..b-1 of the same buffers.
 //
 // FUSED: score + select + compact; otherwise selection only (scores are read from a.scores and nothing is rewritten).
+// SPLIT: the scoring of an event is shared by a cluster of so many CTAs, for calls of few and long events. Each streams its
+// part of K; the others store their scores to the first one's shared memory and leave, the first one selects.
 #pragma once
 #include "akv_event_stream.cuh"
 
@@ -64,14 +66,33 @@ __host__ __device__ inline PfSmem plan_pf_smem(int N, int budget) {
     return p;
 }
 
-template <bool FUSED>
+// Thread-block clusters: rank of this CTA, its arrival at the cluster's barrier, the wait for the others', and a float or an int
+// stored to another CTA's shared memory (at the address of this CTA's own).
+__device__ __forceinline__ int cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return (int)r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t cluster_address(uint32_t own, int rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(own), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_store(uint32_t addr, uint32_t v) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+template <bool FUSED, int SPLIT>
 __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __grid_constant__ EventArgs a, const __grid_constant__ ScoreTab tab) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     __shared__ __align__(16) uint32_t part[2][kStWarps];       // per-warp partial counts, double-buffered
     __shared__ __align__(16) uint4 best_of[2][kStWarps];       // per-warp arg-max: key, 0xFFFFFFFF - slot, row
     const DevLayout& lay = a.lay;
-    const EventId id = decode_event(lay, blockIdx.x);
+    const EventId id = decode_event(lay, blockIdx.x / SPLIT);
+    const int rank = SPLIT > 1 ? cluster_rank() : 0;
     const int n = event_n(a, id.b);
     const int N = lay.N;
     const int bud = event_budget(a, id);
@@ -123,7 +144,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
     }
     if (warp == 0) {
         // (both resident CTAs' columns fit the SM; the right to allocate is given up at once, or the next CTA would not start)
-        if (similarity) tmem_alloc(smem_u32(tmem_holder), kPfCols);
+        if (similarity && rank == 0) tmem_alloc(smem_u32(tmem_holder), kPfCols);
         else tmem_relinquish();
     }
     if (FUSED) {
@@ -133,10 +154,15 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (SPLIT > 1) cluster_arrive();   // (the others may write to this CTA's memory once all have come here)
 
     int bad = 0;
     if (FUSED) {
-        const int stages = (n + kStStageRows - 1) / kStStageRows;
+        // the stages of this CTA: all, or its share of them (in eights, so that rotations are taken afresh where they are
+        // without a split and the scores are the same to the bit)
+        const int all = (n + kStStageRows - 1) / kStStageRows;
+        const int share = SPLIT > 1 ? ((all + SPLIT - 1) / SPLIT + kChainRounds - 1) / kChainRounds * kChainRounds : all;
+        const int first = rank * share, stages = max(min(all - first, share), 0);
         if (!worker) {
             // ---- producer: K through the ring ---------------------------------------------------------------------
             if (lane == 0) {
@@ -146,7 +172,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
                         atomicExch(&cnt[0], 1);
                         break;
                     }
-                    const int r0 = st * kStStageRows, r1 = min(n, r0 + kStStageRows);
+                    const int r0 = (first + st) * kStStageRows, r1 = min(n, r0 + kStStageRows);
                     mbar_expect_tx(bar_full + 8 * sl, (uint32_t)(r1 - r0) * 256u);
                     // as few copies as the layout allows: the whole stage when its rows are contiguous, whole pages
                     // when pages are, else row by row (starve, a testing aid: none at all, the scoring warps' wait runs out)
@@ -197,13 +223,15 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
             const bool d_fits = (long long)D32 == D;
             ChainScore ca, cb;  // cb uses ca's S
             ca.set_step(D, phitab + f0, sect);
+            if (SPLIT > 1) cluster_wait();
+            const uint32_t s_first = SPLIT > 1 ? cluster_address(smem_u32(s), 0) : 0u;
             for (int st = 0; st < stages; ++st) {
                 const int sl = st & (kPfStages - 1);
                 if (!mbar_wait_bounded(bar_full + 8 * sl, (uint32_t)((st / kPfStages) & 1), a.wait_polls)) {
                     atomicExch(&cnt[0], 1);
                     break;
                 }
-                const int ja = st * kStStageRows + 4 * warp + grp, jb = ja + kStRoundRows;
+                const int ja = (first + st) * kStStageRows + 4 * warp + grp, jb = ja + kStRoundRows;
                 const bool la = ja < n, lb = jb < n;
                 const unsigned char* krow = region + sl * kStStageBytes + (4 * warp + grp) * 256 + (lane & 7) * 16;
                 bool fresh = (st & (kChainRounds - 1)) == 0 || a.no_chain || !d_fits;
@@ -233,22 +261,34 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
                 acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 1);
                 const int j = second ? jb : ja;
                 if ((lane & 3) == 0 && j < n) {
-                    s[j] = acc;
+                    if (SPLIT > 1 && rank != 0) cluster_store(s_first + 4u * (uint32_t)j, __float_as_uint(acc));
+                    else s[j] = acc;
                     if (a.scores) a.scores[(long long)id.e * N + j] = acc;
                 }
             }
         }
+        if (SPLIT > 1 && !worker) {
+            __syncwarp();
+            cluster_wait();
+        }
         __syncthreads();
+        if (SPLIT > 1) {
+            // the first CTA goes on with all scores; what the others did lies in its memory, a wait that ran out there included
+            if (rank != 0 && tid == 0 && cnt[0]) cluster_store(cluster_address(smem_u32(cnt), 0), 1u);
+            cluster_arrive();
+            if (rank == 0) cluster_wait();
+            else if (!cnt[0]) return;
+        }
         if (cnt[0]) {
             // a wait ran out: report it, give copies that may still be in flight a bounded chance to land, leave
             if (tid == 0) {
-                if (a.status) a.status[id.e] = 3;
+                if (a.status && rank == 0) a.status[id.e] = 3;
                 for (int sl = 0; sl < kPfStages; ++sl) {
                     mbar_wait_bounded(bar_full + 8 * sl, 0, a.wait_polls);
                     mbar_wait_bounded(bar_full + 8 * sl, 1, a.wait_polls);
                 }
             }
-            if (similarity && warp == 0) tmem_dealloc(*tmem_holder, kPfCols);
+            if (similarity && rank == 0 && warp == 0) tmem_dealloc(*tmem_holder, kPfCols);
             return;
         }
     } else {

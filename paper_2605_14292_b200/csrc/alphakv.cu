@@ -369,16 +369,49 @@ static bool prefill_path_ok(const EventArgs& a) {
     return a.lay.dtype == AKV_BF16 && a.lay.d == kTcD && a.lay.N > kTcMaxN && a.lay.N <= kPfMaxN && a.flat_sig == nullptr &&
            !a.gqa_max && a.budget <= kPfMaxBudget;
 }
-template <bool FUSED>
-static akv_status_t launch_prefill(akv_handle* h, const EventArgs& a, cudaStream_t st, bool dry = false) {
+template <bool FUSED, int SPLIT>
+static akv_status_t launch_prefill_split(akv_handle* h, const EventArgs& a, cudaStream_t st, bool dry) {
     const PfSmem sp = plan_pf_smem(a.lay.N, a.budget);
     akv_status_t s;
-    if ((s = set_smem(event_prefill_kernel<FUSED>, sp.total)) != AKV_OK) return s;
-    CUDA_TRY(cudaFuncSetAttribute(event_prefill_kernel<FUSED>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                  (int)cudaSharedmemCarveoutMaxShared));
+    auto kernel = event_prefill_kernel<FUSED, SPLIT>;
+    if ((s = set_smem(kernel, sp.total)) != AKV_OK) return s;
+    CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
     if (dry) return AKV_OK;
-    event_prefill_kernel<FUSED><<<a.lay.B * a.lay.L * a.lay.H, kStThreads, sp.total, st>>>(a, h->tab);
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)(a.lay.B * a.lay.L * a.lay.H) * SPLIT);
+    cfg.blockDim = dim3(kStThreads);
+    cfg.dynamicSmemBytes = sp.total;
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = SPLIT;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = SPLIT > 1 ? 1 : 0;
+    CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, a, h->tab));
     return launched(FUSED ? "event_prefill" : "select_prefill");
+}
+// How many CTAs share an event's scoring. Two CTAs fit an SM, so up to as many events as SMs leave half of the places empty. A
+// split pays where scoring is long beside what it costs (the cluster's start, its barrier, the first CTA's selection alone).
+// Measured (148 SMs, us per call with 1, 2 and 4 CTAs per event): 28 events of 1100 rows 56 / 55 / 50, of 4096 85 / 68 / 57; 56
+// events of 2048 rows 66 / 57 / 58, of 4096 90 / 72 / 68; 112 events of 1100 rows 59 / 67 / 80, of 2048 75 / 70 / 82, of 4096
+// 96 / 85 / 104; 148 events of 2048 rows 79 / 76 / 106, of 4096 101 / 88 / 125. With more events than SMs it never pays: 222
+// events of 4096 rows 115 / 151 / 168, 896 of them 379 / 488 / 553.
+static int prefill_split(long long events, int N, int sms) {
+    if (events * 4 <= sms && N >= 1024) return 4;
+    if (events * 2 <= sms && N >= 3072) return 4;
+    return events <= sms && N >= 2048 ? 2 : 1;
+}
+template <bool FUSED>
+static akv_status_t launch_prefill(akv_handle* h, const EventArgs& a, cudaStream_t st, bool dry = false) {
+    if constexpr (FUSED) {
+        const long long E = (long long)a.lay.B * a.lay.L * a.lay.H;
+        const int split = prefill_split(E, a.lay.N, h->sm_count);
+        if (split == 4) return launch_prefill_split<true, 4>(h, a, st, dry);
+        if (split == 2) return launch_prefill_split<true, 2>(h, a, st, dry);
+    }
+    return launch_prefill_split<FUSED, 1>(h, a, st, dry);
 }
 
 static akv_status_t launch_select(akv_handle* h, const EventArgs& a, cudaStream_t st, bool dry = false) {

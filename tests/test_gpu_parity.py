@@ -580,6 +580,32 @@ def test_prefill_sized_pool_beyond_the_active_set(N, budget, scale, twice):
             assert rep.ok, rep.log[:3]
 
 
+@pytest.mark.parametrize("L,H,N", [(1, 4, 1023), (1, 4, 1024), (1, 4, 1025), (1, 37, 1601), (2, 19, 2048), (5, 15, 2047), (5, 15, 2113), (4, 15, 3072),
+                                   (1, 3, 5120)])
+def test_scoring_shared_by_several_ctas(L, H, N):
+    """Few long events: several CTAs share an event's scoring (four from N = 1024, two from 2048, by the number of events). The
+    same events in a call of more than any chip's multiprocessors are scored by one CTA each: every output is the same to the
+    bit, also with irregular positions, candidates that end within one CTA's share, and a wait that runs out."""
+    ev = synth.make_plain(1, L, H, N, 128, 40, 0.5, dtype=synth.BF16, seed=N + H)
+    times = 512 // (L * H)
+    many = synth.make_plain(times, 1, 1, 1, 128, 1, 0.5, dtype=synth.BF16, seed=0)
+    for irregular in (False, True):
+        if irregular:
+            ev.pos[:] = np.sort(np.random.default_rng(N).choice(100_000, size=N, replace=False)).astype(np.int32)
+        for name in ("K", "V", "pos", "p_ref"):
+            setattr(many, name, np.repeat(getattr(ev, name), times, axis=0))
+        many.qstat, many.budget = ev.qstat, ev.budget
+        for n in (N, N - 70, 513, 30):
+            a = run_fused(ev, n_cand=[n], p_ref=not irregular)
+            b = run_fused(many, n_cand=[n] * times, p_ref=not irregular)
+            for k, x in a.items():
+                x, y = (x[..., :n], b[k][..., :n]) if k == "scores" else (x, b[k])
+                assert np.array_equal(x[0], y[0]) and np.array_equal(x[0], y[-1]), (k, n, irregular)
+    starved = run_fused(ev, flags=akv.FLAG_TEST_STARVE_WAIT)
+    assert np.all(starved["status"] == 3)
+    assert np.array_equal(starved["K"], ev.K) and np.array_equal(starved["V"], ev.V) and np.array_equal(starved["pos"], ev.pos)
+
+
 def _takes_stream_kernel(N, budget):
     """bf16, d = 128, per-head signatures: what the prefill kernel's limits leave"""
     text = open(os.path.join(os.path.dirname(akv.__file__), "csrc", "akv_event_prefill.cuh")).read()
