@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
     float* r = reinterpret_cast<float*>(smem + sp.key);  // reuses the score keys' storage
     int* spos = reinterpret_cast<int*>(smem + sp.spos);
     unsigned short* bypool = reinterpret_cast<unsigned short*>(smem + sp.bypool);
-    unsigned char* taken = smem + sp.taken;
+    uint32_t* kept = reinterpret_cast<uint32_t*>(smem + sp.taken);
     int* order = reinterpret_cast<int*>(smem + sp.order);
     float* gain = reinterpret_cast<float*>(smem + sp.gain);
     int* idx = reinterpret_cast<int*>(smem + sp.idx);
@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
     }
     bad = __syncthreads_or(bad);
     // (only now: while scoring, this storage holds the statistic's table, which slower warps may still read)
-    for (int j = tid; j < np4; j += kTcThreads) taken[j] = 0;
+    if (tid < 8) kept[tid] = 0u;
 
     phase_stamp(id.e, 2);
     // ---- s_(b) by bisection over the score keys, then the pool in slot order (warp 0) -------------
@@ -476,24 +476,24 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
         }
     }
     __syncthreads();
-    for (int t = tid; t < picks; t += kTcThreads) {
-        const int j = bypool[order[t]];
-        gain[t] = from_orderable(park_key[t]);
-        order[t] = j;
-        taken[j] = 1;
+    int mine = -1;   // the slot of this thread's pick (a budget is at most the threads)
+    if (tid < picks) {
+        mine = bypool[order[tid]];
+        atomicOr(&kept[mine >> 5], 1u << (mine & 31));
     }
     __syncthreads();
 
     phase_stamp(id.e, 7);
     // ---- sort(S) and outputs -------------------------------------------------------------------------
-    ordered_indices(n, a.budget, taken, idx);
-    __syncthreads();
     const long long ob = (long long)id.e * a.budget;
-    for (int t = tid; t < a.budget; t += kTcThreads) {
-        a.idx_sorted[ob + t] = idx[t];
-        if (a.pick_order) a.pick_order[ob + t] = t < picks ? order[t] : -1;
-        if (a.pick_gain) a.pick_gain[ob + t] = t < picks ? gain[t] : 0.f;
+    if (tid < picks) idx[kept_below(kept, mine)] = mine;
+    else if (tid < a.budget) idx[tid] = -1;
+    if (tid < a.budget) {
+        if (a.pick_order) a.pick_order[ob + tid] = mine;
+        if (a.pick_gain) a.pick_gain[ob + tid] = tid < picks ? from_orderable(park_key[tid]) : 0.f;
     }
+    __syncthreads();
+    if (tid < a.budget) a.idx_sorted[ob + tid] = idx[tid];
     if (tid == 0) {
         if (a.n_kept) a.n_kept[id.e] = picks;
         if (a.status) a.status[id.e] = n < bud ? 2 : (bad ? 1 : 0);

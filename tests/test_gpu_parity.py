@@ -606,6 +606,16 @@ def test_scoring_shared_by_several_ctas(L, H, N):
     assert np.array_equal(starved["K"], ev.K) and np.array_equal(starved["V"], ev.V) and np.array_equal(starved["pos"], ev.pos)
 
 
+@pytest.mark.parametrize("N,budget", [(129, 65), (130, 128), (160, 97), (161, 128), (224, 100), (255, 128), (256, 127)])
+@pytest.mark.parametrize("lam", [0.0, 0.5])
+def test_kept_slots_in_order_at_the_edges_of_words(N, budget, lam):
+    """The 256-row kernel orders kept slots by bits in eight words: event sizes and budgets at and beside the words' edges."""
+    ev = synth.make_plain(2, 1, 2, N, 128, budget, lam, dtype=synth.BF16, seed=N + budget)
+    check_all(ev, run_fused(ev), lam)
+    n_cand = [N, budget + 1]
+    check_all(ev, run_fused(ev, n_cand=n_cand), lam, n_cand=n_cand)
+
+
 def _takes_stream_kernel(N, budget):
     """bf16, d = 128, per-head signatures: what the prefill kernel's limits leave"""
     text = open(os.path.join(os.path.dirname(akv.__file__), "csrc", "akv_event_prefill.cuh")).read()
