@@ -18,23 +18,36 @@
 
 namespace akv {
 
-// n rows of one event from global memory into a dense shared tile by 16-byte asynchronous copies, all in flight
-// at once (a lane keeps its column, a row costs one address); the caller waits and synchronises before reading the tile.
-// slots: the rows' slots, or null for 0..n-1.
+// The rows of one event in the n slots listed, from global memory into a dense shared tile by 16-byte asynchronous copies, all
+// in flight at once (a lane keeps its column, a row costs one address); the caller waits and synchronises before reading the tile.
 template <typename T>
-__device__ __forceinline__ void load_tile_async(T* tile, const T* base, const DevLayout& lay, const EventId& id, int n, const int* slots = nullptr) {
+__device__ __forceinline__ void load_rows_async(T* tile, const T* base, const DevLayout& lay, const EventId& id, int n, const int* slots) {
     const int cpr = lay.d * (int)sizeof(T) / 16;  // 16-byte chunks per row
     const int lanes = min(pow2_ceil(cpr), 32), rows = 32 / lanes, lane = threadIdx.x & 31;
     const uint32_t t0 = smem_u32(tile);
     for (int row = (threadIdx.x >> 5) * rows + lane / lanes; row < n; row += kWarps * rows) {
-        const char* src = reinterpret_cast<const char*>(base + row_offset(lay, id.b, id.l, id.h, slots ? slots[row] : row));
+        const char* src = reinterpret_cast<const char*>(base + row_offset(lay, id.b, id.l, id.h, slots[row]));
         for (int c = lane & (lanes - 1); c < cpr; c += lanes) cp_async16(t0 + (uint32_t)(row * cpr + c) * 16u, src + c * 16);
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
 }
-template <int PENDING>
-__device__ __forceinline__ void cp_async_wait_pending() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+// Rows 0..n-1 of one event from global memory into a dense shared tile by bulk copies that report to `bar`; one warp calls. As
+// few copies as the layout allows: pieces of 32 KB where rows are contiguous (whole pages where pages are), else a row each, the
+// rows over the lanes. (192 rows of K and V in fp32, d = 128: all threads' 16-byte copies took 13.3 of an event's 65 thousand cycles
+// to issue; one event 41.3 -> 37.6 us, 112 of them 46.5 -> 42.0.)
+template <typename T>
+__device__ __forceinline__ void load_tile_bulk(T* tile, const T* base, const DevLayout& lay, const EventId& id, int n, uint32_t bar) {
+    const uint32_t row_bytes = (uint32_t)lay.d * (uint32_t)sizeof(T), t0 = smem_u32(tile);
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) mbar_expect_tx(bar, (uint32_t)n * row_bytes);
+    __syncwarp();
+    int run = 1;   // rows of a copy
+    if (lay.page_size == 0 ? lay.sn == lay.d : lay.s_page_n == lay.d) {
+        run = max(32768 / (int)row_bytes, 1);
+        if (lay.page_size && run > lay.page_size) run = lay.page_size;
+        else if (lay.page_size) run = 1 << (31 - __clz(run));   // (a power of two, like pages: no copy crosses one)
+    }
+    for (int row = lane * run; row < n; row += 32 * run)
+        bulk_g2s(t0 + (uint32_t)row * row_bytes, base + row_offset(lay, id.b, id.l, id.h, row), (uint32_t)min(run, n - row) * row_bytes, bar);
 }
 
 constexpr int kResidentCtas = 2;       // most CTAs per SM that the registers of the kernel with the penalty allow
@@ -280,9 +293,18 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
     T* Kg = reinterpret_cast<T*>(a.K);
     T* Vg = reinterpret_cast<T*>(a.V);
 
-    // stage the event on chip
-    load_tile_async(Kt, Kg, lay, id, n);
-    load_tile_async(Vt, Vg, lay, id, n);
+    // stage the event on chip (the barriers' place is the reductions', which come later)
+    const uint32_t bar_k = smem_u32(red), bar_v = bar_k + 8;
+    if (warp == 0) {
+        if (lane == 0) {
+            mbar_init(bar_k, 1);
+            mbar_init(bar_v, 1);
+            mbar_init_fence();
+        }
+        __syncwarp();
+        load_tile_bulk(Kt, Kg, lay, id, n, bar_k);
+        load_tile_bulk(Vt, Vg, lay, id, n, bar_v);
+    }
     int pmax = INT_MIN;
     for (int j = tid; j < n; j += kThreads) {
         const int p = gpos ? gpos[j] : 0;
@@ -295,8 +317,8 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
     const int members = fold_group(a, id, tab, d, g);
     long long pref = 0;
     if (gpos) pref = a.p_ref ? (long long)a.p_ref[id.b] : (long long)block_max_int(pmax, redi) + 1;
-    cp_async_wait_pending<1>();   // K has landed; V may still be under way
     __syncthreads();
+    bool late = !mbar_wait_bounded(bar_k, 0, kWaitPolls);   // K has landed; V may still be under way
 
     // scores: four rows of a lane group at a time, so that one row's dependent steps fill another's latency
     const int G = pow2_ceil(d >> 3) > 32 ? 32 : pow2_ceil(d >> 3);
@@ -336,8 +358,15 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
             if (valid && lig == 0) keep_score(j, sc);
         }
     }
-    cp_async_wait_pending<0>();
-    __syncthreads();
+    late |= !mbar_wait_bounded(bar_v, 0, kWaitPolls);
+    if (__syncthreads_or(late)) {   // (everybody is past the barriers: their place is free)
+        if (tid == 0 && a.status) a.status[id.e] = 3;
+        return;
+    }
+    if (tid == 0) {
+        mbar_inval(bar_k);
+        mbar_inval(bar_v);
+    }
     // reciprocal norms: a thread per row, each lane from its own block of eight elements on (different banks). A block's
     // squares in two chains of four, the blocks in eight sums: an error of 4.2e-8 at d = 128, as from sixteen lanes' partial
     // sums; one chain of all squares has 1.6e-7.
@@ -471,8 +500,8 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
     }
     // compaction: kept rows go to slots 0..picks-1 of the same buffer, all sources on chip first
     if (!k_tile) {
-        load_tile_async(Kt, Kg, lay, id, picks, idx);
-        cp_async_wait_pending<0>();
+        load_rows_async(Kt, Kg, lay, id, picks, idx);
+        cp_async_wait_all();
         __syncthreads();
     }
     const int cpr = d * (int)sizeof(T) / 16, lanes = min(pow2_ceil(cpr), 32), rows = 32 / lanes;

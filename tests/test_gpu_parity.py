@@ -616,6 +616,44 @@ def test_kept_slots_in_order_at_the_edges_of_words(N, budget, lam):
     check_all(ev, run_fused(ev, n_cand=n_cand), lam, n_cand=n_cand)
 
 
+@pytest.mark.parametrize("dtype,N,d,page", [(synth.F32, 1, 128, 0), (synth.F32, 63, 128, 0), (synth.F32, 65, 128, 0), (synth.F32, 130, 128, 0),
+                                            (synth.F32, 200, 64, 0), (synth.BF16, 256, 64, 0), (synth.F32, 70, 128, 1), (synth.F32, 70, 128, 16),
+                                            (synth.BF16, 90, 72, 32), (synth.F32, 192, 128, 64)])
+@pytest.mark.parametrize("padded", [False, True])
+def test_resident_tiles_by_bulk_copies(dtype, N, d, page, padded):
+    """The resident kernel's tiles arrive in copies of 32 KB, whole pages or single rows (padded: rows that do not lie one
+    behind the other): sizes at and beside a copy's end, candidates that end inside one, pages in any order."""
+    ev = synth.make_plain(2, 1, 2, N, d, max(1, N // 3), 0.5, dtype=dtype, seed=N + d)
+    width = d + (8 if padded else 0)
+    rng = np.random.default_rng(N)
+
+    def place(x):   # -> the tensor that holds the rows, and the view the call takes
+        t = torch.zeros((2, 1, 2, N, width), dtype=torch.float32 if dtype == synth.F32 else torch.bfloat16, device="cuda")
+        t[..., :d] = dev(x)
+        if not page:
+            return t[..., :d]
+        pps = -(-N // page)
+        pool = torch.zeros((1, 2 * pps, 2, page, width), dtype=t.dtype, device="cuda")
+        rows = torch.zeros((2, 1, 2, pps * page, width), dtype=t.dtype, device="cuda")
+        rows[:, :, :, :N] = t
+        for b in range(2):
+            pool[0, torch.as_tensor(table[b], device="cuda").long()] = rows[b, 0].view(2, pps, page, width).permute(1, 0, 2, 3)
+        return pool[..., :d]
+
+    table = rng.permutation(2 * (-(-N // page) if page else 1)).reshape(2, -1).astype(np.int32)
+    K, V, pos = place(ev.K), place(ev.V), dev(ev.pos)
+    lay = akv.Layout.paged(K, dev(table), N) if page else akv.Layout.dense(K)
+    n_cand = [N, max(1, N - 5)]
+    sel = akv.alpha_compress_event(K, V, pos, dev(ev.qstat), ev.budget, akv.Options(lam=0.5), p_ref=dev(ev.p_ref), n_cand=dev(np.asarray(n_cand, dtype=np.int32)),
+                                   layout=lay, want_scores=True)
+    plain = run_fused(ev, n_cand=n_cand)
+    check_all(ev, plain, 0.5, n_cand=n_cand)
+    assert np.array_equal(sel.pick_order.cpu().numpy(), plain["order"]) and np.array_equal(sel.idx_sorted.cpu().numpy(), plain["idx"])
+    for b in range(2):
+        assert np.array_equal(sel.scores.cpu().numpy()[b, ..., :n_cand[b]], plain["scores"][b, ..., :n_cand[b]])
+    assert np.array_equal(pos.cpu().numpy(), plain["pos"])
+
+
 def _takes_stream_kernel(N, budget):
     """bf16, d = 128, per-head signatures: what the prefill kernel's limits leave"""
     text = open(os.path.join(os.path.dirname(akv.__file__), "csrc", "akv_event_prefill.cuh")).read()
