@@ -54,17 +54,17 @@ KERNELS = {"C1": "event_resident_kernel<float>", "C2": "event_pool_kernel<fused>
 # capture of another revision is reported as null.
 NCU_TRAFFIC = {
     # one launch of 4096 events captured whole (profiles/event_tri_kernel_bf16_C3.md)
-    "C3": {"bytes": 320790272 + 97728000, "revision": "7942d50ef41b"},
+    "C3": {"bytes": 320505344 + 97829632, "revision": "16bbe4dc64a6"},
     # one launch of 4096 events (16 sequences) captured; a step is 4 x 32 launches of that size
     # (profiles/event_pool_kernel_bf16_C5.md)
-    "C5": {"bytes": (488350976 + 229420288) * 128, "revision": "7942d50ef41b"},
+    "C5": {"bytes": (487292416 + 229692160) * 128, "revision": "16bbe4dc64a6"},
     # the same kernel and capture, scaled to 112 events
-    "C2": {"bytes": (488350976 + 229420288) * 112 // 4096, "revision": "7942d50ef41b"},
+    "C2": {"bytes": (487292416 + 229692160) * 112 // 4096, "revision": "16bbe4dc64a6"},
     # the three launches (lambda 0, 0.5, 1) of a 2-sequence batch captured; the bench batch has 8 sequences
     # (profiles/event_prefill_kernel_bf16_C4.md)
-    "C4": {"bytes": ((251866112 + 3623168) + (255989760 + 3400704) + (262314752 + 3449856)) * 4, "revision": "7942d50ef41b"},
+    "C4": {"bytes": ((251964928 + 4013824) + (256004864 + 4015872) + (262309120 + 4198912)) * 4, "revision": "16bbe4dc64a6"},
     # the step's three launches captured whole (profiles/gram_shared_kernel_f32_C6.md)
-    "C6": {"bytes": (117467904 + 3454976) + 2136320 + (180876544 + 70199040), "revision": "7942d50ef41b"},
+    "C6": {"bytes": (117470464 + 3307520) + 2136832 + (181025792 + 72201728), "revision": "16bbe4dc64a6"},
 }
 
 
