@@ -32,10 +32,10 @@ __device__ __forceinline__ void load_rows_async(T* tile, const T* base, const De
 }
 // Rows 0..n-1 of one event from global memory into a dense shared tile by bulk copies that report to `bar`; one warp calls. As
 // few copies as the layout allows: pieces of 32 KB where rows are contiguous (whole pages where pages are), else a row each, the
-// rows over the lanes. (192 rows of K and V in fp32, d = 128: all threads' 16-byte copies took 13.3 of an event's 65 thousand cycles
+// rows over the lanes (starve, a testing aid: none at all, the wait for them runs out). (192 rows of K and V in fp32, d = 128: all threads' 16-byte copies took 13.3 of an event's 65 thousand cycles
 // to issue; one event 41.3 -> 37.6 us, 112 of them 46.5 -> 42.0.)
 template <typename T>
-__device__ __forceinline__ void load_tile_bulk(T* tile, const T* base, const DevLayout& lay, const EventId& id, int n, uint32_t bar) {
+__device__ __forceinline__ void load_tile_bulk(T* tile, const T* base, const DevLayout& lay, const EventId& id, int n, uint32_t bar, bool starve) {
     const uint32_t row_bytes = (uint32_t)lay.d * (uint32_t)sizeof(T), t0 = smem_u32(tile);
     const int lane = threadIdx.x & 31;
     if (lane == 0) mbar_expect_tx(bar, (uint32_t)n * row_bytes);
@@ -46,7 +46,7 @@ __device__ __forceinline__ void load_tile_bulk(T* tile, const T* base, const Dev
         if (lay.page_size && run > lay.page_size) run = lay.page_size;
         else if (lay.page_size) run = 1 << (31 - __clz(run));   // (a power of two, like pages: no copy crosses one)
     }
-    for (int row = lane * run; row < n; row += 32 * run)
+    for (int row = lane * run; row < n && !starve; row += 32 * run)
         bulk_g2s(t0 + (uint32_t)row * row_bytes, base + row_offset(lay, id.b, id.l, id.h, row), (uint32_t)min(run, n - row) * row_bytes, bar);
 }
 
@@ -302,8 +302,8 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
             mbar_init_fence();
         }
         __syncwarp();
-        load_tile_bulk(Kt, Kg, lay, id, n, bar_k);
-        load_tile_bulk(Vt, Vg, lay, id, n, bar_v);
+        load_tile_bulk(Kt, Kg, lay, id, n, bar_k, a.starve);
+        load_tile_bulk(Vt, Vg, lay, id, n, bar_v, a.starve);
     }
     int pmax = INT_MIN;
     for (int j = tid; j < n; j += kThreads) {
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
     long long pref = 0;
     if (gpos) pref = a.p_ref ? (long long)a.p_ref[id.b] : (long long)block_max_int(pmax, redi) + 1;
     __syncthreads();
-    bool late = !mbar_wait_bounded(bar_k, 0, kWaitPolls);   // K has landed; V may still be under way
+    bool late = !mbar_wait_bounded(bar_k, 0, a.wait_polls);   // K has landed; V may still be under way
 
     // scores: four rows of a lane group at a time, so that one row's dependent steps fill another's latency
     const int G = pow2_ceil(d >> 3) > 32 ? 32 : pow2_ceil(d >> 3);
@@ -358,9 +358,14 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
             if (valid && lig == 0) keep_score(j, sc);
         }
     }
-    late |= !mbar_wait_bounded(bar_v, 0, kWaitPolls);
+    late |= !mbar_wait_bounded(bar_v, 0, a.wait_polls);
     if (__syncthreads_or(late)) {   // (everybody is past the barriers: their place is free)
-        if (tid == 0 && a.status) a.status[id.e] = 3;
+        // a wait ran out: report it, give copies that may still be in flight a bounded chance to land, leave
+        if (tid == 0) {
+            if (a.status) a.status[id.e] = 3;
+            mbar_wait_bounded(bar_k, 0, a.wait_polls);
+            mbar_wait_bounded(bar_v, 0, a.wait_polls);
+        }
         return;
     }
     if (tid == 0) {

@@ -476,6 +476,18 @@ def test_bounded_wait_runs_out_and_reports_status_3(maker):
     check_all(ev, good, ev.lam)
 
 
+@pytest.mark.parametrize("dtype,N,d,budget", [(synth.F32, 192, 128, 64), (synth.F32, 40, 72, 40), (synth.BF16, 256, 64, 128)])
+@pytest.mark.parametrize("lam", [0.0, 0.5])
+def test_resident_waits_run_out_and_report_status_3(dtype, N, d, budget, lam):
+    """The same of the kernel whose K and V tiles stay in shared memory, with and without the penalty: nothing is requested,
+    its two waits run out, the cache is left alone and the next call is a normal one."""
+    ev = synth.make_plain(2, 2, 2, N, d, budget, lam, dtype=dtype, seed=N + d)
+    g = run_fused(ev, flags=akv.FLAG_TEST_STARVE_WAIT)
+    assert np.all(g["status"] == 3)
+    assert np.array_equal(g["K"], ev.K) and np.array_equal(g["V"], ev.V) and np.array_equal(g["pos"], ev.pos)
+    check_all(ev, run_fused(ev), lam)
+
+
 def test_workspace_query_matches_the_route():
     bf = akv.Layout(2, 2, 2, 192, 128, akv.api.AKV_BF16, (2 * 2 * 192 * 128, 2 * 192 * 128, 192 * 128, 128))
     assert akv.workspace_bytes(bf, 64) == 0                                  # on chip, one launch
