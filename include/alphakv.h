@@ -83,7 +83,8 @@ typedef struct {
 #define AKV_FLAG_NO_PRUNE 2u     /* never shrink the candidate pool before the loop (testing aid) */
 /* Testing aid for the bounded waits of the on-chip kernels: no K row is requested (by alpha_select, which reads no
  * keys: no product is issued) and the waits poll only a few times, so every wait runs out with nothing in flight;
- * each event then reports status 3. The fused calls leave K, V and pos as they were; alpha_select writes -1 to
+ * each event then reports status 3. Where several CTAs share an event's scoring, the first one gets its rows and only the
+ * others' waits run out. The fused calls leave K, V and pos as they were; alpha_select writes -1 to
  * every entry of idx_sorted and 0 to n_kept, so that kv_compact moves nothing. Kernels without such waits ignore it. */
 #define AKV_FLAG_TEST_STARVE_WAIT 4u
 /* Testing aid: when an event's positions are an arithmetic progression the fused on-chip kernels turn

@@ -66,15 +66,22 @@ __host__ __device__ inline PfSmem plan_pf_smem(int N, int budget) {
     return p;
 }
 
-// Thread-block clusters: rank of this CTA, its arrival at the cluster's barrier, the wait for the others', and a float or an int
-// stored to another CTA's shared memory (at the address of this CTA's own).
+// Thread-block clusters: rank of this CTA, its arrival at the cluster's barrier and the wait for the others' (the aligned forms:
+// a warp's lanes come together first, whatever branches they come from), and a float or an int stored to another CTA's shared
+// memory (at the address of this CTA's own).
 __device__ __forceinline__ int cluster_rank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return (int)r;
 }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ uint32_t cluster_address(uint32_t own, int rank) {
     uint32_t r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(own), "r"(rank));
@@ -163,12 +170,15 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
         const int all = (n + kStStageRows - 1) / kStStageRows;
         const int share = SPLIT > 1 ? ((all + SPLIT - 1) / SPLIT + kChainRounds - 1) / kChainRounds * kChainRounds : all;
         const int first = rank * share, stages = max(min(all - first, share), 0);
+        // (the testing aid: where others have stages too only they are starved, and the first CTA has to learn of it from them)
+        const bool starve = a.starve && (SPLIT == 1 || rank != 0 || all <= share);
+        const int polls = SPLIT > 1 && !starve ? kWaitPolls : a.wait_polls;
         if (!worker) {
             // ---- producer: K through the ring ---------------------------------------------------------------------
             if (lane == 0) {
                 for (int st = 0; st < stages; ++st) {
                     const int sl = st & (kPfStages - 1);
-                    if (st >= kPfStages && !mbar_wait_bounded(bar_empty + 8 * sl, (uint32_t)((st / kPfStages - 1) & 1), a.wait_polls)) {
+                    if (st >= kPfStages && !mbar_wait_bounded(bar_empty + 8 * sl, (uint32_t)((st / kPfStages - 1) & 1), polls)) {
                         atomicExch(&cnt[0], 1);
                         break;
                     }
@@ -176,7 +186,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
                     mbar_expect_tx(bar_full + 8 * sl, (uint32_t)(r1 - r0) * 256u);
                     // as few copies as the layout allows: the whole stage when its rows are contiguous, whole pages
                     // when pages are, else row by row (starve, a testing aid: none at all, the scoring warps' wait runs out)
-                    for (int row = r0; row < r1 && !a.starve;) {
+                    for (int row = r0; row < r1 && !starve;) {
                         int run = 1;
                         if (dense && lay.sn == kTcD) run = r1 - row;
                         else if (!dense && lay.s_page_n == kTcD) run = min(r1 - row, lay.page_size - row % lay.page_size);
@@ -227,7 +237,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
             const uint32_t s_first = SPLIT > 1 ? cluster_address(smem_u32(s), 0) : 0u;
             for (int st = 0; st < stages; ++st) {
                 const int sl = st & (kPfStages - 1);
-                if (!mbar_wait_bounded(bar_full + 8 * sl, (uint32_t)((st / kPfStages) & 1), a.wait_polls)) {
+                if (!mbar_wait_bounded(bar_full + 8 * sl, (uint32_t)((st / kPfStages) & 1), polls)) {
                     atomicExch(&cnt[0], 1);
                     break;
                 }
@@ -267,10 +277,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
                 }
             }
         }
-        if (SPLIT > 1 && !worker) {
-            __syncwarp();
-            cluster_wait();
-        }
+        if (SPLIT > 1 && !worker) cluster_wait();
         __syncthreads();
         if (SPLIT > 1) {
             // the first CTA goes on with all scores; what the others did lies in its memory, a wait that ran out there included

@@ -618,6 +618,22 @@ def test_scoring_shared_by_several_ctas(L, H, N):
     assert np.array_equal(starved["K"], ev.K) and np.array_equal(starved["V"], ev.V) and np.array_equal(starved["pos"], ev.pos)
 
 
+@pytest.mark.parametrize("L,H,N", [(1, 4, 1100), (1, 37, 4096), (2, 19, 4096), (1, 111, 3000), (4, 37, 4500)])
+def test_first_cta_learns_that_another_gave_up(L, H, N):
+    """With the starve flag the first CTA of a cluster has its rows and scores them; only the others' waits run out. That reaches
+    it through its shared memory: the event reports status 3, writes nothing, and the next call is a normal one."""
+    ev = synth.make_plain(1, L, H, N, 128, 40, 0.5, dtype=synth.BF16, seed=N + H)
+    for lam in (0.5, 0.0):
+        starved = run_fused(ev, lam=lam, flags=akv.FLAG_TEST_STARVE_WAIT)
+        assert np.all(starved["status"] == 3)
+        # (scores of the first CTA's rows are there, in eights of stages; no others)
+        assert np.all(starved["scores"][..., :512] != 0.0) and np.all(starved["scores"][..., -1] == 0.0)
+        for k in ("K", "V", "pos"):
+            assert np.array_equal(starved[k], getattr(ev, k)), k
+    good = run_fused(ev)
+    check_all(ev, good, 0.5, events=[0, L * H - 1])
+
+
 @pytest.mark.parametrize("N,budget", [(129, 65), (130, 128), (160, 97), (161, 128), (224, 100), (255, 128), (256, 127)])
 @pytest.mark.parametrize("lam", [0.0, 0.5])
 def test_kept_slots_in_order_at_the_edges_of_words(N, budget, lam):
