@@ -136,7 +136,8 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
     const int* gpos = event_pos(a.pos, id);
     const bool rotate = gpos != nullptr;
 
-    phase_stamp(id.e, 0);  // phases: 0 start, 1 tables + positions, 2 K scored, 3 s_(b), 4 active set / top-k, 5 triangle, 6 picks, 7 outputs, 8 end
+    // (a cluster's first CTA alone stamps its phases: the others' clocks are those of other SMs)
+    if (rank == 0) phase_stamp(id.e, 0);  // phases: 0 start, 1 tables + positions, 2 K scored, 3 s_(b), 4 active set / top-k, 5 triangle, 6 picks, 7 outputs, 8 end
     // ---- set-up: barriers, tensor memory, tables ----------------------------------------------------------
     if (tid == 0) {
         for (int i = 0; i < kPfStages; ++i) {
@@ -224,7 +225,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
             const bool uniform = cnt[2] == 0;
             long long pref = 0;
             if (rotate) pref = a.p_ref ? (long long)p_ref : (long long)cnt[1] + 1;
-            phase_stamp(id.e, 1);
+            if (rank == 0) phase_stamp(id.e, 1);
             // ---- scores -------------------------------------------------------------------------------------------
             const int grp = lane >> 3, f0 = (lane & 7) * 8;
             // A lane group scores two rows of every stage, 32 slots apart, as two independent chains; each chain steps by
