@@ -295,10 +295,12 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
 
     // stage the event on chip (the barriers' place is the reductions', which come later)
     const uint32_t bar_k = smem_u32(red), bar_v = bar_k + 8;
+    volatile int* late = reinterpret_cast<volatile int*>(red) + 4;   // a wait for them ran out
     if (warp == 0) {
         if (lane == 0) {
             mbar_init(bar_k, 1);
             mbar_init(bar_v, 1);
+            *late = 0;
             mbar_init_fence();
         }
         __syncwarp();
@@ -318,7 +320,7 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
     long long pref = 0;
     if (gpos) pref = a.p_ref ? (long long)a.p_ref[id.b] : (long long)block_max_int(pmax, redi) + 1;
     __syncthreads();
-    bool late = !mbar_wait_bounded(bar_k, 0, a.wait_polls);   // K has landed; V may still be under way
+    if (!mbar_wait_bounded(bar_k, 0, a.wait_polls)) *late = 1;   // K has landed; V may still be under way
 
     // scores: four rows of a lane group at a time, so that one row's dependent steps fill another's latency
     const int G = pow2_ceil(d >> 3) > 32 ? 32 : pow2_ceil(d >> 3);
@@ -358,8 +360,9 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
             if (valid && lig == 0) keep_score(j, sc);
         }
     }
-    late |= !mbar_wait_bounded(bar_v, 0, a.wait_polls);
-    if (__syncthreads_or(late)) {   // (everybody is past the barriers: their place is free)
+    if (!mbar_wait_bounded(bar_v, 0, a.wait_polls)) *late = 1;
+    __syncthreads();
+    if (*late) {   // (everybody is past the barriers: their place is free)
         // a wait ran out: report it, give copies that may still be in flight a bounded chance to land, leave
         if (tid == 0) {
             if (a.status) a.status[id.e] = 3;
@@ -404,6 +407,11 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
     // selection
     const int bud = event_budget(a, id);
     const int picks = min(bud, n);
+    // (nothing below can fail: written here, so that the selection need not hold what it says)
+    if (tid == 0) {
+        if (a.n_kept) a.n_kept[id.e] = picks;
+        if (a.status) a.status[id.e] = n < bud ? 2 : (bad ? 1 : 0);
+    }
     // ---- pool + triangle + one-warp loop, when it fits --------------------------------------------------------
     bool done = false, k_tile = true;   // k_tile: the K rows are still in theirs
     if (PENALTY && picks > 1) {
@@ -498,10 +506,6 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
         a.idx_sorted[ob + t] = idx[t];
         if (a.pick_order) a.pick_order[ob + t] = t < picks ? order[t] : -1;
         if (a.pick_gain) a.pick_gain[ob + t] = t < picks ? gain[t] : 0.f;
-    }
-    if (tid == 0) {
-        if (a.n_kept) a.n_kept[id.e] = picks;
-        if (a.status) a.status[id.e] = n < bud ? 2 : (bad ? 1 : 0);
     }
     // compaction: kept rows go to slots 0..picks-1 of the same buffer, all sources on chip first
     if (!k_tile) {
