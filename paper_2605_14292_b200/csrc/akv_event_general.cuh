@@ -18,37 +18,49 @@
 
 namespace akv {
 
-// The rows of one event in the n slots listed, from global memory into a dense shared tile by 16-byte asynchronous copies, all
-// in flight at once (a lane keeps its column, a row costs one address); the caller waits and synchronises before reading the tile.
+// The rows of one event in the n slots listed (slots null: 0..n-1), from global memory into a dense shared tile by 16-byte
+// asynchronous copies, all in flight at once (a lane keeps its column, a row costs one address), as one group of copies; the caller
+// waits and synchronises before reading the tile.
 template <typename T>
 __device__ __forceinline__ void load_rows_async(T* tile, const T* base, const DevLayout& lay, const EventId& id, int n, const int* slots) {
     const int cpr = lay.d * (int)sizeof(T) / 16;  // 16-byte chunks per row
     const int lanes = min(pow2_ceil(cpr), 32), rows = 32 / lanes, lane = threadIdx.x & 31;
     const uint32_t t0 = smem_u32(tile);
     for (int row = (threadIdx.x >> 5) * rows + lane / lanes; row < n; row += kWarps * rows) {
-        const char* src = reinterpret_cast<const char*>(base + row_offset(lay, id.b, id.l, id.h, slots[row]));
+        const char* src = reinterpret_cast<const char*>(base + row_offset(lay, id.b, id.l, id.h, slots ? slots[row] : row));
         for (int c = lane & (lanes - 1); c < cpr; c += lanes) cp_async16(t0 + (uint32_t)(row * cpr + c) * 16u, src + c * 16);
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
 }
-// Rows 0..n-1 of one event from global memory into a dense shared tile by bulk copies that report to `bar`; one warp calls. As
-// few copies as the layout allows: pieces of 32 KB where rows are contiguous (whole pages where pages are), else a row each, the
-// rows over the lanes (starve, a testing aid: none at all, the wait for them runs out). (192 rows of K and V in fp32, d = 128: all threads' 16-byte copies took 13.3 of an event's 65 thousand cycles
-// to issue; one event 41.3 -> 37.6 us, 112 of them 46.5 -> 42.0.)
+template <int PENDING>
+__device__ __forceinline__ void cp_async_wait_pending() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+}
+// Rows that one bulk copy can take: up to 32 KB where rows are contiguous (at most a page, where pages are), else one.
+__device__ __forceinline__ int rows_per_copy(const DevLayout& lay, int row_bytes) {
+    if (lay.page_size == 0 ? lay.sn != lay.d : lay.s_page_n != lay.d) return 1;
+    const int run = max(32768 / row_bytes, 1);
+    if (lay.page_size == 0) return run;
+    return run > lay.page_size ? lay.page_size : 1 << (31 - __clz(run));   // (a power of two, like pages: no copy crosses one)
+}
+// Rows 0..n-1 of one event from global memory into a dense shared tile by bulk copies of `run` rows each, which report to `bar`; one
+// warp calls, its lanes share the copies. (192 rows of K and V in fp32, d = 128, contiguous: all threads' 16-byte copies took 13.3 of
+// an event's 65 thousand cycles to issue; one event 38.9 -> 34.8 us, 896 of them 240 -> 209.)
 template <typename T>
-__device__ __forceinline__ void load_tile_bulk(T* tile, const T* base, const DevLayout& lay, const EventId& id, int n, uint32_t bar, bool starve) {
+__device__ __forceinline__ void load_tile_bulk(T* tile, const T* base, const DevLayout& lay, const EventId& id, int n, uint32_t bar, int run) {
     const uint32_t row_bytes = (uint32_t)lay.d * (uint32_t)sizeof(T), t0 = smem_u32(tile);
     const int lane = threadIdx.x & 31;
     if (lane == 0) mbar_expect_tx(bar, (uint32_t)n * row_bytes);
     __syncwarp();
-    int run = 1;   // rows of a copy
-    if (lay.page_size == 0 ? lay.sn == lay.d : lay.s_page_n == lay.d) {
-        run = max(32768 / (int)row_bytes, 1);
-        if (lay.page_size && run > lay.page_size) run = lay.page_size;
-        else if (lay.page_size) run = 1 << (31 - __clz(run));   // (a power of two, like pages: no copy crosses one)
-    }
-    for (int row = lane * run; row < n && !starve; row += 32 * run)
+    for (int row = lane * run; row < n; row += 32 * run)
         bulk_g2s(t0 + (uint32_t)row * row_bytes, base + row_offset(lay, id.b, id.l, id.h, row), (uint32_t)min(run, n - row) * row_bytes, bar);
 }
+// Smallest copy that is worth a bulk copy: where rows lie apart or pages are small, one warp's many small ones are slower than all
+// threads' 16-byte copies. 896 events, us per call with bulk copies / 16-byte ones: copies of 64 bytes 115 / 87 (256 rows of 16
+// bf16, pages of 2), of 128 bytes 146 / 111 (192 of 64 bf16, rows apart), of 256 130 / 118 (pages of 2), of 512 117 / 117 (pages
+// of 4), 281 / 242 (192 of 128 fp32, rows apart) and 363 / 332 (160 of 256 bf16, rows apart), of 1024 111 / 115 (192 of 64 bf16, pages of
+// 8), 256 / 281 (192 of 128 fp32, pages of 2) and 344 / 367 (160 of 256 bf16, pages of 2).
+constexpr int kLeastBulk = 1024;
 
 constexpr int kResidentCtas = 2;       // most CTAs per SM that the registers of the kernel with the penalty allow
 constexpr int kResidentCtasTopk = 3;   // ... and of the one without: no triangle (896 events of 128 bf16 rows of 64: 107 us, with the
@@ -304,8 +316,22 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
             mbar_init_fence();
         }
         __syncwarp();
-        load_tile_bulk(Kt, Kg, lay, id, n, bar_k, a.starve);
-        load_tile_bulk(Vt, Vg, lay, id, n, bar_v, a.starve);
+    }
+    const int run = rows_per_copy(lay, d * (int)sizeof(T));
+    if (a.starve) {
+        // (a testing aid: nothing is requested and nobody reports to the barriers, the waits for them run out)
+    } else if (run * d * (int)sizeof(T) >= kLeastBulk) {
+        if (warp == 0) {
+            load_tile_bulk(Kt, Kg, lay, id, n, bar_k, run);
+            load_tile_bulk(Vt, Vg, lay, id, n, bar_v, run);
+        }
+    } else {
+        if (tid == 0) {   // (the copies are awaited as groups)
+            mbar_expect_tx(bar_k, 0);
+            mbar_expect_tx(bar_v, 0);
+        }
+        load_rows_async(Kt, Kg, lay, id, n, nullptr);
+        load_rows_async(Vt, Vg, lay, id, n, nullptr);
     }
     int pmax = INT_MIN;
     for (int j = tid; j < n; j += kThreads) {
@@ -319,6 +345,7 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
     const int members = fold_group(a, id, tab, d, g);
     long long pref = 0;
     if (gpos) pref = a.p_ref ? (long long)a.p_ref[id.b] : (long long)block_max_int(pmax, redi) + 1;
+    cp_async_wait_pending<1>();
     __syncthreads();
     if (!mbar_wait_bounded(bar_k, 0, a.wait_polls)) *late = 1;   // K has landed; V may still be under way
 
@@ -360,6 +387,7 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
             if (valid && lig == 0) keep_score(j, sc);
         }
     }
+    cp_async_wait_pending<0>();
     if (!mbar_wait_bounded(bar_v, 0, a.wait_polls)) *late = 1;
     __syncthreads();
     if (*late) {   // (everybody is past the barriers: their place is free)
@@ -510,7 +538,7 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
     // compaction: kept rows go to slots 0..picks-1 of the same buffer, all sources on chip first
     if (!k_tile) {
         load_rows_async(Kt, Kg, lay, id, picks, idx);
-        cp_async_wait_all();
+        cp_async_wait_pending<0>();
         __syncthreads();
     }
     const int cpr = d * (int)sizeof(T) / 16, lanes = min(pow2_ceil(cpr), 32), rows = 32 / lanes;

@@ -486,6 +486,13 @@ def test_resident_waits_run_out_and_report_status_3(dtype, N, d, budget, lam):
     assert np.all(g["status"] == 3)
     assert np.array_equal(g["K"], ev.K) and np.array_equal(g["V"], ev.V) and np.array_equal(g["pos"], ev.pos)
     check_all(ev, run_fused(ev), lam)
+    # rows apart: their copies are awaited in another way, beside the same two waits
+    K, V = torch.zeros((2, 2, 2, 2, N, d + 8), dtype=torch.float32 if dtype == synth.F32 else torch.bfloat16, device="cuda")[..., :d]
+    pos = dev(ev.pos)
+    K.copy_(dev(ev.K)); V.copy_(dev(ev.V))
+    sel = akv.alpha_compress_event(K, V, pos, dev(ev.qstat), budget, akv.Options(lam=lam, flags=akv.FLAG_TEST_STARVE_WAIT), p_ref=dev(ev.p_ref))
+    assert bool((sel.status == 3).all())
+    assert np.array_equal(akv.to_host_bits(K), ev.K) and np.array_equal(akv.to_host_bits(V), ev.V) and np.array_equal(pos.cpu().numpy(), ev.pos)
 
 
 def test_workspace_query_matches_the_route():
@@ -646,11 +653,13 @@ def test_kept_slots_in_order_at_the_edges_of_words(N, budget, lam):
 
 @pytest.mark.parametrize("dtype,N,d,page", [(synth.F32, 1, 128, 0), (synth.F32, 63, 128, 0), (synth.F32, 65, 128, 0), (synth.F32, 130, 128, 0),
                                             (synth.F32, 200, 64, 0), (synth.BF16, 256, 64, 0), (synth.F32, 70, 128, 1), (synth.F32, 70, 128, 16),
-                                            (synth.BF16, 90, 72, 32), (synth.F32, 192, 128, 64)])
+                                            (synth.BF16, 90, 72, 32), (synth.F32, 192, 128, 64), (synth.F32, 71, 128, 2), (synth.BF16, 200, 64, 4),
+                                            (synth.BF16, 200, 64, 8), (synth.F32, 65, 256, 0), (synth.BF16, 250, 8, 0), (synth.BF16, 250, 8, 64)])
 @pytest.mark.parametrize("padded", [False, True])
 def test_resident_tiles_by_bulk_copies(dtype, N, d, page, padded):
     """The resident kernel's tiles arrive in copies of 32 KB, whole pages or single rows (padded: rows that do not lie one
-    behind the other): sizes at and beside a copy's end, candidates that end inside one, pages in any order."""
+    behind the other), by bulk copies from 1 KB on, below by all threads: sizes at and beside a copy's end, candidates that end
+    inside one, pages in any order."""
     ev = synth.make_plain(2, 1, 2, N, d, max(1, N // 3), 0.5, dtype=dtype, seed=N + d)
     width = d + (8 if padded else 0)
     rng = np.random.default_rng(N)
