@@ -22,6 +22,7 @@
 // part of K; the others store their scores to the first one's shared memory and leave, the first one selects.
 #pragma once
 #include "akv_event_stream.cuh"
+#include "akv_split_rule.cuh"
 
 namespace akv {
 
@@ -169,7 +170,8 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
         // the stages of this CTA: all, or its share of them (in eights, so that rotations are taken afresh where they are
         // without a split and the scores are the same to the bit)
         const int all = (n + kStStageRows - 1) / kStStageRows;
-        const int share = SPLIT > 1 ? ((all + SPLIT - 1) / SPLIT + kChainRounds - 1) / kChainRounds * kChainRounds : all;
+        static_assert(kSplitStages == kChainRounds && kSplitStageRows == kStStageRows, "the rule of the split counts these stages");
+        const int share = SPLIT > 1 ? ((all + SPLIT - 1) / SPLIT + kSplitStages - 1) / kSplitStages * kSplitStages : all;
         const int first = rank * share, stages = max(min(all - first, share), 0);
         // (the testing aid: where others have stages too only they are starved, and the first CTA has to learn of it from them)
         const bool starve = a.starve && (SPLIT == 1 || rank != 0 || all <= share);

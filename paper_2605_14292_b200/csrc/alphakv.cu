@@ -392,22 +392,11 @@ static akv_status_t launch_prefill_split(akv_handle* h, const EventArgs& a, cuda
     CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, a, h->tab));
     return launched(FUSED ? "event_prefill" : "select_prefill");
 }
-// How many CTAs share an event's scoring. Two CTAs fit an SM, so up to as many events as SMs leave half of the places empty. A
-// split pays where scoring is long beside what it costs (the cluster's start, its barrier, the first CTA's selection alone).
-// Measured (148 SMs, us per call with 1, 2 and 4 CTAs per event): 28 events of 1100 rows 56 / 55 / 50, of 4096 85 / 68 / 57; 56
-// events of 2048 rows 66 / 57 / 58, of 4096 90 / 72 / 68; 112 events of 1100 rows 59 / 67 / 80, of 2048 75 / 70 / 82, of 4096
-// 96 / 85 / 104; 148 events of 2048 rows 79 / 76 / 106, of 4096 101 / 88 / 125. With more events than SMs it never pays: 222
-// events of 4096 rows 115 / 151 / 168, 896 of them 379 / 488 / 553.
-static int prefill_split(long long events, int N, int sms) {
-    if (events * 4 <= sms && N >= 1024) return 4;
-    if (events * 2 <= sms && N >= 3072) return 4;
-    return events <= sms && N >= 2048 ? 2 : 1;
-}
 template <bool FUSED>
 static akv_status_t launch_prefill(akv_handle* h, const EventArgs& a, cudaStream_t st, bool dry = false) {
     if constexpr (FUSED) {
         const long long E = (long long)a.lay.B * a.lay.L * a.lay.H;
-        const int split = prefill_split(E, a.lay.N, h->sm_count);
+        const int split = prefill_split(E, a.lay.N, h->sm_count, !a.greedy, a.n_cand != nullptr);
         if (split == 4) return launch_prefill_split<true, 4>(h, a, st, dry);
         if (split == 2) return launch_prefill_split<true, 2>(h, a, st, dry);
     }
