@@ -55,11 +55,12 @@ __device__ __forceinline__ void load_tile_bulk(T* tile, const T* base, const Dev
     for (int row = lane * run; row < n; row += 32 * run)
         bulk_g2s(t0 + (uint32_t)row * row_bytes, base + row_offset(lay, id.b, id.l, id.h, row), (uint32_t)min(run, n - row) * row_bytes, bar);
 }
-// Smallest copy that is worth a bulk copy: where rows lie apart or pages are small, one warp's many small ones are slower than all
-// threads' 16-byte copies. 896 events, us per call with bulk copies / 16-byte ones: copies of 64 bytes 115 / 87 (256 rows of 16
-// bf16, pages of 2), of 128 bytes 146 / 111 (192 of 64 bf16, rows apart), of 256 130 / 118 (pages of 2), of 512 117 / 117 (pages
-// of 4), 281 / 242 (192 of 128 fp32, rows apart) and 363 / 332 (160 of 256 bf16, rows apart), of 1024 111 / 115 (192 of 64 bf16, pages of
-// 8), 256 / 281 (192 of 128 fp32, pages of 2) and 344 / 367 (160 of 256 bf16, pages of 2).
+// Smallest copy of a paged cache that is worth a bulk copy; rows that lie apart in a dense one never are. One warp's many small
+// copies are slower than all threads' 16-byte ones, whose addresses cost more where they go through a block table. 896 events, us per call
+// with bulk copies / 16-byte ones. Pages: copies of 64 bytes 115 / 87 (256 rows of 16 bf16, pages of 2), of 256 130 / 118 (192 of 64 bf16,
+// pages of 2), of 512 117 / 117 (pages of 4) and 303 / 297 (192 of 128 fp32, pages of 1), of 1024 111 / 115 (192 of 64 bf16, pages of 8),
+// 256 / 281 (192 of 128 fp32, pages of 2) and 242 / 244 (96 of 256 fp32, pages of 1). Rows apart: of 128 bytes 146 / 111, of 512 281 / 242
+// (192 of 128 fp32) and 363 / 332 (160 of 256 bf16), of 1024 233 / 223 (96 of 256 fp32).
 constexpr int kLeastBulk = 1024;
 
 constexpr int kResidentCtas = 2;       // most CTAs per SM that the registers of the kernel with the penalty allow
@@ -320,7 +321,7 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
     const int run = rows_per_copy(lay, d * (int)sizeof(T));
     if (a.starve) {
         // (a testing aid: nothing is requested and nobody reports to the barriers, the waits for them run out)
-    } else if (run * d * (int)sizeof(T) >= kLeastBulk) {
+    } else if (lay.page_size ? run * d * (int)sizeof(T) >= kLeastBulk : run > 1) {
         if (warp == 0) {
             load_tile_bulk(Kt, Kg, lay, id, n, bar_k, run);
             load_tile_bulk(Vt, Vg, lay, id, n, bar_v, run);
