@@ -229,9 +229,13 @@ static void build_tables(akv_handle* h, int d, float base, int W) {
     h->tab_d = d; h->tab_base = base; h->tab_W = W;
 }
 
+// Lets a kernel's launch take `bytes` of dynamic shared memory. The limit belongs to the kernel, not to the call, and other threads'
+// calls set it too, between this one's setting and its launch. So it is the same for every call (what the device allows a CTA, minus
+// the kernel's static arrays), never the size that one of them needs.
+constexpr int kStaticSmem = 1024;   // most that a kernel with dynamic shared memory has in static arrays
 template <typename K>
-static akv_status_t set_smem(K kernel, unsigned bytes) {
-    if (bytes > 48 * 1024) CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+static akv_status_t set_smem(const akv_handle* h, K kernel, unsigned bytes, int static_bytes = 0) {
+    if (bytes > 48 * 1024) CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - static_bytes));
     return AKV_OK;
 }
 
@@ -299,7 +303,7 @@ static akv_status_t launch_select_pool(akv_handle* h, const EventArgs& a, cudaSt
     if (tile_rows > a.lay.N) tile_rows = a.lay.N;
     if (!a.greedy) tile_rows = 0;
     const PoolSmem sp = plan_pool_smem(a.lay.N, a.budget, row_bytes, tile_rows);
-    akv_status_t s = set_smem(select_pool_kernel<T, FLAT>, sp.total);
+    akv_status_t s = set_smem(h, select_pool_kernel<T, FLAT>, sp.total);
     if (s != AKV_OK || dry) return s;
     select_pool_kernel<T, FLAT><<<E, kThreads, sp.total, st>>>(a, tile_rows);
     return launched("select_pool");
@@ -324,7 +328,7 @@ static akv_status_t launch_tc(akv_handle* h, const EventArgs& a0, cudaStream_t s
     a.tmem_cols = !a.greedy ? 0 : (a.lay.N <= 128 || a.budget <= 64) ? 128 : 256;
     if ((int)sp.total > h->smem_optin) return fail(AKV_ERR_UNSUPPORTED, "budget %d needs too much shared memory", a.budget);
     akv_status_t s;
-    if ((s = set_smem(event_tc_kernel<FUSED>, sp.total)) != AKV_OK) return s;
+    if ((s = set_smem(h, event_tc_kernel<FUSED>, sp.total)) != AKV_OK) return s;
     CUDA_TRY(cudaFuncSetAttribute(event_tc_kernel<FUSED>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                   (int)cudaSharedmemCarveoutMaxShared));
     if (dry) return AKV_OK;
@@ -349,14 +353,14 @@ static akv_status_t launch_tri(akv_handle* h, const EventArgs& a, cudaStream_t s
     if ((int)sp.total > h->smem_optin) return fail(AKV_ERR_UNSUPPORTED, "budget %d needs too much shared memory", a.budget);
     akv_status_t s;
     if (BIG) {
-        if ((s = set_smem(event_pool_kernel<FUSED>, sp.total)) != AKV_OK) return s;
+        if ((s = set_smem(h, event_pool_kernel<FUSED>, sp.total)) != AKV_OK) return s;
         CUDA_TRY(cudaFuncSetAttribute(event_pool_kernel<FUSED>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                       (int)cudaSharedmemCarveoutMaxShared));
         if (dry) return AKV_OK;
         event_pool_kernel<FUSED><<<E, kTcThreads, sp.total, st>>>(a, h->tab);
         return launched(FUSED ? "event_pool" : "select_pool_active");
     }
-    if ((s = set_smem(event_tri_kernel<FUSED>, sp.total)) != AKV_OK) return s;
+    if ((s = set_smem(h, event_tri_kernel<FUSED>, sp.total)) != AKV_OK) return s;
     CUDA_TRY(cudaFuncSetAttribute(event_tri_kernel<FUSED>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                   (int)cudaSharedmemCarveoutMaxShared));
     if (dry) return AKV_OK;
@@ -374,7 +378,7 @@ static akv_status_t launch_prefill_split(akv_handle* h, const EventArgs& a, cuda
     const PfSmem sp = plan_pf_smem(a.lay.N, a.budget);
     akv_status_t s;
     auto kernel = event_prefill_kernel<FUSED, SPLIT>;
-    if ((s = set_smem(kernel, sp.total)) != AKV_OK) return s;
+    if ((s = set_smem(h, kernel, sp.total, kStaticSmem)) != AKV_OK) return s;
     CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
     if (dry) return AKV_OK;
     cudaLaunchConfig_t cfg;
@@ -422,15 +426,14 @@ static akv_status_t launch_compact(akv_handle* h, const CompactArgs& a0, cudaStr
     a.chunk_rows = rows;
     const unsigned bytes = (unsigned)rows * (2 * rowB + 8);
     if (a.lay.dtype == AKV_BF16) {
-        akv_status_t s = set_smem(compact_kernel<__nv_bfloat16>, bytes);
+        akv_status_t s = set_smem(h, compact_kernel<__nv_bfloat16>, bytes);
         if (s != AKV_OK || dry) return s;
         compact_kernel<__nv_bfloat16><<<E, kThreads, bytes, st>>>(a);
     } else {
-        akv_status_t s = set_smem(compact_kernel<float>, bytes);
+        akv_status_t s = set_smem(h, compact_kernel<float>, bytes);
         if (s != AKV_OK || dry) return s;
         compact_kernel<float><<<E, kThreads, bytes, st>>>(a);
     }
-    (void)h;
     return launched("compact");
 }
 
@@ -566,7 +569,7 @@ static akv_status_t kv_compact_impl(akv_handle_t* h, const akv_layout_t* lay, vo
 // scores in global memory.
 enum EventRoute { ROUTE_TRI, ROUTE_TRI_BIG, ROUTE_TC, ROUTE_PREFILL, ROUTE_STREAM, ROUTE_RESIDENT, ROUTE_THREE };
 // shared memory the streaming kernel may plan with: what the device allows minus its static arrays
-static int stream_smem_limit(int smem_optin) { return smem_optin - 1024; }
+static int stream_smem_limit(int smem_optin) { return smem_optin - kStaticSmem; }
 static bool stream_path_ok(const EventArgs& a, int smem_optin) {
     if (!(a.lay.dtype == AKV_BF16 && a.lay.d == kTcD && a.lay.N > kTcMaxN && a.lay.N <= 65535 && a.flat_sig == nullptr && !a.gqa_max)) return false;
     const StSmem sp = plan_st_smem(a.lay.N, a.budget, stream_smem_limit(smem_optin));
@@ -659,7 +662,7 @@ static akv_status_t alpha_compress_event_impl(akv_handle_t* h, const akv_layout_
     if (route == ROUTE_STREAM) {
         const int limit = stream_smem_limit(h->smem_optin);
         const StSmem sp = plan_st_smem(a.lay.N, a.budget, limit);
-        if ((s = set_smem(event_stream_kernel, sp.total)) != AKV_OK) return s;
+        if ((s = set_smem(h, event_stream_kernel, sp.total, kStaticSmem)) != AKV_OK) return s;
         event_stream_kernel<<<a.lay.B * a.lay.L * a.lay.H, kStThreads, sp.total, st>>>(a, h->tab, limit);
         return launched("event_stream");
     }
@@ -679,7 +682,7 @@ static akv_status_t alpha_compress_event_impl(akv_handle_t* h, const akv_layout_
         const unsigned total = res.total + (unsigned)(extra > 0 ? extra : 0);
         auto kernel = lay->dtype == AKV_BF16 ? (a.greedy ? event_resident_kernel<__nv_bfloat16, true> : event_resident_kernel<__nv_bfloat16, false>)
                                              : (a.greedy ? event_resident_kernel<float, true> : event_resident_kernel<float, false>);
-        if ((s = set_smem(kernel, total)) != AKV_OK) return s;
+        if ((s = set_smem(h, kernel, total)) != AKV_OK) return s;
         kernel<<<E, kThreads, total, st>>>(a, h->tab, extra > 0 ? extra : 0);
         return launched("event");
     }
@@ -779,7 +782,7 @@ static akv_status_t alpha_gram_shared_impl(akv_handle_t* h, const akv_layout_t* 
     const int tiles = (y.N + 127) / 128;
     const long long blocks = groups * tiles * tiles;
     if (blocks > INT_MAX) return fail(AKV_ERR_UNSUPPORTED, "alpha_gram_shared: %lld tiles exceed the grid limit", blocks);
-    if ((s = set_smem(gram_shared_kernel, kGramSmem)) != AKV_OK) return s;
+    if ((s = set_smem(h, gram_shared_kernel, kGramSmem, kStaticSmem)) != AKV_OK) return s;
     gram_shared_kernel<<<(unsigned)blocks, kGramThreads, kGramSmem, (cudaStream_t)stream>>>(sig, n_cand, seq_div, y.N, gram, status);
     return launched("gram_shared");
 }
