@@ -643,6 +643,58 @@ def test_first_cta_learns_that_another_gave_up(L, H, N):
     check_all(ev, good, 0.5, events=[0, L * H - 1])
 
 
+@pytest.mark.parametrize("L,H,N,lam", [(2, 2, 1100, 0.0), (2, 2, 1100, 0.5), (2, 19, 2048, 0.0), (2, 19, 2113, 0.5), (5, 15, 3072, 0.0), (5, 15, 2048, 0.5)])
+def test_shared_scoring_of_all_kinds_of_call(L, H, N, lam):
+    """Four or two CTAs per event, with and without the penalty: budgets per head, a non-finite key in every CTA's part and pages in
+    any order, against the same events in a call that takes one CTA each, to the bit, and a few events against the oracle."""
+    ev = synth.make_plain(1, L, H, N, 128, 40, lam, dtype=synth.BF16, seed=N + H)
+    rng = np.random.default_rng(N)
+    times = 512 // (L * H)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    split = akv_split.prefill_split(L * H, N, sms, topk=lam == 0.0)
+    assert split > 1 and akv_split.prefill_split(L * H * times, N, sms, topk=lam == 0.0) == 1
+    many = synth.make_plain(times, 1, 1, 1, 128, 1, lam, dtype=synth.BF16, seed=0)
+    many.qstat, many.budget = ev.qstat, ev.budget
+
+    def both(**kw):
+        for name in ("K", "V", "pos", "p_ref"):
+            setattr(many, name, np.repeat(getattr(ev, name), times, axis=0))
+        a, b = run_fused(ev, lam=lam, **kw), run_fused(many, lam=lam, **kw)
+        for k, x in a.items():
+            assert np.array_equal(x[0], b[k][-1], equal_nan=x.dtype == np.float32), k
+        return a
+
+    check_all(ev, both(), lam, events=[0, L * H - 1])
+    budgets = rng.integers(1, 41, size=(L, H)).astype(np.int32)
+    budgets[0, 0], budgets[-1, -1] = 40, 1
+    check_all(ev, both(budgets=budgets), lam, events=[0, L * H - 1], budgets=budgets)
+    # the same rows in pages
+    K, V, pos, q, pref = (dev(x) for x in (ev.K, ev.V, ev.pos, ev.qstat, ev.p_ref))
+    plain = run_fused(ev, lam=lam)
+    for page in (64, 16):
+        pps = -(-N // page)
+        table = torch.as_tensor(rng.permutation(pps), device="cuda").to(torch.int32).view(1, pps)
+        pools = torch.zeros((2, L, pps, H, page, 128), dtype=torch.bfloat16, device="cuda")
+        for x, pool in zip((K, V), pools):
+            rows = torch.zeros((L, H, pps * page, 128), dtype=torch.bfloat16, device="cuda")
+            rows[:, :, :N] = x[0]
+            pool[:, table[0].long()] = rows.view(L, H, pps, page, 128).permute(0, 2, 1, 3, 4)
+        p = pos.clone()
+        sel = akv.alpha_compress_event(pools[0], pools[1], p, q, 40, akv.Options(lam=lam), p_ref=pref, layout=akv.Layout.paged(pools[0], table, N), want_scores=True)
+        for k, x in (("order", sel.pick_order), ("idx", sel.idx_sorted), ("gain", sel.pick_gain), ("scores", sel.scores), ("pos", p)):
+            assert np.array_equal(x.cpu().numpy(), plain[k]), (k, page)
+        for name, pool in zip(("K", "V"), pools):
+            rows = pool[:, table[0].long()].permute(0, 2, 1, 3, 4).reshape(L, H, pps * page, 128)[:, :, :N]
+            assert np.array_equal(akv.to_host_bits(rows.contiguous()), plain[name][0]), (name, page)
+    # a key without a finite score in every CTA's part
+    share = 64 * akv_split.split_share((N + 63) // 64, split)
+    bad = [c * share + 5 for c in range(split) if c * share + 5 < N]
+    assert len(bad) > 1
+    ev.K[..., bad, 3] = 0x7F80 if ev.K.dtype == np.uint16 else np.inf
+    g = both()
+    assert np.all(g["status"] == 1) and not set(bad) & set(g["idx"].ravel().tolist())
+
+
 @pytest.mark.parametrize("N,budget", [(129, 65), (130, 128), (160, 97), (161, 128), (224, 100), (255, 128), (256, 127)])
 @pytest.mark.parametrize("lam", [0.0, 0.5])
 def test_kept_slots_in_order_at_the_edges_of_words(N, budget, lam):
@@ -850,7 +902,8 @@ def test_shared_cosine_matrix(mode, N):
             assert np.all(rest == 0)                                  # rows beyond the candidates are left alone
 
 
-@pytest.mark.parametrize("mode,N,budget", [("flat", 256, 128), ("flat", 192, 64), ("layer", 256, 100), ("flat", 130, 20)])
+@pytest.mark.parametrize("mode,N,budget", [("flat", 256, 128), ("flat", 192, 64), ("layer", 256, 100), ("flat", 130, 20), ("flat", 8, 3),
+                                           ("layer", 31, 31), ("flat", 32, 17), ("flat", 33, 8)])
 def test_fused_event_with_shared_cosine_matrix(mode, N, budget):
     """Shared signatures in the fused path: signature pass, one cosine matrix per sequence (and layer), then every
     event of the sequence in ONE launch that reads its cosines from that matrix. Checked against the oracle with
