@@ -7,8 +7,8 @@
 // the K tile, which scoring is done with (the kept K rows are then read again for the compaction), the triangle is filled
 // by plain fp32 dot products and Algorithm 1 runs as the one-warp loop of the tensor-memory kernels. A pool that does not
 // fit is taken in rounds of active sets (picks_in_rounds). Otherwise, and for lambda = 0, the CTA-wide loop with rows of the
-// cosine matrix on demand (greedy_cta). (896 events of 256 bf16 rows of 64, 128 kept, lambda = 0.5: 345 us in rounds, 1471 in
-// the CTA-wide loop, 556 with the whole triangle and one CTA per SM.)
+// cosine matrix on demand (greedy_cta). (896 events of 256 bf16 rows of 64, 128 kept, lambda = 0.5, the
+// call alone: 345 us in rounds, 1471 in the CTA-wide loop, 556 with the whole triangle and one CTA per SM.)
 //
 // The dot products are bound by shared-memory reads, so a thread takes 8 x 4 pairs of rows at a time (12 reads for
 // 128 multiply-adds a step instead of 2 for 4), walking the head dimension from its own starting column so that a warp's loads

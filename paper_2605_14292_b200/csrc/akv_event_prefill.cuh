@@ -18,8 +18,8 @@
 //   4. Kept K and V rows are staged on chip and written to slots 0..b-1 of the same buffers.
 //
 // FUSED: score + select + compact; otherwise selection only (scores are read from a.scores and nothing is rewritten).
-// SPLIT: the scoring of an event is shared by a cluster of so many CTAs, for calls of few and long events. Each streams its
-// part of K; the others store their scores to the first one's shared memory and leave, the first one selects.
+// SPLIT: the scoring of an event is shared by a cluster of so many CTAs, for calls of few and long events (akv_split_rule.cuh says
+// which). Each streams its part of K; the others store their scores to the first one's shared memory and leave, the first one selects.
 #pragma once
 #include "akv_event_stream.cuh"
 #include "akv_split_rule.cuh"
@@ -202,8 +202,8 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
         } else {
             // ---- positions on chip; D: the spacing of rows one stage apart at the newest end, which a cache filled token
             // by token has everywhere (found once, the scoring loop then chains without looking at positions)
-            // (every load of a thread is requested before the first is used: 896 events of 4096 rows 382.5 -> 378.6 us, without picks
-            // 283.8 -> 279.9)
+            // (every load of a thread is requested before the first is used: 896 events of 4096 rows 383.0 -> 379.4 us, without picks
+            // 284.2 -> 280.6, a gain of 1 %, hardly more than runs of the same code differ by)
             const int p_last = rotate && n > kStStageRows ? gpos[n - 1] : 0, p_back = rotate && n > kStStageRows ? gpos[n - 1 - kStStageRows] : 0;
             const int p_ref = rotate && a.p_ref ? a.p_ref[id.b] : 0;
             int p[kPfKeys];
