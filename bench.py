@@ -54,17 +54,17 @@ KERNELS = {"C1": "event_resident_kernel<float>", "C2": "event_pool_kernel<fused>
 # capture of another revision is reported as null.
 NCU_TRAFFIC = {
     # one launch of 4096 events captured whole (profiles/event_tri_kernel_bf16_C3.md)
-    "C3": {"bytes": 320505344 + 97829632, "revision": "16bbe4dc64a6"},
+    "C3": {"bytes": 321168384 + 97798144, "revision": "89e57f158592"},
     # one launch of 4096 events (16 sequences) captured; a step is 4 x 32 launches of that size
     # (profiles/event_pool_kernel_bf16_C5.md)
-    "C5": {"bytes": (487292416 + 229692160) * 128, "revision": "16bbe4dc64a6"},
+    "C5": {"bytes": (490664704 + 228997376) * 128, "revision": "89e57f158592"},
     # the same kernel and capture, scaled to 112 events
-    "C2": {"bytes": (487292416 + 229692160) * 112 // 4096, "revision": "16bbe4dc64a6"},
+    "C2": {"bytes": (490664704 + 228997376) * 112 // 4096, "revision": "89e57f158592"},
     # the three launches (lambda 0, 0.5, 1) of a 2-sequence batch captured; the bench batch has 8 sequences
     # (profiles/event_prefill_kernel_bf16_C4.md)
-    "C4": {"bytes": ((251964928 + 4013824) + (256004864 + 4015872) + (262309120 + 4198912)) * 4, "revision": "16bbe4dc64a6"},
+    "C4": {"bytes": ((251835392 + 3809024) + (256178688 + 3383040) + (262305280 + 3479808)) * 4, "revision": "89e57f158592"},
     # the step's three launches captured whole (profiles/gram_shared_kernel_f32_C6.md)
-    "C6": {"bytes": (117470464 + 3307520) + 2136832 + (181025792 + 72201728), "revision": "16bbe4dc64a6"},
+    "C6": {"bytes": (117467392 + 3519488) + 2136576 + (181068544 + 73741568), "revision": "89e57f158592"},
 }
 
 
