@@ -168,14 +168,11 @@ class Layout:
                       block_table, (sp, sh, sn))
 
     def c(self) -> _Layout:
-        y = _Layout()
-        y.B, y.L, y.H, y.N, y.d, y.dtype = self.B, self.L, self.H, self.N, self.d, self.dtype
-        y.stride_b, y.stride_l, y.stride_h, y.stride_n = self.strides
-        y.page_size = self.page_size
-        y.block_table = _ptr(self.block_table)
-        y.pages_per_seq = 0 if self.block_table is None else int(self.block_table.shape[1])
-        y.stride_page, y.stride_page_h, y.stride_page_n = self.page_strides
-        return y
+        table = self.block_table
+        sb, sl, sh, sn = self.strides
+        sp, sph, spn = self.page_strides
+        return _Layout(self.B, self.L, self.H, self.N, self.d, self.dtype, sb, sl, sh, sn, self.page_size, _ptr(table),
+                       0 if table is None else int(table.shape[1]), sp, sph, spn)
 
     @property
     def n_events(self) -> int:
@@ -191,7 +188,7 @@ def _dtype_code(x: torch.Tensor) -> int:
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()   # (the entry points' argument types make it a pointer)
 
 
 def _need(t: Optional[torch.Tensor], dtype, name: str, cuda=True):
@@ -209,19 +206,25 @@ def _pos_strides(pos: Optional[torch.Tensor], lay: Layout):
     """pos may be [N], [B, N] or [B, L, H, N] (int32, last dim contiguous); returns (b, l, h) strides."""
     if pos is None:
         return 0, 0, 0
-    if pos.dtype != torch.int32 or pos.stride(-1) != 1 or pos.shape[-1] < lay.N:
+    st = pos.stride()
+    if pos.dtype != torch.int32 or st[-1] != 1 or pos.shape[-1] < lay.N:
         raise ValueError("pos must be int32 with a contiguous last dimension of at least N slots")
-    if pos.dim() == 1:
+    if len(st) == 1:
         return 0, 0, 0
-    if pos.dim() == 2:
-        return int(pos.stride(0)), 0, 0
-    if pos.dim() == 4:
-        return int(pos.stride(0)), int(pos.stride(1)), int(pos.stride(2))
+    if len(st) == 2:
+        return st[0], 0, 0
+    if len(st) == 4:
+        return st[:3]
     raise ValueError("pos must have 1, 2 or 4 dimensions")
 
 
-def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+def _call(entry: str, device: torch.device, *args):
+    """One entry point on `device` and its current stream. The device is switched to only where it is another one."""
+    if device.type == "cuda" and device.index == torch.cuda.current_device():
+        _check(getattr(load_library(), entry)(_handle(device), *args, torch._C._cuda_getCurrentRawStream(device.index)))
+        return
+    with torch.cuda.device(device):
+        _check(getattr(load_library(), entry)(_handle(device), *args, torch.cuda.current_stream().cuda_stream))
 
 
 def _lay(x: torch.Tensor, layout: Optional[Layout]) -> Layout:
@@ -239,10 +242,8 @@ def alpha_score(K, qstat, pos=None, p_ref=None, n_cand=None, opts: Optional[Opti
         out = torch.zeros((lay.B, lay.L, lay.H, lay.N), dtype=torch.float32, device=K.device)
     _need(out, torch.float32, "out"); _need(status, torch.int32, "status")
     sb, sl, sh = _pos_strides(pos, lay)
-    with torch.cuda.device(K.device):
-        _check(load_library().alpha_score(_handle(K.device), C.byref(lay.c()), _ptr(K), _ptr(pos), sb, sl, sh,
-                                          _ptr(n_cand), _ptr(qstat), _ptr(p_ref), C.byref(opts.c()), _ptr(out),
-                                          _ptr(status), _stream()))
+    _call("alpha_score", K.device, C.byref(lay.c()), _ptr(K), _ptr(pos), sb, sl, sh, _ptr(n_cand), _ptr(qstat),
+          _ptr(p_ref), C.byref(opts.c()), _ptr(out), _ptr(status))
     return out
 
 
@@ -280,11 +281,9 @@ def alpha_select(scores, V, budget: int, opts: Optional[Options] = None, flat_si
     lay = layout
     _need(scores, torch.float32, "scores"); _need(flat_sig, torch.float32, "flat_sig"); _need(n_cand, torch.int32, "n_cand")
     sel = out or _alloc_sel(lay, budget, scores.device, detail)
-    with torch.cuda.device(scores.device):
-        _check(load_library().alpha_select(_handle(scores.device), C.byref(lay.c()), _ptr(scores), _ptr(V),
-                                           _ptr(flat_sig), _ptr(n_cand), budget, C.byref(opts.c()),
-                                           _ptr(sel.idx_sorted), _ptr(sel.pick_order), _ptr(sel.pick_gain),
-                                           _ptr(sel.n_kept), _ptr(sel.status), _stream()))
+    _call("alpha_select", scores.device, C.byref(lay.c()), _ptr(scores), _ptr(V), _ptr(flat_sig), _ptr(n_cand),
+          budget, C.byref(opts.c()), _ptr(sel.idx_sorted), _ptr(sel.pick_order), _ptr(sel.pick_gain),
+          _ptr(sel.n_kept), _ptr(sel.status))
     return sel
 
 
@@ -295,9 +294,7 @@ def alpha_signature_flat(V, opts: Optional[Options] = None, n_cand=None, layout:
     if out is None:
         out = torch.zeros((lay.B, lay.N, lay.d), dtype=torch.float32, device=V.device)
     _need(out, torch.float32, "out")
-    with torch.cuda.device(V.device):
-        _check(load_library().alpha_signature_flat(_handle(V.device), C.byref(lay.c()), _ptr(V), _ptr(n_cand),
-                                                   C.byref(opts.c()), _ptr(out), _stream()))
+    _call("alpha_signature_flat", V.device, C.byref(lay.c()), _ptr(V), _ptr(n_cand), C.byref(opts.c()), _ptr(out))
     return out
 
 
@@ -309,9 +306,7 @@ def alpha_signature_layer(V, opts: Optional[Options] = None, n_cand=None, layout
     if out is None:
         out = torch.zeros((lay.B, lay.L, lay.N, lay.d), dtype=torch.float32, device=V.device)
     _need(out, torch.float32, "out")
-    with torch.cuda.device(V.device):
-        _check(load_library().alpha_signature_layer(_handle(V.device), C.byref(lay.c()), _ptr(V), _ptr(n_cand),
-                                                    C.byref(opts.c()), _ptr(out), _stream()))
+    _call("alpha_signature_layer", V.device, C.byref(lay.c()), _ptr(V), _ptr(n_cand), C.byref(opts.c()), _ptr(out))
     return out
 
 
@@ -324,9 +319,8 @@ def alpha_gram_shared(sig, layout: Layout, opts: Options, n_cand=None, out=None,
         shape = (lay.B, lay.N, lay.N) if opts.sig_mode == SIG_FLAT else (lay.B, lay.L, lay.N, lay.N)
         out = torch.zeros(shape, dtype=torch.float32, device=sig.device)
     _need(out, torch.float32, "out")
-    with torch.cuda.device(sig.device):
-        _check(load_library().alpha_gram_shared(_handle(sig.device), C.byref(lay.c()), _ptr(sig), _ptr(n_cand),
-                                                C.byref(opts.c()), _ptr(out), _ptr(status), _stream()))
+    _call("alpha_gram_shared", sig.device, C.byref(lay.c()), _ptr(sig), _ptr(n_cand), C.byref(opts.c()), _ptr(out),
+          _ptr(status))
     return out
 
 
@@ -344,9 +338,8 @@ def kv_compact(K, V, pos, idx_sorted, layout: Optional[Layout] = None):
     _need(idx_sorted, torch.int32, "idx_sorted")
     budget = int(idx_sorted.shape[-1])
     sb, sl, sh = _pos_strides(pos, lay)
-    with torch.cuda.device(ref.device):
-        _check(load_library().kv_compact(_handle(ref.device), C.byref(lay.c()), _ptr(K), _ptr(V), _ptr(pos), sb, sl, sh,
-                                         _ptr(idx_sorted), budget, _stream()))
+    _call("kv_compact", ref.device, C.byref(lay.c()), _ptr(K), _ptr(V), _ptr(pos), sb, sl, sh, _ptr(idx_sorted),
+          budget)
 
 
 def alpha_compress_event(K, V, pos, qstat, budget: int, opts: Optional[Options] = None, p_ref=None, n_cand=None,
@@ -362,11 +355,9 @@ def alpha_compress_event(K, V, pos, qstat, budget: int, opts: Optional[Options] 
     if want_scores and sel.scores is None:
         sel.scores = torch.zeros((lay.B, lay.L, lay.H, lay.N), dtype=torch.float32, device=K.device)
     sb, sl, sh = _pos_strides(pos, lay)
-    with torch.cuda.device(K.device):
-        _check(load_library().alpha_compress_event(
-            _handle(K.device), C.byref(lay.c()), _ptr(K), _ptr(V), _ptr(pos), sb, sl, sh, _ptr(n_cand), _ptr(qstat),
-            _ptr(p_ref), _ptr(flat_sig), budget, C.byref(opts.c()), _ptr(sel.idx_sorted), _ptr(sel.pick_order),
-            _ptr(sel.pick_gain), _ptr(sel.scores), _ptr(sel.n_kept), _ptr(sel.status), _stream()))
+    _call("alpha_compress_event", K.device, C.byref(lay.c()), _ptr(K), _ptr(V), _ptr(pos), sb, sl, sh, _ptr(n_cand),
+          _ptr(qstat), _ptr(p_ref), _ptr(flat_sig), budget, C.byref(opts.c()), _ptr(sel.idx_sorted),
+          _ptr(sel.pick_order), _ptr(sel.pick_gain), _ptr(sel.scores), _ptr(sel.n_kept), _ptr(sel.status))
     return sel
 
 
@@ -387,11 +378,9 @@ def alpha_compress_event_static(K, V, pos, qstat, budget: int, opts: Optional[Op
     _need(flat_sig, torch.float32, "flat_sig")
     sel = out or _alloc_sel(lay, budget, K.device, detail)
     sb, sl, sh = _pos_strides(pos, lay)
-    with torch.cuda.device(K.device):
-        _check(load_library().alpha_compress_event_static(
-            _handle(K.device), C.byref(lay.c()), _ptr(K), _ptr(V), _ptr(pos), sb, sl, sh, _ptr(n_cand), _ptr(qstat),
-            _ptr(p_ref), _ptr(flat_sig), budget, C.byref(opts.c()), _ptr(sel.idx_sorted), _ptr(sel.pick_order),
-            _ptr(sel.pick_gain), _ptr(sel.n_kept), _ptr(sel.status), _stream()))
+    _call("alpha_compress_event_static", K.device, C.byref(lay.c()), _ptr(K), _ptr(V), _ptr(pos), sb, sl, sh,
+          _ptr(n_cand), _ptr(qstat), _ptr(p_ref), _ptr(flat_sig), budget, C.byref(opts.c()), _ptr(sel.idx_sorted),
+          _ptr(sel.pick_order), _ptr(sel.pick_gain), _ptr(sel.n_kept), _ptr(sel.status))
     return sel
 
 
