@@ -68,6 +68,28 @@ constexpr int kResidentCtasTopk = 3;   // ... and of the one without: no triangl
                                        // other's 128 registers 156)
 constexpr int kResidentLeastSet = 64;  // rows from which an active set is worth its triangle
 
+// Where a row's values lie: four at a time from global memory, or from shared memory by 32-bit address (a generic pointer's loads
+// and arithmetic cost more).
+struct GlobalRow {
+    const float* p;
+    __device__ __forceinline__ GlobalRow operator+(int n) const { return {p + n}; }
+    __device__ __forceinline__ void load(float (&x)[4]) const { load4(p, x); }
+};
+template <typename T>
+struct SharedRow {
+    uint32_t at;
+    __device__ __forceinline__ SharedRow operator+(int n) const { return {at + (uint32_t)(n * (int)sizeof(T))}; }
+    __device__ __forceinline__ void load(float (&x)[4]) const {
+        if constexpr (sizeof(T) == 4) {
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]) : "r"(at));
+        } else {
+            uint32_t a, b;
+            asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "r"(at));
+            x[0] = bf16lo(a); x[1] = bf16hi(a); x[2] = bf16lo(b); x[3] = bf16hi(b);
+        }
+    }
+};
+
 // Raw dot products of every pair of the R rows listed in `rows` (i >= j) -> the triangle `tri`, 8 x 4 at a time: thread x
 // takes blocks x, x + 256, ...; row band b of eight rows has 2 b + 2 blocks, so it starts at block b (b + 1). row_of: slot ->
 // values.
@@ -87,19 +109,19 @@ __device__ __forceinline__ void fill_triangle(RowOf row_of, const unsigned short
 #pragma unroll
         for (int q = 0; q < 4; ++q) vj[q] = row_of(rows[min(4 * bj + q, R - 1)]);
         int gq = tid % G4;
+#pragma unroll 1
         for (int c = 0; c < G4; ++c) {
-            float xj[4][4];
+            float xi[8][4], xj[4][4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) load4(vj[q] + 4 * gq, xj[q]);
+            for (int q = 0; q < 4; ++q) (vj[q] + 4 * gq).load(xj[q]);
 #pragma unroll
-            for (int p = 0; p < 8; ++p) {
-                float xi[4];
-                load4(vi[p] + 4 * gq, xi);
+            for (int p = 0; p < 8; ++p) (vi[p] + 4 * gq).load(xi[p]);
+#pragma unroll
+            for (int p = 0; p < 8; ++p)
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) acc[p][q] = fmaf(xi[e], xj[q][e], acc[p][q]);
-            }
+                    for (int e = 0; e < 4; ++e) acc[p][q] = fmaf(xi[p][e], xj[q][e], acc[p][q]);
             gq = gq + 1 == G4 ? 0 : gq + 1;
         }
 #pragma unroll
@@ -242,8 +264,8 @@ __device__ __noinline__ int picks_in_rounds(const EventArgs& a, unsigned char* s
         const bool beside = 2 * R * (R + 1) <= room_beside;
         if (!beside) over_k = kRoundsOverK;
         float* tri = reinterpret_cast<float*>(beside ? smem + sp.total + (state_beside ? rs.total : 0u) : smem + sp.tileK + (state_beside ? 0u : rs.total));
-        if (sig) fill_triangle([&](int j) { return sig + (long long)j * d; }, act, R, d, tri);
-        else fill_triangle([&](int j) { return Vt + (size_t)j * d; }, act, R, d, tri);
+        if (sig) fill_triangle([&](int j) { return GlobalRow{sig + (long long)j * d}; }, act, R, d, tri);
+        else fill_triangle([&](int j) { return SharedRow<T>{smem_u32(Vt) + (uint32_t)(j * d * (int)sizeof(T))}; }, act, R, d, tri);
         __syncthreads();
         if (warp == 0) {
             const bool ok = picks_cosine<8, true>(lane, R, picks - made, s, act, ar, a.lam, tri, park_key + made, order + made, bound, am, made_holder, am,
@@ -306,6 +328,7 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
     T* Kg = reinterpret_cast<T*>(a.K);
     T* Vg = reinterpret_cast<T*>(a.V);
 
+    phase_stamp(id.e, 0);  // phases: 0 start, 1 K landed, 2 scores, V landed, 3 norms, 4 pool, 5 triangle, 6 picks, 7 outputs, 8 end
     // stage the event on chip (the barriers' place is the reductions', which come later)
     const uint32_t bar_k = smem_u32(red), bar_v = bar_k + 8;
     volatile int* late = reinterpret_cast<volatile int*>(red) + 4;   // a wait for them ran out
@@ -349,6 +372,7 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
     cp_async_wait_pending<1>();
     __syncthreads();
     if (!mbar_wait_bounded(bar_k, 0, a.wait_polls)) *late = 1;   // K has landed; V may still be under way
+    phase_stamp(id.e, 1);
 
     // scores: four rows of a lane group at a time, so that one row's dependent steps fill another's latency
     const int G = pow2_ceil(d >> 3) > 32 ? 32 : pow2_ceil(d >> 3);
@@ -404,6 +428,7 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
         mbar_inval(bar_k);
         mbar_inval(bar_v);
     }
+    phase_stamp(id.e, 2);
     // reciprocal norms: a thread per row, each lane from its own block of eight elements on (different banks). A block's
     // squares in two chains of four, the blocks in eight sums: an error of 4.2e-8 at d = 128, as from sixteen lanes' partial
     // sums; one chain of all squares has 1.6e-7.
@@ -432,6 +457,7 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
         }
     }
     bad = __syncthreads_or(bad);
+    phase_stamp(id.e, 3);
 
     // selection
     const int bud = event_budget(a, id);
@@ -447,25 +473,37 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
         unsigned short* bypool = reinterpret_cast<unsigned short*>(m);
         float* sb_holder = reinterpret_cast<float*>(red);
         int* pool_holder = redi;
-        // s_(b): the value v with fewer than `picks` scores above it and at least `picks` not below it
-        uint32_t* keys = reinterpret_cast<uint32_t*>(m);   // (padded to a multiple of four with keys below every real one)
-        const int n4 = (n + 3) & ~3;
-        for (int j = tid; j < n4; j += kThreads) keys[j] = j < n ? orderable(s[j]) : 0u;
-        __syncthreads();
-        for (int j = tid; j < n; j += kThreads) {
-            const uint32_t kj = keys[j];
-            int gt = 0, ge = 0;
+        float sb;
+        if (n <= kThreads) {
+            // s_(b) from below to 2^-9 of its value, which is all that pruning needs: a key per thread, a bit per count, and the
+            // barrier does the counting. (The exact value by counting every other key, as below: 5.1 of one event's 55 thousand
+            // cycles, 3.1 so; 896 events of 192 fp32 rows 205 -> 195 us, of 256 bf16 rows of 64 332 -> 322.)
+            const uint32_t kj = tid < n ? orderable(s[tid]) : 0u;
+            uint32_t kb = 0u;
+            for (int lo = 31; lo >= 14; --lo)
+                if (__syncthreads_count(kj >= (kb | (1u << lo))) >= picks) kb |= 1u << lo;
+            sb = kb < 0x00800000u ? -INFINITY : from_orderable(kb);
+        } else {
+            // s_(b): the value v with fewer than `picks` scores above it and at least `picks` not below it
+            uint32_t* keys = reinterpret_cast<uint32_t*>(m);   // (padded to a multiple of four with keys below every real one)
+            const int n4 = (n + 3) & ~3;
+            for (int j = tid; j < n4; j += kThreads) keys[j] = j < n ? orderable(s[j]) : 0u;
+            __syncthreads();
+            for (int j = tid; j < n; j += kThreads) {
+                const uint32_t kj = keys[j];
+                int gt = 0, ge = 0;
 #pragma unroll 4
-            for (int i = 0; i < n4; i += 4) {
-                const uint4 k4 = *reinterpret_cast<const uint4*>(keys + i);
-                gt += (k4.x > kj) + (k4.y > kj) + (k4.z > kj) + (k4.w > kj);
-                ge += (k4.x >= kj) + (k4.y >= kj) + (k4.z >= kj) + (k4.w >= kj);
+                for (int i = 0; i < n4; i += 4) {
+                    const uint4 k4 = *reinterpret_cast<const uint4*>(keys + i);
+                    gt += (k4.x > kj) + (k4.y > kj) + (k4.z > kj) + (k4.w > kj);
+                    ge += (k4.x >= kj) + (k4.y >= kj) + (k4.z >= kj) + (k4.w >= kj);
+                }
+                if (gt < picks && picks <= ge) *sb_holder = s[j];
             }
-            if (gt < picks && picks <= ge) *sb_holder = s[j];
+            __syncthreads();
+            sb = *sb_holder;
         }
-        __syncthreads();
-        const float sb = *sb_holder;
-        const float thr = a.no_prune ? -INFINITY : fmaf(-1.001f, a.lam, sb) - 1e-6f * fabsf(sb);
+        const float thr = a.no_prune || sb == -INFINITY ? -INFINITY : fmaf(-1.001f, a.lam, sb) - 1e-6f * fabsf(sb);
         if (warp == 0) {
             int base = 0;
             for (int j0 = 0; j0 < n; j0 += 32) {
@@ -486,17 +524,20 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
             k_tile = beside;
             float* tri = reinterpret_cast<float*>(beside ? smem + sp.total : smem + sp.tileK);
             const float* sig = a.flat_sig ? event_sig(a, id) : nullptr;
+            phase_stamp(id.e, 4);
             // the norms, by slot until now, by pool row from here on
             const float own_r = tid < P && !sig ? r[bypool[tid]] : 1.f;
             __syncthreads();
             if (tid < P) r[tid] = own_r;
-            if (sig) fill_triangle([&](int j) { return sig + (long long)j * d; }, bypool, P, d, tri);
-            else fill_triangle([&](int j) { return (const T*)Vt + (size_t)j * d; }, bypool, P, d, tri);
+            if (sig) fill_triangle([&](int j) { return GlobalRow{sig + (long long)j * d}; }, bypool, P, d, tri);
+            else fill_triangle([&](int j) { return SharedRow<T>{smem_u32(Vt) + (uint32_t)(j * d * (int)sizeof(T))}; }, bypool, P, d, tri);
             __syncthreads();
+            phase_stamp(id.e, 5);
             uint32_t* park_key = reinterpret_cast<uint32_t*>(gain);
             if (warp == 0) {
-                if (P <= 128) picks_cosine<4, false>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order);
-                else picks_cosine<8, false>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order);
+                // (in pairs: 896 events of 192 fp32 rows 196.6 -> 192.5 us; one event's loop 12.1 -> 10.4 thousand cycles)
+                if (P <= 128) picks_in_pairs<4, false>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order);
+                else picks_in_pairs<8, false>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order);
             }
             __syncthreads();
             for (int t = tid; t < picks; t += kThreads) {
@@ -526,6 +567,7 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
             greedy_cta<T>(n, picks, a.lam, PENALTY, d, s, r, m, taken, order, gain, rows, red);
         }
     }
+    phase_stamp(id.e, 6);
     ordered_indices(n, a.budget, taken, idx);
     __syncthreads();
 
@@ -536,6 +578,7 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
         if (a.pick_order) a.pick_order[ob + t] = t < picks ? order[t] : -1;
         if (a.pick_gain) a.pick_gain[ob + t] = t < picks ? gain[t] : 0.f;
     }
+    phase_stamp(id.e, 7);
     // compaction: kept rows go to slots 0..picks-1 of the same buffer, all sources on chip first
     if (!k_tile) {
         load_rows_async(Kt, Kg, lay, id, picks, idx);
@@ -557,6 +600,7 @@ __global__ void __launch_bounds__(kThreads, PENALTY ? kResidentCtas : kResidentC
         int* wpos = a.pos.p + id.b * a.pos.sb + id.l * a.pos.sl + id.h * a.pos.sh;
         for (int t = tid; t < picks; t += kThreads) wpos[t] = spos[idx[t]];
     }
+    phase_stamp(id.e, 8);
 }
 
 }  // namespace akv

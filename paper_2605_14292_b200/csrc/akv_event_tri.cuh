@@ -372,6 +372,176 @@ __device__ __forceinline__ bool picks_cosine(int lane, int P, int picks, const f
     return true;
 }
 
+// The same loop where few events share an SM and the chain of one pick after another counts more than its instructions. A step
+// finds the best two candidates before either is folded in: the second is the next pick exactly if the first leaves its own maximum
+// as it is, for all other values only fall (after t picks it does in all but one step of t, roughly); a step that finds it raised
+// takes the first alone. 174 cycles a pick with six candidates per lane where picks_cosine takes 193, 160 with four where it takes 190, one event per SM;
+// but about 1.1 times the instructions: with six of the small kernel's events per SM a call is 1 to 4 % slower for it, and in the
+// prefill kernel 4 to 7 %. (Moving the candidates that are left to fewer per lane, with a loop for each number: slower everywhere,
+// 22.3 -> 25.5 thousand cycles of an event alone on its SM, 358 -> 415 us for 896 events of 4096 rows: code that is not yet in the
+// instruction caches costs more than the candidates saved.)
+template <int CPL, bool BOUNDED>
+__device__ __forceinline__ bool picks_in_pairs(int lane, int P, int picks, const float* s, const unsigned short* bypool, float* r, float lam,
+                                               float* tri, uint32_t* park_key, int* park_row, uint32_t bound_key = 0u,
+                                               float* m_out = nullptr, int* t_out = nullptr, const float* m_in = nullptr,
+                                               const int* tie_slot = nullptr) {
+    constexpr int kSteps = 2;   // steps per look at the bound
+    const uint32_t tb = smem_u32(tri), rb = smem_u32(r);
+    const float ninf = __int_as_float(0xff800000), pinf = __int_as_float(0x7f800000);
+    float sv[CPL], lr[CPL], M[CPL];
+    int rc4[CPL], trow[CPL];   // 4 * row, and the shared-memory address of that row of the triangle
+    uint32_t tag[CPL];         // the row's offset in the triangle and the row: the lower tag is the lower row
+    const int last = max(P - 1, 0);
+#pragma unroll
+    for (int k = 0; k < CPL; ++k) {
+        const int rho = lane + 32 * k;
+        const bool in = rho < P;
+        const int rc = min(rho, last);  // clamped: the loads stay inside the triangle, the loop needs no branch
+        sv[k] = in ? fmaxf(s[bypool[rc]], kLowestScore) : ninf;
+        M[k] = m_in && in ? m_in[rc] : 0.f;
+        const float rk = fmaxf(r[rc], 1e-30f);   // positive, so that a maximum of +inf and a value of -inf come about
+        lr[k] = in ? fmaxf(penalty_rate(lam, rk), 1e-30f) : 1.f;   // (finite: no value below is ever NaN, so a winner's row is always found)
+        rc4[k] = 4 * rc;
+        trow[k] = (int)(tb + 4u * (uint32_t)tri_row(rc));
+        tag[k] = ((4u * (uint32_t)tri_row(rc)) << 8) | (uint32_t)rc;
+        if (in) {
+            tri[tri_row(rho) + rho] = pinf;
+            r[rho] = rk;
+        }
+    }
+    __syncwarp();
+    const float bound = BOUNDED && bound_key ? from_orderable(bound_key) : ninf;
+    // the winner: its value, its row and the row's offset (all lanes)
+    auto winner = [&](float& whi, uint32_t& w) {
+        float v[CPL];
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) v[k] = fmaf(-lr[k], M[k], sv[k]);
+        float lm = v[0];
+#pragma unroll
+        for (int k = 1; k < CPL; ++k) lm = fmaxf(lm, v[k]);
+        whi = warp_max_f32(lm);
+        uint32_t best = 0xFFFFFFFFu;
+#pragma unroll
+        for (int k = CPL - 1; k >= 0; --k) best = v[k] == whi ? tag[k] : best;
+        w = __reduce_min_sync(0xFFFFFFFFu, best);
+    };
+    // row i of the triangle at this lane's candidates, and its norm
+    auto load_row = [&](uint32_t w, float& ri, float (&x)[CPL]) {
+        const int i4 = (int)((w & 255u) << 2), irow = (int)(tb + (w >> 8));
+        ri = lds_in_order(rb + (uint32_t)i4);
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) x[k] = lds_in_order((uint32_t)__viaddmax_s32(trow[k], i4, irow + rc4[k]));
+    };
+    auto park = [&](int t, float val, uint32_t w) {
+        park_key[t] = __float_as_uint(val);   // (as a key once the loop is left)
+        park_row[t] = (int)(w & 255u);
+    };
+    // One pick, or two: the best two candidates are found before either is folded in. The second is the next pick exactly if
+    // the first leaves its own maximum as it is, for all other values only fall. Returns the lowest value taken.
+    auto step = [&](int& t) -> float {
+        float v[CPL], u[CPL], x[CPL], y[CPL];
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) v[k] = fmaf(-lr[k], M[k], sv[k]);
+        float lm = v[0];
+#pragma unroll
+        for (int k = 1; k < CPL; ++k) lm = fmaxf(lm, v[k]);
+        const float w1hi = warp_max_f32(lm);
+        // the lane's best two (while the reduction is under way)
+        uint32_t lt = tag[CPL - 1];
+#pragma unroll
+        for (int k = CPL - 2; k >= 0; --k) lt = v[k] == lm ? tag[k] : lt;
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) u[k] = tag[k] == lt ? ninf : v[k];
+        float lm2 = u[0];
+#pragma unroll
+        for (int k = 1; k < CPL; ++k) lm2 = fmaxf(lm2, u[k]);
+        uint32_t lt2 = tag[CPL - 1];
+#pragma unroll
+        for (int k = CPL - 2; k >= 0; --k) lt2 = u[k] == lm2 ? tag[k] : lt2;
+        const uint32_t w1 = __reduce_min_sync(0xFFFFFFFFu, lm == w1hi ? lt : 0xFFFFFFFFu);
+        const bool own = lt == w1;
+        const float lmB = own ? lm2 : lm;
+        const uint32_t ltB = own ? lt2 : lt;
+        const float w2hi = warp_max_f32(lmB);
+        float ri, rj;
+        load_row(w1, ri, x);
+        const uint32_t w2 = __reduce_min_sync(0xFFFFFFFFu, lmB == w2hi ? ltB : 0xFFFFFFFFu);
+        bool raised = false;   // the first raises the maximum of this lane's best other candidate
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) {
+            x[k] *= ri;
+            raised |= tag[k] == ltB && x[k] > M[k];
+        }
+        load_row(w2, rj, y);
+        const bool two = !__any_sync(0xFFFFFFFFu, ltB == w2 && raised);
+        rj = two ? rj : 0.f;
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) M[k] = fmaxf(fmaxf(M[k], x[k]), rj * y[k]);   // (0 * inf: NaN, which fmaxf drops)
+        if (lane == 0 && t < picks) park(t, w1hi, w1);
+        if (lane == 0 && two && t + 1 < picks) park(t + 1, w2hi, w2);
+        t += two ? 2 : 1;
+        return two ? w2hi : w1hi;
+    };
+    int t = 0;
+    bool at_bound = false;
+#pragma unroll 1
+    while (t < picks && !at_bound) {
+        float M0[CPL];
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) M0[k] = M[k];
+        const int t0 = t;
+        float low = 0.f;
+#pragma unroll
+        for (int u = 0; u < kSteps; ++u) low = step(t);   // (picks beyond the last one are not parked)
+        if (!(low > bound)) {
+            // one of them, or one beyond the last pick, was not above the bound (or nothing is left to pick)
+#pragma unroll
+            for (int k = 0; k < CPL; ++k) M[k] = M0[k];
+            t = t0;
+#pragma unroll 1
+            for (int u = 0; u < 2 * kSteps && t < picks; ++u, ++t) {
+                float whi;
+                uint32_t w;
+                winner(whi, w);
+                at_bound = !(whi > bound || (BOUNDED && tie_slot && whi == bound && whi > ninf && (int)bypool[w & 255u] < *tie_slot));
+                if (at_bound) break;
+                if (lane == 0) park(t, whi, w);
+                float ri, x[CPL];
+                load_row(w, ri, x);
+#pragma unroll
+                for (int k = 0; k < CPL; ++k) M[k] = fmaxf(M[k], ri * x[k]);
+            }
+        }
+    }
+    t = min(t, picks);
+    __syncwarp();
+    for (int i = lane; i < t; i += 32) {
+        const float val = __uint_as_float(park_key[i]);
+        park_key[i] = orderable(val <= -2.9e38f ? ninf : val);
+    }
+    if (at_bound) {
+        __syncwarp();
+        if (!BOUNDED || bound_key == 0u) {
+            // no bound: every value left is -inf (cosines overflowed)
+            if (lane == 0) {
+                for (; t < picks; ++t) {
+                    park_key[t] = orderable(ninf);
+                    park_row[t] = lowest_free_row(park_row, t);
+                }
+            }
+            return true;
+        }
+        if (m_out) {
+#pragma unroll
+            for (int k = 0; k < CPL; ++k)
+                if (lane + 32 * k < P) m_out[lane + 32 * k] = M[k];
+        }
+        if (t_out && lane == 0) *t_out = t;
+        return false;
+    }
+    return true;
+}
+
 // The picks that are missing after the loop over an active set reached its bound with `made` picks done. Those stand (no
 // left-out candidate could have won them). The rest, a few as a rule, are taken over the whole pool with rows of the cosine
 // matrix as plain dot products, from the state the loop left: its running maxima for the rows it had (m_act), and for the

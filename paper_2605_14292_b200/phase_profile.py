@@ -26,6 +26,8 @@ PHASES = {
                         "sort + outputs", "compaction"],
     "event_prefill_kernel": ["tables + positions", "K streamed and scored", "s_(b)", "active set / top-k", "V rows, products, triangle",
                              "picks", "sort + outputs", "compaction"],
+    "event_resident_kernel": ["K landed", "scores, V landed", "norms", "s_(b) + pool", "triangle", "picks (one warp)", "sort + outputs",
+                              "compaction"],
     "event_stream_kernel": ["tables + positions", "K streamed and scored", "s_(b)", "pool / top-k", "V rows + norms",
                             "picks", "sort + outputs", "compaction"],
 }
@@ -33,7 +35,7 @@ PHASES = {
 
 def main():
     ap = argparse.ArgumentParser()
-    ap.add_argument("--config", default="C3", choices=["C2", "C3", "C4", "C5"])
+    ap.add_argument("--config", default="C3", choices=["C1", "C2", "C3", "C4", "C5"])
     ap.add_argument("--batch", type=int, default=None)
     ap.add_argument("--lam", type=float, default=0.5)
     ap.add_argument("--flat", action="store_true", help="Eq. 1's flat signature with one cosine matrix per sequence (C2 shape)")
@@ -43,7 +45,9 @@ def main():
     lib.akv_debug_phase_buffer.argtypes = [C.c_void_p]
     slots = int(lib.akv_debug_phase_slots())
     dev = torch.device("cuda")
-    if args.config == "C2":
+    if args.config == "C1":
+        ev, kernel = synth.make_c1(), "event_resident_kernel"
+    elif args.config == "C2":
         ev, kernel = synth.make_c2(B=args.batch or 1), "event_pool_kernel"
     elif args.config == "C3":
         ev, kernel = synth.make_c3(B=args.batch or 16), "event_tri_kernel"

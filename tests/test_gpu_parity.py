@@ -338,6 +338,30 @@ def test_k_rows_beyond_the_tile_arrive_in_freed_slots(N, budget):
     check_all(ev, g, ev.lam, n_cand=n_cand)
 
 
+def in_pairs(ev, seed):
+    """Rows in pairs of one value row, their keys and positions equal in every second pair (equal scores): the best candidate
+    raises the maximum of the next one again and again. The first third at irregular positions, like kept rows."""
+    rng = np.random.default_rng(seed)
+    B, L, H, N, _ = ev.shape
+    gaps = rng.integers(1, 30, size=(B, L, H, N // 3)).cumsum(-1)
+    ev.pos[..., :N // 3] = gaps
+    ev.pos[..., N // 3:] += 30 * N
+    ev.p_ref[:] = 32 * N
+    odd = np.arange(1, N, 2)
+    ev.V[..., odd, :] = ev.V[..., odd - 1, :]
+    ev.K[..., odd[::2], :] = ev.K[..., odd[::2] - 1, :]
+    ev.pos[..., odd[::2]] = ev.pos[..., odd[::2] - 1]
+    return ev
+
+
+@pytest.mark.parametrize("N,budget", [(2, 2), (3, 2), (33, 33), (64, 40), (128, 128), (129, 90), (192, 64), (256, 100)])
+@pytest.mark.parametrize("lam", [0.5, 2.0])
+def test_resident_kernel_picks_in_pairs(N, budget, lam):
+    """Algorithm 1 two picks at a time: rows that come in pairs, down to the smallest sets and to all rows kept."""
+    ev = in_pairs(synth.make_plain(1, 2, 2, N, 64, budget, lam, dtype=synth.F32, seed=N), N)
+    check_all(ev, run_fused(ev), lam)
+
+
 @pytest.mark.parametrize("page,pages_per_seq", [(64, 4), (32, 6), (256, 1)])
 def test_paged_event_longer_than_the_tile(page, pages_per_seq):
     """Paged cache (page sizes are powers of two), budget 64: K pages are copied whole, a 256-slot page in two
