@@ -30,8 +30,14 @@ __device__ __forceinline__ void bulk_store_wait_read() {
 
 // FUSED: score + select + compact; otherwise selection only (scores are read from a.scores and
 // nothing is rewritten).
-template <bool FUSED>
-__global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_constant__ EventArgs a, const __grid_constant__ ScoreTab tab) {
+// WIDE: eight warps for an event that has an SM to itself (a call of no more events than SMs; also what event_tri_kernel takes, from
+// 129 rows on), else four warps and three events per SM. Alone on its SM an event is a chain of phases that too few warps hide: of 256
+// rows to 128, 55.2 -> 49.0 thousand cycles (scores 12.5 -> 10.4, picks in pairs 24.7 -> 22.5, triangle 3.2 -> 2.6, compaction 5.1 -> 4.4);
+// 112 of them 34.7 -> 31.2 us, in pages 39.1 -> 36.5, top-k 22.6 -> 18.5; of 192 rows to 64 (before: event_tri_kernel) 22.6 -> 22.0, of
+// 256 to 64 in pages 29.3 -> 26.8, but of 100 to 32 16.8 -> 17.1.
+template <bool FUSED, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) event_pool_kernel(const __grid_constant__ EventArgs a, const __grid_constant__ ScoreTab tab) {
+    constexpr int NT = WIDE ? kPoolWide : kTcThreads, NW = NT / 32;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const DevLayout& lay = a.lay;
@@ -128,7 +134,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
         const int* gpos = event_pos(a.pos, id);
         const bool rotate = gpos != nullptr;
         int pmax = INT_MIN;
-        for (int j = tid; j < n; j += kTcThreads) {
+        for (int j = tid; j < n; j += NT) {
             const int p = rotate ? gpos[j] : 0;
             spos[j] = p;
             pmax = max(pmax, p);
@@ -147,38 +153,44 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
         tc_fence_after();
         tbase = have_tmem ? *tmem_holder : 0u;
         long long pref = 0;
-        if (rotate) pref = a.p_ref ? (long long)a.p_ref[id.b] : (long long)max(max(redi[0], redi[1]), max(redi[2], redi[3])) + 1;
+        if (rotate) {
+            int top = redi[0];
+#pragma unroll
+            for (int w = 1; w < NW; ++w) top = max(top, redi[w]);
+            pref = a.p_ref ? (long long)a.p_ref[id.b] : (long long)top + 1;
+        }
         // lane covers frequencies f0..f0+7 of the row handled by its group of eight lanes
         const int grp = lane >> 3, f0 = (lane & 7) * 8;
-        // spacing of rows 16 slots apart at the newest end of the event: what a token-by-token cache has everywhere
-        const long long D16 = n > 16 ? (long long)spos[n - 1] - (long long)spos[n - 17] : 0;
+        // spacing of rows kRound (16 or 32) slots apart at the newest end of the event: what a token-by-token cache has everywhere
+        constexpr int kRound = 4 * NW;
+        const long long step = n > kRound ? (long long)spos[n - 1] - (long long)spos[n - 1 - kRound] : 0;
         ChainScore cs;
-        cs.set_step(D16, phitab + f0, sect);
-        // whether every row sits D16 after the row 16 slots before it (found once; the chains then need no look at
+        cs.set_step(step, phitab + f0, sect);
+        // whether every row sits step after the row kRound slots before it (found once; the chains then need no look at
         // the positions)
         bool uni = true;
-        for (int j = 16 + tid; j < n; j += kTcThreads) uni &= (long long)spos[j] - (long long)spos[j - 16] == D16;
+        for (int j = kRound + tid; j < n; j += NT) uni &= (long long)spos[j] - (long long)spos[j - kRound] == step;
         const bool uniform = __syncthreads_and(uni);
-        const int rounds = (n + 15) >> 4;
+        const int rounds = (n + kRound - 1) / kRound;
         timeout = !mbar_wait_bounded(barK, 0, a.wait_polls);
         phase_stamp(id.e, 10);  // (K rows have arrived)
         {
             // The tile holds the whole event. A lane group scores two rows side by side, row j of the first half
-            // of the rounds and row j + 16 * half of the second: two independent chains that share the turn S, so
+            // of the rounds and row j + kRound * half of the second: two independent chains that share the turn S, so
             // that one chain's dependent arithmetic fills the other's latency.
             const int half = (rounds + 1) >> 1;
             ChainScore cb;
             AKV_PHASE_ACC_DECL(cyc_anchor);
 #pragma unroll 1
             for (int round = 0; round < half; ++round) {
-                const int ja = 16 * round + 4 * warp + grp, jb = ja + 16 * half;
+                const int ja = kRound * round + 4 * warp + grp, jb = ja + kRound * half;
                 const bool la = ja < n, lb = jb < n;
                 // each chain on its own: after an event the kept rows' positions are irregular (fresh rotation every
                 // round) while the rows appended since are consecutive (chained)
                 bool fa = round == 0 || a.no_chain, fb = fa;
                 if (!fa && !uniform) {
-                    fa = !__all_sync(0xFFFFFFFFu, !la || (long long)spos[ja] - (long long)spos[ja - 16] == D16);
-                    fb = !__all_sync(0xFFFFFFFFu, !lb || (long long)spos[jb] - (long long)spos[jb - 16] == D16);
+                    fa = !__all_sync(0xFFFFFFFFu, !la || (long long)spos[ja] - (long long)spos[ja - kRound] == step);
+                    fb = !__all_sync(0xFFFFFFFFu, !lb || (long long)spos[jb] - (long long)spos[jb - kRound] == step);
                 }
                 AKV_PHASE_ACC_BEGIN(cyc_anchor);
                 if (fa) {
@@ -226,7 +238,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
             phase_stamp(id.e, 12);  // (scoring loop left)
         }
     } else {
-        for (int j = tid; j < n; j += kTcThreads) {
+        for (int j = tid; j < n; j += NT) {
             const float sc = a.scores[(long long)id.e * N + j];
             const bool fin = isfinite(sc);
             bad |= !fin;
@@ -235,7 +247,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
             key[j] = orderable(sj);
         }
     }
-    for (int j = n + tid; j < np4; j += kTcThreads) key[j] = 0u;  // below every real key
+    for (int j = n + tid; j < np4; j += NT) key[j] = 0u;  // below every real key
     timeout = __syncthreads_or(timeout);
     if (timeout) {
         if (tid == 0 && a.status) a.status[id.e] = 3;
@@ -249,7 +261,52 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
 
     phase_stamp(id.e, 2);
     // ---- s_(b) by bisection over the score keys, then the pool in slot order (warp 0) -------------
-    if (warp == 0) {
+    // (a pool that budgets of at most 64 have: 127 rows, so that the loop has four candidates per lane)
+    const int most = WIDE && a.budget <= 64 ? kTriMaxPool : kPoolActive;
+    if constexpr (WIDE) {
+        // A key per thread, counts by the barrier itself: a bit per round. (One warp with eight keys per lane: 3.7 thousand cycles
+        // of an event, these 3.3.)
+        const uint32_t kj = tid < np4 ? key[tid] : 0u;
+        uint32_t kb = 0u;
+        if (picks > 0)
+            for (int lo = 31; lo >= (similarity ? 14 : 0); --lo)
+                if (__syncthreads_count(kj >= (kb | (1u << lo))) >= picks) kb |= 1u << lo;
+        const float sb = from_orderable(kb);
+        const float thr = a.no_prune || kb < 0x00800000u ? -INFINITY : fmaf(-1.001f, a.lam, sb) - 1e-6f * fabsf(sb);
+        const bool pooled = kj != 0u && !(from_orderable(kj) < thr);
+        ActiveBound bound{0u, 0};
+        if (similarity && __syncthreads_count(pooled) > most)
+            bound = active_bound(orderable(thr), kb, most, most + 1, most - most / 8, [&](uint32_t v1, uint32_t v2, uint32_t v3, int& c1, int& c2, int& c3) {
+                c1 = __syncthreads_count(kj >= v1);
+                c2 = __syncthreads_count(kj >= v2);
+                c3 = __syncthreads_count(kj >= v3);
+            });
+        if (tid == 0) {
+            *tie_holder = 0;
+            *bound_holder = bound.key;
+            *thr_holder = thr;
+        }
+        if (bound.ties) {
+            __syncthreads();
+            if (warp == 0) {
+                const int base = list_with_ties(key, np4, bound.key, bound.ties, bypool, tie_holder);
+                if (lane == 0) *pool_holder = base;
+            }
+        } else {
+            // in slot order: a bit per slot, a row's place is the number of bits below
+            const bool in = similarity ? pooled && kj > bound.key : kj != 0u && kj >= kb;
+            const uint32_t mask = __ballot_sync(0xFFFFFFFFu, in);
+            if (lane == 0) kept[warp] = mask;
+            __syncthreads();
+            if (in) bypool[kept_below(kept, tid)] = (unsigned short)tid;
+            if (tid == 0) {
+                int base = 0;
+#pragma unroll
+                for (int w = 0; w < NW; ++w) base += __popc(kept[w]);
+                *pool_holder = base;
+            }
+        }
+    } else if (warp == 0) {
         uint32_t kk[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
@@ -313,6 +370,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
         }
     }
     __syncthreads();  // every key has been read: its storage becomes r below
+    if (WIDE && tid < 8) kept[tid] = 0u;   // (the pool's bits until now)
     const int P = *pool_holder;
 
     phase_stamp(id.e, 3);
@@ -327,7 +385,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
         int col[kPoolCpl];
 #pragma unroll
         for (int k = 0; k < kPoolCpl; ++k) col[k] = lane + 32 * k < P ? bypool[lane + 32 * k] : 0;
-        for (int ra = warp; ra < P; ra += kTcThreads / 32) {
+        for (int ra = warp; ra < P; ra += NT / 32) {
             const float* grow = G + (long long)bypool[ra] * N;
             const uint32_t dst = tile_u32 + 4u * (uint32_t)(tri_row(ra) + lane);
 #pragma unroll
@@ -335,18 +393,18 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
                 if (lane + 32 * k <= ra) cp_async4(dst + 128u * (uint32_t)k, grow + col[k]);
         }
         cp_async_wait_all();
-        for (int ra = tid; ra < P; ra += kTcThreads) r[ra] = 1.f;
+        for (int ra = tid; ra < P; ra += NT) r[ra] = 1.f;
     } else if (similarity) {
-        // thread -> 16-byte column c of rows r0, r0 + 8, ...: the swizzle term (c ^ row) & 7 is the same for
+        // thread -> 16-byte column c of rows r0, r0 + 8 or 16, ...: the swizzle term (c ^ row) & 7 is the same for
         // all of them, so a row costs one pool lookup, one address and one copy
         const int c = tid & 15, r0 = tid >> 4;
         const uint32_t dst0 = tile_u32 + tile_chunk(r0, c, half_bytes);
         if (dense) {
             const __nv_bfloat16* vcol = Vg + ev_off + c * 8;
-            for (int rho = r0; rho < P; rho += 8)
+            for (int rho = r0; rho < P; rho += NT / 16)
                 cp_async16(dst0 + (uint32_t)(rho - r0) * 128u, vcol + (long long)bypool[rho] * lay.sn);
         } else {
-            for (int rho = r0; rho < P; rho += 8)
+            for (int rho = r0; rho < P; rho += NT / 16)
                 cp_async16(dst0 + (uint32_t)(rho - r0) * 128u, Vg + rowoff(bypool[rho]) + c * 8);
         }
 
@@ -389,19 +447,20 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
     timeout = __syncthreads_or(timeout);  // also: the product has read the whole tile before the triangle lands on it
     if (timeout) {
         if (tid == 0 && a.status) a.status[id.e] = 3;
-        if (!FUSED) select_gave_up(a, id.e, kTcThreads);
+        if (!FUSED) select_gave_up(a, id.e, NT);
         if (have_tmem && warp == 0) tmem_dealloc(tbase, kPoolCols);
         return;
     }
     phase_stamp(id.e, 5);
     if (product) {
         // lower triangle -> shared memory; row rho = 32 warp + lane needs columns 0..rho
-        const int rho = 32 * warp + lane;
-        if (32 * warp < P) {
+        // (eight warps: the second four take the rows from 128 on)
+        const int quarter = warp & 3, rho = 32 * quarter + lane;
+        const uint32_t lanes = tbase + ((uint32_t)(32 * quarter) << 16);
+        if (warp < 4 && 32 * quarter < P) {
             const int trow = tri_row(rho);
-            const uint32_t lanes = tbase + ((uint32_t)(warp * 32) << 16);
             // column blocks left of the diagonal one: every column is below the row
-            for (int cb = 0; cb < warp; ++cb) {
+            for (int cb = 0; cb < quarter; ++cb) {
                 uint32_t v[32];
                 tmem_ld32(lanes + (uint32_t)(32 * cb), v);
                 tmem_ld_wait();
@@ -413,21 +472,20 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
             // the diagonal block: columns up to the row itself, whose last entry is the squared norm
             {
                 uint32_t v[32];
-                tmem_ld32(lanes + (uint32_t)(32 * warp), v);
+                tmem_ld32(lanes + (uint32_t)(32 * quarter), v);
                 tmem_ld_wait();
                 if (rho < P) {
 #pragma unroll
                     for (int k = 0; k < 32; ++k)
-                        if (k <= lane) tri[trow + 32 * warp + k] = __uint_as_float(v[k]);
+                        if (k <= lane) tri[trow + 32 * quarter + k] = __uint_as_float(v[k]);
                     r[rho] = 1.f / (sqrtf(tri[trow + rho]) + a.eps);  // read back: this thread stored it
                 }
             }
         }
-        if (nb > 0) {
+        if (nb > 0 && (!WIDE || warp >= 4)) {
             // rows from 128 on. Left of column 128: row a's entry in column b is row b's entry in column a (every
             // thread moves its own row's columns 128..). From column 128 on: the second product, whose lane L holds
             // row base2 + L against rows 128.. in the columns after the first product's.
-            const uint32_t lanes = tbase + ((uint32_t)(warp * 32) << 16);
             for (int cb = 0; cb < (nb + 31) >> 5; ++cb) {
                 uint32_t v[32];
                 tmem_ld32(lanes + 128u + (uint32_t)(32 * cb), v);
@@ -463,16 +521,23 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
     // after the loop.
     uint32_t* park_key = reinterpret_cast<uint32_t*>(gain);
     if (!similarity) {
-        picks_by_rank<kTcThreads>(tid, P, picks, key, bypool, park_key, order);
+        picks_by_rank<NT>(tid, P, picks, key, bypool, park_key, order);
     } else {
         if (warp == 0) {
-            const bool ok = picks_cosine<kPoolCpl, true>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order, *bound_holder,
-                                                         reinterpret_cast<float*>(tile + kContMact), redi, nullptr, tie_holder);
+            float* m_act = reinterpret_cast<float*>(tile + kContMact);
+            const uint32_t bound = *bound_holder;
+            bool ok;
+            if constexpr (!WIDE)
+                ok = picks_cosine<kPoolCpl, true>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order, bound, m_act, redi, nullptr, tie_holder);
+            else if (P <= 128)
+                ok = picks_in_pairs<4, true>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order, bound, m_act, redi, nullptr, tie_holder);
+            else
+                ok = picks_in_pairs<kPoolCpl, true>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order, bound, m_act, redi, nullptr, tie_holder);
             if (lane == 0) *pick_holder = ok ? picks : *redi;
         }
         __syncthreads();
         if (*pick_holder < picks) {
-            picks_over_whole_pool<true>(a, smem, n, P, picks, *pick_holder);
+            picks_over_whole_pool<true, NT>(a, smem, n, P, picks, *pick_holder);
         }
     }
     __syncthreads();
@@ -508,18 +573,18 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
     // resident CTA per SM.
     int* wpos = a.pos.p ? a.pos.p + id.b * a.pos.sb + id.l * a.pos.sl + id.h * a.pos.sh : nullptr;
     if (picks <= 64) {
-        // thread -> 16-byte column c of kept rows r0, r0 + 8, ...
+        // thread -> 16-byte column c of kept rows r0, r0 + 8 or 16, ...
         const int c = tid & 15, r0 = tid >> 4;
         const uint32_t slot0 = (uint32_t)(r0 * 256 + c * 16);
         const long long col = (dense ? ev_off : 0) + c * 8;
-        for (int t = r0; t < picks; t += 8) {
+        for (int t = r0; t < picks; t += NT / 16) {
             const long long off = col + (dense ? (long long)idx[t] * lay.sn : rowoff(idx[t]));
             cp_async16(tile_u32 + slot0 + (uint32_t)(t - r0) * 256u, Kg + off);
             cp_async16(tile_u32 + 16384u + slot0 + (uint32_t)(t - r0) * 256u, Vg + off);
         }
         cp_async_wait_all();
         __syncthreads();  // every load above has been performed
-        for (int t = r0; t < picks; t += 8) {
+        for (int t = r0; t < picks; t += NT / 16) {
             const long long off = col + (dense ? (long long)t * lay.sn : rowoff(t));
             const unsigned char* src = tile + slot0 + (t - r0) * 256;
             *reinterpret_cast<uint4*>(Kg + off) = *reinterpret_cast<const uint4*>(src);
@@ -531,7 +596,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
         // Stores: slots 0..picks-1 are contiguous in a dense cache (and page by page in a paged one), so one
         // thread writes them back with a few bulk copies. (Gathering by one bulk copy per row measured slower.)
         const uint32_t vhalf = kPoolTileBytes / 2u;
-        for (int x = tid; x < picks * 16; x += kTcThreads) {
+        for (int x = tid; x < picks * 16; x += NT) {
             const long long off = rowoff(idx[x >> 4]) + (x & 15) * 8;
             cp_async16(tile_u32 + (uint32_t)x * 16u, Kg + off);
             cp_async16(tile_u32 + vhalf + (uint32_t)x * 16u, Vg + off);
@@ -552,7 +617,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
                 bulk_store_wait_read();  // shared memory is read out before the CTA may leave
             }
         } else {
-            for (int x = tid; x < picks * 16; x += kTcThreads) {
+            for (int x = tid; x < picks * 16; x += NT) {
                 const long long off = rowoff(x >> 4) + (x & 15) * 8;
                 copy16(reinterpret_cast<char*>(Kg + off), tile + x * 16);
                 copy16(reinterpret_cast<char*>(Vg + off), tile + vhalf + x * 16);
@@ -560,7 +625,7 @@ __global__ void __launch_bounds__(kTcThreads, 3) event_pool_kernel(const __grid_
         }
     }
     if (wpos)
-        for (int t = tid; t < picks; t += kTcThreads) wpos[t] = spos[idx[t]];
+        for (int t = tid; t < picks; t += NT) wpos[t] = spos[idx[t]];
     phase_stamp(id.e, 9);
 }
 

@@ -31,6 +31,14 @@ constexpr int kTriTileRows = 128;           // K rows resident at a time = rows 
 constexpr unsigned kTriTileBytes = 32768u;  // 128 rows of 256 bytes; holds the triangle of up to 127 rows
 constexpr int kTriMaxPool = 127;            // largest pool whose cosine matrix goes through the tile
 
+// event_pool_kernel's (akv_event_pool.cuh): a tile of 64 KB, for a whole event's K rows, then the triangle of an active set of up to 180 rows (see the kernel);
+// three CTAs per SM.
+constexpr unsigned kPoolTileBytes = 65536u;
+constexpr int kPoolActive = 180;            // most rows whose cosine matrix goes through the tile
+constexpr uint32_t kPoolCols = 256u;        // tensor-memory columns (a power of two >= the matrix's columns)
+constexpr int kPoolWide = 256;              // threads of a CTA that has an SM to itself
+constexpr int kPoolCpl = 6;                 // candidates per lane of the one-warp loop
+
 struct TriSmem {
     unsigned tile, s, key, spos, bypool, taken, order, gain, idx, sect, misc, total;   // taken: a flag per slot, or (event_pool_kernel) a bit
 };
@@ -55,13 +63,6 @@ __host__ __device__ inline TriSmem plan_event_smem(int N, int budget, unsigned t
     return p;
 }
 __host__ __device__ inline TriSmem plan_tri_smem(int N, int budget) { return plan_event_smem(N, budget, kTriTileBytes); }
-
-// event_pool_kernel's (akv_event_pool.cuh): a tile of 64 KB, for a whole event's K rows, then the triangle of an active set of up to 180 rows (see the kernel);
-// three CTAs per SM.
-constexpr unsigned kPoolTileBytes = 65536u;
-constexpr int kPoolActive = 180;            // most rows whose cosine matrix goes through the tile
-constexpr uint32_t kPoolCols = 256u;        // tensor-memory columns (a power of two >= the matrix's columns)
-constexpr int kPoolCpl = 6;                 // candidates per lane of the one-warp loop
 
 __host__ __device__ inline TriSmem plan_pool_event_smem(int N, int budget) { return plan_event_smem(N, budget, kPoolTileBytes); }
 
@@ -552,7 +553,7 @@ constexpr unsigned kContMact = 8192u;      // m_act, 1 KB
 //
 // Out of line and with few arguments (the rest is found again from them), so that it costs the kernels that call it
 // neither registers nor a stretch of cold code between the phases (inlined: 2.5 % of event_tri_kernel).
-template <bool POOL>
+template <bool POOL, int NT>
 __device__ __noinline__ void picks_over_whole_pool(const EventArgs& a, unsigned char* smem, int n, int active, int picks, int made) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const DevLayout& lay = a.lay;
@@ -580,15 +581,15 @@ __device__ __noinline__ void picks_over_whole_pool(const EventArgs& a, unsigned 
     int* chosen = reinterpret_cast<int*>(left + 256);                          // slots of the picks made
     unsigned char* state = reinterpret_cast<unsigned char*>(chosen + 128);     // by slot: 1 in the old active set
     int* n_left = reinterpret_cast<int*>(state + 256);
-    for (int j = tid; j < 256; j += kTcThreads) state[j] = 0;
+    for (int j = tid; j < 256; j += NT) state[j] = 0;
     if (tid == 0) *n_left = 0;
     __syncthreads();
-    for (int rho = tid; rho < active; rho += kTcThreads) {
+    for (int rho = tid; rho < active; rho += NT) {
         const int j = bypool[rho];
         state[j] = 1;
         m_slot[j] = m_act[rho];
     }
-    for (int t = tid; t < made; t += kTcThreads) chosen[t] = bypool[order[t]];
+    for (int t = tid; t < made; t += NT) chosen[t] = bypool[order[t]];
     __syncthreads();
     if (warp == 0) {
         int base = 0;
@@ -604,7 +605,7 @@ __device__ __noinline__ void picks_over_whole_pool(const EventArgs& a, unsigned 
     }
     __syncthreads();
     const int P = holders[0];
-    for (int rho = tid; rho < P; rho += kTcThreads) {
+    for (int rho = tid; rho < P; rho += NT) {
         const int j = bypool[rho];
         inv[j] = (unsigned short)rho;
         if (state[j]) {
@@ -626,7 +627,7 @@ __device__ __noinline__ void picks_over_whole_pool(const EventArgs& a, unsigned 
         r[rho] = 1.f / (sqrtf(ss) + a.eps);
     }
     __syncthreads();
-    for (int t = tid; t < made; t += kTcThreads) order[t] = inv[chosen[t]];
+    for (int t = tid; t < made; t += NT) order[t] = inv[chosen[t]];
     __syncthreads();
     auto dot = [&](int i, const __nv_bfloat16* vi, int c) -> float {   // of two pool rows (vi: row i's values)
         if (G) return G[(long long)bypool[i] * lay.N + bypool[c]];
@@ -645,7 +646,7 @@ __device__ __noinline__ void picks_over_whole_pool(const EventArgs& a, unsigned 
     // left-out rows against the picks made: m = max(0, max_t r_t <V_c, V_t>), every (row, pick) pair its own dot
     // product, the maximum by an integer atomic (the values are non-negative floats)
     const int pairs = *n_left * made;
-    for (int x = tid; x < pairs; x += kTcThreads) {
+    for (int x = tid; x < pairs; x += NT) {
         const int c = left[x / made], i = order[x % made];
         const float v = fmaxf(r[i] * dot(i, vrow_of(bypool[i]), c), 0.f);
         atomicMax(reinterpret_cast<int*>(m_init) + c, __float_as_int(v));
@@ -678,7 +679,7 @@ __device__ __noinline__ void picks_over_whole_pool(const EventArgs& a, unsigned 
         const int irho = holders[1];
         // row irho of the cosine matrix
         const __nv_bfloat16* vpick = vrow_of(bypool[irho]);
-        for (int rho = tid; rho < P; rho += kTcThreads) rowbuf[rho] = dot(irho, vpick, rho);
+        for (int rho = tid; rho < P; rho += NT) rowbuf[rho] = dot(irho, vpick, rho);
         __syncthreads();
         if (warp == 0) {
             const float ri = r[irho];
@@ -1040,7 +1041,7 @@ __global__ void __launch_bounds__(kTcThreads) event_tri_kernel(const __grid_cons
         }
         __syncthreads();
         if (*pick_holder < picks) {
-            picks_over_whole_pool<false>(a, smem, n, P, picks, *pick_holder);
+            picks_over_whole_pool<false, kTcThreads>(a, smem, n, P, picks, *pick_holder);
         }
     }
     __syncthreads();

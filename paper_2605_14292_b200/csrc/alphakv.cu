@@ -349,15 +349,18 @@ static bool pool_shared_ok(const EventArgs& a) {
 template <bool FUSED, bool BIG>
 static akv_status_t launch_tri(akv_handle* h, const EventArgs& a, cudaStream_t st, bool dry = false) {
     const int E = a.lay.B * a.lay.L * a.lay.H;
+    if constexpr (!BIG)   // an SM for every event: the large kernel's eight warps (see there; events of up to 128 rows gain nothing)
+        if (E <= h->sm_count && a.lay.N > 128) return launch_tri<FUSED, true>(h, a, st, dry);
     const TriSmem sp = BIG ? plan_pool_event_smem(a.lay.N, a.budget) : plan_tri_smem(a.lay.N, a.budget);
     if ((int)sp.total > h->smem_optin) return fail(AKV_ERR_UNSUPPORTED, "budget %d needs too much shared memory", a.budget);
     akv_status_t s;
     if (BIG) {
-        if ((s = set_smem(h, event_pool_kernel<FUSED>, sp.total)) != AKV_OK) return s;
-        CUDA_TRY(cudaFuncSetAttribute(event_pool_kernel<FUSED>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                      (int)cudaSharedmemCarveoutMaxShared));
+        const bool wide = E <= h->sm_count;   // an SM for every event
+        auto kernel = wide ? event_pool_kernel<FUSED, true> : event_pool_kernel<FUSED, false>;
+        if ((s = set_smem(h, kernel, sp.total)) != AKV_OK) return s;
+        CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
         if (dry) return AKV_OK;
-        event_pool_kernel<FUSED><<<E, kTcThreads, sp.total, st>>>(a, h->tab);
+        kernel<<<E, wide ? kPoolWide : kTcThreads, sp.total, st>>>(a, h->tab);
         return launched(FUSED ? "event_pool" : "select_pool_active");
     }
     if ((s = set_smem(h, event_tri_kernel<FUSED>, sp.total)) != AKV_OK) return s;

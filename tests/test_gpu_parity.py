@@ -354,6 +354,26 @@ def in_pairs(ev, seed):
     return ev
 
 
+@pytest.mark.parametrize("N,budget,lam", [(129, 20, 0.5), (144, 64, 1.0), (160, 128, 0.5), (192, 64, 0.0), (250, 33, 1.0), (255, 65, 0.0),
+                                          (256, 64, 0.5), (256, 128, 0.5), (256, 128, 2.0)])
+def test_events_with_an_sm_each_and_several_to_an_sm(N, budget, lam):
+    """bf16, d = 128: calls of no more events than SMs take the kernel of eight warps, others those of four; both against the
+    oracle, with all candidates, ragged counts and when their waits run out."""
+    few = in_pairs(synth.make_plain(2, 1, 3, N, 128, budget, lam, dtype=synth.BF16, seed=N + budget), N)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    times = sms // 6 + 1
+    many = synth.make_plain(2 * times, 1, 3, 1, 128, 1, lam, dtype=synth.BF16, seed=0)
+    many.qstat, many.budget = few.qstat, budget
+    for name in ("K", "V", "pos", "p_ref"):
+        setattr(many, name, np.tile(getattr(few, name), (times,) + (1,) * (getattr(few, name).ndim - 1)))
+    for ev, events in ((few, range(6)), (many, (0, 4, 6 * times - 1))):
+        check_all(ev, run_fused(ev), lam, events=events)
+        n_cand = [N - 1, N // 2 + 1] * (len(ev.p_ref) // 2)
+        check_all(ev, run_fused(ev, n_cand=n_cand), lam, events=events, n_cand=n_cand)
+        g = run_fused(ev, flags=akv.FLAG_TEST_STARVE_WAIT)
+        assert np.all(g["status"] == 3) and np.array_equal(g["K"], ev.K) and np.array_equal(g["V"], ev.V) and np.array_equal(g["pos"], ev.pos)
+
+
 @pytest.mark.parametrize("N,budget", [(2, 2), (3, 2), (33, 33), (64, 40), (128, 128), (129, 90), (192, 64), (256, 100)])
 @pytest.mark.parametrize("lam", [0.5, 2.0])
 def test_resident_kernel_picks_in_pairs(N, budget, lam):
