@@ -527,8 +527,9 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
             float* m_act = reinterpret_cast<float*>(tile + kContMact);
             const uint32_t bound = *bound_holder;
             bool ok;
+            // (eight picks per look at the bound instead of four: 16 384 events of 256 rows to 128 1645 -> 1626 us, 448 of them 76.8 -> 74.7)
             if constexpr (!WIDE)
-                ok = picks_cosine<kPoolCpl, true>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order, bound, m_act, redi, nullptr, tie_holder);
+                ok = picks_cosine<kPoolCpl, true, 8>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order, bound, m_act, redi, nullptr, tie_holder);
             else if (P <= 128)
                 ok = picks_in_pairs<4, true>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order, bound, m_act, redi, nullptr, tie_holder);
             else

@@ -240,8 +240,8 @@ __device__ __forceinline__ int lowest_free_row(const int* picked, int t) {
 // of two reductions and one load. Per candidate and pick: an fma, a max, a compare and a select to find the winner's row,
 // two integer instructions for the address (an entry's index is max(tri_row(c) + i, tri_row(i) + c) whichever of c and i
 // is the higher), a load, a product with the picked row's norm and a max. The row and its offset travel as one word. A
-// branch on the winner costs 50 cycles, so the bound is looked at once per four picks (winners only fall), and where it
-// was reached those four are taken again one by one. (Norms applied to the whole triangle beforehand instead: 5 cycles
+// branch on the winner costs 50 cycles, so the bound is looked at once per four picks or eight (winners only fall), and
+// where it was reached those are taken again one by one. (Norms applied to the whole triangle beforehand instead: 5 cycles
 // less a pick, but 2 to 6 thousand more for the triangle.)
 //
 // BOUNDED: the P rows are only the best-scored part of the pool, and every candidate left out scores at most
@@ -250,12 +250,12 @@ __device__ __forceinline__ int lowest_free_row(const int* picked, int t) {
 // left out that may equal it; at the first pick that does not, it stops and returns false. The picks made so
 // far stand; with m_out / t_out given the running maxima (by pool row; +inf for the rows already picked) and the number
 // of picks are left for the caller to continue from. m_in: maxima to start from (null: 0). `tri` (its diagonal) and `r` are modified. At most 256 rows.
-template <int CPL, bool BOUNDED>
+// kGroup: picks per look at the bound (divides 32).
+template <int CPL, bool BOUNDED, int kGroup = 4>
 __device__ __forceinline__ bool picks_cosine(int lane, int P, int picks, const float* s, const unsigned short* bypool, float* r, float lam,
                                              float* tri, uint32_t* park_key, int* park_row, uint32_t bound_key = 0u,
                                              float* m_out = nullptr, int* t_out = nullptr, const float* m_in = nullptr,
                                              const int* tie_slot = nullptr) {
-    constexpr int kGroup = 4;   // picks per look at the bound (divides 32)
     const uint32_t tb = smem_u32(tri), rb = smem_u32(r);
     const float ninf = __int_as_float(0xff800000), pinf = __int_as_float(0x7f800000);
     float sv[CPL], lr[CPL], M[CPL];
@@ -327,7 +327,7 @@ __device__ __forceinline__ bool picks_cosine(int lane, int P, int picks, const f
                 fold(w);
             }
             if (!(whi > bound)) {
-                // one of the four, or one beyond the last pick, was not above the bound (or nothing is left to pick)
+                // one of the group, or one beyond the last pick, was not above the bound (or nothing is left to pick)
 #pragma unroll
                 for (int k = 0; k < CPL; ++k) M[k] = M0[k];
 #pragma unroll 1
