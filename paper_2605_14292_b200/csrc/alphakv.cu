@@ -376,8 +376,9 @@ static bool prefill_path_ok(const EventArgs& a) {
     return a.lay.dtype == AKV_BF16 && a.lay.d == kTcD && a.lay.N > kTcMaxN && a.lay.N <= kPfMaxN && a.flat_sig == nullptr &&
            !a.gqa_max && a.budget <= kPfMaxBudget;
 }
+// (events of the call from a.first_event on)
 template <bool FUSED, int SPLIT>
-static akv_status_t launch_prefill_split(akv_handle* h, const EventArgs& a, cudaStream_t st, bool dry) {
+static akv_status_t launch_prefill_split(akv_handle* h, const EventArgs& a, long long events, cudaStream_t st, bool dry) {
     const PfSmem sp = plan_pf_smem(a.lay.N, a.budget);
     akv_status_t s;
     auto kernel = event_prefill_kernel<FUSED, SPLIT>;
@@ -386,28 +387,49 @@ static akv_status_t launch_prefill_split(akv_handle* h, const EventArgs& a, cuda
     if (dry) return AKV_OK;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)(a.lay.B * a.lay.L * a.lay.H) * SPLIT);
+    cfg.gridDim = dim3((unsigned)events * SPLIT);
     cfg.blockDim = dim3(kStThreads);
     cfg.dynamicSmemBytes = sp.total;
     cfg.stream = st;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = SPLIT;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = SPLIT > 1 ? 1 : 0;
+    cudaLaunchAttribute attr[2];
+    cfg.attrs = attr;
+    if (SPLIT > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = SPLIT;
+        attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
+        ++cfg.numAttrs;
+    }
+    if (a.behind) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+        ++cfg.numAttrs;
+    }
     CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, a, h->tab));
     return launched(FUSED ? "event_prefill" : "select_prefill");
 }
 template <bool FUSED>
-static akv_status_t launch_prefill(akv_handle* h, const EventArgs& a, cudaStream_t st, bool dry = false) {
+static akv_status_t launch_prefill(akv_handle* h, const EventArgs& a0, cudaStream_t st, bool dry = false) {
+    EventArgs a = a0;
+    const long long E = (long long)a.lay.B * a.lay.L * a.lay.H;
     if constexpr (FUSED) {
-        const long long E = (long long)a.lay.B * a.lay.L * a.lay.H;
+        // The events of a nearly empty last wave, sharing their scoring, as a launch of their own behind the full waves
+        const long long tail = prefill_tail(E, a.lay.N, h->sm_count, !a.greedy, a.n_cand != nullptr);
+        if (tail) {
+            EventArgs b = a0;
+            b.behind = 1;
+            b.first_event = (int)(E - tail);
+            a.followed = 1;
+            const bool four = prefill_split(tail, a.lay.N, h->sm_count, !a.greedy, a.n_cand != nullptr) == 4;
+            auto second = [&](bool check) { return four ? launch_prefill_split<true, 4>(h, b, tail, st, check) : launch_prefill_split<true, 2>(h, b, tail, st, check); };
+            akv_status_t s = second(true);   // (what can be refused is, before the first launch)
+            if (s == AKV_OK) s = launch_prefill_split<true, 1>(h, a, E - tail, st, dry);
+            return s != AKV_OK || dry ? s : second(false);
+        }
         const int split = prefill_split(E, a.lay.N, h->sm_count, !a.greedy, a.n_cand != nullptr);
-        if (split == 4) return launch_prefill_split<true, 4>(h, a, st, dry);
-        if (split == 2) return launch_prefill_split<true, 2>(h, a, st, dry);
+        if (split == 4) return launch_prefill_split<true, 4>(h, a, E, st, dry);
+        if (split == 2) return launch_prefill_split<true, 2>(h, a, E, st, dry);
     }
-    return launch_prefill_split<FUSED, 1>(h, a, st, dry);
+    return launch_prefill_split<FUSED, 1>(h, a, E, st, dry);
 }
 
 static akv_status_t launch_select(akv_handle* h, const EventArgs& a, cudaStream_t st, bool dry = false) {

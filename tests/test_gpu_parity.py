@@ -687,6 +687,42 @@ def test_first_cta_learns_that_another_gave_up(L, H, N):
     check_all(ev, good, 0.5, events=[0, L * H - 1])
 
 
+@pytest.mark.parametrize("rest,N,budget", [(1, 3009, 17), (40, 3072, 128), (70, 3100, 64)])
+def test_last_events_of_a_topk_call_in_a_launch_of_their_own(rest, N, budget):
+    """Top-k over many long events: the few beyond the full waves share their scoring and come in a second launch, which ends after
+    the first; every event as in a small call, to the bit, also when captured and replayed."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    E, base = 2 * sms + rest, 7
+    assert akv_split.prefill_tail(E, N, sms, topk=True) == rest and akv_split.prefill_tail(E, N, sms, topk=False) == 0
+    ev = synth.make_plain(1, 1, base, N, 128, budget, 0.0, dtype=synth.BF16, seed=N)
+    small = run_fused(ev)
+    check_all(ev, small, 0.0, events=[0, base - 1])
+    which = torch.arange(E, device="cuda") % base
+    K0, V0, pos0, q = (dev(x).index_select(dim, which) for x, dim in ((ev.K, 2), (ev.V, 2), (ev.pos, 2), (ev.qstat, 1)))
+    K, V, pos = K0.clone(), V0.clone(), pos0.clone()
+    opts, pref = akv.Options(lam=0.0), dev(ev.p_ref)
+    before = akv.launch_count()
+    sel = akv.alpha_compress_event(K, V, pos, q, budget, opts, p_ref=pref)
+    idx = sel.idx_sorted.clone()          # (the next thing on the stream)
+    assert akv.launch_count() == before + 2
+
+    def same():
+        for got, want in ((K.view(torch.int16), small["K"].view(np.int16)), (V.view(torch.int16), small["V"].view(np.int16)), (pos, small["pos"]),
+                          (sel.pick_order, small["order"]), (sel.pick_gain, small["gain"]), (idx, small["idx"]), (sel.status, small["status"])):
+            assert torch.equal(got, torch.from_numpy(want).cuda().index_select(2, which))
+
+    same()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        K.copy_(K0); V.copy_(V0); pos.copy_(pos0)
+        akv.alpha_compress_event(K, V, pos, q, budget, opts, p_ref=pref, out=sel)
+        idx.copy_(sel.idx_sorted)
+    for _ in range(2):
+        sel.pick_order.zero_(); idx.zero_()
+        graph.replay()
+        same()
+
+
 @pytest.mark.parametrize("L,H,N,lam", [(2, 2, 1100, 0.0), (2, 2, 1100, 0.5), (2, 19, 2048, 0.0), (2, 19, 2113, 0.5), (5, 15, 3072, 0.0), (5, 15, 2048, 0.5)])
 def test_shared_scoring_of_all_kinds_of_call(L, H, N, lam):
     """Four or two CTAs per event, with and without the penalty: budgets per head, a non-finite key in every CTA's part and pages in

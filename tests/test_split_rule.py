@@ -2,7 +2,7 @@
 calls that were measured slower for it."""
 import pytest
 
-from akv_split import prefill_split, split_share
+from akv_split import prefill_split, prefill_tail, split_share
 
 
 @pytest.mark.parametrize("sms", [148, 132, 80])
@@ -31,3 +31,14 @@ def test_a_split_shortens_every_share(sms, topk, ragged):
     (28, 4096, False, False, 4), (28, 1100, True, False, 4), (37, 1100, False, False, 4), (56, 4096, False, True, 4), (74, 2049, True, False, 2)])
 def test_calls_that_were_measured(events, N, topk, ragged, split):
     assert prefill_split(events, N, 148, topk, ragged) == split
+
+
+# (events, rows, top-k, ragged, how many of them are left to a second launch): 148 multiprocessors, 296 places
+@pytest.mark.parametrize("events,N,topk,ragged,tail", [
+    (896, 4096, True, False, 8), (896, 4096, False, False, 0), (304, 3072, True, False, 8), (304, 2113, True, False, 0), (370, 5000, True, False, 74),
+    (371, 4096, True, False, 0), (296 + 112, 3136, True, False, 0), (592, 4096, True, False, 0), (296, 4096, True, False, 0), (8, 4096, True, False, 0),
+    (304, 4096, True, True, 0), (296 + 148, 4096, True, False, 0), (296 + 200, 4096, True, False, 0)])
+def test_events_left_to_a_second_launch(events, N, topk, ragged, tail):
+    assert prefill_tail(events, N, 148, topk, ragged) == tail
+    if tail:
+        assert prefill_split(tail, N, 148, topk, ragged) > 1
