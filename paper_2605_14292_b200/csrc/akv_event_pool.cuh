@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
     const int N = lay.N;
     const int bud = event_budget(a, id);
     const int picks = min(bud, n);
-    const TriSmem sp = plan_pool_event_smem(N, a.budget);
+    const TriSmem sp = plan_pool_event_smem(N, a.budget, lay.page_size != 0);
     unsigned char* tile = smem + sp.tile;
     float* tri = reinterpret_cast<float*>(tile);  // lower triangle of the cosine matrix, after the product
     float* s = reinterpret_cast<float*>(smem + sp.s);
@@ -77,8 +77,16 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
     // row addressing: dense events are one base offset plus a row stride
     const bool dense = lay.page_size == 0;
     const long long ev_off = dense ? id.b * lay.sb + id.l * lay.sl + id.h * lay.sh : 0;
+    // paged: where the event's pages start, looked up once by as many lanes of every warp at the same time (the block table's
+    // entries come from L2; looked up row by row and copy by copy: 16 384 events of 256 rows to 128 in pages of 64 1631 us, 1600 so,
+    // 8192 in pages of 16 798 and 771)
+    long long* page_off = reinterpret_cast<long long*>(smem + sp.pages);
+    const bool few_pages = !dense && ((N - 1) >> lay.page_shift) < kPageOffsets;
+    if (few_pages && tid < kPageOffsets && (tid << lay.page_shift) < N) page_off[tid] = row_offset(lay, id.b, id.l, id.h, tid << lay.page_shift);
+    __syncwarp();
     auto rowoff = [&](int j) -> long long {
-        return dense ? ev_off + (long long)j * lay.sn : row_offset(lay, id.b, id.l, id.h, j);
+        if (dense) return ev_off + (long long)j * lay.sn;
+        return few_pages ? page_off[j >> lay.page_shift] + (long long)(j & (lay.page_size - 1)) * lay.s_page_n : row_offset(lay, id.b, id.l, id.h, j);
     };
     __nv_bfloat16* Kg = reinterpret_cast<__nv_bfloat16*>(a.K);
     __nv_bfloat16* Vg = reinterpret_cast<__nv_bfloat16*>(a.V);
@@ -597,10 +605,16 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
         // Stores: slots 0..picks-1 are contiguous in a dense cache (and page by page in a paged one), so one
         // thread writes them back with a few bulk copies. (Gathering by one bulk copy per row measured slower.)
         const uint32_t vhalf = kPoolTileBytes / 2u;
-        for (int x = tid; x < picks * 16; x += NT) {
+        auto gather = [&](int x) {
             const long long off = rowoff(idx[x >> 4]) + (x & 15) * 8;
             cp_async16(tile_u32 + (uint32_t)x * 16u, Kg + off);
             cp_async16(tile_u32 + vhalf + (uint32_t)x * 16u, Vg + off);
+        };
+        if constexpr (WIDE) {
+            for (int x = tid; x < picks * 16; x += NT) gather(x);
+        } else {
+#pragma unroll 4
+            for (int x = tid; x < picks * 16; x += NT) gather(x);   // (several rows' look-ups at once; with one event per SM no gain)
         }
         cp_async_wait_all();
         fence_proxy_async();  // the bulk stores below read what these copies wrote

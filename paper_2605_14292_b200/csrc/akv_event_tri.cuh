@@ -40,10 +40,11 @@ constexpr int kPoolWide = 256;              // threads of a CTA that has an SM t
 constexpr int kPoolCpl = 6;                 // candidates per lane of the one-warp loop
 
 struct TriSmem {
-    unsigned tile, s, key, spos, bypool, taken, order, gain, idx, sect, misc, total;   // taken: a flag per slot, or (event_pool_kernel) a bit
+    unsigned tile, s, key, spos, bypool, taken, order, gain, idx, sect, misc, pages, total;   // taken: a flag per slot, or (event_pool_kernel) a bit
 };
 // Layout after the 1024-byte aligned base. `key` (score keys) and `r` (reciprocal norms) share storage.
-__host__ __device__ inline TriSmem plan_event_smem(int N, int budget, unsigned tile_bytes) {
+constexpr int kPageOffsets = 16;   // pages of an event whose offsets are kept on chip
+__host__ __device__ inline TriSmem plan_event_smem(int N, int budget, unsigned tile_bytes, bool paged) {
     TriSmem p;
     const unsigned np = (unsigned)((N + 3) & ~3);
     unsigned o = 0;
@@ -59,12 +60,13 @@ __host__ __device__ inline TriSmem plan_event_smem(int N, int budget, unsigned t
     if (o - p.bypool < 1024u) o = p.bypool + 1024u;  // bypool..idx also hold the folded statistic and the phase steps (1 KB) while scoring
     p.sect = o;   o += 256;       // cosine and sine of the 32 sector angles
     p.misc = o;   o += 64;        // mbarriers (K, product, late K rows), tmem base, pool size, bound, threshold, block-max scratch
+    p.pages = o;  o += paged ? 8 * kPageOffsets : 0;
     p.total = o + 1024;           // room to align the base to 1024 bytes
     return p;
 }
-__host__ __device__ inline TriSmem plan_tri_smem(int N, int budget) { return plan_event_smem(N, budget, kTriTileBytes); }
+__host__ __device__ inline TriSmem plan_tri_smem(int N, int budget, bool paged) { return plan_event_smem(N, budget, kTriTileBytes, paged); }
 
-__host__ __device__ inline TriSmem plan_pool_event_smem(int N, int budget) { return plan_event_smem(N, budget, kPoolTileBytes); }
+__host__ __device__ inline TriSmem plan_pool_event_smem(int N, int budget, bool paged) { return plan_event_smem(N, budget, kPoolTileBytes, paged); }
 
 // 32 consecutive columns of this thread's TMEM lane.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
@@ -558,7 +560,7 @@ __device__ __noinline__ void picks_over_whole_pool(const EventArgs& a, unsigned 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const DevLayout& lay = a.lay;
     const EventId id = decode_event(lay, blockIdx.x);
-    const TriSmem sp = POOL ? plan_pool_event_smem(lay.N, a.budget) : plan_tri_smem(lay.N, a.budget);
+    const TriSmem sp = POOL ? plan_pool_event_smem(lay.N, a.budget, lay.page_size != 0) : plan_tri_smem(lay.N, a.budget, lay.page_size != 0);
     const float* G = POOL && a.gram ? a.gram + id.b * a.gram_sb + id.l * a.gram_sl : nullptr;
     const float* s = reinterpret_cast<const float*>(smem + sp.s);
     unsigned short* bypool = reinterpret_cast<unsigned short*>(smem + sp.bypool);
@@ -704,7 +706,7 @@ __global__ void __launch_bounds__(kTcThreads) event_tri_kernel(const __grid_cons
     const int N = lay.N;
     const int bud = event_budget(a, id);
     const int picks = min(bud, n);
-    const TriSmem sp = plan_tri_smem(N, a.budget);
+    const TriSmem sp = plan_tri_smem(N, a.budget, lay.page_size != 0);
     unsigned char* tile = smem + sp.tile;
     float* tri = reinterpret_cast<float*>(tile);  // lower triangle of the cosine matrix, after the product
     float* s = reinterpret_cast<float*>(smem + sp.s);
@@ -736,8 +738,15 @@ __global__ void __launch_bounds__(kTcThreads) event_tri_kernel(const __grid_cons
     // row addressing: dense events are one base offset plus a row stride
     const bool dense = lay.page_size == 0;
     const long long ev_off = dense ? id.b * lay.sb + id.l * lay.sl + id.h * lay.sh : 0;
+    // paged: where the event's pages start, looked up once by as many lanes of every warp at the same time (the block table's
+    // entries come from L2; looked up row by row and copy by copy: 4096 events of 192 rows to 64 in pages of 64 191 us, 183 so)
+    long long* page_off = reinterpret_cast<long long*>(smem + sp.pages);
+    const bool few_pages = !dense && ((N - 1) >> lay.page_shift) < kPageOffsets;
+    if (few_pages && tid < kPageOffsets && (tid << lay.page_shift) < N) page_off[tid] = row_offset(lay, id.b, id.l, id.h, tid << lay.page_shift);
+    __syncwarp();
     auto rowoff = [&](int j) -> long long {
-        return dense ? ev_off + (long long)j * lay.sn : row_offset(lay, id.b, id.l, id.h, j);
+        if (dense) return ev_off + (long long)j * lay.sn;
+        return few_pages ? page_off[j >> lay.page_shift] + (long long)(j & (lay.page_size - 1)) * lay.s_page_n : row_offset(lay, id.b, id.l, id.h, j);
     };
     __nv_bfloat16* Kg = reinterpret_cast<__nv_bfloat16*>(a.K);
     __nv_bfloat16* Vg = reinterpret_cast<__nv_bfloat16*>(a.V);

@@ -351,7 +351,7 @@ static akv_status_t launch_tri(akv_handle* h, const EventArgs& a, cudaStream_t s
     const int E = a.lay.B * a.lay.L * a.lay.H;
     if constexpr (!BIG)   // an SM for every event: the large kernel's eight warps (see there; events of up to 128 rows gain nothing)
         if (E <= h->sm_count && a.lay.N > 128) return launch_tri<FUSED, true>(h, a, st, dry);
-    const TriSmem sp = BIG ? plan_pool_event_smem(a.lay.N, a.budget) : plan_tri_smem(a.lay.N, a.budget);
+    const TriSmem sp = BIG ? plan_pool_event_smem(a.lay.N, a.budget, a.lay.page_size != 0) : plan_tri_smem(a.lay.N, a.budget, a.lay.page_size != 0);
     if ((int)sp.total > h->smem_optin) return fail(AKV_ERR_UNSUPPORTED, "budget %d needs too much shared memory", a.budget);
     akv_status_t s;
     if (BIG) {

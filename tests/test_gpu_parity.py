@@ -374,6 +374,31 @@ def test_events_with_an_sm_each_and_several_to_an_sm(N, budget, lam):
         assert np.all(g["status"] == 3) and np.array_equal(g["K"], ev.K) and np.array_equal(g["V"], ev.V) and np.array_equal(g["pos"], ev.pos)
 
 
+@pytest.mark.parametrize("page,N,budget", [(16, 256, 128), (16, 250, 64), (16, 241, 100), (8, 128, 40), (8, 130, 64), (8, 256, 128), (256, 131, 70)])
+def test_pages_on_both_sides_of_those_whose_offsets_are_kept(page, N, budget):
+    """Up to sixteen pages of an event have their offsets on chip: one less, as many and one more, in no order, for events with an
+    SM each and several to an SM; against the same rows in a dense cache, to the bit."""
+    for B in (1, 40):
+        ev = synth.make_plain(B, 2, 2, N, 128, budget, 0.5, dtype=synth.BF16, seed=N + page)
+        plain = run_fused(ev)
+        pps = -(-N // page)
+        table = torch.randperm(B * pps, device="cuda").to(torch.int32).view(B, pps)
+        pools = []
+        for x in (dev(ev.K), dev(ev.V)):
+            rows = torch.zeros((B, 2, 2, pps * page, 128), dtype=torch.bfloat16, device="cuda")
+            rows[..., :N, :] = x
+            pool = torch.zeros((2, B * pps, 2, page, 128), dtype=torch.bfloat16, device="cuda")
+            pool[:, table.long().flatten()] = rows.view(B, 2, 2, pps, page, 128).permute(1, 0, 3, 2, 4, 5).reshape(2, B * pps, 2, page, 128)
+            pools.append(pool)
+        pos, lay = dev(ev.pos), akv.Layout.paged(pools[0], table, N)
+        sel = akv.alpha_compress_event(pools[0], pools[1], pos, dev(ev.qstat), budget, akv.Options(lam=0.5), p_ref=dev(ev.p_ref), layout=lay)
+        assert np.array_equal(sel.pick_order.cpu().numpy(), plain["order"]) and np.array_equal(sel.pick_gain.cpu().numpy(), plain["gain"])
+        assert np.array_equal(pos.cpu().numpy(), plain["pos"])
+        for pool, name in zip(pools, "KV"):
+            rows = pool[:, table.long().flatten()].view(2, B, pps, 2, page, 128).permute(1, 0, 3, 2, 4, 5).reshape(B, 2, 2, pps * page, 128)
+            assert np.array_equal(akv.to_host_bits(rows[..., :N, :].contiguous()), plain[name]), name
+
+
 @pytest.mark.parametrize("N,budget", [(2, 2), (3, 2), (33, 33), (64, 40), (128, 128), (129, 90), (192, 64), (256, 100)])
 @pytest.mark.parametrize("lam", [0.5, 2.0])
 def test_resident_kernel_picks_in_pairs(N, budget, lam):
