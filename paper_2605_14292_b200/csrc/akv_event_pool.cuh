@@ -5,7 +5,7 @@
 //
 //   The picks hardly ever reach beyond the best-scored few dozen rows past the budget. The cosine matrix is
 //   therefore formed only for the pool's best-scored rows, 158 to 180 of them (64 KB of triangle: three CTAs
-//   per SM), and only their V rows are read. Every candidate left out scores at most `bound` (see active_bound),
+//   per SM; 138 to 158 and 49 KB: four), and only their V rows are read. Every candidate left out scores at most `bound` (see active_bound),
 //   and its Eq. 2 value never exceeds its score: the loop over the active set is exact as long as its
 //   winning value stays above that bound. In the rare event where it does not, the picks made so far stand and
 //   the remaining ones (a few, as a rule) are taken over the whole pool with rows of the cosine matrix as plain
@@ -30,14 +30,20 @@ __device__ __forceinline__ void bulk_store_wait_read() {
 
 // FUSED: score + select + compact; otherwise selection only (scores are read from a.scores and
 // nothing is rewritten).
-// WIDE: eight warps for an event that has an SM to itself (a call of no more events than SMs; also what event_tri_kernel takes, from
-// 129 rows on), else four warps and three events per SM. Alone on its SM an event is a chain of phases that too few warps hide: of 256
+// FORM (PoolShape): kPoolWideForm, eight warps for an event that has an SM to itself (a call of no more events than SMs; also what
+// event_tri_kernel takes, from 129 rows on). Alone on its SM an event is a chain of phases that too few warps hide: of 256
 // rows to 128, 55.2 -> 49.0 thousand cycles (scores 12.5 -> 10.4, picks in pairs 24.7 -> 22.5, triangle 3.2 -> 2.6, compaction 5.1 -> 4.4);
 // 112 of them 34.7 -> 31.2 us, in pages 39.1 -> 36.5, top-k 22.6 -> 18.5; of 192 rows to 64 (before: event_tri_kernel) 22.6 -> 22.0, of
-// 256 to 64 in pages 29.3 -> 26.8, but of 100 to 32 16.8 -> 17.1.
-template <bool FUSED, bool WIDE>
-__global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) event_pool_kernel(const __grid_constant__ EventArgs a, const __grid_constant__ ScoreTab tab) {
-    constexpr int NT = WIDE ? kPoolWide : kTcThreads, NW = NT / 32;
+// 256 to 64 in pages 29.3 -> 26.8, but of 100 to 32 16.8 -> 17.1. kPoolThree, four warps and three events per SM; kPoolFour, four events
+// per SM: latency bounds a call of many events (34 % of the issue slots used), so what counts is how many an SM holds. For that the last
+// 64 K rows come late, the triangle has 158 rows and the last kept V rows wait in registers: 16 384 events of 256 rows to 128 in
+// pages 1598 -> 1479 us (launch_tri says which calls). PAGED: with the layout known to the compiler, and 16 to 40 registers
+// more that the residency allows, another 1479 -> 1426, 1792 events with a shared matrix (all of the call) 222 -> 198.
+template <bool FUSED, int FORM, bool PAGED>
+__global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kCtas) event_pool_kernel(const __grid_constant__ EventArgs a, const __grid_constant__ ScoreTab tab) {
+    using Shape = PoolShape<FORM>;
+    constexpr bool WIDE = FORM == kPoolWideForm, FOUR = FORM == kPoolFour;
+    constexpr int NT = Shape::kThreads, NW = NT / 32;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const DevLayout& lay = a.lay;
@@ -46,7 +52,7 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
     const int N = lay.N;
     const int bud = event_budget(a, id);
     const int picks = min(bud, n);
-    const TriSmem sp = plan_pool_event_smem(N, a.budget, lay.page_size != 0);
+    const TriSmem sp = plan_pool_event_smem<FORM>(N, a.budget, PAGED);
     unsigned char* tile = smem + sp.tile;
     float* tri = reinterpret_cast<float*>(tile);  // lower triangle of the cosine matrix, after the product
     float* s = reinterpret_cast<float*>(smem + sp.s);
@@ -69,21 +75,25 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
     float* thr_holder = reinterpret_cast<float*>(smem + sp.misc + 56);          // the pool's score threshold
     int* tie_holder = reinterpret_cast<int*>(smem + sp.misc + 60);              // see picks_cosine: tie_slot
     const uint32_t tile_u32 = smem_u32(tile);
-    const uint32_t half_bytes = kPoolTileBytes / 2u;  // the operand's two 128-byte column halves
+    constexpr uint32_t half_bytes = Shape::kOperandRows * 128u;  // the operand's two 128-byte column halves
+    const uint32_t barL = barK + 48;  // K rows that wait for a free slot
+    const int n_late = FOUR && FUSED && n > Shape::kRows ? n - Shape::kRows : 0;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool similarity = a.greedy != 0 && picks > 1;   // (the first pick is the highest score in any case)
     const int np4 = (N + 3) & ~3;
     // row addressing: dense events are one base offset plus a row stride
-    const bool dense = lay.page_size == 0;
+    constexpr bool dense = !PAGED;
     const long long ev_off = dense ? id.b * lay.sb + id.l * lay.sl + id.h * lay.sh : 0;
     // paged: where the event's pages start, looked up once by as many lanes of every warp at the same time (the block table's
     // entries come from L2; looked up row by row and copy by copy: 16 384 events of 256 rows to 128 in pages of 64 1631 us, 1600 so,
     // 8192 in pages of 16 798 and 771)
     long long* page_off = reinterpret_cast<long long*>(smem + sp.pages);
     const bool few_pages = !dense && ((N - 1) >> lay.page_shift) < kPageOffsets;
-    if (few_pages && tid < kPageOffsets && (tid << lay.page_shift) < N) page_off[tid] = row_offset(lay, id.b, id.l, id.h, tid << lay.page_shift);
-    __syncwarp();
+    if (few_pages) {
+        if (tid < kPageOffsets && (tid << lay.page_shift) < N) page_off[tid] = row_offset(lay, id.b, id.l, id.h, tid << lay.page_shift);
+        __syncwarp();
+    }
     auto rowoff = [&](int j) -> long long {
         if (dense) return ev_off + (long long)j * lay.sn;
         return few_pages ? page_off[j >> lay.page_shift] + (long long)(j & (lay.page_size - 1)) * lay.s_page_n : row_offset(lay, id.b, id.l, id.h, j);
@@ -113,9 +123,10 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
     if (tid == 0) {
         mbar_init(barK, 1);
         mbar_init(barM, 1);
+        if (FOUR) mbar_init(barL, 1);
         mbar_init_fence();
         // the K rows are asked for before anything else: the wait for tensor memory below overlaps their flight
-        if (FUSED) request_k_rows(0, n, 0, barK);
+        if (FUSED) request_k_rows(0, n - n_late, 0, barK);
     }
     if (FUSED && warp == 1) fill_sector_table(sect, lane);
     // (this kernel claims half of the SM's columns: two of the three resident CTAs hold theirs at a time, the
@@ -170,7 +181,7 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
         // lane covers frequencies f0..f0+7 of the row handled by its group of eight lanes
         const int grp = lane >> 3, f0 = (lane & 7) * 8;
         // spacing of rows kRound (16 or 32) slots apart at the newest end of the event: what a token-by-token cache has everywhere
-        constexpr int kRound = 4 * NW;
+        constexpr int kRound = FOUR ? 8 * NW : 4 * NW;
         const long long step = n > kRound ? (long long)spos[n - 1] - (long long)spos[n - 1 - kRound] : 0;
         ChainScore cs;
         cs.set_step(step, phitab + f0, sect);
@@ -186,13 +197,21 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
             // The tile holds the whole event. A lane group scores two rows side by side, row j of the first half
             // of the rounds and row j + kRound * half of the second: two independent chains that share the turn S, so
             // that one chain's dependent arithmetic fills the other's latency.
-            const int half = (rounds + 1) >> 1;
+            // (four CTAs per SM: rows 16 slots apart instead, in order, so that the slots of the first 64 are free early for the late rows)
+            const int half = FOUR ? rounds : (rounds + 1) >> 1;
             ChainScore cb;
             AKV_PHASE_ACC_DECL(cyc_anchor);
 #pragma unroll 1
             for (int round = 0; round < half; ++round) {
-                const int ja = kRound * round + 4 * warp + grp, jb = ja + kRound * half;
+                const int ja = kRound * round + 4 * warp + grp, jb = FOUR ? ja + 16 : ja + kRound * half;
                 const bool la = ja < n, lb = jb < n;
+                if (FOUR && n_late > 0) {
+                    if (round == 2) {   // rows 0..63 have been scored
+                        __syncthreads();
+                        if (tid == 0) request_k_rows(Shape::kRows, n, 0, barL);
+                    }
+                    if (round == Shape::kRows / 32) timeout |= !mbar_wait_bounded(barL, 0, a.wait_polls);
+                }
                 // each chain on its own: after an event the kept rows' positions are irregular (fresh rotation every
                 // round) while the rows appended since are consecutive (chained)
                 bool fa = round == 0 || a.no_chain, fb = fa;
@@ -214,11 +233,11 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
                 AKV_PHASE_ACC_END(cyc_anchor);
                 float acca = 0.f, accb = 0.f;
                 if (la) {
-                    const unsigned char* krow = tile + ja * 256 + (lane & 7) * 16;
+                    const unsigned char* krow = tile + (FOUR && ja >= Shape::kRows ? ja - Shape::kRows : ja) * 256 + (lane & 7) * 16;
                     acca = cs.dot(*reinterpret_cast<const uint4*>(krow), *reinterpret_cast<const uint4*>(krow + 128));
                 }
                 if (lb) {
-                    const unsigned char* krow = tile + jb * 256 + (lane & 7) * 16;
+                    const unsigned char* krow = tile + (FOUR && jb >= Shape::kRows ? jb - Shape::kRows : jb) * 256 + (lane & 7) * 16;
                     accb = cb.dot(*reinterpret_cast<const uint4*>(krow), *reinterpret_cast<const uint4*>(krow + 128));
                 }
 #pragma unroll
@@ -260,6 +279,7 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
     if (timeout) {
         if (tid == 0 && a.status) a.status[id.e] = 3;
         mbar_wait_bounded(barK, 0, a.wait_polls);  // give copies still in flight another bounded chance to land
+        if (n_late > 0) mbar_wait_bounded(barL, 0, a.wait_polls);
         if (have_tmem && warp == 0) tmem_dealloc(tbase, kPoolCols);
         return;
     }
@@ -270,7 +290,7 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
     phase_stamp(id.e, 2);
     // ---- s_(b) by bisection over the score keys, then the pool in slot order (warp 0) -------------
     // (a pool that budgets of at most 64 have: 127 rows, so that the loop has four candidates per lane)
-    const int most = WIDE && a.budget <= 64 ? kTriMaxPool : kPoolActive;
+    const int most = WIDE && a.budget <= 64 ? kTriMaxPool : Shape::kActive;
     if constexpr (WIDE) {
         // A key per thread, counts by the barrier itself: a bit per round. (One warp with eight keys per lane: 3.7 thousand cycles
         // of an event, these 3.3.)
@@ -345,7 +365,7 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
         const float sb = from_orderable(kb);
         // -inf keeps everyone (also where kb, whose low bits are open, is below every finite value's key)
         const float thr = a.no_prune || kb < 0x00800000u ? -INFINITY : fmaf(-1.001f, a.lam, sb) - 1e-6f * fabsf(sb);
-        // Active set: the pool's best-scored rows, at most kPoolActive of them; no key left out is above bound.key (0: none
+        // Active set: the pool's best-scored rows, at most Shape::kActive of them; no key left out is above bound.key (0: none
         // is left out). A candidate's Eq. 2 value never exceeds its score: the loop over the active set is exact as long as
         // its winning value stays above the bound (it nearly always does: with lambda = 0.5 the picks reach a few ranks
         // beyond the budget).
@@ -355,7 +375,7 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
 #pragma unroll
             for (int k = 0; k < 8; ++k) pool_size += kk[k] != 0u && !(from_orderable(kk[k]) < thr);
             pool_size = __reduce_add_sync(0xFFFFFFFFu, pool_size);
-            if (pool_size > kPoolActive) bound = warp_active_bound(kk, orderable(thr), kb, kPoolActive);
+            if (pool_size > Shape::kActive) bound = warp_active_bound(kk, orderable(thr), kb, Shape::kActive);
         }
         int base = 0;
         if (lane == 0) *tie_holder = 0;
@@ -390,14 +410,14 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
         // keeps their slots in registers). Asynchronous 4-byte copies straight into the triangle: nothing waits until all of a
         // warp's rows are under way (1792 events of 256 rows to 128: 18.1 thousand cycles of an event with the loads through registers,
         // four rows at a time, 10.4 thousand so; the call with signatures and matrix 297 -> 271 us).
-        int col[kPoolCpl];
+        int col[Shape::kCpl];
 #pragma unroll
-        for (int k = 0; k < kPoolCpl; ++k) col[k] = lane + 32 * k < P ? bypool[lane + 32 * k] : 0;
+        for (int k = 0; k < Shape::kCpl; ++k) col[k] = lane + 32 * k < P ? bypool[lane + 32 * k] : 0;
         for (int ra = warp; ra < P; ra += NT / 32) {
             const float* grow = G + (long long)bypool[ra] * N;
             const uint32_t dst = tile_u32 + 4u * (uint32_t)(tri_row(ra) + lane);
 #pragma unroll
-            for (int k = 0; k < kPoolCpl; ++k)
+            for (int k = 0; k < Shape::kCpl; ++k)
                 if (lane + 32 * k <= ra) cp_async4(dst + 128u * (uint32_t)k, grow + col[k]);
         }
         cp_async_wait_all();
@@ -537,16 +557,16 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
             bool ok;
             // (eight picks per look at the bound instead of four: 16 384 events of 256 rows to 128 1645 -> 1626 us, 448 of them 76.8 -> 74.7)
             if constexpr (!WIDE)
-                ok = picks_cosine<kPoolCpl, true, 8>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order, bound, m_act, redi, nullptr, tie_holder);
+                ok = picks_cosine<Shape::kCpl, true, 8>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order, bound, m_act, redi, nullptr, tie_holder);
             else if (P <= 128)
                 ok = picks_in_pairs<4, true>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order, bound, m_act, redi, nullptr, tie_holder);
             else
-                ok = picks_in_pairs<kPoolCpl, true>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order, bound, m_act, redi, nullptr, tie_holder);
+                ok = picks_in_pairs<Shape::kCpl, true>(lane, P, picks, s, bypool, r, a.lam, tri, park_key, order, bound, m_act, redi, nullptr, tie_holder);
             if (lane == 0) *pick_holder = ok ? picks : *redi;
         }
         __syncthreads();
         if (*pick_holder < picks) {
-            picks_over_whole_pool<true, NT>(a, smem, n, P, picks, *pick_holder);
+            picks_over_whole_pool<FORM, NT>(a, smem, n, P, picks, *pick_holder);
         }
     }
     __syncthreads();
@@ -600,33 +620,51 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
             *reinterpret_cast<uint4*>(Vg + off) = *reinterpret_cast<const uint4*>(src + 16384);
         }
     } else {
-        static_assert(128u * 512u <= kPoolTileBytes, "the kept rows of the largest budget fit the tile");
-        // The tile holds the kept rows of K and of V side by side: one round of 16-byte gathers, one barrier.
+        // The tile holds the kept rows of K and of V side by side: one round of 16-byte gathers, one barrier. (With four CTAs per
+        // SM the last V rows that do not fit there wait in registers.)
         // Stores: slots 0..picks-1 are contiguous in a dense cache (and page by page in a paged one), so one
         // thread writes them back with a few bulk copies. (Gathering by one bulk copy per row measured slower.)
-        const uint32_t vhalf = kPoolTileBytes / 2u;
-        auto gather = [&](int x) {
+        constexpr uint32_t vhalf = 32768u;
+        constexpr int kFit = (int)((Shape::kTile - vhalf) / 256u) < 128 ? (int)((Shape::kTile - vhalf) / 256u) : 128;
+        constexpr int kHeld = ((128 - kFit) * 16 + NT - 1) / NT;
+        const int fit = min(picks, kFit);
+        auto gather = [&](int x, bool v) {
             const long long off = rowoff(idx[x >> 4]) + (x & 15) * 8;
             cp_async16(tile_u32 + (uint32_t)x * 16u, Kg + off);
-            cp_async16(tile_u32 + vhalf + (uint32_t)x * 16u, Vg + off);
+            if (v) cp_async16(tile_u32 + vhalf + (uint32_t)x * 16u, Vg + off);
         };
         if constexpr (WIDE) {
-            for (int x = tid; x < picks * 16; x += NT) gather(x);
+            for (int x = tid; x < picks * 16; x += NT) gather(x, true);
         } else {
 #pragma unroll 4
-            for (int x = tid; x < picks * 16; x += NT) gather(x);   // (several rows' look-ups at once; with one event per SM no gain)
+            for (int x = tid; x < picks * 16; x += NT) gather(x, !FOUR || x < fit * 16);   // (several rows' look-ups at once; with one event per SM no gain)
+        }
+        uint4 held[kHeld > 0 ? kHeld : 1];
+#pragma unroll
+        for (int i = 0; i < kHeld; ++i) {
+            const int x = fit * 16 + tid + i * NT;
+            held[i] = x < picks * 16 ? *reinterpret_cast<const uint4*>(Vg + rowoff(idx[x >> 4]) + (x & 15) * 8) : make_uint4(0u, 0u, 0u, 0u);
         }
         cp_async_wait_all();
         fence_proxy_async();  // the bulk stores below read what these copies wrote
-        __syncthreads();      // every kept row is on chip before the first store
+        // every kept row is on chip before the first store (those in registers too: the barrier's operand depends on them)
+        if constexpr (kHeld > 0) {
+            uint32_t arrived = 0u;
+#pragma unroll
+            for (int i = 0; i < kHeld; ++i) arrived |= held[i].x | held[i].w;
+            __syncthreads_or(arrived == 0x7FC07FC1u);
+        } else {
+            __syncthreads();
+        }
         const bool runs = dense ? lay.sn == kTcD : lay.s_page_n == kTcD;
         if (runs) {
             if (tid == 0) {
                 for (int row = 0; row < picks;) {
                     const int run = dense ? picks - row : min(picks - row, lay.page_size - row % lay.page_size);
                     const long long off = rowoff(row);
+                    const int vrun = min(run, fit - row);
                     bulk_s2g(Kg + off, tile_u32 + (uint32_t)row * 256u, (uint32_t)run * 256u);
-                    bulk_s2g(Vg + off, tile_u32 + vhalf + (uint32_t)row * 256u, (uint32_t)run * 256u);
+                    if (!FOUR || vrun > 0) bulk_s2g(Vg + off, tile_u32 + vhalf + (uint32_t)row * 256u, (uint32_t)vrun * 256u);
                     row += run;
                 }
                 bulk_store_wait_read();  // shared memory is read out before the CTA may leave
@@ -635,8 +673,13 @@ __global__ void __launch_bounds__(WIDE ? kPoolWide : kTcThreads, WIDE ? 1 : 3) e
             for (int x = tid; x < picks * 16; x += NT) {
                 const long long off = rowoff(x >> 4) + (x & 15) * 8;
                 copy16(reinterpret_cast<char*>(Kg + off), tile + x * 16);
-                copy16(reinterpret_cast<char*>(Vg + off), tile + vhalf + x * 16);
+                if (!FOUR || x < fit * 16) copy16(reinterpret_cast<char*>(Vg + off), tile + vhalf + x * 16);
             }
+        }
+#pragma unroll
+        for (int i = 0; i < kHeld; ++i) {
+            const int x = fit * 16 + tid + i * NT;
+            if (x < picks * 16) *reinterpret_cast<uint4*>(Vg + rowoff(x >> 4) + (x & 15) * 8) = held[i];
         }
     }
     if (wpos)

@@ -92,19 +92,19 @@ __device__ __forceinline__ void cluster_store(uint32_t addr, uint32_t v) {
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
-// A call of two launches (see launch_prefill), one CTA per event and several: the first lets the second start as soon as all of its own CTAs have, the second ends
+// TAIL: a call of two launches (see launch_prefill), one CTA per event and several. The first lets the second start as soon as all of its own CTAs have, the second ends
 // only when the first has, so that whatever follows on the stream comes after both.
 __device__ __forceinline__ void let_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_launch_ahead() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-template <bool FUSED, int SPLIT>
+template <bool FUSED, int SPLIT, bool TAIL>
 __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __grid_constant__ EventArgs a, const __grid_constant__ ScoreTab tab) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     __shared__ __align__(16) uint32_t part[2][kStWarps];       // per-warp partial counts, double-buffered
     __shared__ __align__(16) uint4 best_of[2][kStWarps];       // per-warp arg-max: key, 0xFFFFFFFF - slot, row
     const DevLayout& lay = a.lay;
-    const EventId id = decode_event(lay, (SPLIT > 1 ? a.first_event : 0) + (int)blockIdx.x / SPLIT);
+    const EventId id = decode_event(lay, TAIL && SPLIT > 1 ? a.first_event + (int)blockIdx.x / SPLIT : blockIdx.x / SPLIT);
     const int rank = SPLIT > 1 ? cluster_rank() : 0;
     const int n = event_n(a, id.b);
     const int N = lay.N;
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
         cnt[0] = 0;
         cnt[1] = INT_MIN;
         cnt[2] = 0;
-        if (SPLIT == 1 && a.followed) let_dependents_launch();
+        if (TAIL && SPLIT == 1) let_dependents_launch();
     }
     if (warp == 0) {
         // (both resident CTAs' columns fit the SM; the right to allocate is given up at once, or the next CTA would not start)
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
                 }
             }
             if (similarity && rank == 0 && warp == 0) tmem_dealloc(*tmem_holder, kPfCols);
-            if (SPLIT > 1 && a.behind && tid == 0) wait_for_launch_ahead();
+            if (TAIL && SPLIT > 1 && tid == 0) wait_for_launch_ahead();
             return;
         }
     } else {
@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
                 if (warp == 0) tmem_dealloc(tbase, kPfCols);
                 if (tid == 0 && a.status) a.status[id.e] = 3;
                 if (!FUSED) select_gave_up(a, id.e, kStWork);
-                if (SPLIT > 1 && a.behind && tid == 0) wait_for_launch_ahead();
+                if (TAIL && SPLIT > 1 && tid == 0) wait_for_launch_ahead();
                 return;
             }
             // lower triangle -> shared memory: warps 0..3 the first product's columns up to the row itself, warps 4..7 its
@@ -800,7 +800,7 @@ __global__ void __launch_bounds__(kStThreads, 2) event_prefill_kernel(const __gr
         *reinterpret_cast<uint4*>(Vg + off) = *reinterpret_cast<const uint4*>(region + 32768 + x * 16);
     }
     if (wpos && tid < picks) wpos[tid] = pv;
-    if (SPLIT > 1 && a.behind && tid == 0) wait_for_launch_ahead();
+    if (TAIL && SPLIT > 1 && tid == 0) wait_for_launch_ahead();
     phase_stamp(id.e, 8);
 }
 

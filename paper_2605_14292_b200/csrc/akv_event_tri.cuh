@@ -31,20 +31,12 @@ constexpr int kTriTileRows = 128;           // K rows resident at a time = rows 
 constexpr unsigned kTriTileBytes = 32768u;  // 128 rows of 256 bytes; holds the triangle of up to 127 rows
 constexpr int kTriMaxPool = 127;            // largest pool whose cosine matrix goes through the tile
 
-// event_pool_kernel's (akv_event_pool.cuh): a tile of 64 KB, for a whole event's K rows, then the triangle of an active set of up to 180 rows (see the kernel);
-// three CTAs per SM.
-constexpr unsigned kPoolTileBytes = 65536u;
-constexpr int kPoolActive = 180;            // most rows whose cosine matrix goes through the tile
-constexpr uint32_t kPoolCols = 256u;        // tensor-memory columns (a power of two >= the matrix's columns)
-constexpr int kPoolWide = 256;              // threads of a CTA that has an SM to itself
-constexpr int kPoolCpl = 6;                 // candidates per lane of the one-warp loop
-
 struct TriSmem {
     unsigned tile, s, key, spos, bypool, taken, order, gain, idx, sect, misc, pages, total;   // taken: a flag per slot, or (event_pool_kernel) a bit
 };
 // Layout after the 1024-byte aligned base. `key` (score keys) and `r` (reciprocal norms) share storage.
 constexpr int kPageOffsets = 16;   // pages of an event whose offsets are kept on chip
-__host__ __device__ inline TriSmem plan_event_smem(int N, int budget, unsigned tile_bytes, bool paged) {
+__host__ __device__ inline TriSmem plan_event_smem(int N, int budget, unsigned tile_bytes, bool paged, unsigned taken_bytes) {
     TriSmem p;
     const unsigned np = (unsigned)((N + 3) & ~3);
     unsigned o = 0;
@@ -53,7 +45,7 @@ __host__ __device__ inline TriSmem plan_event_smem(int N, int budget, unsigned t
     p.key = o;    o += align16(np * 4);
     p.spos = o;   o += align16(np * 4);
     p.bypool = o; o += align16(np * 2);
-    p.taken = o;  o += align16(np < 32 ? 32 : np);
+    p.taken = o;  o += align16(taken_bytes);
     p.order = o;  o += align16((unsigned)budget * 4);
     p.gain = o;   o += align16((unsigned)budget * 4);
     p.idx = o;    o += align16((unsigned)budget * 4);
@@ -64,9 +56,30 @@ __host__ __device__ inline TriSmem plan_event_smem(int N, int budget, unsigned t
     p.total = o + 1024;           // room to align the base to 1024 bytes
     return p;
 }
-__host__ __device__ inline TriSmem plan_tri_smem(int N, int budget, bool paged) { return plan_event_smem(N, budget, kTriTileBytes, paged); }
+__host__ __device__ inline TriSmem plan_tri_smem(int N, int budget, bool paged) { return plan_event_smem(N, budget, kTriTileBytes, paged, N < 32 ? 32u : (unsigned)((N + 3) & ~3)); }
 
-__host__ __device__ inline TriSmem plan_pool_event_smem(int N, int budget, bool paged) { return plan_event_smem(N, budget, kPoolTileBytes, paged); }
+
+// event_pool_kernel's (akv_event_pool.cuh) forms: how many of an event's rows a CTA has on chip, and with how many threads.
+enum PoolForm { kPoolThree, kPoolWideForm, kPoolFour };
+constexpr uint32_t kPoolCols = 256u;        // tensor-memory columns (a power of two >= the matrix's columns)
+constexpr int kPoolWide = 256;              // threads of a CTA that has an SM to itself
+template <int FORM>
+struct PoolShape {
+    // a whole event's K rows, then the triangle of an active set of up to 180 rows; three CTAs per SM, or one of eight warps
+    static constexpr int kThreads = FORM == kPoolWideForm ? kPoolWide : kTcThreads, kCtas = FORM == kPoolWideForm ? 1 : 3;
+    static constexpr unsigned kTile = 65536u;
+    static constexpr int kActive = 180, kCpl = 6, kRows = 256, kOperandRows = 256;
+};
+template <>
+struct PoolShape<kPoolFour> {
+    // 192 K rows (the others arrive in the slots of the first), then the triangle of up to 158 rows; four CTAs per SM: 57 312 bytes for
+    // 256 rows in pages to 128, of the 57 344 that four leave each
+    static constexpr int kThreads = kTcThreads, kCtas = 4;
+    static constexpr unsigned kTile = 50688u;
+    static constexpr int kActive = 158, kCpl = 5, kRows = 192, kOperandRows = 160;
+};
+template <int FORM>
+__host__ __device__ inline TriSmem plan_pool_event_smem(int N, int budget, bool paged) { return plan_event_smem(N, budget, PoolShape<FORM>::kTile, paged, 32u); }
 
 // 32 consecutive columns of this thread's TMEM lane.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
@@ -555,12 +568,13 @@ constexpr unsigned kContMact = 8192u;      // m_act, 1 KB
 //
 // Out of line and with few arguments (the rest is found again from them), so that it costs the kernels that call it
 // neither registers nor a stretch of cold code between the phases (inlined: 2.5 % of event_tri_kernel).
-template <bool POOL, int NT>
+template <int FORM, int NT>
 __device__ __noinline__ void picks_over_whole_pool(const EventArgs& a, unsigned char* smem, int n, int active, int picks, int made) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const DevLayout& lay = a.lay;
     const EventId id = decode_event(lay, blockIdx.x);
-    const TriSmem sp = POOL ? plan_pool_event_smem(lay.N, a.budget, lay.page_size != 0) : plan_tri_smem(lay.N, a.budget, lay.page_size != 0);
+    constexpr bool POOL = FORM >= 0;   // (below 0: event_tri_kernel)
+    const TriSmem sp = POOL ? plan_pool_event_smem<POOL ? FORM : 0>(lay.N, a.budget, lay.page_size != 0) : plan_tri_smem(lay.N, a.budget, lay.page_size != 0);
     const float* G = POOL && a.gram ? a.gram + id.b * a.gram_sb + id.l * a.gram_sl : nullptr;
     const float* s = reinterpret_cast<const float*>(smem + sp.s);
     unsigned short* bypool = reinterpret_cast<unsigned short*>(smem + sp.bypool);
@@ -695,8 +709,9 @@ __device__ __noinline__ void picks_over_whole_pool(const EventArgs& a, unsigned 
 }
 
 // FUSED: score + select + compact; otherwise selection only (scores are read from a.scores and
-// nothing is rewritten).
-template <bool FUSED>
+// nothing is rewritten). (The dense form decides by the layout all the same: with that known at compile time the call of 4096 events
+// of 192 rows is 0.8 % slower, which registers go where.)
+template <bool FUSED, bool PAGED>
 __global__ void __launch_bounds__(kTcThreads) event_tri_kernel(const __grid_constant__ EventArgs a, const __grid_constant__ ScoreTab tab) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -706,7 +721,7 @@ __global__ void __launch_bounds__(kTcThreads) event_tri_kernel(const __grid_cons
     const int N = lay.N;
     const int bud = event_budget(a, id);
     const int picks = min(bud, n);
-    const TriSmem sp = plan_tri_smem(N, a.budget, lay.page_size != 0);
+    const TriSmem sp = plan_tri_smem(N, a.budget, PAGED);
     unsigned char* tile = smem + sp.tile;
     float* tri = reinterpret_cast<float*>(tile);  // lower triangle of the cosine matrix, after the product
     float* s = reinterpret_cast<float*>(smem + sp.s);
@@ -736,17 +751,19 @@ __global__ void __launch_bounds__(kTcThreads) event_tri_kernel(const __grid_cons
     const bool similarity = a.greedy != 0 && picks > 1;   // (the first pick is the highest score in any case)
     const int np4 = (N + 3) & ~3;
     // row addressing: dense events are one base offset plus a row stride
-    const bool dense = lay.page_size == 0;
+    const bool dense = !PAGED && lay.page_size == 0;
     const long long ev_off = dense ? id.b * lay.sb + id.l * lay.sl + id.h * lay.sh : 0;
-    // paged: where the event's pages start, looked up once by as many lanes of every warp at the same time (the block table's
-    // entries come from L2; looked up row by row and copy by copy: 4096 events of 192 rows to 64 in pages of 64 191 us, 183 so)
+    // paged: where the event's pages start, looked up once by as many lanes at the same time (the block table's entries come from L2;
+    // looked up row by row and copy by copy: 4096 events of 192 rows to 64 in pages of 64 191 us, 182 so)
     long long* page_off = reinterpret_cast<long long*>(smem + sp.pages);
-    const bool few_pages = !dense && ((N - 1) >> lay.page_shift) < kPageOffsets;
-    if (few_pages && tid < kPageOffsets && (tid << lay.page_shift) < N) page_off[tid] = row_offset(lay, id.b, id.l, id.h, tid << lay.page_shift);
-    __syncwarp();
+    const bool few_pages = PAGED && ((N - 1) >> lay.page_shift) < kPageOffsets;
+    if (PAGED && few_pages) {
+        if (tid < kPageOffsets && (tid << lay.page_shift) < N) page_off[tid] = row_offset(lay, id.b, id.l, id.h, tid << lay.page_shift);
+        __syncwarp();
+    }
     auto rowoff = [&](int j) -> long long {
-        if (dense) return ev_off + (long long)j * lay.sn;
-        return few_pages ? page_off[j >> lay.page_shift] + (long long)(j & (lay.page_size - 1)) * lay.s_page_n : row_offset(lay, id.b, id.l, id.h, j);
+        if (PAGED && few_pages) return page_off[j >> lay.page_shift] + (long long)(j & (lay.page_size - 1)) * lay.s_page_n;
+        return dense ? ev_off + (long long)j * lay.sn : row_offset(lay, id.b, id.l, id.h, j);
     };
     __nv_bfloat16* Kg = reinterpret_cast<__nv_bfloat16*>(a.K);
     __nv_bfloat16* Vg = reinterpret_cast<__nv_bfloat16*>(a.V);
@@ -1050,7 +1067,7 @@ __global__ void __launch_bounds__(kTcThreads) event_tri_kernel(const __grid_cons
         }
         __syncthreads();
         if (*pick_holder < picks) {
-            picks_over_whole_pool<false, kTcThreads>(a, smem, n, P, picks, *pick_holder);
+            picks_over_whole_pool<-1, kTcThreads>(a, smem, n, P, picks, *pick_holder);
         }
     }
     __syncthreads();

@@ -27,9 +27,7 @@ struct EventArgs {
     int gqa_max;            // 1: a key's score is the largest over the group, 0: their mean
     int starve;             // testing aid: request no K row and, where there is no K to read, issue no product, so that the bounded waits run out
     int wait_polls;         // polls after which a bounded wait gives up
-    int first_event;        // prefill kernel: the first event of this launch
-    int followed;           // prefill kernel: another launch of the same call may start once this one's CTAs have
-    int behind;             // prefill kernel: this launch is that other one, and does not end before the one ahead of it has
+    int first_event;        // prefill kernel: the first event of the second of two launches
     int* idx_sorted;
     int* pick_order;
     float* pick_gain;

@@ -351,23 +351,37 @@ static akv_status_t launch_tri(akv_handle* h, const EventArgs& a, cudaStream_t s
     const int E = a.lay.B * a.lay.L * a.lay.H;
     if constexpr (!BIG)   // an SM for every event: the large kernel's eight warps (see there; events of up to 128 rows gain nothing)
         if (E <= h->sm_count && a.lay.N > 128) return launch_tri<FUSED, true>(h, a, st, dry);
-    const TriSmem sp = BIG ? plan_pool_event_smem(a.lay.N, a.budget, a.lay.page_size != 0) : plan_tri_smem(a.lay.N, a.budget, a.lay.page_size != 0);
-    if ((int)sp.total > h->smem_optin) return fail(AKV_ERR_UNSUPPORTED, "budget %d needs too much shared memory", a.budget);
     akv_status_t s;
-    if (BIG) {
-        const bool wide = E <= h->sm_count;   // an SM for every event
-        auto kernel = wide ? event_pool_kernel<FUSED, true> : event_pool_kernel<FUSED, false>;
-        if ((s = set_smem(h, kernel, sp.total)) != AKV_OK) return s;
-        CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
-        if (dry) return AKV_OK;
-        kernel<<<E, wide ? kPoolWide : kTcThreads, sp.total, st>>>(a, h->tab);
-        return launched(FUSED ? "event_pool" : "select_pool_active");
+    if constexpr (BIG) {
+        auto launch = [&](auto kernel, unsigned bytes, int threads) -> akv_status_t {
+            if ((int)bytes > h->smem_optin) return fail(AKV_ERR_UNSUPPORTED, "budget %d needs too much shared memory", a.budget);
+            if ((s = set_smem(h, kernel, bytes)) != AKV_OK) return s;
+            CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
+            if (dry) return AKV_OK;
+            kernel<<<E, threads, bytes, st>>>(a, h->tab);
+            return launched(FUSED ? "event_pool" : "select_pool_active");
+        };
+        const bool paged = a.lay.page_size != 0;
+        if (E <= h->sm_count)
+            return launch(paged ? event_pool_kernel<FUSED, kPoolWideForm, true> : event_pool_kernel<FUSED, kPoolWideForm, false>,
+                          plan_pool_event_smem<kPoolWideForm>(a.lay.N, a.budget, paged).total, kPoolWide);
+        // Four events to an SM where three would not hold the call, as long as the loop hardly ever looks beyond the 158 rows that they have
+        // room for: with weak penalties, or budgets that leave room for strong ones. Us per call, three / four: 560 events of 256 rows to
+        // 128 75.8 / 64.5, 4096 of 180 to 70 250 / 229, of 256 to 128 at lambda 0.25 352 / 326, with near-duplicates at 0.5 403 / 385, at 0.75
+        // 363 / 393, at 1.0 363 / 655, 4096 to 96 at 1.0 325 / 269, to 80 307 / 262; 444 of 256 to 100 52.3 / 56.5, 336 51.3 / 51.4; top-k 201 / 206.
+        if (E > 3 * h->sm_count && a.greedy && (a.lam <= 0.5f || (a.lam <= 1.f && a.budget <= 96)))
+            return launch(paged ? event_pool_kernel<FUSED, kPoolFour, true> : event_pool_kernel<FUSED, kPoolFour, false>,
+                          plan_pool_event_smem<kPoolFour>(a.lay.N, a.budget, paged).total, kTcThreads);
+        return launch(paged ? event_pool_kernel<FUSED, kPoolThree, true> : event_pool_kernel<FUSED, kPoolThree, false>,
+                      plan_pool_event_smem<kPoolThree>(a.lay.N, a.budget, paged).total, kTcThreads);
     }
-    if ((s = set_smem(h, event_tri_kernel<FUSED>, sp.total)) != AKV_OK) return s;
-    CUDA_TRY(cudaFuncSetAttribute(event_tri_kernel<FUSED>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                  (int)cudaSharedmemCarveoutMaxShared));
+    const TriSmem sp = plan_tri_smem(a.lay.N, a.budget, a.lay.page_size != 0);
+    if ((int)sp.total > h->smem_optin) return fail(AKV_ERR_UNSUPPORTED, "budget %d needs too much shared memory", a.budget);
+    auto kernel = a.lay.page_size ? event_tri_kernel<FUSED, true> : event_tri_kernel<FUSED, false>;
+    if ((s = set_smem(h, kernel, sp.total)) != AKV_OK) return s;
+    CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
     if (dry) return AKV_OK;
-    event_tri_kernel<FUSED><<<E, kTcThreads, sp.total, st>>>(a, h->tab);
+    kernel<<<E, kTcThreads, sp.total, st>>>(a, h->tab);
     return launched(FUSED ? "event_tri" : "select_tri");
 }
 
@@ -377,11 +391,11 @@ static bool prefill_path_ok(const EventArgs& a) {
            !a.gqa_max && a.budget <= kPfMaxBudget;
 }
 // (events of the call from a.first_event on)
-template <bool FUSED, int SPLIT>
+template <bool FUSED, int SPLIT, bool TAIL = false>
 static akv_status_t launch_prefill_split(akv_handle* h, const EventArgs& a, long long events, cudaStream_t st, bool dry) {
     const PfSmem sp = plan_pf_smem(a.lay.N, a.budget);
     akv_status_t s;
-    auto kernel = event_prefill_kernel<FUSED, SPLIT>;
+    auto kernel = event_prefill_kernel<FUSED, SPLIT, TAIL>;
     if ((s = set_smem(h, kernel, sp.total, kStaticSmem)) != AKV_OK) return s;
     CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
     if (dry) return AKV_OK;
@@ -399,7 +413,7 @@ static akv_status_t launch_prefill_split(akv_handle* h, const EventArgs& a, long
         attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
         ++cfg.numAttrs;
     }
-    if (a.behind) {
+    if (TAIL && SPLIT > 1) {
         attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
         ++cfg.numAttrs;
@@ -408,21 +422,18 @@ static akv_status_t launch_prefill_split(akv_handle* h, const EventArgs& a, long
     return launched(FUSED ? "event_prefill" : "select_prefill");
 }
 template <bool FUSED>
-static akv_status_t launch_prefill(akv_handle* h, const EventArgs& a0, cudaStream_t st, bool dry = false) {
-    EventArgs a = a0;
+static akv_status_t launch_prefill(akv_handle* h, const EventArgs& a, cudaStream_t st, bool dry = false) {
     const long long E = (long long)a.lay.B * a.lay.L * a.lay.H;
     if constexpr (FUSED) {
         // The events of a nearly empty last wave, sharing their scoring, as a launch of their own behind the full waves
         const long long tail = prefill_tail(E, a.lay.N, h->sm_count, !a.greedy, a.n_cand != nullptr);
         if (tail) {
-            EventArgs b = a0;
-            b.behind = 1;
+            EventArgs b = a;
             b.first_event = (int)(E - tail);
-            a.followed = 1;
             const bool four = prefill_split(tail, a.lay.N, h->sm_count, !a.greedy, a.n_cand != nullptr) == 4;
-            auto second = [&](bool check) { return four ? launch_prefill_split<true, 4>(h, b, tail, st, check) : launch_prefill_split<true, 2>(h, b, tail, st, check); };
+            auto second = [&](bool check) { return four ? launch_prefill_split<true, 4, true>(h, b, tail, st, check) : launch_prefill_split<true, 2, true>(h, b, tail, st, check); };
             akv_status_t s = second(true);   // (what can be refused is, before the first launch)
-            if (s == AKV_OK) s = launch_prefill_split<true, 1>(h, a, E - tail, st, dry);
+            if (s == AKV_OK) s = launch_prefill_split<true, 1, true>(h, a, E - tail, st, dry);
             return s != AKV_OK || dry ? s : second(false);
         }
         const int split = prefill_split(E, a.lay.N, h->sm_count, !a.greedy, a.n_cand != nullptr);

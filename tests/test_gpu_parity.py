@@ -355,18 +355,20 @@ def in_pairs(ev, seed):
 
 
 @pytest.mark.parametrize("N,budget,lam", [(129, 20, 0.5), (144, 64, 1.0), (160, 128, 0.5), (192, 64, 0.0), (250, 33, 1.0), (255, 65, 0.0),
-                                          (256, 64, 0.5), (256, 128, 0.5), (256, 128, 2.0)])
+                                          (256, 64, 0.5), (256, 128, 0.5), (256, 128, 2.0), (192, 70, 0.5), (193, 71, 0.25), (224, 128, 0.5)])
 def test_events_with_an_sm_each_and_several_to_an_sm(N, budget, lam):
-    """bf16, d = 128: calls of no more events than SMs take the kernel of eight warps, others those of four; both against the
-    oracle, with all candidates, ragged counts and when their waits run out."""
+    """bf16, d = 128: calls of no more events than SMs take the kernel of eight warps, others those of four, three or four (more than
+    three per SM, no strong penalty) of them to an SM; all against the oracle, with all candidates, ragged counts and when their waits
+    run out."""
     few = in_pairs(synth.make_plain(2, 1, 3, N, 128, budget, lam, dtype=synth.BF16, seed=N + budget), N)
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    times = sms // 6 + 1
-    many = synth.make_plain(2 * times, 1, 3, 1, 128, 1, lam, dtype=synth.BF16, seed=0)
-    many.qstat, many.budget = few.qstat, budget
-    for name in ("K", "V", "pos", "p_ref"):
-        setattr(many, name, np.tile(getattr(few, name), (times,) + (1,) * (getattr(few, name).ndim - 1)))
-    for ev, events in ((few, range(6)), (many, (0, 4, 6 * times - 1))):
+    for times in (1, sms // 6 + 1, 3 * sms // 6 + 1):
+        ev, events = few, range(6)
+        if times > 1:
+            ev, events = synth.make_plain(2 * times, 1, 3, 1, 128, 1, lam, dtype=synth.BF16, seed=0), (0, 4, 6 * times - 1)
+            ev.qstat, ev.budget = few.qstat, budget
+            for name in ("K", "V", "pos", "p_ref"):
+                setattr(ev, name, np.tile(getattr(few, name), (times,) + (1,) * (getattr(few, name).ndim - 1)))
         check_all(ev, run_fused(ev), lam, events=events)
         n_cand = [N - 1, N // 2 + 1] * (len(ev.p_ref) // 2)
         check_all(ev, run_fused(ev, n_cand=n_cand), lam, events=events, n_cand=n_cand)
@@ -378,7 +380,7 @@ def test_events_with_an_sm_each_and_several_to_an_sm(N, budget, lam):
 def test_pages_on_both_sides_of_those_whose_offsets_are_kept(page, N, budget):
     """Up to sixteen pages of an event have their offsets on chip: one less, as many and one more, in no order, for events with an
     SM each and several to an SM; against the same rows in a dense cache, to the bit."""
-    for B in (1, 40):
+    for B in (1, 40, 120):
         ev = synth.make_plain(B, 2, 2, N, 128, budget, 0.5, dtype=synth.BF16, seed=N + page)
         plain = run_fused(ev)
         pps = -(-N // page)
@@ -1038,6 +1040,25 @@ def test_fused_event_with_shared_cosine_matrix(mode, N, budget):
                                 sel.idx_sorted[b, l, h].cpu().numpy(), Kn[b, l, h], Vn[b, l, h], pn[b, l, h], sig=ref_sig)
                 n_same += int(torch.equal(sel.pick_order[b, l, h], ref.pick_order[b, l, h]))
     assert n_same >= 11                                               # the two routes round differently: near-ties may differ
+    assert int(sel.status.abs().max()) == 0 and int(sel.n_kept.min()) == budget
+
+
+@pytest.mark.parametrize("N,budget", [(256, 128), (193, 90)])
+def test_shared_cosine_matrix_with_four_events_to_an_sm(N, budget):
+    """The same of a call of more than three events per SM."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    B, lam = sms // 2 + 1, 0.5
+    ev = synth.make_c3(seed=N, B=B, L=2, H=3, N=N, budget=budget)
+    K, V, pos = dev(ev.K), dev(ev.V), dev(ev.pos)
+    sig = akv.alpha_signature_flat(V)
+    gram = akv.alpha_gram_shared(sig, akv.Layout.dense(V), akv.Options(sig_mode=akv.SIG_FLAT))
+    sel = akv.alpha_compress_event(K, V, pos, dev(ev.qstat), budget, akv.Options(lam=lam, sig_mode=akv.SIG_FLAT, shared_gram=gram), p_ref=dev(ev.p_ref),
+                                   flat_sig=sig, want_scores=True)
+    Kn, Vn, pn = akv.to_host_bits(K), akv.to_host_bits(V), pos.cpu().numpy()
+    for b, l, h in ((0, 0, 0), (B // 2, 1, 1), (B - 1, 1, 2)):
+        chk.check_event(ev.K[b, l, h], ev.V[b, l, h], ev.pos[b, l, h], ev.qstat[l, h], int(ev.p_ref[b]), budget, lam,
+                        sel.scores[b, l, h].cpu().numpy(), sel.pick_order[b, l, h].cpu().numpy(), sel.idx_sorted[b, l, h].cpu().numpy(),
+                        Kn[b, l, h], Vn[b, l, h], pn[b, l, h], sig=O.signatures_flat(ev.V[b]))
     assert int(sel.status.abs().max()) == 0 and int(sel.n_kept.min()) == budget
 
 
