@@ -285,7 +285,7 @@ static akv_status_t launch_score(akv_handle* h, const EventArgs& a, cudaStream_t
         if (s != AKV_OK) return s;
     }
     const unsigned grid = (unsigned)blocks;
-    if (d128) score_rows_kernel<<<grid, kThreads, 0, st>>>(a, h->tab);
+    if (d128) (a.lay.page_size ? score_rows_kernel<true> : score_rows_kernel<false>)<<<grid, kThreads, 0, st>>>(a, h->tab);
     else if (a.lay.dtype == AKV_BF16) score_kernel<__nv_bfloat16><<<grid, kThreads, 0, st>>>(a, h->tab);
     else score_kernel<float><<<grid, kThreads, 0, st>>>(a, h->tab);
     return launched("score");

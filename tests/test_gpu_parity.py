@@ -221,6 +221,23 @@ def test_score_select_compact_chain_equals_fused(dtype):
     assert int(status.abs().max()) == 0
 
 
+@pytest.mark.parametrize("N,page", [(5, 4), (256, 64), (257, 16), (1000, 128)])
+def test_scores_of_a_paged_cache_are_the_dense_ones(N, page):
+    """bf16, d = 128: the score kernel's two layouts, with a block table in no order, to the bit."""
+    ev = synth.make_plain(2, 2, 3, N, 128, 2, 0.5, dtype=synth.BF16, seed=N)
+    K, pos, q, pref = dev(ev.K), dev(ev.pos), dev(ev.qstat), dev(ev.p_ref)
+    pps = -(-N // page)
+    table = torch.randperm(2 * pps, device="cuda").to(torch.int32).view(2, pps)
+    rows = torch.zeros((2, 2, 3, pps * page, 128), dtype=torch.bfloat16, device="cuda")
+    rows[..., :N, :] = K
+    pool = torch.zeros((2, 2 * pps, 3, page, 128), dtype=torch.bfloat16, device="cuda")
+    pool[:, table.long().flatten()] = rows.view(2, 2, 3, pps, page, 128).permute(1, 0, 3, 2, 4, 5).reshape(2, 2 * pps, 3, page, 128)
+    dense = akv.alpha_score(K, q, pos=pos, p_ref=pref)
+    assert torch.equal(dense, akv.alpha_score(pool, q, pos=pos, p_ref=pref, layout=akv.Layout.paged(pool, table, N)))
+    ref = O.triattention_score(ev.K[1, 1, 2], ev.pos[1, 1, 2], ev.qstat[1, 2], int(ev.p_ref[1]), 1, 10000.0)
+    chk.check_scores(dense[1, 1, 2].cpu().numpy(), ref, chk.score_scale(ev.K[1, 1, 2], ev.qstat[1, 2], 128))
+
+
 def test_score_only_broadcast_positions_and_rotated_cache():
     ev = synth.make_plain(2, 3, 2, 70, 128, 10, 0.5, dtype=synth.BF16, seed=22)
     K, q = dev(ev.K), dev(ev.qstat)
