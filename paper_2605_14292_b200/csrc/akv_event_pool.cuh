@@ -38,7 +38,8 @@ __device__ __forceinline__ void bulk_store_wait_read() {
 // per SM: latency bounds a call of many events (34 % of the issue slots used), so what counts is how many an SM holds. For that the last
 // 64 K rows come late, the triangle has 158 rows and the last kept V rows wait in registers: 16 384 events of 256 rows to 128 in
 // pages 1598 -> 1479 us (launch_tri says which calls). PAGED: with the layout known to the compiler, and 16 to 40 registers
-// more that the residency allows, another 1479 -> 1426, 1792 events with a shared matrix (all of the call) 222 -> 198.
+// more that the residency allows, another 1479 -> 1426, 1792 events with a shared matrix (all of the call) 222 -> 198; but three events
+// per SM in pages 1598 -> 1703, so that those decide at run time.
 template <bool FUSED, int FORM, bool PAGED>
 __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kCtas) event_pool_kernel(const __grid_constant__ EventArgs a, const __grid_constant__ ScoreTab tab) {
     using Shape = PoolShape<FORM>;
@@ -83,7 +84,7 @@ __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kC
     const bool similarity = a.greedy != 0 && picks > 1;   // (the first pick is the highest score in any case)
     const int np4 = (N + 3) & ~3;
     // row addressing: dense events are one base offset plus a row stride
-    constexpr bool dense = !PAGED;
+    const bool dense = PAGED && FORM == kPoolThree ? lay.page_size == 0 : !PAGED;   // (see above: three events per SM, in pages)
     const long long ev_off = dense ? id.b * lay.sb + id.l * lay.sl + id.h * lay.sh : 0;
     // paged: where the event's pages start, looked up once by as many lanes of every warp at the same time (the block table's
     // entries come from L2; looked up row by row and copy by copy: 16 384 events of 256 rows to 128 in pages of 64 1631 us, 1600 so,

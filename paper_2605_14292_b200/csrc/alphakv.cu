@@ -366,10 +366,12 @@ static akv_status_t launch_tri(akv_handle* h, const EventArgs& a, cudaStream_t s
             return launch(paged ? event_pool_kernel<FUSED, kPoolWideForm, true> : event_pool_kernel<FUSED, kPoolWideForm, false>,
                           plan_pool_event_smem<kPoolWideForm>(a.lay.N, a.budget, paged).total, kPoolWide);
         // Four events to an SM where three would not hold the call, as long as the loop hardly ever looks beyond the 158 rows that they have
-        // room for: with weak penalties, or budgets that leave room for strong ones. Us per call, three / four: 560 events of 256 rows to
-        // 128 75.8 / 64.5, 4096 of 180 to 70 250 / 229, of 256 to 128 at lambda 0.25 352 / 326, with near-duplicates at 0.5 403 / 385, at 0.75
-        // 363 / 393, at 1.0 363 / 655, 4096 to 96 at 1.0 325 / 269, to 80 307 / 262; 444 of 256 to 100 52.3 / 56.5, 336 51.3 / 51.4; top-k 201 / 206.
-        if (E > 3 * h->sm_count && a.greedy && (a.lam <= 0.5f || (a.lam <= 1.f && a.budget <= 96)))
+        // room for, which budgets of at most 96 leave it. Us per call, three / four: 4096 events of 180 rows to 70 250 / 229, of 256 to 96 at
+        // lambda 1.0 325 / 269, to 80 307 / 262; 444 of 256 to 100 52.3 / 56.5, 336 51.3 / 51.4; top-k 201 / 206. Not for larger budgets, although
+        // random rows gain (16 384 of 256 to 128 at lambda 0.5 1598 / 1479): where a cache holds many values twice the picks go deeper, and the
+        // decode cadence whose appended rows repeat takes 70.8 ms instead of 52.7 for 32 rounds.
+        // (With a shared matrix the rows left out cost little: any budget, 222 / 198.)
+        if (E > 3 * h->sm_count && a.greedy && (a.gram ? a.lam <= 0.5f : a.lam <= 1.f && a.budget <= 96))
             return launch(paged ? event_pool_kernel<FUSED, kPoolFour, true> : event_pool_kernel<FUSED, kPoolFour, false>,
                           plan_pool_event_smem<kPoolFour>(a.lay.N, a.budget, paged).total, kTcThreads);
         return launch(paged ? event_pool_kernel<FUSED, kPoolThree, true> : event_pool_kernel<FUSED, kPoolThree, false>,

@@ -372,10 +372,10 @@ def in_pairs(ev, seed):
 
 
 @pytest.mark.parametrize("N,budget,lam", [(129, 20, 0.5), (144, 64, 1.0), (160, 128, 0.5), (192, 64, 0.0), (250, 33, 1.0), (255, 65, 0.0),
-                                          (256, 64, 0.5), (256, 128, 0.5), (256, 128, 2.0), (192, 70, 0.5), (193, 71, 0.25), (224, 128, 0.5)])
+                                          (256, 64, 0.5), (256, 128, 0.5), (256, 128, 2.0), (192, 70, 0.5), (193, 71, 1.0), (256, 96, 0.5)])
 def test_events_with_an_sm_each_and_several_to_an_sm(N, budget, lam):
     """bf16, d = 128: calls of no more events than SMs take the kernel of eight warps, others those of four, three or four (more than
-    three per SM, no strong penalty) of them to an SM; all against the oracle, with all candidates, ragged counts and when their waits
+    three per SM, budgets of at most 96) of them to an SM; all against the oracle, with all candidates, ragged counts and when their waits
     run out."""
     few = in_pairs(synth.make_plain(2, 1, 3, N, 128, budget, lam, dtype=synth.BF16, seed=N + budget), N)
     sms = torch.cuda.get_device_properties(0).multi_processor_count
