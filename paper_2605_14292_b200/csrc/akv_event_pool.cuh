@@ -86,13 +86,14 @@ __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kC
     // row addressing: dense events are one base offset plus a row stride
     const bool dense = PAGED && FORM == kPoolThree ? lay.page_size == 0 : !PAGED;   // (see above: three events per SM, in pages)
     const long long ev_off = dense ? id.b * lay.sb + id.l * lay.sl + id.h * lay.sh : 0;
-    // paged: where the event's pages start, looked up once by as many lanes of every warp at the same time (the block table's
+    // paged: where the event's pages start, looked up once by as many lanes of warp 0 at the same time (the block table's
     // entries come from L2; looked up row by row and copy by copy: 16 384 events of 256 rows to 128 in pages of 64 1631 us, 1600 so,
-    // 8192 in pages of 16 798 and 771)
+    // 8192 in pages of 16 798 and 771). The other warps read them behind the next block-wide barrier.
     long long* page_off = reinterpret_cast<long long*>(smem + sp.pages);
-    const bool few_pages = !dense && ((N - 1) >> lay.page_shift) < kPageOffsets;
+    const int pages = dense ? 0 : event_pages(N, lay.page_shift);
+    const bool few_pages = !dense && pages <= kPageOffsets;
     if (few_pages) {
-        if (tid < kPageOffsets && (tid << lay.page_shift) < N) page_off[tid] = row_offset(lay, id.b, id.l, id.h, tid << lay.page_shift);
+        if (tid < pages) page_off[tid] = row_offset(lay, id.b, id.l, id.h, tid << lay.page_shift);
         __syncwarp();
     }
     auto rowoff = [&](int j) -> long long {

@@ -24,6 +24,7 @@
 #pragma once
 #include "akv_active_set.cuh"
 #include "akv_event_tc.cuh"
+#include "akv_pages.cuh"
 
 namespace akv {
 
@@ -753,12 +754,14 @@ __global__ void __launch_bounds__(kTcThreads) event_tri_kernel(const __grid_cons
     // row addressing: dense events are one base offset plus a row stride
     const bool dense = !PAGED && lay.page_size == 0;
     const long long ev_off = dense ? id.b * lay.sb + id.l * lay.sl + id.h * lay.sh : 0;
-    // paged: where the event's pages start, looked up once by as many lanes at the same time (the block table's entries come from L2;
-    // looked up row by row and copy by copy: 4096 events of 192 rows to 64 in pages of 64 191 us, 182 so)
+    // paged: where the event's pages start, looked up once by as many lanes of warp 0 at the same time (the block table's entries come from L2;
+    // looked up row by row and copy by copy: 4096 events of 192 rows to 64 in pages of 64 191 us, 182 so). The other warps read
+    // them behind the next block-wide barrier.
     long long* page_off = reinterpret_cast<long long*>(smem + sp.pages);
-    const bool few_pages = PAGED && ((N - 1) >> lay.page_shift) < kPageOffsets;
+    const int pages = PAGED ? event_pages(N, lay.page_shift) : 0;
+    const bool few_pages = PAGED && pages <= kPageOffsets;
     if (PAGED && few_pages) {
-        if (tid < kPageOffsets && (tid << lay.page_shift) < N) page_off[tid] = row_offset(lay, id.b, id.l, id.h, tid << lay.page_shift);
+        if (tid < pages) page_off[tid] = row_offset(lay, id.b, id.l, id.h, tid << lay.page_shift);
         __syncwarp();
     }
     auto rowoff = [&](int j) -> long long {

@@ -418,6 +418,27 @@ def test_pages_on_both_sides_of_those_whose_offsets_are_kept(page, N, budget):
             assert np.array_equal(akv.to_host_bits(rows[..., :N, :].contiguous()), plain[name]), name
 
 
+@pytest.mark.parametrize("shift", [28, 29, 30])
+@pytest.mark.parametrize("N,budget", [(100, 40), (192, 64), (256, 128), (256, 140)])
+def test_one_page_that_could_hold_far_more_slots_than_the_event_has(N, budget, shift):
+    """A whole sequence in one page, whose size is stated as up to 2^30 slots; against the same rows in a dense cache, to the bit."""
+    for B in (2, 80):
+        ev = synth.make_plain(B, 2, 2, N, 128, budget, 0.5, dtype=synth.BF16, seed=N)
+        plain = run_fused(ev)
+        table = torch.randperm(B, device="cuda").to(torch.int32).view(B, 1)
+        pools = [torch.empty((2, B, 2, N, 128), dtype=torch.bfloat16, device="cuda") for _ in "KV"]
+        for pool, x in zip(pools, (dev(ev.K), dev(ev.V))):
+            pool[:, table.long().flatten()] = x.transpose(0, 1)
+        sl, sp, sh, sn, _ = pools[0].stride()
+        lay = akv.Layout(B, 2, 2, N, 128, synth.BF16, (0, sl, 0, 0), 1 << shift, table, (sp, sh, sn))
+        pos = dev(ev.pos)
+        sel = akv.alpha_compress_event(pools[0], pools[1], pos, dev(ev.qstat), budget, akv.Options(lam=0.5), p_ref=dev(ev.p_ref), layout=lay)
+        assert np.array_equal(sel.pick_order.cpu().numpy(), plain["order"]) and np.array_equal(sel.pick_gain.cpu().numpy(), plain["gain"])
+        assert np.array_equal(pos.cpu().numpy(), plain["pos"])
+        for pool, name in zip(pools, "KV"):
+            assert np.array_equal(akv.to_host_bits(pool[:, table.long().flatten()].transpose(0, 1).contiguous()), plain[name]), name
+
+
 @pytest.mark.parametrize("N,budget", [(2, 2), (3, 2), (33, 33), (64, 40), (128, 128), (129, 90), (192, 64), (256, 100)])
 @pytest.mark.parametrize("lam", [0.5, 2.0])
 def test_resident_kernel_picks_in_pairs(N, budget, lam):
