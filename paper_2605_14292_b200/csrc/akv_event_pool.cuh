@@ -30,11 +30,12 @@ __device__ __forceinline__ void bulk_store_wait_read() {
 
 // FUSED: score + select + compact; otherwise selection only (scores are read from a.scores and
 // nothing is rewritten).
-// FORM (PoolShape): kPoolWideForm, eight warps for an event that has an SM to itself (a call of no more events than SMs; also what
-// event_tri_kernel takes, from 129 rows on). Alone on its SM an event is a chain of phases that too few warps hide: of 256
+// FORM (PoolShape): kPoolWideForm, eight warps for an event that has an SM to itself (a call of no more events than SMs). Alone on
+// its SM an event is a chain of phases that too few warps hide: of 256
 // rows to 128, 55.2 -> 49.0 thousand cycles (scores 12.5 -> 10.4, picks in pairs 24.7 -> 22.5, triangle 3.2 -> 2.6, compaction 5.1 -> 4.4);
-// 112 of them 34.7 -> 31.2 us, in pages 39.1 -> 36.5, top-k 22.6 -> 18.5; of 192 rows to 64 (before: event_tri_kernel) 22.6 -> 22.0, of
-// 256 to 64 in pages 29.3 -> 26.8, but of 100 to 32 16.8 -> 17.1. kPoolThree, four warps and three events per SM; kPoolFour, four events
+// 112 of them 34.7 -> 31.2 us, in pages 39.1 -> 36.5, top-k 22.6 -> 18.5. Not for what event_tri_kernel takes: alone, 112 events of 192 rows
+// to 64 gain 2 us of 27 (in pages 4 of 29), but that kernel has six events on an SM, and four streams with such a call each take 41 us there, 50 here
+// (in pages 43 and 80). kPoolThree, four warps and three events per SM; kPoolFour, four events
 // per SM: latency bounds a call of many events (34 % of the issue slots used), so what counts is how many an SM holds. For that the last
 // 64 K rows come late, the triangle has 158 rows and the last kept V rows wait in registers: 16 384 events of 256 rows to 128 in
 // pages 1598 -> 1479 us (launch_tri says which calls). PAGED: with the layout known to the compiler, and 16 to 40 registers
@@ -291,8 +292,7 @@ __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kC
 
     phase_stamp(id.e, 2);
     // ---- s_(b) by bisection over the score keys, then the pool in slot order (warp 0) -------------
-    // (a pool that budgets of at most 64 have: 127 rows, so that the loop has four candidates per lane)
-    const int most = WIDE && a.budget <= 64 ? kTriMaxPool : Shape::kActive;
+    constexpr int most = Shape::kActive;
     if constexpr (WIDE) {
         // A key per thread, counts by the barrier itself: a bit per round. (One warp with eight keys per lane: 3.7 thousand cycles
         // of an event, these 3.3.)

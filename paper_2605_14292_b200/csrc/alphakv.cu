@@ -349,8 +349,6 @@ static bool pool_shared_ok(const EventArgs& a) {
 template <bool FUSED, bool BIG>
 static akv_status_t launch_tri(akv_handle* h, const EventArgs& a, cudaStream_t st, bool dry = false) {
     const int E = a.lay.B * a.lay.L * a.lay.H;
-    if constexpr (!BIG)   // an SM for every event: the large kernel's eight warps (see there; events of up to 128 rows gain nothing)
-        if (E <= h->sm_count && a.lay.N > 128) return launch_tri<FUSED, true>(h, a, st, dry);
     akv_status_t s;
     if constexpr (BIG) {
         auto launch = [&](auto kernel, unsigned bytes, int threads) -> akv_status_t {

@@ -1,4 +1,5 @@
 """GPU-vs-oracle parity, through the C ABI (via the thin binding), element by element."""
+import copy
 import os
 import re
 
@@ -391,6 +392,41 @@ def test_events_with_an_sm_each_and_several_to_an_sm(N, budget, lam):
         check_all(ev, run_fused(ev, n_cand=n_cand), lam, events=events, n_cand=n_cand)
         g = run_fused(ev, flags=akv.FLAG_TEST_STARVE_WAIT)
         assert np.all(g["status"] == 3) and np.array_equal(g["K"], ev.K) and np.array_equal(g["V"], ev.V) and np.array_equal(g["pos"], ev.pos)
+
+
+def tiled(ev, times):
+    """The same events `times` over, as one call of more sequences."""
+    big = copy.copy(ev)
+    for name in ("K", "V", "pos", "p_ref"):
+        x = getattr(ev, name)
+        setattr(big, name, np.tile(x, (times,) + (1,) * (x.ndim - 1)))
+    return big
+
+
+def beyond_one_and_three_per_sm(events):
+    """How often a call of so many events has to be repeated for more events than SMs, and for more than three per SM."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return sms // events + 1, 3 * sms // events + 1
+
+
+def same_bits(few, many):
+    """The results of a call against those of its events many times over."""
+    for k, x in few.items():
+        x, y = np.ascontiguousarray(x), np.ascontiguousarray(many[k])
+        same = (y.view(np.uint8).reshape(-1, x.nbytes) == x.view(np.uint8).reshape(1, -1)).all(1)
+        assert same.all(), f"{k}: {int((~same).sum())} of {same.size} copies differ"
+
+
+@pytest.mark.parametrize("N,budget,lam", [(100, 40, 0.5), (128, 128, 0.5), (129, 20, 0.5), (160, 64, 1.0), (192, 64, 0.0), (192, 64, 0.5), (256, 64, 2.0)])
+@pytest.mark.parametrize("regular", [True, False])
+def test_an_event_has_the_same_bits_in_every_call(N, budget, lam, regular):
+    """bf16, d = 128: scores, picks, gains and kept rows of an event do not depend on how many other events the call has."""
+    ev = synth.make_c3(seed=N, B=1, L=2, H=3, N=N, budget=budget)
+    if not regular:
+        ev = in_pairs(ev, N)
+    few = run_fused(ev, lam=lam)
+    for times in beyond_one_and_three_per_sm(6):
+        same_bits(few, run_fused(tiled(ev, times), lam=lam))
 
 
 @pytest.mark.parametrize("page,N,budget", [(16, 256, 128), (16, 250, 64), (16, 241, 100), (8, 128, 40), (8, 130, 64), (8, 256, 128), (256, 131, 70)])
