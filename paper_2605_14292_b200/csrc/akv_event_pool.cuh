@@ -15,6 +15,7 @@
 //   cosines against one another; their cosines against rows < 128 are those rows' columns 128.. by symmetry.
 #pragma once
 #include "akv_event_tri.cuh"
+#include "akv_score_order.cuh"
 
 namespace akv {
 
@@ -79,7 +80,9 @@ __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kC
     const uint32_t tile_u32 = smem_u32(tile);
     constexpr uint32_t half_bytes = Shape::kOperandRows * 128u;  // the operand's two 128-byte column halves
     const uint32_t barL = barK + 48;  // K rows that wait for a free slot
-    const int n_late = FOUR && FUSED && n > Shape::kRows ? n - Shape::kRows : 0;
+    const int steps = score_steps(n), second = 16 * steps;   // the second chain's first row
+    const int late0 = 16 * (steps - kLateSteps);             // of a chain's rows, the first that comes late
+    const int n_late = FOUR && FUSED && n > Shape::kRows ? n - 2 * late0 : 0;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool similarity = a.greedy != 0 && picks > 1;   // (the first pick is the highest score in any case)
@@ -114,11 +117,10 @@ __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kC
     // when its rows are contiguous, whole pages when pages are, else row by row), all issued by one
     // thread (a bulk copy is a per-warp instruction)
     auto request_k_rows = [&](int r0, int r1, int slot0, uint32_t bar) {
-        mbar_expect_tx(bar, (uint32_t)(r1 - r0) * 256u);
         for (int row = r0; row < r1 && !a.starve;) {  // starve (testing aid): nothing is requested, the waits run out
             int run = 1;
             if (dense && lay.sn == kTcD) run = min(r1 - row, 128);
-            else if (!dense && lay.s_page_n == kTcD) run = min(r1 - row, lay.page_size - row % lay.page_size);
+            else if (!dense && lay.s_page_n == kTcD) run = min(r1 - row, lay.page_size - (row & (lay.page_size - 1)));
             bulk_g2s(tile_u32 + (uint32_t)(slot0 + row - r0) * 256u, Kg + rowoff(row), (uint32_t)run * 256u, bar);
             row += run;
         }
@@ -129,7 +131,15 @@ __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kC
         if (FOUR) mbar_init(barL, 1);
         mbar_init_fence();
         // the K rows are asked for before anything else: the wait for tensor memory below overlaps their flight
-        if (FUSED) request_k_rows(0, n - n_late, 0, barK);
+        if (FUSED) {
+            mbar_expect_tx(barK, (uint32_t)(n - n_late) * 256u);
+            if (n_late > 0) {
+                request_k_rows(0, late0, 0, barK);
+                request_k_rows(second, second + late0, kChainSlots, barK);
+            } else {
+                request_k_rows(0, n, 0, barK);
+            }
+        }
     }
     if (FUSED && warp == 1) fill_sector_table(sect, lane);
     // (this kernel claims half of the SM's columns: two of the three resident CTAs hold theirs at a time, the
@@ -183,64 +193,67 @@ __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kC
         }
         // lane covers frequencies f0..f0+7 of the row handled by its group of eight lanes
         const int grp = lane >> 3, f0 = (lane & 7) * 8;
-        // spacing of rows kRound (16 or 32) slots apart at the newest end of the event: what a token-by-token cache has everywhere
-        constexpr int kRound = FOUR ? 8 * NW : 4 * NW;
-        const long long step = n > kRound ? (long long)spos[n - 1] - (long long)spos[n - 1 - kRound] : 0;
+        // spacing of rows 16 slots apart at the newest end of the event: what a token-by-token cache has everywhere
+        const long long D16 = n > 16 ? (long long)spos[n - 1] - (long long)spos[n - 17] : 0;
         ChainScore cs;
-        cs.set_step(step, phitab + f0, sect);
-        // whether every row sits step after the row kRound slots before it (found once; the chains then need no look at
+        cs.set_step(D16, phitab + f0, sect);
+        // whether every row sits D16 after the row 16 slots before it (found once; the chains then need no look at
         // the positions)
         bool uni = true;
-        for (int j = kRound + tid; j < n; j += NT) uni &= (long long)spos[j] - (long long)spos[j - kRound] == step;
+        for (int j = 16 + tid; j < n; j += NT) uni &= (long long)spos[j] - (long long)spos[j - 16] == D16;
         const bool uniform = __syncthreads_and(uni);
-        const int rounds = (n + kRound - 1) / kRound;
+        // A lane group scores two rows side by side, so that one's dependent arithmetic fills the other's latency: a row of each chain (see
+        // score_steps), or, with four of the eight warps on a chain each, a row and the next one of the same chain.
+        const int row = 4 * (warp & 3) + grp;
+        auto spaced = [&](int j) { return j >= n || (long long)spos[j] - (long long)spos[j - 16] == D16; };
         timeout = !mbar_wait_bounded(barK, 0, a.wait_polls);
         phase_stamp(id.e, 10);  // (K rows have arrived)
         {
-            // The tile holds the whole event. A lane group scores two rows side by side, row j of the first half
-            // of the rounds and row j + kRound * half of the second: two independent chains that share the turn S, so
-            // that one chain's dependent arithmetic fills the other's latency.
-            // (four CTAs per SM: rows 16 slots apart instead, in order, so that the slots of the first 64 are free early for the late rows)
-            const int half = FOUR ? rounds : (rounds + 1) >> 1;
             ChainScore cb;
             AKV_PHASE_ACC_DECL(cyc_anchor);
 #pragma unroll 1
-            for (int round = 0; round < half; ++round) {
-                const int ja = kRound * round + 4 * warp + grp, jb = FOUR ? ja + 16 : ja + kRound * half;
-                const bool la = ja < n, lb = jb < n;
+            for (int i = 0; i < steps; i += WIDE ? 2 : 1) {
+                const int ja = 16 * i + row + (WIDE ? (warp >> 2) * second : 0), jb = ja + (WIDE ? 16 : second);
+                const bool la = ja < n, lb = jb < n && (!WIDE || i + 1 < steps);
                 if (FOUR && n_late > 0) {
-                    if (round == 2) {   // rows 0..63 have been scored
+                    if (i == kLateSteps) {   // the slots are free
                         __syncthreads();
-                        if (tid == 0) request_k_rows(Shape::kRows, n, 0, barL);
+                        if (tid == 0) {
+                            mbar_expect_tx(barL, (uint32_t)n_late * 256u);
+                            request_k_rows(late0, second, 0, barL);
+                            request_k_rows(second + late0, n, kChainSlots, barL);
+                        }
                     }
-                    if (round == Shape::kRows / 32) timeout |= !mbar_wait_bounded(barL, 0, a.wait_polls);
+                    if (i == steps - kLateSteps) timeout |= !mbar_wait_bounded(barL, 0, a.wait_polls);
                 }
                 // each chain on its own: after an event the kept rows' positions are irregular (fresh rotation every
-                // round) while the rows appended since are consecutive (chained)
-                bool fa = round == 0 || a.no_chain, fb = fa;
-                if (!fa && !uniform) {
-                    fa = !__all_sync(0xFFFFFFFFu, !la || (long long)spos[ja] - (long long)spos[ja - kRound] == step);
-                    fb = !__all_sync(0xFFFFFFFFu, !lb || (long long)spos[jb] - (long long)spos[jb - kRound] == step);
+                // step) while the rows appended since are consecutive (chained)
+                bool fa = i == 0 || a.no_chain, fb = WIDE ? a.no_chain != 0 : fa;
+                if (!(WIDE ? fb : fa) && !uniform) {
+                    if (!WIDE || i > 0) fa = !__all_sync(0xFFFFFFFFu, spaced(ja));
+                    fb = !__all_sync(0xFFFFFFFFu, spaced(jb));
                 }
                 AKV_PHASE_ACC_BEGIN(cyc_anchor);
                 if (fa) {
                     if (la) cs.anchor(pref - (long long)spos[ja], gtab + f0, phitab + f0, sect);
                 } else {
+                    if (WIDE) cs.turn_to(cb);
                     cs.advance();
                 }
                 if (fb) {
                     if (lb) cb.anchor(pref - (long long)spos[jb], gtab + f0, phitab + f0, sect);
                 } else {
+                    if (WIDE) cb.turn_to(cs);
                     cb.advance_by(cs);
                 }
                 AKV_PHASE_ACC_END(cyc_anchor);
                 float acca = 0.f, accb = 0.f;
                 if (la) {
-                    const unsigned char* krow = tile + (FOUR && ja >= Shape::kRows ? ja - Shape::kRows : ja) * 256 + (lane & 7) * 16;
+                    const unsigned char* krow = tile + (FOUR && n_late > 0 ? ja + late_slot_shift(i, steps, 0) : ja) * 256 + (lane & 7) * 16;
                     acca = cs.dot(*reinterpret_cast<const uint4*>(krow), *reinterpret_cast<const uint4*>(krow + 128));
                 }
                 if (lb) {
-                    const unsigned char* krow = tile + (FOUR && jb >= Shape::kRows ? jb - Shape::kRows : jb) * 256 + (lane & 7) * 16;
+                    const unsigned char* krow = tile + (FOUR && n_late > 0 ? jb + late_slot_shift(i, steps, 1) : jb) * 256 + (lane & 7) * 16;
                     accb = cb.dot(*reinterpret_cast<const uint4*>(krow), *reinterpret_cast<const uint4*>(krow + 128));
                 }
 #pragma unroll
@@ -253,7 +266,7 @@ __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kC
                     for (int h = 0; h < 2; ++h) {
                         const int j = h ? jb : ja;
                         const float acc = h ? accb : acca;
-                        if (j < n) {
+                        if (h ? lb : la) {
                             if (a.scores) a.scores[(long long)id.e * N + j] = acc;
                             const bool fin = isfinite(acc);
                             bad |= !fin;
@@ -288,11 +301,10 @@ __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kC
     }
     bad = __syncthreads_or(bad);
     // (only now: while scoring, this storage holds the statistic's table, which slower warps may still read)
-    if (tid < 8) kept[tid] = 0u;
+    if (!WIDE && tid < 8) kept[tid] = 0u;
 
     phase_stamp(id.e, 2);
     // ---- s_(b) by bisection over the score keys, then the pool in slot order (warp 0) -------------
-    constexpr int most = Shape::kActive;
     if constexpr (WIDE) {
         // A key per thread, counts by the barrier itself: a bit per round. (One warp with eight keys per lane: 3.7 thousand cycles
         // of an event, these 3.3.)
@@ -305,8 +317,8 @@ __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kC
         const float thr = a.no_prune || kb < 0x00800000u ? -INFINITY : fmaf(-1.001f, a.lam, sb) - 1e-6f * fabsf(sb);
         const bool pooled = kj != 0u && !(from_orderable(kj) < thr);
         ActiveBound bound{0u, 0};
-        if (similarity && __syncthreads_count(pooled) > most)
-            bound = active_bound(orderable(thr), kb, most, most + 1, most - most / 8, [&](uint32_t v1, uint32_t v2, uint32_t v3, int& c1, int& c2, int& c3) {
+        if (similarity && __syncthreads_count(pooled) > a.active)
+            bound = active_bound(orderable(thr), kb, a.active, a.active + 1, a.active - a.active / 8, [&](uint32_t v1, uint32_t v2, uint32_t v3, int& c1, int& c2, int& c3) {
                 c1 = __syncthreads_count(kj >= v1);
                 c2 = __syncthreads_count(kj >= v2);
                 c3 = __syncthreads_count(kj >= v3);
@@ -367,7 +379,7 @@ __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kC
         const float sb = from_orderable(kb);
         // -inf keeps everyone (also where kb, whose low bits are open, is below every finite value's key)
         const float thr = a.no_prune || kb < 0x00800000u ? -INFINITY : fmaf(-1.001f, a.lam, sb) - 1e-6f * fabsf(sb);
-        // Active set: the pool's best-scored rows, at most Shape::kActive of them; no key left out is above bound.key (0: none
+        // Active set: the pool's best-scored rows, at most a.active of them; no key left out is above bound.key (0: none
         // is left out). A candidate's Eq. 2 value never exceeds its score: the loop over the active set is exact as long as
         // its winning value stays above the bound (it nearly always does: with lambda = 0.5 the picks reach a few ranks
         // beyond the budget).
@@ -377,7 +389,7 @@ __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kC
 #pragma unroll
             for (int k = 0; k < 8; ++k) pool_size += kk[k] != 0u && !(from_orderable(kk[k]) < thr);
             pool_size = __reduce_add_sync(0xFFFFFFFFu, pool_size);
-            if (pool_size > Shape::kActive) bound = warp_active_bound(kk, orderable(thr), kb, Shape::kActive);
+            if (pool_size > a.active) bound = warp_active_bound(kk, orderable(thr), kb, a.active);
         }
         int base = 0;
         if (lane == 0) *tie_holder = 0;
@@ -662,7 +674,7 @@ __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kC
         if (runs) {
             if (tid == 0) {
                 for (int row = 0; row < picks;) {
-                    const int run = dense ? picks - row : min(picks - row, lay.page_size - row % lay.page_size);
+                    const int run = dense ? picks - row : min(picks - row, lay.page_size - (row & (lay.page_size - 1)));
                     const long long off = rowoff(row);
                     const int vrun = min(run, fit - row);
                     bulk_s2g(Kg + off, tile_u32 + (uint32_t)row * 256u, (uint32_t)run * 256u);

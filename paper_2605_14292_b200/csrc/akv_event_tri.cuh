@@ -73,7 +73,7 @@ struct PoolShape {
 };
 template <>
 struct PoolShape<kPoolFour> {
-    // 192 K rows (the others arrive in the slots of the first), then the triangle of up to 158 rows; four CTAs per SM: 57 312 bytes for
+    // 192 K rows (the others arrive in the slots of the first, see late_slot_shift), then the triangle of up to 158 rows; four CTAs per SM: 57 312 bytes for
     // 256 rows in pages to 128, of the 57 344 that four leave each
     static constexpr int kThreads = kTcThreads, kCtas = 4;
     static constexpr unsigned kTile = 50688u;
@@ -783,7 +783,7 @@ __global__ void __launch_bounds__(kTcThreads) event_tri_kernel(const __grid_cons
         for (int row = r0; row < r1 && !a.starve;) {  // starve (testing aid): nothing is requested, the waits run out
             int run = 1;
             if (dense && lay.sn == kTcD) run = min(r1 - row, 128);
-            else if (!dense && lay.s_page_n == kTcD) run = min(r1 - row, lay.page_size - row % lay.page_size);
+            else if (!dense && lay.s_page_n == kTcD) run = min(r1 - row, lay.page_size - (row & (lay.page_size - 1)));
             bulk_g2s(tile_u32 + (uint32_t)(slot0 + row - r0) * 256u, Kg + rowoff(row), (uint32_t)run * 256u, bar);
             row += run;
         }

@@ -27,6 +27,7 @@ struct EventArgs {
     int gqa_max;            // 1: a key's score is the largest over the group, 0: their mean
     int starve;             // testing aid: request no K row and, where there is no K to read, issue no product, so that the bounded waits run out
     int wait_polls;         // polls after which a bounded wait gives up
+    int active;             // event_pool_kernel: most rows of an active set
     int first_event;        // prefill kernel: the first event of the second of two launches
     int* idx_sorted;
     int* pick_order;

@@ -69,6 +69,11 @@ struct ChainScore {
             Gx[p] = nx; Gy[p] = ny;
         }
     }
+    // the row that another state is at
+    __device__ __forceinline__ void turn_to(const ChainScore& o) {
+#pragma unroll
+        for (int p = 0; p < 4; ++p) { Gx[p] = o.Gx[p]; Gy[p] = o.Gy[p]; }
+    }
     // the lane's partial sum of Re(G conj(k)) over its 8 frequencies
     __device__ __forceinline__ float dot(const uint4& wr, const uint4& wi) const {
         const uint32_t wre[4] = {wr.x, wr.y, wr.z, wr.w}, wim[4] = {wi.x, wi.y, wi.z, wi.w};

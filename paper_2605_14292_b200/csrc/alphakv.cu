@@ -346,11 +346,16 @@ static bool tri_big_ok(const EventArgs& a) { return tc_path_ok(a) && !tri_path_o
 static bool pool_shared_ok(const EventArgs& a) {
     return a.gram != nullptr && a.lay.dtype == AKV_BF16 && a.lay.d == kTcD && a.lay.N <= kTcMaxN && a.budget <= 128 && !a.gqa_max;
 }
+// Calls that four events per SM may take: where the loop hardly ever looks beyond the 158 rows that those have room for.
+static bool pool_four_ok(const EventArgs& a) { return a.greedy && (a.gram ? a.lam <= 0.5f : a.lam <= 1.f && a.budget <= 96); }
 template <bool FUSED, bool BIG>
-static akv_status_t launch_tri(akv_handle* h, const EventArgs& a, cudaStream_t st, bool dry = false) {
+static akv_status_t launch_tri(akv_handle* h, const EventArgs& a0, cudaStream_t st, bool dry = false) {
+    EventArgs a = a0;
     const int E = a.lay.B * a.lay.L * a.lay.H;
     akv_status_t s;
     if constexpr (BIG) {
+        // (by the options alone: an event's active set is the same however many others the call has)
+        a.active = pool_four_ok(a) ? PoolShape<kPoolFour>::kActive : PoolShape<kPoolThree>::kActive;
         auto launch = [&](auto kernel, unsigned bytes, int threads) -> akv_status_t {
             if ((int)bytes > h->smem_optin) return fail(AKV_ERR_UNSUPPORTED, "budget %d needs too much shared memory", a.budget);
             if ((s = set_smem(h, kernel, bytes)) != AKV_OK) return s;
@@ -369,7 +374,7 @@ static akv_status_t launch_tri(akv_handle* h, const EventArgs& a, cudaStream_t s
         // random rows gain (16 384 of 256 to 128 at lambda 0.5 1598 / 1479): where a cache holds many values twice the picks go deeper, and the
         // decode cadence whose appended rows repeat takes 70.8 ms instead of 52.7 for 32 rounds.
         // (With a shared matrix the rows left out cost little: any budget, 222 / 198.)
-        if (E > 3 * h->sm_count && a.greedy && (a.gram ? a.lam <= 0.5f : a.lam <= 1.f && a.budget <= 96))
+        if (E > 3 * h->sm_count && pool_four_ok(a))
             return launch(paged ? event_pool_kernel<FUSED, kPoolFour, true> : event_pool_kernel<FUSED, kPoolFour, false>,
                           plan_pool_event_smem<kPoolFour>(a.lay.N, a.budget, paged).total, kTcThreads);
         return launch(paged ? event_pool_kernel<FUSED, kPoolThree, true> : event_pool_kernel<FUSED, kPoolThree, false>,

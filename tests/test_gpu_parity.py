@@ -417,16 +417,43 @@ def same_bits(few, many):
         assert same.all(), f"{k}: {int((~same).sum())} of {same.size} copies differ"
 
 
-@pytest.mark.parametrize("N,budget,lam", [(100, 40, 0.5), (128, 128, 0.5), (129, 20, 0.5), (160, 64, 1.0), (192, 64, 0.0), (192, 64, 0.5), (256, 64, 2.0)])
+@pytest.mark.parametrize("N,budget,lam", [(100, 40, 0.5), (128, 128, 0.5), (129, 20, 0.5), (160, 64, 1.0), (192, 64, 0.0), (192, 64, 0.5), (256, 64, 2.0),
+                                          (129, 100, 0.5), (144, 70, 1.0), (176, 96, 0.5), (193, 90, 0.5), (208, 128, 1.0), (224, 96, 1.0), (225, 65, 0.0),
+                                          (240, 80, 0.5), (241, 96, 2.0), (256, 96, 1.0), (256, 128, 0.0), (256, 128, 0.5), (256, 128, 2.0)])
 @pytest.mark.parametrize("regular", [True, False])
 def test_an_event_has_the_same_bits_in_every_call(N, budget, lam, regular):
     """bf16, d = 128: scores, picks, gains and kept rows of an event do not depend on how many other events the call has."""
-    ev = synth.make_c3(seed=N, B=1, L=2, H=3, N=N, budget=budget)
+    ev = synth.make_c3(seed=N, B=2, L=1, H=3, N=N, budget=budget)
     if not regular:
         ev = in_pairs(ev, N)
     few = run_fused(ev, lam=lam)
+    check_all(ev, few, lam)
     for times in beyond_one_and_three_per_sm(6):
         same_bits(few, run_fused(tiled(ev, times), lam=lam))
+    for n_cand in ([N, N // 2], [N - 17, N - 1]):
+        few = run_fused(ev, lam=lam, n_cand=n_cand)
+        for times in beyond_one_and_three_per_sm(6):
+            same_bits(few, run_fused(tiled(ev, times), lam=lam, n_cand=n_cand * times))
+
+
+@pytest.mark.parametrize("N,budget,lam", [(100, 40, 0.5), (192, 64, 0.5), (193, 90, 0.25), (256, 128, 0.5), (256, 128, 1.5)])
+@pytest.mark.parametrize("twice", [True, False])
+def test_an_event_has_the_same_bits_in_every_call_with_a_shared_matrix(N, budget, lam, twice):
+    ev = _duplicated_rows(N, lam, B=1, L=2, H=3, N=N // 2 * 2, budget=budget) if twice else synth.make_c3(seed=N, B=1, L=2, H=3, N=N, budget=budget)
+
+    def run(e):
+        K, V, pos = dev(e.K), dev(e.V), dev(e.pos)
+        sig = akv.alpha_signature_flat(V)
+        gram = akv.alpha_gram_shared(sig, akv.Layout.dense(V), akv.Options(sig_mode=akv.SIG_FLAT))
+        sel = akv.alpha_compress_event(K, V, pos, dev(e.qstat), budget, akv.Options(lam=lam, sig_mode=akv.SIG_FLAT, shared_gram=gram), p_ref=dev(e.p_ref),
+                                       flat_sig=sig, want_scores=True)
+        return dict(K=akv.to_host_bits(K), V=akv.to_host_bits(V), pos=pos.cpu().numpy(), idx=sel.idx_sorted.cpu().numpy(), order=sel.pick_order.cpu().numpy(),
+                    gain=sel.pick_gain.cpu().numpy(), scores=sel.scores.cpu().numpy(), n_kept=sel.n_kept.cpu().numpy(), status=sel.status.cpu().numpy())
+
+    few = run(ev)
+    assert few["status"].max() == 0
+    for times in beyond_one_and_three_per_sm(6):
+        same_bits(few, run(tiled(ev, times)))
 
 
 @pytest.mark.parametrize("page,N,budget", [(16, 256, 128), (16, 250, 64), (16, 241, 100), (8, 128, 40), (8, 130, 64), (8, 256, 128), (256, 131, 70)])
