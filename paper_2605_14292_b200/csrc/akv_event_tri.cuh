@@ -66,8 +66,10 @@ constexpr uint32_t kPoolCols = 256u;        // tensor-memory columns (a power of
 constexpr int kPoolWide = 256;              // threads of a CTA that has an SM to itself
 template <int FORM>
 struct PoolShape {
-    // a whole event's K rows, then the triangle of an active set of up to 180 rows; three CTAs per SM, or one of eight warps
-    static constexpr int kThreads = FORM == kPoolWideForm ? kPoolWide : kTcThreads, kCtas = FORM == kPoolWideForm ? 1 : 3;
+    // a whole event's K rows, then the triangle of an active set of up to 180 rows; three CTAs per SM, or two of eight warps (a call
+    // puts one on an SM, but calls in other streams come beside it: with registers for one only, two streams with 112 events of 256 rows
+    // to 128 in pages each took 63 us instead of 41, four 121 instead of 74; for three, one such call alone took 41 instead of 33)
+    static constexpr int kThreads = FORM == kPoolWideForm ? kPoolWide : kTcThreads, kCtas = FORM == kPoolWideForm ? 2 : 3;
     static constexpr unsigned kTile = 65536u;
     static constexpr int kActive = 180, kCpl = 6, kRows = 256, kOperandRows = 256;
 };
