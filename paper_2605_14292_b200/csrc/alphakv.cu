@@ -346,7 +346,10 @@ static bool tri_big_ok(const EventArgs& a) { return tc_path_ok(a) && !tri_path_o
 static bool pool_shared_ok(const EventArgs& a) {
     return a.gram != nullptr && a.lay.dtype == AKV_BF16 && a.lay.d == kTcD && a.lay.N <= kTcMaxN && a.budget <= 128 && !a.gqa_max;
 }
-// Calls that four events per SM may take: where the loop hardly ever looks beyond the 158 rows that those have room for.
+// Calls that four events per SM may take: where the loop hardly ever looks beyond the 158 rows that those have room for, which budgets of at most
+// 96 leave it. Not for larger ones, although random rows gain (16 384 events of 256 rows to 128 at lambda 0.5 1598 / 1479 us): where a
+// cache holds many values twice the picks go deeper, and the decode cadence whose appended rows repeat takes 70.8 ms instead of 52.7 for 32
+// rounds. With a shared matrix the rows left out cost little: any budget. Top-k gains nothing (4096 events of 256 rows to 96 201 / 206).
 static bool pool_four_ok(const EventArgs& a) { return a.greedy && (a.gram ? a.lam <= 0.5f : a.lam <= 1.f && a.budget <= 96); }
 template <bool FUSED, bool BIG>
 static akv_status_t launch_tri(akv_handle* h, const EventArgs& a0, cudaStream_t st, bool dry = false) {
@@ -368,13 +371,13 @@ static akv_status_t launch_tri(akv_handle* h, const EventArgs& a0, cudaStream_t 
         if (E <= h->sm_count)
             return launch(paged ? event_pool_kernel<FUSED, kPoolWideForm, true> : event_pool_kernel<FUSED, kPoolWideForm, false>,
                           plan_pool_event_smem<kPoolWideForm>(a.lay.N, a.budget, paged).total, kPoolWide);
-        // Four events to an SM where three would not hold the call, as long as the loop hardly ever looks beyond the 158 rows that they have
-        // room for, which budgets of at most 96 leave it. Us per call, three / four: 4096 events of 180 rows to 70 250 / 229, of 256 to 96 at
-        // lambda 1.0 325 / 269, to 80 307 / 262; 444 of 256 to 100 52.3 / 56.5, 336 51.3 / 51.4; top-k 201 / 206. Not for larger budgets, although
-        // random rows gain (16 384 of 256 to 128 at lambda 0.5 1598 / 1479): where a cache holds many values twice the picks go deeper, and the
-        // decode cadence whose appended rows repeat takes 70.8 ms instead of 52.7 for 32 rounds.
-        // (With a shared matrix the rows left out cost little: any budget, 222 / 198.)
-        if (E > 3 * h->sm_count && pool_four_ok(a))
+        // Four events to an SM where three would not hold the call, but for pages not up to five per SM when four do not hold it either: both then
+        // take two waves. Us per call, three / four per SM, 148 SMs: 444 events of 256 rows to 96 51.2 / 51.2, 460 63.6 / 53.3, 592 67.6 / 56.2, 660
+        // 68.5 / 68.5, 740 69.6 / 70.4, 744 79.9 / 71.7, 888 84.0 / 73.8, 4096 of 180 to 70 250 / 229; in pages of 64 460 67.6 / 57.4,
+        // 592 68.4 / 59.4, 594 68.7 / 78.5, 740 71.9 / 79.9, 744 82.7 / 80.6, 1184 103 / 101, 2368 198 / 181; with a shared matrix, of 256 to 128, 592
+        // 78.5 / 53.3, 700 82.0 / 80.6, 888 86.9 / 86.0, in pages 592 78.9 / 54.2, 740 82.9 / 84.8, 896 111 / 89, 2368 222 / 198.
+        const bool two_waves = paged && E > 4 * h->sm_count && E <= 5 * h->sm_count;
+        if (E > 3 * h->sm_count && !two_waves && pool_four_ok(a))
             return launch(paged ? event_pool_kernel<FUSED, kPoolFour, true> : event_pool_kernel<FUSED, kPoolFour, false>,
                           plan_pool_event_smem<kPoolFour>(a.lay.N, a.budget, paged).total, kTcThreads);
         return launch(paged ? event_pool_kernel<FUSED, kPoolThree, true> : event_pool_kernel<FUSED, kPoolThree, false>,
