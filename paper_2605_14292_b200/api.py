@@ -218,10 +218,19 @@ def _pos_strides(pos: Optional[torch.Tensor], lay: Layout):
     raise ValueError("pos must have 1, 2 or 4 dimensions")
 
 
+def _stream_getter():
+    """The current stream of a device as a number, without a Stream object around it; a torch without that function (it is not part
+    of its interface) gives the object."""
+    return getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
+_raw_stream = _stream_getter()
+
+
 def _call(entry: str, device: torch.device, *args):
     """One entry point on `device` and its current stream. The device is switched to only where it is another one."""
     if device.type == "cuda" and device.index == torch.cuda.current_device():
-        _check(getattr(load_library(), entry)(_handle(device), *args, torch._C._cuda_getCurrentRawStream(device.index)))
+        _check(getattr(load_library(), entry)(_handle(device), *args, _raw_stream(device.index)))
         return
     with torch.cuda.device(device):
         _check(getattr(load_library(), entry)(_handle(device), *args, torch.cuda.current_stream().cuda_stream))

@@ -3,8 +3,10 @@ and the host-side validation returns error codes without launching anything."""
 import ctypes as C
 import os
 import re
+from types import SimpleNamespace
 
 import pytest
+import torch
 
 import __graft_entry__ as entry
 from paper_2605_14292_b200 import api
@@ -62,3 +64,20 @@ def test_workspace_query_validates_before_it_touches_the_device(lib):
     assert lib.akv_workspace_bytes(C.byref(lay), 17, C.byref(opt), C.byref(out)) == 3 and out.value == 0
     assert b"budget" in lib.akv_last_error(None)
     assert lib.akv_workspace_bytes(None, 4, C.byref(opt), C.byref(out)) == 1
+
+
+def test_calls_take_the_current_stream_with_and_without_torchs_raw_function(monkeypatch):
+    """The function that gives a stream as a number is not part of torch's interface: where it is missing the Stream object gives it."""
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda index: SimpleNamespace(cuda_stream=700 + index))
+    monkeypatch.setattr(api, "_handle", lambda device: "handle")
+    for raw, stream in ((lambda index: 500 + index, 503), (None, 703)):
+        if raw is None:
+            monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+        else:
+            monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", raw, raising=False)
+        monkeypatch.setattr(api, "_raw_stream", api._stream_getter())
+        calls = []
+        monkeypatch.setattr(api, "load_library", lambda: SimpleNamespace(entry=lambda *args: calls.append(args) or 0))
+        api._call("entry", torch.device("cuda", 3), 1, 2)
+        assert calls == [("handle", 1, 2, stream)]
