@@ -29,7 +29,36 @@ def dev(x):
     return akv.to_device(x, "cuda")
 
 
-def run_fused(ev, lam=None, flags=0, n_cand=None, p_ref=True, W=None, budgets=None):
+def tiled(ev, times):
+    """The same events `times` over, as one call of more sequences."""
+    big = copy.copy(ev)
+    for name in ("K", "V", "pos", "p_ref"):
+        x = getattr(ev, name)
+        setattr(big, name, np.tile(x, (times,) + (1,) * (x.ndim - 1)))
+    return big
+
+
+def beyond_one_and_three_per_sm(events):
+    """How often a call of so many events has to be repeated for more events than SMs, and for more than three per SM."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return sms // events + 1, 3 * sms // events + 1
+
+
+def same_bits(few, many, keys=None):
+    """The results of a call against those of its events many times over."""
+    for k in keys or few:
+        x, y = np.ascontiguousarray(few[k]), np.ascontiguousarray(many[k])
+        same = (y.view(np.uint8).reshape(-1, x.nbytes) == x.view(np.uint8).reshape(1, -1)).all(1)
+        assert same.all(), f"{k}: {int((~same).sum())} of {same.size} copies differ"
+
+
+def takes_forms(ev):
+    """Shapes whose kernel (event_pool_kernel) has forms for one, three and four events per SM."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return ev.dtype == synth.BF16 and ev.shape[-1] == 128 and 128 < ev.shape[3] <= 256 and 64 < ev.budget <= 128 and ev.n_events <= sms
+
+
+def run_fused_once(ev, lam=None, flags=0, n_cand=None, p_ref=True, W=None, budgets=None):
     lam = ev.lam if lam is None else lam
     K, V, pos, q = dev(ev.K), dev(ev.V), dev(ev.pos), dev(ev.qstat)
     pref = dev(ev.p_ref) if p_ref else None
@@ -42,6 +71,17 @@ def run_fused(ev, lam=None, flags=0, n_cand=None, p_ref=True, W=None, budgets=No
     return dict(K=akv.to_host_bits(K), V=akv.to_host_bits(V), pos=pos.cpu().numpy(), idx=sel.idx_sorted.cpu().numpy(),
                 order=sel.pick_order.cpu().numpy(), gain=sel.pick_gain.cpu().numpy(), scores=sel.scores.cpu().numpy(),
                 n_kept=sel.n_kept.cpu().numpy(), status=sel.status.cpu().numpy())
+
+
+def run_fused(ev, lam=None, flags=0, n_cand=None, p_ref=True, W=None, budgets=None):
+    """The fused call on a copy of the events, as host arrays. Where the kernel's form depends on the number of events the call is also made with
+    the same events so often that the other forms take them: the results are the same to the bit."""
+    g = run_fused_once(ev, lam, flags, n_cand, p_ref, W, budgets)
+    if takes_forms(ev):
+        written = ("K", "V", "pos", "status") if flags & akv.FLAG_TEST_STARVE_WAIT else None
+        for times in beyond_one_and_three_per_sm(ev.n_events):
+            same_bits(g, run_fused_once(tiled(ev, times), lam, flags, None if n_cand is None else list(n_cand) * times, p_ref, W, budgets), written)
+    return g
 
 
 def check_all(ev, g, lam, events=None, n_cand=None, p_ref=True, W=None, threads=8, budgets=None):
@@ -375,9 +415,9 @@ def in_pairs(ev, seed):
 @pytest.mark.parametrize("N,budget,lam", [(129, 20, 0.5), (144, 64, 1.0), (160, 128, 0.5), (192, 64, 0.0), (250, 33, 1.0), (255, 65, 0.0),
                                           (256, 64, 0.5), (256, 128, 0.5), (256, 128, 2.0), (192, 70, 0.5), (193, 71, 1.0), (256, 96, 0.5)])
 def test_events_with_an_sm_each_and_several_to_an_sm(N, budget, lam):
-    """bf16, d = 128: calls of no more events than SMs take the kernel of eight warps, others those of four, three or four (more than
-    three per SM, budgets of at most 96) of them to an SM; all against the oracle, with all candidates, ragged counts and when their waits
-    run out."""
+    """bf16, d = 128, budgets beyond 64: calls of no more events than SMs take the form of eight warps, others those of four, three or four (more
+    than three per SM, budgets of at most 96) of them to an SM; smaller budgets one kernel. All against the oracle, with all candidates, ragged
+    counts and when their waits run out."""
     few = in_pairs(synth.make_plain(2, 1, 3, N, 128, budget, lam, dtype=synth.BF16, seed=N + budget), N)
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     for times in (1, sms // 6 + 1, 3 * sms // 6 + 1):
@@ -394,29 +434,6 @@ def test_events_with_an_sm_each_and_several_to_an_sm(N, budget, lam):
         assert np.all(g["status"] == 3) and np.array_equal(g["K"], ev.K) and np.array_equal(g["V"], ev.V) and np.array_equal(g["pos"], ev.pos)
 
 
-def tiled(ev, times):
-    """The same events `times` over, as one call of more sequences."""
-    big = copy.copy(ev)
-    for name in ("K", "V", "pos", "p_ref"):
-        x = getattr(ev, name)
-        setattr(big, name, np.tile(x, (times,) + (1,) * (x.ndim - 1)))
-    return big
-
-
-def beyond_one_and_three_per_sm(events):
-    """How often a call of so many events has to be repeated for more events than SMs, and for more than three per SM."""
-    sms = torch.cuda.get_device_properties(0).multi_processor_count
-    return sms // events + 1, 3 * sms // events + 1
-
-
-def same_bits(few, many):
-    """The results of a call against those of its events many times over."""
-    for k, x in few.items():
-        x, y = np.ascontiguousarray(x), np.ascontiguousarray(many[k])
-        same = (y.view(np.uint8).reshape(-1, x.nbytes) == x.view(np.uint8).reshape(1, -1)).all(1)
-        assert same.all(), f"{k}: {int((~same).sum())} of {same.size} copies differ"
-
-
 @pytest.mark.parametrize("N,budget,lam", [(100, 40, 0.5), (128, 128, 0.5), (129, 20, 0.5), (160, 64, 1.0), (192, 64, 0.0), (192, 64, 0.5), (256, 64, 2.0),
                                           (129, 100, 0.5), (144, 70, 1.0), (176, 96, 0.5), (193, 90, 0.5), (208, 128, 1.0), (224, 96, 1.0), (225, 65, 0.0),
                                           (240, 80, 0.5), (241, 96, 2.0), (256, 96, 1.0), (256, 128, 0.0), (256, 128, 0.5), (256, 128, 2.0)])
@@ -426,14 +443,14 @@ def test_an_event_has_the_same_bits_in_every_call(N, budget, lam, regular):
     ev = synth.make_c3(seed=N, B=2, L=1, H=3, N=N, budget=budget)
     if not regular:
         ev = in_pairs(ev, N)
-    few = run_fused(ev, lam=lam)
+    few = run_fused_once(ev, lam=lam)
     check_all(ev, few, lam)
     for times in beyond_one_and_three_per_sm(6):
-        same_bits(few, run_fused(tiled(ev, times), lam=lam))
+        same_bits(few, run_fused_once(tiled(ev, times), lam=lam))
     for n_cand in ([N, N // 2], [N - 17, N - 1]):
-        few = run_fused(ev, lam=lam, n_cand=n_cand)
+        few = run_fused_once(ev, lam=lam, n_cand=n_cand)
         for times in beyond_one_and_three_per_sm(6):
-            same_bits(few, run_fused(tiled(ev, times), lam=lam, n_cand=n_cand * times))
+            same_bits(few, run_fused_once(tiled(ev, times), lam=lam, n_cand=n_cand * times))
 
 
 @pytest.mark.parametrize("N,budget,lam", [(100, 40, 0.5), (192, 64, 0.5), (193, 90, 0.25), (256, 128, 0.5), (256, 128, 1.5)])
@@ -441,12 +458,25 @@ def test_an_event_has_the_same_bits_in_every_call(N, budget, lam, regular):
 def test_an_event_has_the_same_bits_in_every_call_with_a_shared_matrix(N, budget, lam, twice):
     ev = _duplicated_rows(N, lam, B=1, L=2, H=3, N=N // 2 * 2, budget=budget) if twice else synth.make_c3(seed=N, B=1, L=2, H=3, N=N, budget=budget)
 
-    def run(e):
-        K, V, pos = dev(e.K), dev(e.V), dev(e.pos)
+    def run(e, page=0):
+        K, V, pos, lay = dev(e.K), dev(e.V), dev(e.pos), None
         sig = akv.alpha_signature_flat(V)
         gram = akv.alpha_gram_shared(sig, akv.Layout.dense(V), akv.Options(sig_mode=akv.SIG_FLAT))
+        if page:
+            B, L, H, n, d = e.shape
+            pps = -(-n // page)
+            table = torch.randperm(B * pps, device="cuda").to(torch.int32).view(B, pps)
+            pools = torch.zeros((2, L, B * pps, H, page, d), dtype=torch.bfloat16, device="cuda")
+            for pool, x in zip(pools, (K, V)):
+                rows = torch.zeros((B, L, H, pps * page, d), dtype=torch.bfloat16, device="cuda")
+                rows[..., :n, :] = x
+                pool[:, table.long().flatten()] = rows.view(B, L, H, pps, page, d).permute(1, 0, 3, 2, 4, 5).reshape(L, B * pps, H, page, d)
+            K, V, lay = pools[0], pools[1], akv.Layout.paged(pools[0], table, n)
         sel = akv.alpha_compress_event(K, V, pos, dev(e.qstat), budget, akv.Options(lam=lam, sig_mode=akv.SIG_FLAT, shared_gram=gram), p_ref=dev(e.p_ref),
-                                       flat_sig=sig, want_scores=True)
+                                       flat_sig=sig, want_scores=True, layout=lay)
+        if page:
+            K, V = (x[:, table.long().flatten()].view(L, B, pps, H, page, d).permute(1, 0, 3, 2, 4, 5).reshape(B, L, H, pps * page, d)[..., :n, :].contiguous()
+                    for x in (K, V))
         return dict(K=akv.to_host_bits(K), V=akv.to_host_bits(V), pos=pos.cpu().numpy(), idx=sel.idx_sorted.cpu().numpy(), order=sel.pick_order.cpu().numpy(),
                     gain=sel.pick_gain.cpu().numpy(), scores=sel.scores.cpu().numpy(), n_kept=sel.n_kept.cpu().numpy(), status=sel.status.cpu().numpy())
 
@@ -454,15 +484,19 @@ def test_an_event_has_the_same_bits_in_every_call_with_a_shared_matrix(N, budget
     assert few["status"].max() == 0
     for times in beyond_one_and_three_per_sm(6):
         same_bits(few, run(tiled(ev, times)))
+        for page in (64, 8):
+            same_bits(few, run(tiled(ev, times), page))
 
 
-@pytest.mark.parametrize("page,N,budget", [(16, 256, 128), (16, 250, 64), (16, 241, 100), (8, 128, 40), (8, 130, 64), (8, 256, 128), (256, 131, 70)])
+@pytest.mark.parametrize("page,N,budget", [(16, 256, 128), (16, 250, 64), (16, 241, 100), (8, 128, 40), (8, 130, 64), (8, 256, 128), (256, 131, 70),
+                                           (16, 256, 96), (8, 256, 96), (64, 193, 71), (32, 225, 90), (16, 241, 65)])
 def test_pages_on_both_sides_of_those_whose_offsets_are_kept(page, N, budget):
     """Up to sixteen pages of an event have their offsets on chip: one less, as many and one more, in no order, for events with an
-    SM each and several to an SM; against the same rows in a dense cache, to the bit."""
+    SM each and several to an SM (four, budgets of at most 96: with late K rows from 193 rows on and V rows in registers from 71 kept ones
+    on); against the same rows in a dense cache, to the bit."""
     for B in (1, 40, 120):
         ev = synth.make_plain(B, 2, 2, N, 128, budget, 0.5, dtype=synth.BF16, seed=N + page)
-        plain = run_fused(ev)
+        plain = run_fused_once(ev)
         pps = -(-N // page)
         table = torch.randperm(B * pps, device="cuda").to(torch.int32).view(B, pps)
         pools = []
@@ -479,6 +513,27 @@ def test_pages_on_both_sides_of_those_whose_offsets_are_kept(page, N, budget):
         for pool, name in zip(pools, "KV"):
             rows = pool[:, table.long().flatten()].view(2, B, pps, 2, page, 128).permute(1, 0, 3, 2, 4, 5).reshape(B, 2, 2, pps * page, 128)
             assert np.array_equal(akv.to_host_bits(rows[..., :N, :].contiguous()), plain[name]), name
+
+
+@pytest.mark.parametrize("N,budget,lam", [(192, 64, 0.5), (193, 71, 0.5), (224, 96, 1.0), (256, 96, 0.5), (256, 128, 0.5), (256, 128, 0.0)])
+def test_rows_that_lie_apart_and_selection_alone_in_every_form(N, budget, lam):
+    """With an SM for each event, and with three and four of them to an SM: a cache whose rows are 136 elements apart, and alpha_select on scores
+    given, as in the fused call on contiguous rows, to the bit."""
+    ev = synth.make_c3(seed=N + budget, B=2, L=1, H=3, N=N, budget=budget)
+    few = run_fused_once(ev, lam=lam)
+    for times in (1,) + beyond_one_and_three_per_sm(6):
+        e = tiled(ev, times)
+        K, V = (torch.empty(e.shape[:-1] + (136,), dtype=torch.bfloat16, device="cuda")[..., :128].copy_(dev(x)) for x in (e.K, e.V))
+        pos, opts = dev(e.pos), akv.Options(lam=lam)
+        scores = dev(np.ascontiguousarray(np.tile(few["scores"], (times, 1, 1, 1))))
+        sel = akv.alpha_select(scores, V, budget, opts, layout=akv.Layout.dense(V))
+        same_bits({k: few[k] for k in ("idx", "order", "gain", "n_kept", "status")},
+                  dict(idx=sel.idx_sorted.cpu().numpy(), order=sel.pick_order.cpu().numpy(), gain=sel.pick_gain.cpu().numpy(),
+                       n_kept=sel.n_kept.cpu().numpy(), status=sel.status.cpu().numpy()))
+        sel = akv.alpha_compress_event(K, V, pos, dev(e.qstat), budget, opts, p_ref=dev(e.p_ref), layout=akv.Layout.dense(K), want_scores=True)
+        same_bits(few, dict(K=akv.to_host_bits(K.contiguous()), V=akv.to_host_bits(V.contiguous()), pos=pos.cpu().numpy(), idx=sel.idx_sorted.cpu().numpy(),
+                            order=sel.pick_order.cpu().numpy(), gain=sel.pick_gain.cpu().numpy(), scores=sel.scores.cpu().numpy(),
+                            n_kept=sel.n_kept.cpu().numpy(), status=sel.status.cpu().numpy()))
 
 
 @pytest.mark.parametrize("shift", [28, 29, 30])
@@ -605,12 +660,14 @@ def test_per_layer_signature_mode(dtype, N, d):
                                 sel.idx_sorted[b, l, h].cpu().numpy(), Kn[b, l, h], Vn[b, l, h], pn[b, l, h], sig=ref_sig)
 
 
-@pytest.mark.parametrize("maker", ["c3_192", "c2_256", "f32_96", "f32_600"])
+@pytest.mark.parametrize("maker", ["c3_192", "c3_256", "c2_256", "f32_96", "f32_600"])
 def test_per_head_budgets(maker):
     """A budget per (layer, head): every kernel family keeps budgets[l, h] rows per event, pads its index rows
     to the largest budget with -1 and reports the kept count; uniform budgets equal the scalar call."""
     if maker == "c3_192":
         ev = synth.make_c3(seed=41, B=2, L=3, H=2, N=192, budget=64)
+    elif maker == "c3_256":
+        ev = synth.make_c3(seed=45, B=2, L=3, H=2, N=256, budget=96)
     elif maker == "c2_256":
         ev = synth.make_c2(seed=42, B=2, L=3, H=2)
     elif maker == "f32_96":
@@ -851,6 +908,44 @@ def test_last_events_of_a_topk_call_in_a_launch_of_their_own(rest, N, budget):
         same()
 
 
+@pytest.mark.parametrize("rest", [1, 40])
+@pytest.mark.parametrize("kind", ["starved", "budgets", "pages"])
+def test_kinds_of_topk_call_whose_last_events_have_a_launch_of_their_own(kind, rest):
+    """Waits that run out (the second launch's CTAs leave early, and still only behind the first launch), a budget per head, pages in any
+    order: both launches look them up for their own events."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    E, base, N, budget, page = 2 * sms + rest, 7, 3072, 64, 64
+    assert akv_split.prefill_tail(E, N, sms, topk=True) == rest
+    ev = synth.make_plain(1, 1, base, N, 128, budget, 0.0, dtype=synth.BF16, seed=rest)
+    few = (np.arange(base, dtype=np.int32) * 9 + 5) % budget + 1
+    small = run_fused_once(ev, budgets=few[None] if kind == "budgets" else None)
+    which = torch.arange(E, device="cuda") % base
+    K, V, pos, q = (dev(x).index_select(dim, which) for x, dim in ((ev.K, 2), (ev.V, 2), (ev.pos, 2), (ev.qstat, 1)))
+    opts, lay = akv.Options(lam=0.0), None
+    if kind == "starved":
+        opts.flags = akv.FLAG_TEST_STARVE_WAIT
+    elif kind == "budgets":
+        opts.head_budgets = torch.from_numpy(few).cuda()[which][None].contiguous()
+    else:
+        table = torch.randperm(N // page, device="cuda").to(torch.int32)[None]
+        place = table.long().flatten().argsort()
+        K, V = (x.view(1, E, N // page, page, 128)[:, :, place].transpose(1, 2).contiguous() for x in (K, V))
+        lay = akv.Layout.paged(K, table, N)
+    K0, V0, pos0, before = K.clone(), V.clone(), pos.clone(), akv.launch_count()
+    sel = akv.alpha_compress_event(K, V, pos, q, budget, opts, p_ref=dev(ev.p_ref), layout=lay)
+    status, Kc, Vc = sel.status.clone(), K.clone(), V.clone()      # (the next things on the stream)
+    assert akv.launch_count() == before + 2
+    if kind == "starved":
+        assert bool((status == 3).all()) and torch.equal(Kc, K0) and torch.equal(Vc, V0) and torch.equal(pos, pos0)
+        return
+    if kind == "pages":
+        Kc, Vc = (x[:, table.long().flatten()].transpose(1, 2).reshape(1, 1, E, N, 128) for x in (Kc, Vc))
+    for got, want in ((Kc.view(torch.int16), small["K"].view(np.int16)), (Vc.view(torch.int16), small["V"].view(np.int16)), (pos, small["pos"]),
+                      (sel.pick_order, small["order"]), (sel.pick_gain, small["gain"]), (sel.idx_sorted, small["idx"]), (status, small["status"]),
+                      (sel.n_kept, small["n_kept"])):
+        assert torch.equal(got, torch.from_numpy(want).cuda().index_select(2, which))
+
+
 @pytest.mark.parametrize("L,H,N,lam", [(2, 2, 1100, 0.0), (2, 2, 1100, 0.5), (2, 19, 2048, 0.0), (2, 19, 2113, 0.5), (5, 15, 3072, 0.0), (5, 15, 2048, 0.5)])
 def test_shared_scoring_of_all_kinds_of_call(L, H, N, lam):
     """Four or two CTAs per event, with and without the penalty: budgets per head, a non-finite key in every CTA's part and pages in
@@ -903,7 +998,7 @@ def test_shared_scoring_of_all_kinds_of_call(L, H, N, lam):
     assert np.all(g["status"] == 1) and not set(bad) & set(g["idx"].ravel().tolist())
 
 
-@pytest.mark.parametrize("N,budget", [(129, 65), (130, 128), (160, 97), (161, 128), (224, 100), (255, 128), (256, 127)])
+@pytest.mark.parametrize("N,budget", [(129, 65), (130, 128), (160, 97), (161, 128), (193, 71), (224, 100), (225, 96), (255, 128), (256, 127)])
 @pytest.mark.parametrize("lam", [0.0, 0.5])
 def test_kept_slots_in_order_at_the_edges_of_words(N, budget, lam):
     """The 256-row kernel orders kept slots by bits in eight words: event sizes and budgets at and beside the words' edges."""
@@ -1171,17 +1266,19 @@ def _duplicated_rows(seed, lam, B=2, L=2, H=2, N=256, budget=128):
     return ev
 
 
-@pytest.mark.parametrize("lam", [2.0, 1.5])
-def test_active_set_bound_reached_and_the_loop_continues_over_the_whole_pool(lam):
-    """N = 256 -> b = 128 with duplicated V rows: the one-warp loop over the best-scored rows reaches its bound;
+@pytest.mark.parametrize("lam,budget,active", [(2.0, 128, 180), (1.5, 128, 180), (1.0, 96, 158)])
+def test_active_set_bound_reached_and_the_loop_continues_over_the_whole_pool(lam, budget, active):
+    """N = 256 with duplicated V rows: the one-warp loop over the best-scored rows reaches its bound;
     the picks made stand, the rest are taken over the whole pool. Every pick is checked against the oracle."""
-    ev = _duplicated_rows(33, lam)
+    ev = _duplicated_rows(33, lam, budget=budget)
+    if budget < 128:
+        ev.qstat *= 0.05         # (scores that differ by less than the penalty)
     g = run_fused(ev, lam=lam)
     log = check_all(ev, g, lam)
-    # the picks did go deep: some kept row's score rank lies beyond the 180 rows an active set holds at most
+    # the picks did go deep: some kept row's score rank lies beyond the rows an active set holds at most
     s = g["scores"][0, 0, 0]
     rank = np.argsort(np.argsort(-s))
-    assert rank[g["idx"][0, 0, 0]].max() >= 181
+    assert rank[g["idx"][0, 0, 0]].max() > active
     print("duplicated rows, lambda", lam, "near-tie divergences:", log)
 
 
@@ -1211,14 +1308,14 @@ def _close_scores(N, budget, lam, width, seed, B=2, L=1, H=2):
 
 @pytest.mark.parametrize("lam", [0.5, 1.0])
 @pytest.mark.parametrize("width", [0.0, 1e-3, 3e-3])
-@pytest.mark.parametrize("N,budget", [(192, 64), (128, 128), (256, 128), (300, 128), (1000, 64), (5120, 128)])
+@pytest.mark.parametrize("N,budget", [(192, 64), (128, 128), (256, 128), (256, 96), (300, 128), (1000, 64), (5120, 128)])
 def test_scores_close_together(N, budget, width, lam):
     """The best-scored rows that an active set holds are then told apart by the last bits of their scores, or by their slots."""
     ev = _close_scores(N, budget, lam, width, seed=N)
     check_all(ev, run_fused(ev), lam)
 
 
-@pytest.mark.parametrize("N,budget", [(192, 64), (256, 128), (1000, 128)])
+@pytest.mark.parametrize("N,budget", [(192, 64), (256, 128), (256, 96), (1000, 128)])
 def test_zero_cache_and_non_finite_scores(N, budget):
     """A zero-filled cache keeps its lowest slots; so does one whose scores are all NaN, with status 1."""
     ev = synth.make_plain(1, 2, 2, N, 128, budget, 0.5, dtype=synth.BF16, seed=N)
@@ -1235,7 +1332,7 @@ def test_zero_cache_and_non_finite_scores(N, budget):
 
 
 @pytest.mark.parametrize("lam", [0.0, 0.5])
-@pytest.mark.parametrize("N,budget", [(192, 64), (256, 128), (256, 140), (1000, 100), (1000, 140), (5200, 100)])
+@pytest.mark.parametrize("N,budget", [(192, 64), (256, 128), (250, 90), (256, 140), (1000, 100), (1000, 140), (5200, 100)])
 def test_a_few_non_finite_scores_on_the_tensor_memory_kernels(N, budget, lam):
     """Flagged and never preferred: with the rows of infinite and NaN scores out of the candidates the result is the same."""
     ev = synth.make_plain(1, 1, 2, N, 128, budget, lam, dtype=synth.BF16, seed=N + budget)
@@ -1253,7 +1350,7 @@ def test_a_few_non_finite_scores_on_the_tensor_memory_kernels(N, budget, lam):
     assert rep.ok, rep.log[:3]
 
 
-@pytest.mark.parametrize("dtype,N,budget", [(synth.BF16, 192, 64), (synth.BF16, 256, 128), (synth.BF16, 256, 140), (synth.BF16, 1000, 128),
+@pytest.mark.parametrize("dtype,N,budget", [(synth.BF16, 192, 64), (synth.BF16, 256, 128), (synth.BF16, 256, 96), (synth.BF16, 256, 140), (synth.BF16, 1000, 128),
                                             (synth.BF16, 1000, 140), (synth.F32, 128, 64), (synth.F32, 128, 128)])
 def test_zero_value_rows_with_eps_zero(dtype, N, budget):
     """eps = 0 and zero value rows: their reciprocal norm is infinite, their cosine counts as 0 (the oracle's with a tiny eps).
@@ -1303,29 +1400,36 @@ def test_active_set_bound_reached_with_a_shared_cosine_matrix():
 
 
 # ------------------------------------------------------------------ grouped-query statistics
-@pytest.mark.parametrize("N,budget,G", [(192, 64, 7), (256, 128, 4), (256, 140, 2), (700, 60, 8)])
+@pytest.mark.parametrize("N,budget,G", [(192, 64, 7), (256, 128, 4), (256, 96, 3), (256, 140, 2), (700, 60, 8)])
 def test_mean_of_grouped_statistics_on_the_tensor_memory_kernels(N, budget, G):
     """The mean over a KV head's query heads is the score of their mean statistic, so these calls take the kernels of
     ungrouped ones (one for each of the four shapes)."""
     ev = synth.make_plain(2, 2, 3, N, 128, budget, 0.5, dtype=synth.BF16, seed=N + G)
     Q = np.random.default_rng(G).standard_normal((2, 3 * G, 128)).astype(np.float32)
-    K, V, pos, pref = dev(ev.K), dev(ev.V), dev(ev.pos), dev(ev.p_ref)
-    sel = akv.alpha_compress_event(K, V, pos, dev(Q), budget, akv.Options(lam=0.5, gqa_group=G), p_ref=pref, want_scores=True)
-    torch.cuda.synchronize()
-    Kn, Vn, pn = akv.to_host_bits(K), akv.to_host_bits(V), pos.cpu().numpy()
+
+    def run(e):
+        K, V, pos = dev(e.K), dev(e.V), dev(e.pos)
+        sel = akv.alpha_compress_event(K, V, pos, dev(Q), budget, akv.Options(lam=0.5, gqa_group=G), p_ref=dev(e.p_ref), want_scores=True)
+        return dict(K=akv.to_host_bits(K), V=akv.to_host_bits(V), pos=pos.cpu().numpy(), scores=sel.scores.cpu().numpy(), order=sel.pick_order.cpu().numpy(),
+                    idx=sel.idx_sorted.cpu().numpy(), gain=sel.pick_gain.cpu().numpy())
+
+    g = run(ev)
+    if takes_forms(ev):
+        for times in beyond_one_and_three_per_sm(ev.n_events):
+            same_bits(g, run(tiled(ev, times)))
     for b in range(2):
         for l in range(2):
             for h in range(3):
                 q = Q[l, h * G:(h + 1) * G].astype(np.float64).mean(0)
                 chk.check_event(ev.K[b, l, h], ev.V[b, l, h], ev.pos[b, l, h], q, int(ev.p_ref[b]), budget, 0.5,
-                                sel.scores[b, l, h].cpu().numpy(), sel.pick_order[b, l, h].cpu().numpy(),
-                                sel.idx_sorted[b, l, h].cpu().numpy(), Kn[b, l, h], Vn[b, l, h], pn[b, l, h])
+                                g["scores"][b, l, h], g["order"][b, l, h], g["idx"][b, l, h], g["K"][b, l, h], g["V"][b, l, h], g["pos"][b, l, h])
 
 
-@pytest.mark.parametrize("N,budget", [(192, 64), (256, 128), (256, 140), (700, 60), (5200, 60)])
-def test_grouped_statistics_are_scored_with_fresh_rotations(N, budget):
+@pytest.mark.parametrize("B", [1, 40, 120])
+@pytest.mark.parametrize("N,budget", [(192, 64), (256, 128), (256, 96), (256, 140), (700, 60), (5200, 60)])
+def test_grouped_statistics_are_scored_with_fresh_rotations(N, budget, B):
     """The scores of grouped calls keep the general kernels' precision: no rotation is carried from row to row."""
-    ev = synth.make_plain(1, 2, 2, N, 128, budget, 0.5, dtype=synth.BF16, seed=N)
+    ev = synth.make_plain(B if N <= 256 else 1, 2, 2, N, 128, budget, 0.5, dtype=synth.BF16, seed=N)
     Q = np.random.default_rng(N).standard_normal((2, 2 * 4, 128)).astype(np.float32)
     s = []
     for flags in (0, akv.FLAG_NO_CHAIN):
