@@ -31,17 +31,15 @@ __device__ __forceinline__ void bulk_store_wait_read() {
 
 // FUSED: score + select + compact; otherwise selection only (scores are read from a.scores and
 // nothing is rewritten).
-// FORM (PoolShape): kPoolWideForm, eight warps for an event that has an SM to itself (a call of no more events than SMs). Alone on
-// its SM an event is a chain of phases that too few warps hide: of 256
-// rows to 128, 55.2 -> 49.0 thousand cycles (scores 12.5 -> 10.4, picks in pairs 24.7 -> 22.5, triangle 3.2 -> 2.6, compaction 5.1 -> 4.4);
-// 112 of them 34.7 -> 31.2 us, in pages 39.1 -> 36.5, top-k 22.6 -> 18.5. Not for what event_tri_kernel takes: alone, 112 events of 192 rows
-// to 64 gain 2 us of 27 (in pages 4 of 29), but that kernel has six events on an SM, and four streams with such a call each take 41 us there, 50 here
-// (in pages 43 and 80). kPoolThree, four warps and three events per SM; kPoolFour, four events
-// per SM: latency bounds a call of many events (34 % of the issue slots used), so what counts is how many an SM holds. For that the last
-// 64 K rows come late, the triangle has 158 rows and the last kept V rows wait in registers: 16 384 events of 256 rows to 128 in
-// pages 1598 -> 1479 us (launch_tri says which calls). PAGED: with the layout known to the compiler, and 16 to 40 registers
-// more that the residency allows, another 1479 -> 1426, 1792 events with a shared matrix (all of the call) 222 -> 198; but three events
-// per SM in pages 1598 -> 1703, so that those decide at run time.
+// FORM (PoolShape): kPoolWideForm, eight warps for a call of no more events than SMs. Alone on its SM an event is a chain of phases that
+// too few warps hide: of 256 rows to 128, 55.2 -> 49.0 thousand cycles (scores 12.5 -> 10.4, picks in pairs 24.7 -> 22.5, triangle 3.2 -> 2.6,
+// compaction 5.1 -> 4.4); 112 of them 35.1 -> 31.0 us, in pages 37.1 -> 33.0, top-k 20.7 -> 18.7. Not for what event_tri_kernel takes:
+// alone, 112 events of 192 rows to 64 gain 2 us of 27 (in pages 4 of 29), but that kernel has six events on an SM, and four streams with such
+// a call each take 41 us there, 50 here (in pages 43 and 80). kPoolThree, four warps and three events per SM. kPoolFour, four events per
+// SM: latency bounds a call of many events (34 % of the issue slots used), so what counts is how many an SM holds. For that the last K rows come
+// late, the triangle has 158 rows and the last kept V rows wait in registers: 2368 events of 256 rows to 96 191 -> 164 us, in pages
+// 198 -> 181 (launch_tri says which calls). PAGED: with the layout known to the compiler 1792 events with a shared matrix take 198 us (all of the
+// call) instead of 222. All forms score the rows in the same chains and have the same active set: an event has the same bits in each.
 template <bool FUSED, int FORM, bool PAGED>
 __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kCtas) event_pool_kernel(const __grid_constant__ EventArgs a, const __grid_constant__ ScoreTab tab) {
     using Shape = PoolShape<FORM>;
@@ -88,7 +86,9 @@ __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kC
     const bool similarity = a.greedy != 0 && picks > 1;   // (the first pick is the highest score in any case)
     const int np4 = (N + 3) & ~3;
     // row addressing: dense events are one base offset plus a row stride
-    const bool dense = PAGED && FORM == kPoolThree ? lay.page_size == 0 : !PAGED;   // (see above: three events per SM, in pages)
+    // (Three events per SM in pages look at the layout although it is known: with a constant here 16 384 events of 256 rows to 128 take
+    // 2007 us a pass instead of 1911. Not for its registers, 138 instead of 106: held to 122 or to 96 of them it takes 2023 and 2118.)
+    const bool dense = PAGED && FORM == kPoolThree ? lay.page_size == 0 : !PAGED;
     const long long ev_off = dense ? id.b * lay.sb + id.l * lay.sl + id.h * lay.sh : 0;
     // paged: where the event's pages start, looked up once by as many lanes of warp 0 at the same time (the block table's
     // entries come from L2; looked up row by row and copy by copy: 16 384 events of 256 rows to 128 in pages of 64 1631 us, 1600 so,
@@ -142,8 +142,8 @@ __global__ void __launch_bounds__(PoolShape<FORM>::kThreads, PoolShape<FORM>::kC
         }
     }
     if (FUSED && warp == 1) fill_sector_table(sect, lane);
-    // (this kernel claims half of the SM's columns: two of the three resident CTAs hold theirs at a time, the
-    // third waits in the allocation until one has moved its triangle out; claiming late instead measured 2 % slower)
+    // (this kernel claims half of the SM's columns: two of the CTAs on an SM hold theirs at a time, the others wait in the
+    // allocation until one has moved its triangle out; claiming late instead measured 2 % slower)
     const bool have_tmem = similarity && !G;
     if (!have_tmem && warp == 0) tmem_relinquish();  // this event takes no tensor memory
     if (have_tmem && warp == 0) tmem_alloc(smem_u32(tmem_holder), kPoolCols);

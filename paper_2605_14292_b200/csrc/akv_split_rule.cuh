@@ -42,7 +42,8 @@ inline int prefill_split(long long events, int N, int sms, bool topk, bool ragge
 }
 
 // How many of a call's events, the last ones, are left to a launch of their own: those beyond the full waves of two per SM, where
-// sharing their scoring shortens the call: where each of the CTAs that share has an SM, for candidates known to be many. It does for top-k, whose selection is short: with a penalty such an event is mostly
+// sharing their scoring shortens the call: at most half as many as SMs (two CTAs each from 66 of 148 SMs on, four below, so one or two on an SM), for
+// candidates known to be many. It does for top-k, whose selection is short: with a penalty such an event is mostly
 // selection, and the places that fall free early have it half done by the time that the last full wave ends. Measured, us per call in one
 // launch / two, 296 events and 8, 37, 65, 74 more, lambda 0: 2113 rows 83 / 87, 93 / 100, 85 / 93, 85 / 93, 3072 rows 102 / 97, 114 / 110,
 // 103 / 102, 104 / 102, 4096 rows 124 / 108, 138 / 126, 127 / 118, 127 / 118, 5000 rows 146 / 126, 160 / 147, 148 / 136, 148 / 134, 896 events
