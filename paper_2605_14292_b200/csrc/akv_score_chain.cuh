@@ -6,10 +6,11 @@
 namespace akv {
 
 // (cos, sin) of the angle 2 pi ph / 2^32: nearest of the 32 sector angles from the shared-memory table,
-// remainder by the short polynomials of score_lane8
+// remainder (in units of 2 pi / 2^37, to the last place: with 4.5716245e-11, 1.2e-6 off, a carried turn was off by up to 1.2e-7,
+// and scores by 3.1e-7 of their size, 2-norm over 2-norm, instead of 1.8e-7 at chains of eight) by the short polynomials of score_lane8
 __device__ __forceinline__ float2 phase_cos_sin(uint32_t ph, const float2* sect) {
     const float2 e = sect[(ph + 0x04000000u) >> 27];
-    const float w = (float)(int32_t)(ph << 5) * 4.5716245e-11f, z = w * w;
+    const float w = (float)(int32_t)(ph << 5) * 4.571619e-11f, z = w * w;
     const float sw = w * fmaf(z, fmaf(z, 8.3333333e-3f, -0.16666667f), 1.f);
     const float cw = fmaf(z, fmaf(z, 4.1666667e-2f, -0.5f), 1.f);
     return make_float2(e.x * cw - e.y * sw, e.y * cw + e.x * sw);
@@ -135,7 +136,8 @@ __device__ __forceinline__ void fill_statistic_tables(const EventArgs& a, int lh
 // rows), K streamed from global memory once, the next 64 rows requested before the present ones are scored. A lane group
 // scores two rows of every 64 side by side, rotations from the sector table. They are taken afresh for every row: carried on
 // over four rows they cost 7 us less of 137 (448 events of 1000 rows, score, selection and compaction), but the scores' error
-// rises from 1.2e-7 to 1.8e-7 (score_kernel, which took 44 us more: 1.4e-7).
+// rises by half (from 1.2e-7 to 1.8e-7 when that was measured, with the remainder's constant of then; 9.6e-8 as they are now, score_kernel,
+// which took 44 us more, 1.4e-7).
 // Dense and paged layouts are instantiations of their own (58.3 -> 57.7 us of those calls).
 // ---------------------------------------------------------------------------------------------
 constexpr int kScoreRows128 = 256;

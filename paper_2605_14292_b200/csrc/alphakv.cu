@@ -260,8 +260,8 @@ static void fill_score_args(EventArgs& a, const akv_options_t* opt) {
     a.gqa_group = opt->gqa_group < 1 ? 1 : opt->gqa_group;
     a.gqa_max = opt->gqa_reduce == 1 && a.gqa_group > 1;
     // Several statistics per KV head: every row's rotation afresh, as in the general kernels that take the group's maximum.
-    // Carried rotations are faster (2048 events of 192 rows, 64 kept: 94 us beside 132), but their scores are off by 4.6e-7 of
-    // their size instead of 1.2e-7 (the general kernel: 1.4e-7), and no caller of these asked for that.
+    // Carried rotations are faster (2048 events of 192 rows, 64 kept: 94 us beside 132), but their scores are off by 2.6e-7 of
+    // their size instead of 1.0e-7 (the general kernel: 1.4e-7), and no caller of these asked for that.
     if (a.gqa_group > 1) a.no_chain = 1;
 }
 

@@ -1160,6 +1160,19 @@ def test_chained_and_fresh_scores_agree_on_the_tensor_memory_kernels():
         check_all(ev, b, ev.lam)
 
 
+@pytest.mark.parametrize("N,budget,chain", [(128, 64, 8), (192, 64, 12), (256, 64, 16), (256, 128, 8), (256, 140, 8), (1000, 64, 8), (4096, 128, 8), (6000, 128, 8)])
+def test_error_of_carried_rotations(N, budget, chain):
+    """Scores of evenly spaced rows against float64, 2-norm over 2-norm. Fresh rotations leave 1.0e-7 (sums of 128 products of numbers that are
+    right to 2^-25). A step of a chain adds the turn's error, the same one at every step: its sine and cosine are rounded twice, to
+    2^-25 each, 4.3e-8 together. That is for rms of 0 .. chain - 1 steps. (With 2 pi / 2^37 off by 1.2e-6 a step added 8e-8.)"""
+    ev = synth.make_plain(2, 2, 4, N, 128, budget, 0.5, dtype=synth.BF16, seed=N + budget)
+    s = run_fused_once(ev)["scores"].astype(np.float64)
+    ref = np.stack([[[O.triattention_score(ev.K[b, l, h], ev.pos[b, l, h], ev.qstat[l, h], int(ev.p_ref[b])) for h in range(4)] for l in range(2)]
+                    for b in range(2)])
+    bound = np.hypot(1.05e-7, 4.3e-8 * np.sqrt(np.mean(np.arange(chain) ** 2.0)))
+    assert np.linalg.norm(s - ref) <= bound * np.linalg.norm(ref)
+
+
 # ------------------------------------------------------------------ shared signatures with one cosine matrix per sequence
 @pytest.mark.parametrize("L,H", [(1, 1), (1, 31), (4, 8), (3, 11), (9, 7), (1, 64), (5, 13)])
 @pytest.mark.parametrize("dtype", [synth.BF16, synth.F32])
