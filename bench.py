@@ -53,18 +53,16 @@ KERNELS = {"C1": "event_resident_kernel<float>", "C2": "event_pool_kernel<fused>
 # keyed by workload, each with the source revision of csrc/ it was taken at (see kernel_revision()); a
 # capture of another revision is reported as null.
 NCU_TRAFFIC = {
-    # one launch of 4096 events captured whole (profiles/event_tri_kernel_bf16_C3.md)
-    "C3": {"bytes": 321387776 + 98283264, "revision": "829da00380ff"},
+    # one launch of 4096 events captured whole
+    "C3": {"bytes": 321056256 + 97517824, "revision": "1b951c4aec5e"},
     # one launch of 4096 events (16 sequences) captured; a step is 4 x 32 launches of that size
-    # (profiles/event_pool_kernel_bf16_C5.md)
-    "C5": {"bytes": (487347968 + 230005760) * 128, "revision": "829da00380ff"},
+    "C5": {"bytes": (488305152 + 229420288) * 128, "revision": "1b951c4aec5e"},
     # the same kernel and capture, scaled to 112 events
-    "C2": {"bytes": (487347968 + 230005760) * 112 // 4096, "revision": "829da00380ff"},
+    "C2": {"bytes": (488305152 + 229420288) * 112 // 4096, "revision": "1b951c4aec5e"},
     # the three launches (lambda 0, 0.5, 1) of a 2-sequence batch captured; the bench batch has 8 sequences
-    # (profiles/event_prefill_kernel_bf16_C4.md)
-    "C4": {"bytes": ((251938304 + 6620672) + (256058880 + 3280896) + (262373632 + 3437312)) * 4, "revision": "829da00380ff"},
-    # the step's three launches captured whole (profiles/gram_shared_kernel_f32_C6.md)
-    "C6": {"bytes": (117466624 + 3970560) + 2136320 + (182253312 + 69398784), "revision": "829da00380ff"},
+    "C4": {"bytes": ((251891456 + 4220160) + (256020224 + 3539968) + (262290944 + 3697408)) * 4, "revision": "1b951c4aec5e"},
+    # the step's three launches captured whole
+    "C6": {"bytes": (117468160 + 3197696) + 2136576 + (182097152 + 68966912), "revision": "1b951c4aec5e"},
 }
 
 
