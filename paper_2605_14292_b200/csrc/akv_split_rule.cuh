@@ -42,9 +42,9 @@ inline int prefill_split(long long events, int N, int sms, bool topk, bool ragge
 }
 
 // How many of a call's events, the last ones, are left to a launch of their own: those beyond the full waves of two per SM, where
-// sharing their scoring shortens the call: at most half as many as SMs (two CTAs each from 66 of 148 SMs on, four below, so one or two on an SM), for
-// candidates known to be many. It does for top-k, whose selection is short: with a penalty such an event is mostly
-// selection, and the places that fall free early have it half done by the time that the last full wave ends. Measured, us per call in one
+// sharing their scoring shortens the call, at most half as many as SMs, for candidates known to be many. It does for top-k, whose selection is
+// short: with a penalty such an event is mostly selection, and the places that fall free early have it half done by the time that the last full
+// wave ends. Measured, us per call in one
 // launch / two, 296 events and 8, 37, 65, 74 more, lambda 0: 2113 rows 83 / 87, 93 / 100, 85 / 93, 85 / 93, 3072 rows 102 / 97, 114 / 110,
 // 103 / 102, 104 / 102, 4096 rows 124 / 108, 138 / 126, 127 / 118, 127 / 118, 5000 rows 146 / 126, 160 / 147, 148 / 136, 148 / 134, 896 events
 // of 4096 rows 260 / 243; lambda 0.5: 304 events of 1100 rows 114 / 139, of 4096 179 / 181, 896 of 4096 359 / 372.
@@ -53,5 +53,9 @@ inline long long prefill_tail(long long events, int N, int sms, bool topk, bool 
     if (!topk || ragged || events < places || rest * 2 > sms || (N + kSplitStageRows - 1) / kSplitStageRows < 48) return 0;
     return prefill_split(rest, N, sms, topk, ragged) > 1 ? rest : 0;
 }
+// How many CTAs share such an event: four or two, as long as each has an SM. (Four each up to 65 events, as in a call of their own, take no less,
+// and in two and three streams with such a call each 296 + 64 events of 3072 rows 195 and 282 us instead of 174 and 264, of 4096 223 and 320 instead of
+// 209 and 311; in one launch 166 and 247, 202 and 302.)
+inline int prefill_tail_split(long long tail, int sms) { return tail * 4 <= sms ? 4 : 2; }
 
 }  // namespace akv

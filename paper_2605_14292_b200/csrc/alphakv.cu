@@ -438,7 +438,7 @@ static akv_status_t launch_prefill(akv_handle* h, const EventArgs& a, cudaStream
         if (tail) {
             EventArgs b = a;
             b.first_event = (int)(E - tail);
-            const bool four = prefill_split(tail, a.lay.N, h->sm_count, !a.greedy, a.n_cand != nullptr) == 4;
+            const bool four = prefill_tail_split(tail, h->sm_count) == 4;
             auto second = [&](bool check) { return four ? launch_prefill_split<true, 4, true>(h, b, tail, st, check) : launch_prefill_split<true, 2, true>(h, b, tail, st, check); };
             akv_status_t s = second(true);   // (what can be refused is, before the first launch)
             if (s == AKV_OK) s = launch_prefill_split<true, 1, true>(h, a, E - tail, st, dry);

@@ -9,6 +9,7 @@ HOST = r"""
 #include "akv_split_rule.cuh"
 extern "C" int rule(long long events, int N, int sms, int topk, int ragged) { return akv::prefill_split(events, N, sms, topk, ragged); }
 extern "C" long long tail(long long events, int N, int sms, int topk, int ragged) { return akv::prefill_tail(events, N, sms, topk, ragged); }
+extern "C" int tail_split(long long tail, int sms) { return akv::prefill_tail_split(tail, sms); }
 extern "C" int share(int stages, int split) { return akv::split_share(stages, split); }
 """
 _lib = None
@@ -25,6 +26,7 @@ def _load():
             _lib = C.CDLL(so)
         _lib.rule.argtypes = _lib.tail.argtypes = [C.c_longlong, C.c_int, C.c_int, C.c_int, C.c_int]
         _lib.tail.restype = C.c_longlong
+        _lib.tail_split.argtypes = [C.c_longlong, C.c_int]
     return _lib
 
 
@@ -34,6 +36,10 @@ def prefill_split(events, N, sms=148, topk=False, ragged=False):
 
 def prefill_tail(events, N, sms=148, topk=False, ragged=False):
     return _load().tail(events, N, sms, topk, ragged)
+
+
+def prefill_tail_split(tail, sms=148):
+    return _load().tail_split(tail, sms)
 
 
 def split_share(stages, split):

@@ -2,7 +2,7 @@
 calls that were measured slower for it."""
 import pytest
 
-from akv_split import prefill_split, prefill_tail, split_share
+from akv_split import prefill_split, prefill_tail, prefill_tail_split, split_share
 
 
 @pytest.mark.parametrize("sms", [148, 132, 80])
@@ -42,3 +42,13 @@ def test_events_left_to_a_second_launch(events, N, topk, ragged, tail):
     assert prefill_tail(events, N, 148, topk, ragged) == tail
     if tail:
         assert prefill_split(tail, N, 148, topk, ragged) > 1
+
+
+@pytest.mark.parametrize("sms", [148, 132, 80])
+def test_ctas_that_share_a_last_event_have_an_sm_each(sms):
+    for rest in range(1, 2 * sms):
+        tail = prefill_tail(2 * sms + rest, 4096, sms, topk=True)
+        if tail:
+            split = prefill_tail_split(tail, sms)
+            assert tail == rest and split in (2, 4) and tail * split <= sms
+            assert split == 4 or tail * 4 > sms
