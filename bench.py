@@ -54,15 +54,15 @@ KERNELS = {"C1": "event_resident_kernel<float>", "C2": "event_pool_kernel<fused>
 # capture of another revision is reported as null.
 NCU_TRAFFIC = {
     # one launch of 4096 events captured whole
-    "C3": {"bytes": 321056256 + 97517824, "revision": "1b951c4aec5e"},
+    "C3": {"bytes": 321202176 + 97834752, "revision": "5f8cc4f93547"},
     # one launch of 4096 events (16 sequences) captured; a step is 4 x 32 launches of that size
-    "C5": {"bytes": (488305152 + 229420288) * 128, "revision": "1b951c4aec5e"},
+    "C5": {"bytes": (489884160 + 229008640) * 128, "revision": "5f8cc4f93547"},
     # the same kernel and capture, scaled to 112 events
-    "C2": {"bytes": (488305152 + 229420288) * 112 // 4096, "revision": "1b951c4aec5e"},
+    "C2": {"bytes": (489884160 + 229008640) * 112 // 4096, "revision": "5f8cc4f93547"},
     # the three launches (lambda 0, 0.5, 1) of a 2-sequence batch captured; the bench batch has 8 sequences
-    "C4": {"bytes": ((251891456 + 4220160) + (256020224 + 3539968) + (262290944 + 3697408)) * 4, "revision": "1b951c4aec5e"},
+    "C4": {"bytes": ((251972608 + 3480064) + (256064256 + 3631104) + (262408704 + 3111680)) * 4, "revision": "5f8cc4f93547"},
     # the step's three launches captured whole
-    "C6": {"bytes": (117468160 + 3197696) + 2136576 + (182097152 + 68966912), "revision": "1b951c4aec5e"},
+    "C6": {"bytes": (117468928 + 3780352) + 2137088 + (182178304 + 69079040), "revision": "5f8cc4f93547"},
 }
 
 
